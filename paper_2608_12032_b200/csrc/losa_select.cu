@@ -1,16 +1,12 @@
 // losa_select: retained-mass selection (Eq. 3) and CSR validation.
 //
-// Three small launches over a [rows, nKb] fp32 mass matrix:
-//   1. select_rows_warp_kernel  rows of at most 1024 blocks: one warp per row, the row in
-//                           registers, the threshold value found bit by bit with masked
-//                           fixed-point sums (no sort); the kept set is written as a bitmap
+// Two launches over a [rows, nKb] fp32 mass matrix:
+//   1. select_rows_kernel   one warp per row of at most 1024 blocks, two, four or eight warps for
+//                           longer rows; the row stays in registers, the threshold value is found
+//                           with one histogram pass (no sort); the kept set is written as a bitmap
 //                           over block indices plus its size.
-//      select_rows_kernel   longer rows: one CTA per
-//                           row, sort (mass descending, index ascending) as 64-bit integer
-//                           keys in shared memory, fp64 prefix sum along the sorted order,
-//                           shortest prefix reaching tau; same outputs.
-//   2. scan_counts_kernel   exclusive prefix of the per-row sizes -> offsets.
-//   3. expand_rows_kernel   one warp per row: bitmap -> ascending block indices.
+//   2. expand_rows_kernel   every CTA adds up the sizes of the rows before its own (offsets) and
+//                           turns its rows' bitmaps into ascending block indices.
 // Each mass element is read once and each kept index written once; the bitmap adds 1/16
 // of the mass bytes.  The result is deterministic (no floating-point atomics).
 #include <limits.h>
@@ -20,288 +16,400 @@
 namespace losa {
 namespace {
 
-constexpr int kSelThreads = 256;
-constexpr unsigned long long kPadKey = ~0ull;
+// The kept set of Eq. 3 is "every block heavier than v*, plus the lowest-indexed blocks equal to v*
+// until the sum reaches tau", where v* is the largest value v with sum(mass >= v) >= tau.
+// Non-negative floats order like their bit patterns, so the row is split into bins by the leading
+// bits: the exponent and four mantissa bits.  All values of a bin share their exponent, so a bin's
+// sum is exact in two 32-bit integers - how many values, and the sum of their 19 low mantissa bits
+// (8192 of them stay below 2^32) - which the warps gather with shared-memory integer atomics.  A
+// scan over the bins from the heaviest down, in 2^-60 fixed point, gives the bin of v*; its few
+// values are put into a list, and v* is found among them bit by bit.  Integer addition is exact and
+// order-independent, so the result is deterministic and differs from a sequential fp64 sum by less
+// than 1e-14 (masses below 2^-37 lose low bits).
+//
+// The bins end at the mass limit 8 and begin kBins * 2^(1/16) steps below it (about 2^-35): lighter
+// values share bin 0.  A threshold in bin 0, or a bin with more values than the list holds, is
+// searched bit by bit over the registers instead (31 or 19 masked sums over the row).  The
+// fixed-ratio rule only counts: its bins take one mantissa bit and reach down to zero.
+//
+// What bounds it: instructions per value.  The search bit by bit over the whole row that short rows
+// used before took 31 masked 64-bit sums, and the sort in shared memory that longer rows used moved
+// every value about 70 times: 22296 rows of 3713 blocks took 5.48 ms, of 929 blocks 0.33 ms.
+constexpr int kBins = 608;   // per lane of one warp 19, an odd number: the scan has no bank conflicts
+constexpr int kTauShift = 19, kCountShift = 22;
+constexpr int kTopBin = 0x41000000 >> kTauShift;  // of the largest mass, 8.0
+constexpr int kListCap = 256;
+constexpr double kFixedOne = 1152921504606846976.0;  // 2^60
 
-__device__ __forceinline__ double key_mass(unsigned long long key) {
-  return (double)__uint_as_float(~(uint32_t)(key >> 32));
+struct RowShared {
+  uint32_t cnt[kBins], low[kBins];
+  uint32_t list[kListCap];
+  unsigned long long total[8];   // per warp of the row
+  unsigned long long above;      // weight of the bins heavier than the one of v*
+  double sum[8];
+  int bin, cnt_above, list_len;
+  uint32_t v;
+  int need, s, eq_total;
+  int eq[8];
+};
+
+// (cap: see `tiny` below)
+__device__ __forceinline__ unsigned long long fixed_weight(uint32_t bits, double scale, double cap) {
+  return (unsigned long long)(fmin((double)__uint_as_float(bits), cap) * scale);
 }
 
-__global__ void __launch_bounds__(kSelThreads)
-select_rows_kernel(const float* __restrict__ mass, int nKb, int n2, double tau, int fixed_count,
-                   int32_t* __restrict__ counts, uint32_t* __restrict__ bitmaps, int* status) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  unsigned long long* keys = reinterpret_cast<unsigned long long*>(smem_raw);
-  uint32_t* bitmap = reinterpret_cast<uint32_t*>(keys + n2);
-  __shared__ double warp_total[kSelThreads / 32];
-  __shared__ int first_pos;
-  __shared__ double row_total;
+// warp sum of 64-bit values as three integer reductions of 22-bit limbs (one instruction each)
+__device__ __forceinline__ unsigned long long warp_sum_u64(unsigned long long a) {
+  const unsigned r0 = __reduce_add_sync(0xffffffffu, (unsigned)(a & 0x3fffffull));
+  const unsigned r1 = __reduce_add_sync(0xffffffffu, (unsigned)((a >> 22) & 0x3fffffull));
+  const unsigned r2 = __reduce_add_sync(0xffffffffu, (unsigned)(a >> 44));
+  return (unsigned long long)r0 + ((unsigned long long)r1 << 22) + ((unsigned long long)r2 << 44);
+}
 
-  const int tid = threadIdx.x;
-  const int64_t row = blockIdx.x;
-  const int words = (nKb + 31) >> 5;
-  const float* mrow = mass + row * nKb;
+template <int W>  // warps per row
+__device__ __forceinline__ void row_sync() {
+  if (W == 1) __syncwarp();
+  else __syncthreads();  // (the row has the CTA to itself)
+}
 
-  bool bad = false;
-  for (int i = tid; i < n2; i += kSelThreads) {
-    unsigned long long key = kPadKey;
-    if (i < nKb) {
-      float m = mrow[i];
-      if (!(m >= 0.0f) || m > 8.0f) {  // negative, NaN, or far beyond any mass
-        bad = true;
-        m = 0.0f;
-      }
-      // mass >= 0, so its IEEE bits order like the value; -0 becomes +0
-      const uint32_t bits = (m == 0.0f) ? 0u : __float_as_uint(m);
-      key = ((unsigned long long)(~bits) << 32) | (uint32_t)i;
-    }
-    keys[i] = key;
-  }
-  for (int w = tid; w < words; w += kSelThreads) bitmap[w] = 0u;
-  if (tid == 0) first_pos = INT_MAX;
-  if (bad) report_error(status, LOSA_ERR_BAD_MASS);
+// sum over the row's threads (W > 1: through shared memory; every thread gets the result)
+template <int W>
+__device__ __forceinline__ unsigned long long row_sum_u64(unsigned long long a, RowShared* rs, int warp, int lane) {
+  a = warp_sum_u64(a);
+  if (W == 1) return a;
+  if (lane == 0) rs->total[warp] = a;
   __syncthreads();
-
-  // bitonic sort, ascending keys = descending mass, ties by ascending block index; every thread
-  // owns compare-exchange pairs (i, i | j), so no thread idles
-  for (int k = 2; k <= n2; k <<= 1) {
-    for (int j = k >> 1; j > 0; j >>= 1) {
-      for (int pr = tid; pr < (n2 >> 1); pr += kSelThreads) {
-        const int i = ((pr & ~(j - 1)) << 1) | (pr & (j - 1));
-        const int ixj = i | j;
-        const unsigned long long a = keys[i], b = keys[ixj];
-        const bool up = ((i & k) == 0);
-        if ((a > b) == up) {
-          keys[i] = b;
-          keys[ixj] = a;
-        }
-      }
-      __syncthreads();
-    }
-  }
-
-  // fp64 prefix sum along the sorted order: per-thread chunk, then a block scan of chunk sums
-  const int chunk = (n2 + kSelThreads - 1) / kSelThreads;
-  const int lo = min(tid * chunk, n2), hi = min(lo + chunk, n2);
-  double local = 0.0;
-  for (int i = lo; i < hi; ++i) local += key_mass(keys[i]);
-  double incl = local;
-  const int lane = tid & 31, warp = tid >> 5;
+  unsigned long long t = 0ull;
 #pragma unroll
-  for (int d = 1; d < 32; d <<= 1) {
-    const double up = __shfl_up_sync(0xffffffffu, incl, d);
-    if (lane >= d) incl += up;
-  }
-  if (lane == 31) warp_total[warp] = incl;
+  for (int w = 0; w < W; ++w) t += rs->total[w];
   __syncthreads();
-  double base = 0.0;
-  for (int w = 0; w < warp; ++w) base += warp_total[w];
-  double acc = base + (incl - local);
-  for (int i = lo; i < hi; ++i) {
-    acc += key_mass(keys[i]);
-    if (acc >= tau) {
-      atomicMin(&first_pos, i + 1);
-      break;
-    }
-  }
-  if (tid == kSelThreads - 1) row_total = base + incl;
-  __syncthreads();
-  int s = first_pos;
-  if (tau >= 1.0 || s > nKb) s = nKb;
-  // same rule as the warp-per-row kernel: a row whose masses add up to more than 8 is reported and
-  // keeps every block
-  if (row_total > 8.0) {
-    s = nKb;
-    if (tid == 0) report_error(status, LOSA_ERR_BAD_MASS);
-  }
-  if (fixed_count > 0) s = min(fixed_count, nKb);  // fixed-ratio rule: the k heaviest blocks
-
-  for (int i = lo; i < hi; ++i) {
-    if (i < s) {
-      const uint32_t idx = (uint32_t)keys[i];
-      atomicOr(&bitmap[idx >> 5], 1u << (idx & 31));
-    }
-  }
-  __syncthreads();
-  for (int w = tid; w < words; w += kSelThreads) bitmaps[row * words + w] = bitmap[w];
-  if (tid == 0) counts[row] = s;
+  return t;
 }
 
-// Rows of at most 1024 blocks: one WARP per row, no sort.  The kept set of Eq. 3 is "every block
-// heavier than v*, plus the lowest-indexed blocks equal to v* until the sum reaches tau", where v*
-// is the largest value v with sum(mass >= v) >= tau.  Non-negative floats order like their bit
-// patterns, so v* is found bit by bit (31 steps), each step one masked sum over the row, which
-// the warp holds in registers (lane l owns blocks l, l + 32, ...).  The sums are taken in 2^-60
-// fixed point: integer addition is exact and order-independent, so the result is deterministic
-// and differs from a sequential fp64 sum by less than 1e-15 (masses below 2^-37 lose low bits).
-// The kept set comes out as one ballot per 32 blocks - the bitmap word - and its size.
-template <int K>  // blocks per lane
-__global__ void __launch_bounds__(128)
-select_rows_warp_kernel(const float* __restrict__ mass, int rows, int nKb, double tau, int fixed_count,
-                        int32_t* __restrict__ counts, uint32_t* __restrict__ bitmaps, int* status) {
+// W warps per row, K blocks per lane: warp w of the row owns blocks [w * 32 K, (w + 1) * 32 K), its
+// lane l the blocks l, l + 32, ... of those, so that a ballot is a bitmap word.  One row per CTA, or
+// four at W = 1.
+template <int W, int K>
+__global__ void __launch_bounds__(W == 1 ? 128 : 32 * W)
+select_rows_kernel(const float* __restrict__ mass, int rows, int nKb, double tau, int fixed_count,
+                   int32_t* __restrict__ counts, uint32_t* __restrict__ bitmaps, int* status) {
+  constexpr int kRowsPerCta = (W == 1) ? 4 : 1;
+  constexpr int T = 32 * W;
+  __shared__ RowShared shared[kRowsPerCta];
   const int lane = threadIdx.x & 31;
-  const int64_t row = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  const int warp = (W == 1) ? 0 : threadIdx.x >> 5;     // of the row
+  const int t = warp * 32 + lane;                       // thread of the row
+  RowShared* const rs = &shared[(W == 1) ? threadIdx.x >> 5 : 0];
+  const int64_t row = (int64_t)blockIdx.x * kRowsPerCta + ((W == 1) ? threadIdx.x >> 5 : 0);
   if (row >= rows) return;
   const int words = (nKb + 31) >> 5;
   const float* mrow = mass + row * nKb;
+  const int first = warp * 32 * K + lane;
+  const bool counting = fixed_count > 0;
+  const int shift = counting ? kCountShift : kTauShift;
+  const int base = counting ? 0 : kTopBin - (kBins - 1);
+
   uint32_t bits[K];
-  unsigned long long fx[K];
-  bool bad = false;
-  float row_sum = 0.0f;
 #pragma unroll
   for (int k = 0; k < K; ++k) {
-    const int i = k * 32 + lane;
-    float m = (i < nKb) ? mrow[i] : 0.0f;
+    const int i = first + k * 32;
+    bits[k] = (i < nKb) ? __float_as_uint(__ldg(mrow + i)) : 0u;
+  }
+  for (int i = t; i < kBins; i += T) {
+    rs->cnt[i] = 0u;
+    rs->low[i] = 0u;
+  }
+  if (t == 0) {
+    rs->list_len = 0;
+    rs->bin = -1;
+  }
+  row_sync<W>();
+  bool bad = false;
+  float sum = 0.0f;
+  const uint32_t low_mask = (1u << shift) - 1u;
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    const float m = __uint_as_float(bits[k]);
     if (!(m >= 0.0f) || m > 8.0f) {  // negative, NaN, or far beyond any mass
       bad = true;
-      m = 0.0f;
+      bits[k] = 0u;
     }
-    bits[k] = (m == 0.0f) ? 0u : __float_as_uint(m);  // -0 becomes +0
-    // the weight that is summed: the mass in 2^-60 fixed point (exact product), or 1 per existing
-    // block for the fixed-ratio rule, which counts; blocks past the row's end weigh nothing
-    if (fixed_count > 0) fx[k] = (i < nKb) ? 1ull : 0ull;
-    else fx[k] = (unsigned long long)((double)m * 1152921504606846976.0);
-    row_sum += m;
+    if (bits[k] == 0x80000000u) bits[k] = 0u;  // -0 becomes +0
+    sum += __uint_as_float(bits[k]);
+    if (first + k * 32 < nKb) {
+      const int bin = max((int)(bits[k] >> shift) - base, 0);
+      atomicAdd(&rs->cnt[bin], 1u);
+      if (!counting) atomicAdd(&rs->low[bin], bits[k] & low_mask);
+    }
   }
-  // The fixed-point sums below hold at most 16: a row whose masses add up to more than 8 (a mass
-  // row sums to 1) is reported, and keeps every block, instead of wrapping silently.
+  // The fixed-point sums hold at most 16: a row whose masses add up to more than 8 (a mass row sums
+  // to 1) is reported, and keeps every block, instead of wrapping silently.
+  double row_sum = (double)sum;
 #pragma unroll
   for (int d = 16; d > 0; d >>= 1) row_sum += __shfl_xor_sync(0xffffffffu, row_sum, d);
-  if (fixed_count <= 0 && row_sum > 8.0f) {
-    bad = true;
+  if (W > 1 && lane == 0) rs->sum[warp] = row_sum;
+  row_sync<W>();
+  if (W > 1) {
+    row_sum = 0.0;
 #pragma unroll
-    for (int k = 0; k < K; ++k) fx[k] = 0ull;
+    for (int w = 0; w < W; ++w) row_sum += rs->sum[w];
   }
-  if (__any_sync(0xffffffffu, bad) && lane == 0) report_error(status, LOSA_ERR_BAD_MASS);
+  const bool too_heavy = row_sum > 8.0;
+  if (bad || (t == 0 && too_heavy && (!counting || W > 1))) report_error(status, LOSA_ERR_BAD_MASS);
 
-  // sum (or count, for the fixed-ratio rule) of the blocks with bits >= v, over the whole row
-  auto measure_ge = [&](uint32_t v) -> unsigned long long {
-    unsigned long long a0 = 0ull, a1 = 0ull;
-#pragma unroll
-    for (int k = 0; k < K; k += 2) {
-      a0 += (bits[k] >= v) ? fx[k] : 0ull;
-      a1 += (bits[k + 1] >= v) ? fx[k + 1] : 0ull;
-    }
-    const unsigned long long a = a0 + a1;
-    // warp sum of 64-bit values as three integer reductions of 22-bit limbs (one instruction each)
-    const unsigned r0 = __reduce_add_sync(0xffffffffu, (unsigned)(a & 0x3fffffull));
-    const unsigned r1 = __reduce_add_sync(0xffffffffu, (unsigned)((a >> 22) & 0x3fffffull));
-    const unsigned r2 = __reduce_add_sync(0xffffffffu, (unsigned)(a >> 44));
-    return (unsigned long long)r0 + ((unsigned long long)r1 << 22) + ((unsigned long long)r2 << 44);
-  };
-
-  const unsigned long long target =
-      (fixed_count > 0) ? (unsigned long long)min(fixed_count, nKb)
-                        : (unsigned long long)(fmin(tau, 1.0) * 1152921504606846976.0);
-  int s = nKb, need = 0;
-  uint32_t v = 0u;  // kept: bits > v, and the first `need` (by index) with bits == v
-  const bool all = (fixed_count <= 0 && tau >= 1.0) || measure_ge(0u) < target;  // never reaches tau
+  // A tau far below any useful threshold would be lost in units of 2^-60: its rows are searched over
+  // the registers in units of about 2^-50 tau, with every weight cut off at tau (a block of that mass
+  // reaches the threshold alone), so that sums still fit.  (Every positive float is above 2^-200.)
+  const bool tiny = !counting && tau < 0x1p-20;
+  double scale = kFixedOne, cap = 8.0;
+  if (tiny) {
+    cap = fmax(tau, 0x1p-200);
+    scale = __hiloint2double((1023 + 49 - (((__double2hiint(cap) >> 20) & 0x7ff) - 1023)) << 20, 0);
+  }
+  const unsigned long long target = counting ? (unsigned long long)min(fixed_count, nKb)
+                                             : (unsigned long long)(fmin(tiny ? cap : tau, 1.0) * scale);
+  bool all = !counting && (tau >= 1.0 || too_heavy);  // (too heavy: keeps every block)
+  uint32_t v = 0u;   // kept: bits > v, and the first `need` (by index) with bits == v
+  int need = 0, s = nKb, eq_total = 0;
   if (!all) {
-    for (int b = 30; b >= 0; --b) {
-      const uint32_t cand = v | (1u << b);
-      if (measure_ge(cand) >= target) v = cand;
-    }
-    unsigned long long gt = 0ull;
-    int n_gt = 0, n_eq = 0;
+    // ---- the bin of v*: thread t owns bins [hi - kPer + 1, hi], heaviest bins first
+    constexpr int kPer = (kBins + T - 1) / T;
+    const int hi = kBins - 1 - t * kPer;
+    auto bin_weight = [&](int b) -> unsigned long long {
+      const uint32_t c = rs->cnt[b];
+      if (counting) return c;
+      if (c == 0u || b == 0) return 0ull;
+      const uint32_t lead = (uint32_t)(b + base);  // exponent and four mantissa bits
+      const unsigned long long mant = (unsigned long long)c * ((16u | (lead & 15u)) << kTauShift) + rs->low[b];
+      return mant << ((lead >> 4) - 90u);  // the mantissa's unit is 2^(e - 150); e >= 92 here
+    };
+    unsigned long long mine = 0ull;
+    for (int b = hi; b > hi - kPer && b >= 0; --b) mine += bin_weight(b);
+    unsigned long long incl = mine;
 #pragma unroll
-    for (int k = 0; k < K; ++k) {
-      const bool valid = (k * 32 + lane) < nKb;
-      if (valid && bits[k] > v) {
-        gt += fx[k];
-        ++n_gt;
+    for (int d = 1; d < 32; d <<= 1) {
+      const unsigned long long up = __shfl_up_sync(0xffffffffu, incl, d);
+      if (lane >= d) incl += up;
+    }
+    if (W > 1) {
+      if (lane == 31) rs->total[warp] = incl;
+      __syncthreads();
+#pragma unroll
+      for (int w = 0; w < W; ++w)
+        if (w < warp) incl += rs->total[w];
+    }
+    unsigned long long acc = incl - mine;
+    if (acc < target && incl >= target) {  // exactly one thread, or none
+      for (int b = hi; b > hi - kPer && b >= 0; --b) {
+        const unsigned long long w = bin_weight(b);
+        if (acc + w >= target) {
+          rs->bin = b;
+          rs->above = acc;
+          break;
+        }
+        acc += w;
       }
-      if (valid && bits[k] == v) ++n_eq;
     }
+    row_sync<W>();
+    const int bin = tiny ? -1 : rs->bin;
+    const uint32_t lead = (uint32_t)(bin + base);
+    // ---- v* within the bin
+    bool listed = false;
+    if (bin >= 0) {
+      const uint32_t m = rs->cnt[bin];
+      listed = m <= (uint32_t)kListCap;
+      if (listed) {
 #pragma unroll
-    for (int d = 16; d > 0; d >>= 1) {
-      gt += __shfl_xor_sync(0xffffffffu, gt, d);
-      n_gt += __shfl_xor_sync(0xffffffffu, n_gt, d);
-      n_eq += __shfl_xor_sync(0xffffffffu, n_eq, d);
+        for (int k = 0; k < K; ++k) {
+          const bool in = (first + k * 32 < nKb) && (bits[k] >> shift) == lead;
+          const uint32_t mask = __ballot_sync(0xffffffffu, in);
+          if (mask != 0u) {
+            int at = 0;
+            if (lane == 0) at = atomicAdd(&rs->list_len, __popc(mask));
+            at = __shfl_sync(0xffffffffu, at, 0) + __popc(mask & ((1u << lane) - 1u));
+            if (in) rs->list[at] = bits[k] & low_mask;
+          }
+        }
+        row_sync<W>();
+        if (warp == 0) {
+          // what the bin has to add, in units of the bin's mantissas: rounded up, the sums below are whole
+          const uint32_t lift = counting ? 0u : (lead >> 4) - 90u;
+          const unsigned long long missing =
+              (target - rs->above + ((1ull << lift) - 1ull)) >> lift;
+          const unsigned long long lead_mant = counting ? 1ull : (unsigned long long)((16u | (lead & 15u)) << kTauShift);
+          const int groups = ((int)m + 31) >> 5;
+          uint32_t lv = 0u;
+          auto measure = [&](uint32_t from, int* n_out) -> unsigned long long {
+            uint32_t n = 0u, l = 0u;
+            for (int g = 0; g < groups; ++g) {
+              const int i = g * 32 + lane;
+              const uint32_t x = (i < (int)m) ? rs->list[i] : 0u;
+              const bool ge = (i < (int)m) && x >= from;
+              n += ge ? 1u : 0u;
+              l += ge ? x : 0u;
+            }
+            n = __reduce_add_sync(0xffffffffu, n);
+            *n_out = (int)n;
+            if (counting) return n;
+            l = __reduce_add_sync(0xffffffffu, l);
+            return n * lead_mant + l;
+          };
+          int n_ge = (int)m;  // of the bin's values, those >= lv
+          for (int b = shift - 1; b >= 0; --b) {
+            int n;
+            if (measure(lv | (1u << b), &n) >= missing) {
+              lv |= 1u << b;
+              n_ge = n;
+            }
+          }
+          int n_gt;
+          const unsigned long long gt = measure(lv + 1u, &n_gt);
+          const unsigned long long each = counting ? 1ull : lead_mant + lv;
+          const int n_eq = n_ge - n_gt;
+          const int take = (int)min((missing - gt + each - 1ull) / each, (unsigned long long)n_eq);
+          // blocks of the bins above
+          int c_above = 0;
+          for (int b = bin + 1 + lane; b < kBins; b += 32) c_above += (int)rs->cnt[b];
+          c_above = __reduce_add_sync(0xffffffffu, c_above);
+          if (lane == 0) {
+            rs->v = (lead << shift) | lv;
+            rs->need = take;
+            rs->eq_total = n_eq;
+            rs->s = c_above + n_gt + take;
+          }
+        }
+        row_sync<W>();
+        v = rs->v;
+        need = rs->need;
+        s = rs->s;
+        eq_total = rs->eq_total;
+      }
     }
-    unsigned long long need64;
-    if (fixed_count > 0) {
-      need64 = target - gt;
-    } else {
-      const unsigned long long fv = (unsigned long long)((double)__uint_as_float(v) * 1152921504606846976.0);
-      need64 = (fv == 0ull) ? (unsigned long long)n_eq : (target - gt + fv - 1ull) / fv;
+    if (!listed) {
+      // ---- bit by bit over the row: masked sums (or counts) of the blocks with bits >= v
+      auto measure_ge = [&](uint32_t from) -> unsigned long long {
+        unsigned long long a = 0ull;
+#pragma unroll
+        for (int k = 0; k < K; ++k)
+          if (bits[k] >= from && first + k * 32 < nKb) a += counting ? 1ull : fixed_weight(bits[k], scale, cap);
+        return row_sum_u64<W>(a, rs, warp, lane);
+      };
+      all = measure_ge(0u) < target;  // never reaches tau
+      if (!all) {
+        for (int b = 30; b >= 0; --b) {
+          const uint32_t cand = v | (1u << b);
+          if (measure_ge(cand) >= target) v = cand;
+        }
+        const unsigned long long gt = measure_ge(v + 1u);
+        unsigned long long n = 0ull;  // how many are above v, and how many equal it
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+          const bool valid = first + k * 32 < nKb;
+          if (valid && bits[k] > v) n += 1ull;
+          if (valid && bits[k] == v) n += 1ull << 20;
+        }
+        n = row_sum_u64<W>(n, rs, warp, lane);
+        const int n_gt = (int)(n & 0xfffffull);
+        eq_total = (int)(n >> 20);
+        const unsigned long long fv = counting ? 1ull : fixed_weight(v, scale, cap);
+        const unsigned long long need64 = (fv == 0ull) ? (unsigned long long)eq_total : (target - gt + fv - 1ull) / fv;
+        need = (int)min(need64, (unsigned long long)eq_total);
+        s = n_gt + need;
+      }
     }
-    need = (int)min(need64, (unsigned long long)n_eq);
-    s = n_gt + need;
   }
+  // ---- bitmap words; of the blocks equal to v the first `need` by index
   int seen = 0;  // ties at lower indices
+  if (!all && need < eq_total) {  // (otherwise all ties are kept and their order does not matter)
+    int n = 0;
+#pragma unroll
+    for (int k = 0; k < K; ++k) n += (first + k * 32 < nKb && bits[k] == v) ? 1 : 0;
+    n = __reduce_add_sync(0xffffffffu, n);
+    if (W > 1) {
+      if (lane == 0) rs->eq[warp] = n;
+      __syncthreads();
+#pragma unroll
+      for (int w = 0; w < W; ++w)
+        if (w < warp) seen += rs->eq[w];
+    }
+  }
+  uint32_t out = 0u;  // lane k: word k of this warp's K
 #pragma unroll
   for (int k = 0; k < K; ++k) {
-    const bool valid = (k * 32 + lane) < nKb;
-    const bool eq = valid && !all && bits[k] == v;
-    const uint32_t eqm = __ballot_sync(0xffffffffu, eq);
-    const int rank = seen + __popc(eqm & ((1u << lane) - 1u));
-    const bool keep = valid && (all || bits[k] > v || (eq && rank < need));
-    seen += __popc(eqm);
+    const bool valid = first + k * 32 < nKb;
+    bool keep = valid && (all || bits[k] > v);
+    if (!all) {
+      const bool eq = valid && bits[k] == v;
+      const uint32_t eqm = __ballot_sync(0xffffffffu, eq);
+      keep = keep || (eq && seen + __popc(eqm & ((1u << lane) - 1u)) < need);
+      seen += __popc(eqm);
+    }
     const uint32_t word = __ballot_sync(0xffffffffu, keep);
-    if (lane == 0 && k < words) bitmaps[row * words + k] = word;
+    if (lane == k) out = word;
   }
-  if (lane == 0) counts[row] = s;
+  if (lane < K && warp * K + lane < words) bitmaps[row * words + warp * K + lane] = out;
+  if (t == 0) counts[row] = s;
 }
 
-__global__ void __launch_bounds__(1024)
-scan_counts_kernel(const int32_t* __restrict__ counts, int rows, int32_t* __restrict__ offsets,
-                   int64_t kv_capacity, int* status) {
-  __shared__ int warp_total[32];
-  __shared__ int carry_s;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  if (tid == 0) carry_s = 0;
+// Bitmaps -> ascending indices, `per_cta` consecutive rows per CTA.  The CTA first adds up the sizes
+// of all rows before its own: that is a read of at most 4 bytes per row from L2, and it replaces a
+// launch that scanned the sizes with one CTA.  Then a warp per row, 32 indices at a time: lane b
+// stands for bit b of a bitmap word, so the stores of a word are contiguous.  (One lane per word,
+// each writing its word's indices one after the other, stored 32 separate sectors per instruction.)
+constexpr int kExpandThreads = 512;
+
+__global__ void __launch_bounds__(kExpandThreads)
+expand_rows_kernel(const int32_t* __restrict__ counts, const uint32_t* __restrict__ bitmaps, int rows, int nKb,
+                   int per_cta, int32_t* __restrict__ offsets, int32_t* __restrict__ kv_idx, int64_t kv_capacity,
+                   int* status) {
+  constexpr int kWarps = kExpandThreads / 32;
+  __shared__ int warp_total[kWarps];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int row0 = blockIdx.x * per_cta, row1 = min(rows, row0 + per_cta);
+  const int words = (nKb + 31) >> 5;
+  int before = 0;
+  for (int i = threadIdx.x; i < (row0 >> 2); i += kExpandThreads) {
+    const int4 c = __ldg(reinterpret_cast<const int4*>(counts) + i);
+    before += (c.x + c.y) + (c.z + c.w);
+  }
+  if (threadIdx.x < (row0 & 3)) before += __ldg(counts + (row0 & ~3) + threadIdx.x);
+  before = __reduce_add_sync(0xffffffffu, before);
+  if (lane == 0) warp_total[warp] = before;
   __syncthreads();
-  for (int base = 0; base < rows; base += 1024) {
-    const int i = base + tid;
-    const int c = (i < rows) ? counts[i] : 0;
+  int pos = 0;  // first index of the row
+#pragma unroll
+  for (int w = 0; w < kWarps; ++w) pos += warp_total[w];
+  for (int r0 = row0; r0 < row1; r0 += 32) {
+    // 32 rows: every warp scans their sizes and expands its share of them
+    const int r = r0 + lane;
+    const int c = (r < row1) ? __ldg(counts + r) : 0;
     int incl = c;
 #pragma unroll
     for (int d = 1; d < 32; d <<= 1) {
       const int up = __shfl_up_sync(0xffffffffu, incl, d);
       if (lane >= d) incl += up;
     }
-    if (lane == 31) warp_total[warp] = incl;
-    __syncthreads();
-    int wbase = 0;
-    for (int w = 0; w < warp; ++w) wbase += warp_total[w];
-    const int carry = carry_s;
-    if (i < rows) offsets[i] = carry + wbase + incl - c;
-    __syncthreads();
-    if (tid == 1023) carry_s = carry + wbase + incl;
-    __syncthreads();
-  }
-  if (tid == 0) {
-    offsets[rows] = carry_s;
-    if ((int64_t)carry_s > kv_capacity) report_error(status, LOSA_ERR_CAPACITY);
-  }
-}
-
-__global__ void __launch_bounds__(256)
-expand_rows_kernel(const uint32_t* __restrict__ bitmaps, const int32_t* __restrict__ offsets,
-                   int rows, int nKb, int32_t* __restrict__ kv_idx, int64_t kv_capacity) {
-  const int lane = threadIdx.x & 31;
-  const int64_t row = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (row >= rows) return;
-  const int words = (nKb + 31) >> 5;
-  int64_t pos0 = offsets[row];
-  for (int w0 = 0; w0 < words; w0 += 32) {
-    const int w = w0 + lane;
-    uint32_t word = (w < words) ? bitmaps[row * words + w] : 0u;
-    const int cnt = __popc(word);
-    int incl = cnt;
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-      const int up = __shfl_up_sync(0xffffffffu, incl, d);
-      if (lane >= d) incl += up;
+    const int n = min(32, row1 - r0);
+    if (warp == 0 && lane < n) offsets[r] = pos + incl - c;
+    for (int j = warp; j < n; j += kWarps) {
+      int at = pos + __shfl_sync(0xffffffffu, incl - c, j);
+      const uint32_t* bm = bitmaps + (int64_t)(r0 + j) * words;
+      for (int w0 = 0; w0 < words; w0 += 32) {
+        const uint32_t mine = (w0 + lane < words) ? __ldg(bm + w0 + lane) : 0u;
+        const int m = min(32, words - w0);
+        for (int i = 0; i < m; ++i) {
+          const uint32_t word = __shfl_sync(0xffffffffu, mine, i);
+          const int to = at + __popc(word & ((1u << lane) - 1u));
+          if (((word >> lane) & 1u) && to < kv_capacity) kv_idx[to] = (w0 + i) * 32 + lane;
+          at += __popc(word);
+        }
+      }
     }
-    int64_t pos = pos0 + incl - cnt;
-    while (word) {
-      const int b = __ffs(word) - 1;
-      word &= word - 1;
-      if (pos < kv_capacity) kv_idx[pos] = w * 32 + b;
-      ++pos;
-    }
-    pos0 += __shfl_sync(0xffffffffu, incl, 31);
+    pos += __shfl_sync(0xffffffffu, incl, 31);
+  }
+  if (row1 == rows && threadIdx.x == 0) {
+    offsets[rows] = pos;
+    if ((int64_t)pos > kv_capacity) report_error(status, LOSA_ERR_CAPACITY);
   }
 }
 
@@ -355,12 +463,6 @@ row_recall_kernel(const float* __restrict__ mass, int rows, int nKb,
   }
 }
 
-int next_pow2(int x) {
-  int n = 32;
-  while (n < x) n <<= 1;
-  return n;
-}
-
 size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 }  // namespace
@@ -376,31 +478,22 @@ int launch_select(int rows, int nKb, const float* mass, double tau, int fixed_co
   int32_t* counts = static_cast<int32_t*>(ws);
   uint32_t* bitmaps = reinterpret_cast<uint32_t*>(static_cast<char*>(ws) +
                                                   align_up((size_t)rows * sizeof(int32_t), 256));
-  if (nKb <= 1024) {
-    // one warp per row, the row in registers, no sort
-    const int ctas = (rows + 3) / 4;
-    if (nKb <= 256)
-      select_rows_warp_kernel<8><<<ctas, 128, 0, st>>>(mass, rows, nKb, tau, fixed_count, counts, bitmaps, status);
-    else if (nKb <= 512)
-      select_rows_warp_kernel<16><<<ctas, 128, 0, st>>>(mass, rows, nKb, tau, fixed_count, counts, bitmaps, status);
-    else
-      select_rows_warp_kernel<32><<<ctas, 128, 0, st>>>(mass, rows, nKb, tau, fixed_count, counts, bitmaps, status);
-  } else {
-    const int n2 = next_pow2(nKb);
-    const int words = (nKb + 31) / 32;
-    const size_t smem = (size_t)n2 * 8 + (size_t)words * 4;
-    // (a function attribute belongs to the current device: set on every call, it costs nothing)
-    if (smem > 48 * 1024) {
-      LOSA_CUDA_TRY(cudaFuncSetAttribute(select_rows_kernel,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    }
-    select_rows_kernel<<<rows, kSelThreads, smem, st>>>(mass, nKb, n2, tau, fixed_count, counts, bitmaps,
-                                                        status);
-  }
-  scan_counts_kernel<<<1, 1024, 0, st>>>(counts, rows, offsets, kv_capacity, status);
-  const int warps_per_cta = 8;
-  expand_rows_kernel<<<(rows + warps_per_cta - 1) / warps_per_cta, warps_per_cta * 32, 0, st>>>(
-      bitmaps, offsets, rows, nKb, kv_idx, kv_capacity);
+  // (registers hold 32 blocks per lane at most: longer rows take more warps)
+#define LOSA_SELECT_ROWS(w, k) \
+  select_rows_kernel<w, k><<<(w) == 1 ? (rows + 3) / 4 : rows, (w) == 1 ? 128 : 32 * (w), 0, st>>>( \
+      mass, rows, nKb, tau, fixed_count, counts, bitmaps, status)
+  if (nKb <= 256) LOSA_SELECT_ROWS(1, 8);
+  else if (nKb <= 512) LOSA_SELECT_ROWS(1, 16);
+  else if (nKb <= 1024) LOSA_SELECT_ROWS(1, 32);
+  else if (nKb <= 2048) LOSA_SELECT_ROWS(2, 32);
+  else if (nKb <= 4096) LOSA_SELECT_ROWS(4, 32);
+  else LOSA_SELECT_ROWS(8, 32);
+#undef LOSA_SELECT_ROWS
+  // four CTAs per SM at most (but no fewer rows than warps): adding up the sizes of the rows before
+  // costs every CTA the same, so more of them only read more
+  const int per_cta = max(kExpandThreads / 32, (rows + 591) / 592);
+  expand_rows_kernel<<<(rows + per_cta - 1) / per_cta, kExpandThreads, 0, st>>>(
+      counts, bitmaps, rows, nKb, per_cta, offsets, kv_idx, kv_capacity, status);
   LOSA_CUDA_TRY(cudaGetLastError());
   return LOSA_OK;
 }

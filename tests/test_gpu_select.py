@@ -43,6 +43,39 @@ def test_select_bit_exact_against_oracle(rows, nKb, tau):
     assert off[0] == 0 and off[-1] == sel.count.sum()
 
 
+@pytest.mark.parametrize("nKb", [7, 256, 257, 513, 1024, 1025, 2048, 2049, 4096, 4097, 8192])
+@pytest.mark.parametrize("kind", ["spread", "equal", "binade", "tail", "short"])
+def test_select_at_the_edges_of_its_row_lengths(nKb, kind):
+    """Row lengths around every change of layout, on masses that reach each way of finding the
+    threshold: its histogram bin's list, a bin with more values than the list holds (equal masses, and
+    masses within one sixteenth of a binade), below the bins, and rows that never reach tau.  Sums of
+    both sides are exact to 1e-13, so only rows with a prefix that close to tau could differ."""
+    rng = np.random.default_rng(nKb)
+    if kind == "equal":
+        m = np.full((5, nKb), 2.0 ** -13)
+        taus = (2.0 ** -13 * (nKb // 3 + 1), 0.25)
+    elif kind == "binade":
+        m = (1.0 + rng.integers(0, 2 ** 18, (5, nKb)) / 2.0 ** 22) * 2.0 ** -14
+        taus = (0.3 * nKb * 2.0 ** -14,)
+    elif kind == "tail":  # one heavy block, the threshold among masses about 2^-40
+        m = rng.integers(1, 2 ** 10, (5, nKb)) * 2.0 ** -50
+        m[:, nKb // 2] = 0.5
+        taus = (0.5, 0.5 + 0.4 * float(m[0].sum() - 0.5))
+    else:
+        m = random_mass(5, nKb, 40 + nKb, tail=2.0) * (0.5 if kind == "short" else 1.0)
+        taus = (0.99, 0.4)
+    m = m.astype(np.float32)
+    for tau in taus + (1e-9, 1e-25):
+        off, idx, status = run_select(m, tau)
+        assert status == 0
+        sel = orc.select(m.astype(np.float64), tau)
+        assert util.csr_rows(off, idx[: off[-1]]) == util.csr_rows(sel.offsets, sel.kv_idx), (kind, tau)
+    k = max(1, nKb // 3)
+    off, idx = lib().losa_select_topk(torch.from_numpy(m).cuda().reshape(1, 1, 5, nKb), k)
+    ref_off, ref_idx = orc.select_topk(m.astype(np.float64), k)
+    assert np.array_equal(off.cpu().numpy(), ref_off) and np.array_equal(idx.cpu().numpy()[: 5 * k], ref_idx)
+
+
 def test_select_ties_uniform_and_zero_masses():
     nKb = 10
     m = np.full((4, nKb), 0.1, dtype=np.float32)
