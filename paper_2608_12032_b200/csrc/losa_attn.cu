@@ -18,7 +18,7 @@
 // blocks (two lists, four when R = 64), so a K/V tile needed by both tiles is loaded once, and
 // MMAs are issued only for the query tiles that list one of its blocks.  The items of the last,
 // partly filled wave of the persistent grid are cut into parts of their lists, merged by
-// merge_parts_kernel.
+// the fallback launch.
 //
 // One S = Q K^T covers a whole K/V tile (128-wide MMAs).  At head dimension 128 TMEM holds exactly
 // S and O of both query tiles, P overwrites S, and per query tile the steps S -> softmax ->
@@ -43,7 +43,6 @@
 
 #include <atomic>
 #include <cstddef>
-#include <vector>
 
 #include "losa_common.cuh"
 #include "losa_ptx.cuh"
@@ -98,7 +97,9 @@ constexpr int kProducerWarp = 0, kIssuerWarp = 1, kSchedulerWarp = 3;  // issuer
 constexpr int kTmemCols = 512;
 // Tile list ring: the scheduler warp writes one 32-bit entry per work item header, per K/V tile
 // and one end marker; every other warp reads all of them in order.
-constexpr size_t kCounterBytes = 256;  // head of the workspace: the work-item counter
+constexpr size_t kCounterBytes = 256;  // head of the workspace: the launch's counters
+// work-item counter, length of the fallback list, the fallback launch's item counter, its CTAs that are done
+constexpr int kCounters = 4;
 constexpr size_t kRowstatBytes = (size_t)kMaxPersistentCtas * 2 * 128 * sizeof(float2);
 constexpr size_t kPartMlBytes = kRowstatBytes;  // same shape: [slot][2][128] float2
 constexpr int kTlChunks = 4;
@@ -152,7 +153,7 @@ struct Cfg {
 
 // One entry per problem of a batched launch (several layers or requests of one shape in one
 // persistent launch): the problem's tensor maps, its output and its own CSR pattern.  The table
-// lives in the workspace and is written by the host before the launch.
+// lives in the workspace and is written by write_problems_kernel before the launch.
 struct alignas(128) ProblemEntry {
   CUtensorMap map_q, map_k, map_v;
   CUtensorMap map_kh;  // K with boxes of at most 64 keys (the CTA-pair kernel copies half a K tile per CTA)
@@ -196,9 +197,11 @@ struct Params {
   int* status;
   // Work units whose scores outgrew the fixed reference of the two-threads-per-row kernel: it
   // appends them here, and a second launch (one thread per row, moving reference) recomputes them.
+  // That second launch, which also merges the partial units, draws redo_list[0 .. *redo_count) instead
+  // of all units.
   int* redo_count;
   int* redo_list;
-  int redo;             // this launch processes redo_list[0 .. *redo_count) instead of all units
+  int* redo_done;  // how many CTAs of the second launch are done
   // extents of the buffers the kernels index into (elements), for the checked build
   long long cap_part_rows, cap_table_floats, cap_mass, cap_lse, cap_units;
   uint32_t wait_polls;  // bound of every device-side wait, in polls (ptx::kWaitPolls)
@@ -325,6 +328,96 @@ struct Control {
     ++te;                                                                            \
   } while (0)
 
+// Merge of the partial units: for every row of the split items, combine the parts' unnormalised
+// O, reference maximum and row sum (the usual log-sum-exp merge) and write the attention output.  A
+// warp per row, its lanes the columns; all parts of a row are read at once, whatever their weights
+// turn out to be, because the merge is nothing but the latency of its loads (as a kernel of its own
+// that read the statistics, then part after part, it took 14 us at D = 64 and 20 us at D = 128 for
+// 8 parts; the attention kernel before it 21 us on a 2048-token layer).  AT_ONCE = false: part after
+// part, for the few registers that are left behind the attention kernel's roles.
+template <int D, bool AT_ONCE>
+__device__ __forceinline__ void merge_parts(const Params& p, int cta, int ctas) {
+  constexpr int kCols = D / 32;
+  const int warps = blockDim.x >> 5, lane = threadIdx.x & 31;
+  const int parts = p.split_parts;
+  if (parts <= 1) return;
+  const int rows = (p.nWork - p.split_first) * 256;
+  for (int i = cta * warps + (threadIdx.x >> 5); i < rows; i += ctas * warps) {
+    const int r = i >> 8, qt = (i >> 7) & 1, row = i & 127;
+    const int w = p.split_first + r;
+    const int pbh = w / p.nPairs, pr = w % p.nPairs;
+    const int T = 2 * pr + qt, grow = T * 128 + row;
+    if (grow >= p.N) continue;
+    const int64_t slot0 = ((int64_t)r * parts * 2 + qt) * 128 + row;  // of part s: slot0 + 256 s
+    float2 ml = make_float2(0.f, 0.f);
+    if (lane < parts) ml = __ldcg(p.part_ml + slot0 + lane * 256);
+    auto load = [&](int s, float* v) {
+      const float* src = p.part_o + (slot0 + s * 256) * D + lane * kCols;
+      if constexpr (kCols == 4) {
+        const float4 x = __ldcg(reinterpret_cast<const float4*>(src));
+        v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
+      } else {
+        const float2 x = __ldcg(reinterpret_cast<const float2*>(src));
+        v[0] = x.x; v[1] = x.y;
+      }
+    };
+    float v[AT_ONCE ? kMaxParts : 1][kCols];
+    if constexpr (AT_ONCE) {
+#pragma unroll
+      for (int s = 0; s < kMaxParts; ++s)
+        if (s < parts) load(s, v[s]);
+    }
+    float m = (ml.y > 0.f) ? ml.x : -INFINITY;
+#pragma unroll
+    for (int d = kMaxParts / 2; d > 0; d >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, d));
+    const float mine = (ml.y > 0.f) ? ptx::ex2_approx(ml.x - m) : 0.f;
+    float L = 0.f, acc[kCols];
+#pragma unroll
+    for (int c = 0; c < kCols; ++c) acc[c] = 0.f;
+#pragma unroll(AT_ONCE ? kMaxParts : 1)
+    for (int s = 0; s < kMaxParts; ++s) {
+      if (s < parts) {
+        const float sc = __shfl_sync(0xffffffffu, mine, s);
+        L += __shfl_sync(0xffffffffu, ml.y, s) * sc;
+        if constexpr (!AT_ONCE) load(s, v[0]);
+        if (sc != 0.f) {
+#pragma unroll
+          for (int c = 0; c < kCols; ++c) acc[c] += v[AT_ONCE ? s : 0][c] * sc;
+        }
+      }
+    }
+    const float inv = (L > 0.f) ? 1.f / L : 0.f;
+    const int bh = pbh % (p.B * p.H);
+    void* const o_base = (p.problems != nullptr) ? p.problems[pbh / (p.B * p.H)].o : p.o;
+    const int64_t off = (int64_t)(bh / p.H) * p.sb + (int64_t)(bh % p.H) * p.sh + (int64_t)grow * p.sn + lane * kCols;
+    if (p.o_f32) {
+      float* dst = static_cast<float*>(o_base) + off;
+      if constexpr (kCols == 4)
+        *reinterpret_cast<float4*>(dst) = make_float4(acc[0] * inv, acc[1] * inv, acc[2] * inv, acc[3] * inv);
+      else
+        *reinterpret_cast<float2*>(dst) = make_float2(acc[0] * inv, acc[1] * inv);
+    } else {
+      __nv_bfloat16* dst = static_cast<__nv_bfloat16*>(o_base) + off;
+      if constexpr (kCols == 4)
+        *reinterpret_cast<uint2*>(dst) = make_uint2(ptx::pack_bf16x2(acc[0] * inv, acc[1] * inv),
+                                                    ptx::pack_bf16x2(acc[2] * inv, acc[3] * inv));
+      else
+        *reinterpret_cast<uint32_t*>(dst) = ptx::pack_bf16x2(acc[0] * inv, acc[1] * inv);
+    }
+  }
+}
+
+// Tensor maps of a batched launch were written to the workspace by a kernel, over those of an earlier call.
+__device__ __forceinline__ void acquire_maps(const ProblemEntry* pe) {
+  ptx::tensormap_acquire(&pe->map_q);
+  ptx::tensormap_acquire(&pe->map_k);
+  ptx::tensormap_acquire(&pe->map_v);
+  ptx::tensormap_acquire(&pe->map_kh);
+  ptx::tensormap_acquire(&pe->map_k64);
+  ptx::tensormap_acquire(&pe->map_k128);
+  ptx::tensormap_acquire(&pe->map_v128);
+}
+
 template <int D, int R, int C_, int MODE, int KT, bool SPLIT>
 __global__ void __launch_bounds__(Lay<SPLIT>::kThreads, 1)
 losa_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
@@ -372,6 +465,17 @@ losa_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   if (SPLIT && smem != smem_raw) {
     if (threadIdx.x == 0) report_error(p.status, LOSA_ERR_CUDA);
     return;
+  }
+  if (SPLIT) {
+    ptx::grid_launch_dependents();
+  } else {
+    // Fallback launch: on ordinary inputs there is nothing to recompute, and the CTAs only merge the
+    // partial units and leave, before they set anything up.
+    ptx::grid_dependency_wait();
+    if (*reinterpret_cast<volatile int*>(p.redo_count) == 0) {
+      if (MODE == kDense || MODE == kSparse) merge_parts<D, true>(p, blockIdx.x, gridDim.x);
+      return;
+    }
   }
   uint8_t* sQ = smem;
   uint8_t* sK = sQ + 2 * C::kQBytes;
@@ -440,6 +544,9 @@ losa_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   ptx::tc_fence_after_sync();
   const uint32_t tmem_base = ctl->tmem_base;
 
+  // (the tile lists and the counters come from the kernel before; everything up to here overlaps it)
+  if (SPLIT) ptx::grid_dependency_wait();
+
   // The softmax warpgroups hold a whole S row per thread: the utility warpgroup gives registers
   // up and the softmax warpgroups take them.
   if (warp < 4) {
@@ -449,6 +556,7 @@ losa_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     // (the whole warp walks the tile list; lane 0 alone issues the copies)
     {
       uint32_t nq[2] = {0, 0}, nk = 0, nv = 0, te = 0, ent;
+      int problem = -1;  // batched launch: whose tensor maps this warp has acquired
       LOSA_TL_NEXT(ent);
       while ((ent >> 28) == 1) {
         const int w = (int)(ent & kTlItemMask);
@@ -463,6 +571,10 @@ losa_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           mv = &pe->map_v;
           mkw = &pe->map_k128;
           mvw = &pe->map_v128;
+          if (pbh / (p.B * p.H) != problem) {
+            problem = pbh / (p.B * p.H);
+            acquire_maps(pe);
+          }
         }
 #pragma unroll
         for (int qt = 0; qt < 2; ++qt) {
@@ -859,19 +971,22 @@ losa_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     // Walks the block-index lists of this CTA's work items and publishes, per item, a header
     // and the ascending merge of its tiles; nobody else touches the CSR.
     uint32_t te = 0;
+    bool first_item = true;
     for (;;) {
       // (diagnostic launch, see losa_debug_stall_next_launch: no tile list is ever published, no
       // copy and no MMA is issued, and every other role's first wait runs out)
       if (p.stall) break;
-      // work items are drawn from a global counter, in head-major order, so that a CTA that
-      // finishes early takes the next item instead of idling at the end of the launch
-      int w = 0;
-      if (lane == 0) {
-        w = atomicAdd(p.work_counter, 1);
-        // fallback launch: the units the two-threads-per-row kernel could not finish
-        if (p.redo) w = (w < *p.redo_count) ? p.redo_list[w] : p.nUnits;
+      // After a first item by position, work items are drawn from a global counter, in head-major
+      // order, so that a CTA that finishes early takes the next item instead of idling at the end
+      // of the launch
+      int w = blockIdx.x;
+      if (!first_item) {
+        if (lane == 0) w = (int)gridDim.x + atomicAdd(p.work_counter, 1);
+        w = __shfl_sync(0xffffffffu, w, 0);
       }
-      w = __shfl_sync(0xffffffffu, w, 0);
+      first_item = false;
+      // fallback launch: the units the two-threads-per-row kernel could not finish
+      if (!SPLIT) w = (w < *reinterpret_cast<volatile int*>(p.redo_count)) ? p.redo_list[w] : p.nUnits;
       if (w >= p.nUnits) break;
       // units past split_first are parts of the key range of the last items
       int part = 0, parts = 1;
@@ -890,11 +1005,11 @@ losa_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         // the unit's merged tile list was built before the launch: stream it into the ring,
         // 32 entries per step, so that this warp takes next to no issue slots from the softmax
         // warps of its scheduler partition
-        const int cnt = LOSA_IN_RANGE(unit, p.cap_units) ? min(__ldg(p.tl_count + unit), p.tl_cap) : 0;
+        const int cnt = LOSA_IN_RANGE(unit, p.cap_units) ? min(__ldcg(p.tl_count + unit), p.tl_cap) : 0;
         const uint32_t* src = p.tl_entries + (int64_t)unit * p.tl_cap;
         for (int base = 0; base < cnt; base += 32) {
           const int n = min(32, cnt - base);
-          const uint32_t e = (lane < n) ? __ldg(src + base + lane) : 0u;
+          const uint32_t e = (lane < n) ? __ldcg(src + base + lane) : 0u;
           LOSA_TL_PUT_BULK(e, n);
         }
         continue;
@@ -1692,6 +1807,15 @@ teardown:
     ptx::tc_fence_after_sync();
     ptx::tmem_dealloc(tmem_base, kTmemCols);
   }
+  if (!SPLIT && (MODE == kDense || MODE == kSparse) && p.split_parts > 1) {
+    // the last CTA that is done recomputing merges the partial units alone
+    __threadfence();
+    __syncthreads();
+    if (__syncthreads_or(threadIdx.x == 0 && atomicAdd(p.redo_done, 1) == (int)gridDim.x - 1)) {
+      __threadfence();
+      merge_parts<D, false>(p, 0, 1);
+    }
+  }
 }
 
 #include "losa_attn_pair.cuh"
@@ -1712,10 +1836,17 @@ teardown:
 // idle.  A unit that is a part of an item takes the same share, by position, of every list, so
 // each (query block, key block) pair belongs to exactly one part.  Indices out of range are
 // reported and skipped; an unsorted list still gives a valid tile list.
+//
+// One warp per list fills its bitmap (a list of a small layer is nothing but the latency of its two
+// dependent loads), then the first warp writes the tile list.  The first CTA also zeroes the
+// launch's counters.
 template <int NB, int G>
-__global__ void __launch_bounds__(32) build_tile_lists_kernel(const Params p) {
+__global__ void __launch_bounds__(32 * NB) build_tile_lists_kernel(const Params p) {
   extern __shared__ uint32_t bm[];  // [NB][W] bitmaps
-  const int lane = threadIdx.x, unit = blockIdx.x;
+  ptx::grid_launch_dependents();
+  ptx::grid_dependency_wait();  // (batched launch: the table of the problems)
+  const int lane = threadIdx.x & 31, n = threadIdx.x >> 5, unit = blockIdx.x;
+  if (unit == 0 && threadIdx.x < kCounters) p.work_counter[threadIdx.x] = 0;
   int w = unit, part = 0, parts = 1;
   if (unit >= p.split_first) {
     const int r = unit - p.split_first;
@@ -1733,28 +1864,33 @@ __global__ void __launch_bounds__(32) build_tile_lists_kernel(const Params p) {
     kv_idx = pe->kv_idx;
   }
   const int W = (p.nKb + 31) >> 5;
-  for (int i = lane; i < NB * W; i += 32) bm[i] = 0u;
-  __syncwarp();
-  const int32_t nnz = __ldg(offsets + (int64_t)p.B * p.H * p.nQb);
-#pragma unroll
-  for (int n = 0; n < NB; ++n) {
-    const int g = pr * NB + n;
-    if (g >= p.nQb) continue;
+  uint32_t* const mine = bm + n * W;
+  const int g = pr * NB + n;
+  int b = 0, e = 0;
+  if (g < p.nQb) {
     const int64_t row = (int64_t)bh * p.nQb + g;
-    const int32_t b = __ldg(offsets + row), e = __ldg(offsets + row + 1);
+    const int32_t nnz = __ldg(offsets + (int64_t)p.B * p.H * p.nQb);
+    b = __ldg(offsets + row);
+    e = __ldg(offsets + row + 1);
     if (b < 0 || e < b || e > nnz || e - b > p.nKb) {
       report_error(p.status, LOSA_ERR_BAD_INDEX);
-      continue;
+      b = e = 0;
     }
+  }
+  for (int i = lane; i < W; i += 32) mine[i] = 0u;
+  __syncwarp();
+  {
     const int b2 = b + (int)(((int64_t)(e - b) * part) / parts);
     const int e2 = b + (int)(((int64_t)(e - b) * (part + 1)) / parts);
+#pragma unroll 4
     for (int i = b2 + lane; i < e2; i += 32) {
       const int v = __ldg(kv_idx + i);
-      if ((unsigned)v < (unsigned)p.nKb) atomicOr(&bm[n * W + (v >> 5)], 1u << (v & 31));
+      if ((unsigned)v < (unsigned)p.nKb) atomicOr(&mine[v >> 5], 1u << (v & 31));
       else report_error(p.status, LOSA_ERR_BAD_INDEX);  // skipped, never used as an address
     }
   }
-  __syncwarp();
+  __syncthreads();
+  if (n != 0) return;
   // Order of the entries.  A key block that only ONE of the unit's two query tiles lists is
   // processed by that tile alone, at half the CTA's rate; two such blocks, one of each tile, can
   // be in flight at the same time (the tiles' chains are independent).  So the list holds first
@@ -1786,8 +1922,16 @@ __global__ void __launch_bounds__(32) build_tile_lists_kernel(const Params p) {
   const int tA = (na + G - 1) / G, tB = (nbb + G - 1) / G;   // K/V tiles of the single-tile classes
   const int tmin = min(tA, tB);
   const int total = min(s1 + (tA + tB) * G, p.tl_cap);
-  for (int i = lane; i < total; i += 32) dst[i] = kTlPad;
-  __syncwarp();
+  // padding: the ends of the last K/V tile of each class
+  auto slot_of = [&](int k, int r) {  // position of entry r of class k (1: tile 0 only, 2: tile 1 only)
+    const int t = r / G;
+    return s1 + ((t < tmin) ? 2 * t + (k - 1) : 2 * tmin + (t - tmin)) * G + r % G;
+  };
+  if (lane < G) {
+    if (nb + lane < s1 && nb + lane < total) dst[nb + lane] = kTlPad;
+    if (na + lane < tA * G && slot_of(1, na + lane) < total) dst[slot_of(1, na + lane)] = kTlPad;
+    if (nbb + lane < tB * G && slot_of(2, nbb + lane) < total) dst[slot_of(2, nbb + lane)] = kTlPad;
+  }
   int rb = 0, ra = 0, rbb = 0;  // entries of each class emitted by earlier windows
   for (int w0 = 0; w0 < W; w0 += 32) {
     const int wi = w0 + lane;
@@ -1820,14 +1964,7 @@ __global__ void __launch_bounds__(32) build_tile_lists_kernel(const Params p) {
         uint32_t memb = 0;
 #pragma unroll
         for (int n = 0; n < NB; ++n) memb |= ((m[n] >> bit) & 1u) << n;
-        int pos;
-        if (k == 0) {
-          pos = r;
-        } else {
-          const int t = r / G;  // K/V tile of the class
-          const int slot = (t < tmin) ? 2 * t + (k - 1) : 2 * tmin + (t - tmin);
-          pos = s1 + slot * G + r % G;
-        }
+        const int pos = (k == 0) ? r : slot_of(k, r);
         if (pos < p.tl_cap) dst[pos] = (uint32_t)(wi * 32 + bit) | (memb << 16);
         ++r;
       }
@@ -1837,77 +1974,6 @@ __global__ void __launch_bounds__(32) build_tile_lists_kernel(const Params p) {
     rbb += tot[2];
   }
   if (lane == 0) p.tl_count[unit] = total;
-}
-
-// Merge of the partial units: for every row of the split items, combine the parts' unnormalised
-// O, reference maximum and row sum (the usual log-sum-exp merge) and write the attention output.
-// grid = (split items, 2 query tiles x 8 row chunks), 4 warps; a warp takes 4 rows, its lanes the
-// columns.
-template <int D>
-__global__ void __launch_bounds__(128) merge_parts_kernel(const Params p) {
-  const int r = blockIdx.x, qt = blockIdx.y >> 3, chunk = blockIdx.y & 7;
-  const int w = p.split_first + r;
-  const int pbh = w / p.nPairs, pr = w % p.nPairs;
-  const int T = 2 * pr + qt;
-  if (T >= p.nQt) return;
-  const int bh = pbh % (p.B * p.H);
-  const int b = bh / p.H, h = bh % p.H;
-  void* const o_base = (p.problems != nullptr) ? p.problems[pbh / (p.B * p.H)].o : p.o;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int parts = p.split_parts;
-#pragma unroll
-  for (int rr = 0; rr < 4; ++rr) {
-    const int row = chunk * 16 + warp * 4 + rr;
-    const int grow = T * 128 + row;
-    if (grow >= p.N) break;
-    float sc[kMaxParts];
-    float m = -INFINITY;
-#pragma unroll
-    for (int s = 0; s < kMaxParts; ++s) {
-      sc[s] = 0.f;
-      if (s < parts) {
-        const float2 ml = p.part_ml[(((int64_t)r * parts + s) * 2 + qt) * 128 + row];
-        if (ml.y > 0.f) m = fmaxf(m, ml.x);
-      }
-    }
-    float L = 0.f;
-#pragma unroll
-    for (int s = 0; s < kMaxParts; ++s) {
-      if (s < parts) {
-        const float2 ml = p.part_ml[(((int64_t)r * parts + s) * 2 + qt) * 128 + row];
-        if (ml.y > 0.f) {
-          sc[s] = ptx::ex2_approx(ml.x - m);
-          L += ml.y * sc[s];
-        }
-      }
-    }
-    const float inv = (L > 0.f) ? 1.f / L : 0.f;
-    const int d = lane * 4;
-    if (d < D) {
-      float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-      for (int s = 0; s < kMaxParts; ++s) {
-        if (s < parts && sc[s] != 0.f) {
-          const float4 v = *reinterpret_cast<const float4*>(
-              p.part_o + ((((int64_t)r * parts + s) * 2 + qt) * 128 + row) * D + d);
-          acc.x += v.x * sc[s];
-          acc.y += v.y * sc[s];
-          acc.z += v.z * sc[s];
-          acc.w += v.w * sc[s];
-        }
-      }
-      const int64_t off = (int64_t)b * p.sb + (int64_t)h * p.sh + (int64_t)grow * p.sn + d;
-      if (p.o_f32) {
-        *reinterpret_cast<float4*>(static_cast<float*>(o_base) + off) =
-            make_float4(acc.x * inv, acc.y * inv, acc.z * inv, acc.w * inv);
-      } else {
-        uint2 v;
-        v.x = ptx::pack_bf16x2(acc.x * inv, acc.y * inv);
-        v.y = ptx::pack_bf16x2(acc.z * inv, acc.w * inv);
-        *reinterpret_cast<uint2*>(static_cast<__nv_bfloat16*>(o_base) + off) = v;
-      }
-    }
-  }
 }
 
 // ---------------------------------------------------------------------------- host side
@@ -1952,6 +2018,65 @@ int make_map(CUtensorMap* m, const void* base, const Geometry& g, int box_rows) 
   return LOSA_OK;
 }
 
+// The tensor maps of one problem.  Boxes: the key blocks (kh: at most 64 keys, half a K/V tile), and
+// for 32-key blocks, whose tiles are copied whole where their blocks are consecutive, 64 and 128
+// keys; elsewhere those are not used.  v null: the mass pass, which has none.
+int make_maps(ProblemEntry* e, const Geometry& g, const void* q, const void* k, const void* v) {
+  int rc;
+  if ((rc = make_map(&e->map_q, q, g, 128)) != LOSA_OK) return rc;
+  if ((rc = make_map(&e->map_k, k, g, g.C)) != LOSA_OK) return rc;
+  e->map_v = e->map_k;
+  if (v && (rc = make_map(&e->map_v, v, g, g.C)) != LOSA_OK) return rc;
+  e->map_kh = e->map_k64 = e->map_k128 = e->map_k;
+  e->map_v128 = e->map_v;
+  if (g.C > 64 && (rc = make_map(&e->map_kh, k, g, 64)) != LOSA_OK) return rc;
+  if (g.C < 64) {
+    if ((rc = make_map(&e->map_k64, k, g, 64)) != LOSA_OK) return rc;
+    if ((rc = make_map(&e->map_k128, k, g, 128)) != LOSA_OK) return rc;
+    if (v && (rc = make_map(&e->map_v128, v, g, 128)) != LOSA_OK) return rc;
+  }
+  return LOSA_OK;
+}
+
+// Zeroes the counters of a launch that no other kernel precedes (a kernel and not a memset, so that
+// the attention kernel can be launched as its dependent: 3 us of that kernel's set-up overlap).
+__global__ void __launch_bounds__(32) init_counters_kernel(int* counters) {
+  ptx::grid_launch_dependents();
+  if (threadIdx.x < kCounters) counters[threadIdx.x] = 0;
+}
+
+// Part of a batched launch's table, carried in the kernel's parameters: the call reads its host
+// arguments before it returns, without a copy from pageable memory (which staged and waited, 20 us).
+constexpr int kTableChunk = 8;
+struct ProblemChunk {
+  ProblemEntry e[kTableChunk];
+};
+__global__ void __launch_bounds__(256)
+write_problems_kernel(const __grid_constant__ ProblemChunk chunk, ProblemEntry* table, int n) {
+  ptx::grid_launch_dependents();
+  const uint4* src = reinterpret_cast<const uint4*>(&chunk);
+  uint4* dst = reinterpret_cast<uint4*>(table);
+  for (int i = threadIdx.x; i < n * (int)(sizeof(ProblemEntry) / sizeof(uint4)); i += blockDim.x) dst[i] = src[i];
+}
+
+// Launches `kern`; `dependent`: it may be scheduled before the kernel ahead of it in the stream has
+// finished, and waits for it itself (grid_dependency_wait).
+template <typename... P, typename... A>
+int launch(void (*kern)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st, bool dependent, const A&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads, 1, 1);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = attr;
+  cfg.numAttrs = dependent ? 1 : 0;
+  LOSA_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, args...));
+  return LOSA_OK;
+}
+
 // Configures (once per device) and launches one layout of the attention kernel.
 template <int D, int R, int C_, int MODE, int KT, bool SPLIT>
 int launch_kernel(const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv, const CUtensorMap& mkw,
@@ -1982,9 +2107,7 @@ int launch_kernel(const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMa
     LOSA_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     configured = true;
   }
-  kern<<<grid, L::kThreads, smem, st>>>(mq, mk, mv, mkw, mvw, prm);
-  LOSA_CUDA_TRY(cudaGetLastError());
-  return LOSA_OK;
+  return launch(kern, dim3(grid), L::kThreads, smem, st, true, mq, mk, mv, mkw, mvw, prm);
 }
 
 // Configures (once per device) and launches the CTA-pair kernel on `clusters` pairs; *max_clusters
@@ -2000,7 +2123,9 @@ int launch_pair(const CUtensorMap& mq, const CUtensorMap& mkh, const CUtensorMap
   int dev = 0;
   LOSA_CUDA_TRY(cudaGetDevice(&dev));
   cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = 2;
   attr[0].val.clusterDim.y = 1;
@@ -2032,6 +2157,7 @@ int launch_pair(const CUtensorMap& mq, const CUtensorMap& mkh, const CUtensorMap
     return LOSA_OK;
   }
   cfg.gridDim = dim3(2 * clusters, 1, 1);
+  cfg.numAttrs = 2;
   LOSA_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, mq, mkh, mv, mk64, mv128, prm));
   return LOSA_OK;
 }
@@ -2040,14 +2166,10 @@ template <int D, int R, int C_, int MODE, int KT>
 int launch_t(const Geometry& g, const void* q, const void* k, const void* v, Params prm, int sms,
              cudaStream_t st) {
   using C = Cfg<D, R, C_, MODE, KT>;
-  CUtensorMap mq, mk, mv;
+  ProblemEntry maps;
   int rc;
-  if ((rc = make_map(&mq, q, g, 128)) != LOSA_OK) return rc;
-  if ((rc = make_map(&mk, k, g, C::kC)) != LOSA_OK) return rc;
-  if ((rc = make_map(&mv, C::kHasV ? v : k, g, C::kC)) != LOSA_OK) return rc;
-  CUtensorMap mk128, mv128;  // boxes of a whole 128-key tile, for tiles of consecutive key blocks
-  if ((rc = make_map(&mk128, k, g, 128)) != LOSA_OK) return rc;
-  if ((rc = make_map(&mv128, C::kHasV ? v : k, g, 128)) != LOSA_OK) return rc;
+  if ((rc = make_maps(&maps, g, q, k, C::kHasV ? v : nullptr)) != LOSA_OK) return rc;
+  const CUtensorMap &mq = maps.map_q, &mk = maps.map_k, &mv = maps.map_v;
   int ctas = min(sms, kMaxPersistentCtas);
   // Head dimension 128 with 128-row query blocks, modes with an attention output: pairs of CTAs,
   // one work item per pair at a time (see losa_attn_pair.cuh); the single-CTA kernels stay the
@@ -2060,12 +2182,9 @@ int launch_t(const Geometry& g, const void* q, const void* k, const void* v, Par
                              (MODE == kDense || MODE == kSparse || (LOSA_PAIR_FUSED && MODE == kFused) ||
                               (LOSA_PAIR_MASS && MODE == kMass && C_ < 64));
   bool pair = false;  // (a device that cannot hold a pair of these CTAs runs the single-CTA kernel)
-  CUtensorMap mkh, mk64;
   if constexpr (kPairMode) {
-    if ((rc = make_map(&mkh, k, g, C::kC < 64 ? C::kC : 64)) != LOSA_OK) return rc;
-    if ((rc = make_map(&mk64, k, g, 64)) != LOSA_OK) return rc;
     int fit = 0;
-    if (launch_pair<C_, MODE>(mq, mkh, mv, mk64, mv128, prm, 0, st, &fit) == LOSA_OK && fit >= 1 && sms >= 2) {
+    if (launch_pair<C_, MODE>(mq, maps.map_kh, mv, maps.map_k64, maps.map_v128, prm, 0, st, &fit) == LOSA_OK && fit >= 1 && sms >= 2) {
       pair = true;
       ctas = min(min(sms / 2, fit), kMaxPersistentCtas);
     }
@@ -2078,7 +2197,6 @@ int launch_t(const Geometry& g, const void* q, const void* k, const void* v, Par
   prm.split_first = prm.nWork;
   prm.split_parts = 1;
   constexpr bool kAttnOnly = (MODE == kDense || MODE == kSparse);
-  constexpr bool kTwoPerRow = true;  // every mode runs with two threads per row; one per row is the fallback
   if (kAttnOnly) {
     const int rest = (prm.nWork < ctas) ? prm.nWork : prm.nWork % ctas;
     int parts = rest > 0 ? ctas / rest : 1;
@@ -2090,43 +2208,35 @@ int launch_t(const Geometry& g, const void* q, const void* k, const void* v, Par
     }
   }
   const int grid = min(ctas, prm.nUnits);
+  // Every kernel after the first is launched as a dependent of the one before.
   if (MODE == kSparse) {
     const size_t bm_bytes = (size_t)C::kNB * ((prm.nKb + 31) / 32) * sizeof(uint32_t);  // <= 32 KB
-    build_tile_lists_kernel<C::kNB, C::kG><<<prm.nUnits, 32, bm_bytes, st>>>(prm);
-    LOSA_CUDA_TRY(cudaGetLastError());
-  }
-  if constexpr (kTwoPerRow) {
-    // The modes with an attention output run with two threads per query row and a reference that
-    // never moves; the units whose scores outgrew it (none, on ordinary inputs) are listed, and a second
-    // launch of the one-thread-per-row kernel, which returns at once when the list is empty,
-    // recomputes them with a moving reference.
-    prm.redo = 0;
-    bool launched = false;
-    if constexpr (kPairMode) {
-      if (pair) {
-        if ((rc = launch_pair<C_, MODE>(mq, mkh, mv, mk64, mv128, prm, grid, st, nullptr)) != LOSA_OK) return rc;
-        launched = true;
-      }
-    }
-    if (!launched) {
-      if ((rc = launch_kernel<D, R, C_, MODE, KT, true>(mq, mk, mv, mk128, mv128, prm, grid, st)) != LOSA_OK) return rc;
-    }
-    if (!prm.stall) {
-      prm.redo = 1;
-      prm.work_counter += 2;  // its own counter (zeroed with the first)
-      // (as many CTAs as SMs, whichever kernel ran first)
-      const int rgrid = min(min(sms, kMaxPersistentCtas), prm.nUnits);
-      if ((rc = launch_kernel<D, R, C_, MODE, KT, false>(mq, mk, mv, mk128, mv128, prm, rgrid, st)) != LOSA_OK) return rc;
-    }
+    rc = launch(build_tile_lists_kernel<C::kNB, C::kG>, dim3(prm.nUnits), 32 * C::kNB, bm_bytes, st, prm.nProb > 1, prm);
   } else {
-    prm.redo = 0;
-    if ((rc = launch_kernel<D, R, C_, MODE, KT, false>(mq, mk, mv, mk128, mv128, prm, grid, st)) != LOSA_OK) return rc;
+    rc = launch(init_counters_kernel, dim3(1), 32, 0, st, false, prm.work_counter);
   }
-  if (prm.split_parts > 1) {
-    merge_parts_kernel<D><<<dim3(prm.nWork - prm.split_first, 16), 128, 0, st>>>(prm);
-    LOSA_CUDA_TRY(cudaGetLastError());
+  if (rc != LOSA_OK) return rc;
+  // All modes run with two threads per query row and a reference that never moves; the units whose
+  // scores outgrew it (none, on ordinary inputs) are listed, and a second launch of the
+  // one-thread-per-row kernel recomputes them with a moving reference and merges the partial units.
+  bool launched = false;
+  if constexpr (kPairMode) {
+    if (pair) {
+      if ((rc = launch_pair<C_, MODE>(mq, maps.map_kh, mv, maps.map_k64, maps.map_v128, prm, grid, st, nullptr)) != LOSA_OK)
+        return rc;
+      launched = true;
+    }
   }
-  return LOSA_OK;
+  if (!launched) {
+    rc = launch_kernel<D, R, C_, MODE, KT, true>(mq, mk, mv, maps.map_k128, maps.map_v128, prm, grid, st);
+    if (rc != LOSA_OK) return rc;
+  }
+  if (prm.stall) return LOSA_OK;
+  prm.work_counter += 2;  // the second launch's own counter
+  // (as many CTAs as SMs, whichever kernel ran first, where there is something to merge)
+  const int rgrid = min(sms, kMaxPersistentCtas);
+  return launch_kernel<D, R, C_, MODE, KT, false>(mq, mk, mv, maps.map_k128, maps.map_v128, prm,
+                                                  prm.split_parts > 1 ? rgrid : min(rgrid, prm.nUnits), st);
 }
 
 template <int MODE>
@@ -2243,30 +2353,29 @@ int launch_attn(AttnMode mode, const Geometry& g, const void* q, const void* k, 
     if (n_prob > 1) {
       // the problems' table, behind the tile lists (dense mode has none), written before the launch
       char* tab = tl + (mode == kSparse ? tl_count_bytes(g, n_prob) + tl_entries_bytes(g, n_prob) : 0);
-      std::vector<ProblemEntry> host(n_prob);
-      for (int i = 0; i < n_prob; ++i) {
-        int rc;
-        if ((rc = make_map(&host[i].map_q, layers[i].q, g, 128)) != LOSA_OK) return rc;
-        if ((rc = make_map(&host[i].map_k, layers[i].k, g, g.C)) != LOSA_OK) return rc;
-        if ((rc = make_map(&host[i].map_v, layers[i].v, g, g.C)) != LOSA_OK) return rc;
-        if ((rc = make_map(&host[i].map_kh, layers[i].k, g, g.C < 64 ? g.C : 64)) != LOSA_OK) return rc;
-        if ((rc = make_map(&host[i].map_k64, layers[i].k, g, 64)) != LOSA_OK) return rc;
-        if ((rc = make_map(&host[i].map_k128, layers[i].k, g, 128)) != LOSA_OK) return rc;
-        if ((rc = make_map(&host[i].map_v128, layers[i].v, g, 128)) != LOSA_OK) return rc;
-        host[i].o = layers[i].o;
-        host[i].offsets = layers[i].offsets;
-        host[i].kv_idx = layers[i].kv_idx;
+      ProblemChunk chunk;
+      for (int i0 = 0; i0 < n_prob; i0 += kTableChunk) {
+        const int n = min(kTableChunk, n_prob - i0);
+        for (int i = 0; i < n; ++i) {
+          const losa_layer_t& l = layers[i0 + i];
+          const int rc = make_maps(&chunk.e[i], g, l.q, l.k, l.v);
+          if (rc != LOSA_OK) return rc;
+          chunk.e[i].o = l.o;
+          chunk.e[i].offsets = l.offsets;
+          chunk.e[i].kv_idx = l.kv_idx;
+        }
+        const int rc = launch(write_problems_kernel, dim3(1), 256, 0, st, false, chunk,
+                              reinterpret_cast<ProblemEntry*>(tab) + i0, n);
+        if (rc != LOSA_OK) return rc;
       }
-      // (a copy from pageable memory is staged before the call returns: `host` may go out of scope)
-      LOSA_CUDA_TRY(cudaMemcpyAsync(tab, host.data(), (size_t)n_prob * sizeof(ProblemEntry),
-                                    cudaMemcpyHostToDevice, st));
       prm.problems = reinterpret_cast<const ProblemEntry*>(tab);
       q = layers[0].q;  // the kernel's parameter maps are unused but must be valid
       k = layers[0].k;
       v = layers[0].v;
     }
-    // counter block: [0] work counter, [1] length of the fallback list, [2] the fallback launch's counter
+    // (kCounters)
     prm.redo_count = prm.work_counter + 1;
+    prm.redo_done = prm.work_counter + 3;
     prm.redo_list = reinterpret_cast<int*>(
         tl + (mode == kSparse ? tl_count_bytes(g, n_prob) + tl_entries_bytes(g, n_prob) : 0) +
         (n_prob > 1 ? (size_t)n_prob * sizeof(ProblemEntry) : 0));
@@ -2289,7 +2398,6 @@ int launch_attn(AttnMode mode, const Geometry& g, const void* q, const void* k, 
   const uint32_t stall_polls = g_stall_polls.exchange(0u);
   prm.stall = stall_polls > 0u ? 1 : 0;
   prm.wait_polls = stall_polls > 0u ? stall_polls : ptx::kWaitPolls;
-  LOSA_CUDA_TRY(cudaMemsetAsync(prm.work_counter, 0, 4 * sizeof(int), st));
   switch (mode) {
     case kDense: return dispatch<kDense>(g, q, k, v, prm, sms, st);
     case kSparse: return dispatch<kSparse>(g, q, k, v, prm, sms, st);

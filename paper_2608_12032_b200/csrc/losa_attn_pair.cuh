@@ -152,6 +152,7 @@ losa_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = ptx::cluster_ctarank();  // 0: the CTA that issues the MMAs; also the query tile of the pair
+  ptx::grid_launch_dependents();
   // (the swizzled tiles rely on the declared alignment of the dynamic shared memory)
   const bool misaligned = (ptx::smem_u32(smem_raw) & 1023u) != 0;
 
@@ -232,6 +233,8 @@ losa_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     }
   }
   __syncthreads();
+  // (the tile lists and the counters come from the kernel before; everything up to here overlaps it)
+  ptx::grid_dependency_wait();
 
   if (warp < 4) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(L::kRegsUtility));
@@ -239,6 +242,7 @@ losa_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     if (warp == kProducerWarp) {
       // ------------------------------------------------------------------ TMA producer (both CTAs)
       uint32_t nq = 0, nk = 0, nv = 0, te = 0, ent;
+      int problem = -1;  // batched launch: whose tensor maps this warp has acquired
       PAIR_TL_NEXT(ent);
       while ((ent >> 28) == 1) {
         const int w = (int)(ent & kTlItemMask);
@@ -254,6 +258,10 @@ losa_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           mv = &pe->map_v;
           mkw = &pe->map_k64;
           mvw = &pe->map_v128;
+          if (pbh / (p.B * p.H) != problem) {
+            problem = pbh / (p.B * p.H);
+            acquire_maps(pe);
+          }
         }
         // this CTA's query tile (rows past the end of the sequence are filled with zeros)
         const int T = 2 * pr + (int)rank;
@@ -431,11 +439,15 @@ losa_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     } else if (warp == kSchedulerWarp && rank == 0) {
       // ------------------------------------------------------------------ scheduler of the pair
       uint32_t te = 0;
+      bool first_item = true;
       for (;;) {
         if (p.stall) break;  // diagnostic launch: nothing is published and every wait runs out
-        int w = 0;
-        if (lane == 0) w = atomicAdd(p.work_counter, 1);
-        w = __shfl_sync(0xffffffffu, w, 0);
+        int w = (int)(blockIdx.x >> 1);  // a first item by position, then from the counter
+        if (!first_item) {
+          if (lane == 0) w = (int)(gridDim.x >> 1) + atomicAdd(p.work_counter, 1);
+          w = __shfl_sync(0xffffffffu, w, 0);
+        }
+        first_item = false;
         if (w >= p.nUnits) break;
         int part = 0, parts = 1;
         uint32_t flags = 0;
@@ -450,11 +462,11 @@ losa_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         const int pr = w % p.nPairs;
         PAIR_TL_PUT(kTlItem | flags | (uint32_t)w);
         if (MODE == kSparse) {
-          const int cnt = LOSA_IN_RANGE(unit, p.cap_units) ? min(__ldg(p.tl_count + unit), p.tl_cap) : 0;
+          const int cnt = LOSA_IN_RANGE(unit, p.cap_units) ? min(__ldcg(p.tl_count + unit), p.tl_cap) : 0;
           const uint32_t* src = p.tl_entries + (int64_t)unit * p.tl_cap;
           for (int base = 0; base < cnt; base += 32) {
             const int n = min(32, cnt - base);
-            const uint32_t e = (lane < n) ? __ldg(src + base + lane) : 0u;
+            const uint32_t e = (lane < n) ? __ldcg(src + base + lane) : 0u;
             PAIR_TL_PUT_BULK(e, n);
           }
           continue;

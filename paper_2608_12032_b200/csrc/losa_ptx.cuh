@@ -27,6 +27,19 @@ __device__ __forceinline__ bool elect_one() {
   return is_leader != 0;
 }
 
+// ---------------------------------------------------------------- programmatic dependent launch
+
+// The next kernel of the stream, if launched as a dependent, may be scheduled from here on.
+__device__ __forceinline__ void grid_launch_dependents() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+// Waits until the kernels this one was launched behind have completed and their writes are visible
+// (returns at once in an ordinary launch).
+__device__ __forceinline__ void grid_dependency_wait() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 // ---------------------------------------------------------------- mbarrier
 
 __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
@@ -104,6 +117,11 @@ __device__ __forceinline__ void prefetch_tensormap(const CUtensorMap* m) {
 }
 
 // 4D tiled load global -> this CTA's shared memory, completion on an mbarrier.
+// Before a copy through a tensor map that a kernel wrote to global memory.
+__device__ __forceinline__ void tensormap_acquire(const CUtensorMap* m) {
+  asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(m) : "memory");
+}
+
 __device__ __forceinline__ void tma_load_4d(void* smem_dst, const CUtensorMap* map, uint64_t* bar,
                                             int x, int y, int z, int w) {
   asm volatile(

@@ -114,3 +114,28 @@ def test_batched_call_reports_a_bad_index_of_one_layer_and_checks_its_arguments(
     with pytest.raises(losa.LosaError) as e:
         losa.losa_sparse_attn_batched(dev, R, C, ws=torch.empty(1024, dtype=torch.uint8, device="cuda"))
     assert e.value.code == -3
+
+
+@pytest.mark.parametrize("L", [1, 8, 9, 17])
+def test_batched_call_replays_from_a_graph(L):
+    """The table of the problems travels with the launch: a captured call, replayed after its host
+    arguments are gone, gives the bits of the call itself (table sizes around a launch's share of 8)."""
+    losa = lib()
+    B, H, N, D, R, C = 1, 1, 520, 128, 128, 64
+    dev = make_layers(L, B, H, N, D, R, C, 900)[1]
+    ref = [o.clone() for o in losa.losa_sparse_attn_batched(dev, R, C)]
+    outs = [torch.zeros_like(o) for o in ref]
+    need = losa.losa_workspace_bytes_batched(losa.binding.LOSA_OP_SPARSE_ATTN, losa.make_problem(dev[0][0], R, C), L)
+    ws = torch.empty(need, dtype=torch.uint8, device="cuda")
+    losa.losa_sparse_attn_batched(dev, R, C, outs=outs, ws=ws)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        losa.losa_sparse_attn_batched(dev, R, C, outs=outs, ws=ws)
+    for o in outs:
+        o.zero_()
+    for _ in range(2):
+        graph.replay()
+    torch.cuda.synchronize()
+    assert losa.losa_async_status() == 0
+    assert all(torch.equal(a, b) for a, b in zip(ref, outs))
