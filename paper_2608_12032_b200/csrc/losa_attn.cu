@@ -111,6 +111,10 @@ constexpr uint32_t kTlItemMask = 0x00ffffffu, kTlPartial = 1u << 27;
 // membership bits from bit 16); the last group of an item is padded with this entry: no member,
 // and a block index whose rows lie past the end of the tensor (the copy engine fills zeros).
 constexpr uint32_t kTlPad = 0xffffu;
+constexpr uint32_t kTlRagged = 1u << 20;  // tile entry: the sequence ends inside this key block
+// What is said of a unit's tile list: how many K/V tiles, which query tiles list any (kHdrHas << query
+// tile), and whether query tile 1 lists its first in the second K/V tile
+constexpr uint32_t kHdrTiles = 0x1fffffffu, kHdrLate = 1u << 29, kHdrHas = 1u << 30;
 constexpr int kMaxParts = 8;
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLn2 = 0.6931471805599453f;
@@ -165,7 +169,7 @@ struct alignas(128) ProblemEntry {
 };
 
 struct Params {
-  int B, H, N, nQb, nKb, nQt, nPairs, nWork;
+  int B, H, N, C, nQb, nKb, nQt, nPairs, nWork;
   // Batched launch: work items run over nProb problems, item w belongs to problem
   // w / (B * H * nPairs); `problems` is null for a single problem, whose maps are kernel
   // parameters and whose o / offsets / kv_idx are the fields below.
@@ -177,7 +181,7 @@ struct Params {
   // Sparse mode: the merged tile lists of all units, built by build_tile_lists_kernel before the
   // attention kernel: unit u owns tl_entries[u * tl_cap ...], tl_count[u] of them (padded to whole tiles).
   uint32_t* tl_entries;
-  int32_t* tl_count;
+  int32_t* tl_count;  // (kHdrTiles, kHdrHas, kHdrLate)
   int tl_cap;
   float* part_o;    // [slot][2][128][D] unnormalised O of a partial unit, slot = (item - split_first) * parts + part
   float2* part_ml;  // [slot][2][128] (reference max, row sum) of a partial unit
@@ -1005,7 +1009,8 @@ losa_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         // the unit's merged tile list was built before the launch: stream it into the ring,
         // 32 entries per step, so that this warp takes next to no issue slots from the softmax
         // warps of its scheduler partition
-        const int cnt = LOSA_IN_RANGE(unit, p.cap_units) ? min(__ldcg(p.tl_count + unit), p.tl_cap) : 0;
+        const int cnt = LOSA_IN_RANGE(unit, p.cap_units)
+                            ? min((int)((uint32_t)__ldcg(p.tl_count + unit) & kHdrTiles) * kG, p.tl_cap) : 0;
         const uint32_t* src = p.tl_entries + (int64_t)unit * p.tl_cap;
         for (int base = 0; base < cnt; base += 32) {
           const int n = min(32, cnt - base);
@@ -1932,6 +1937,7 @@ __global__ void __launch_bounds__(32 * NB) build_tile_lists_kernel(const Params 
     if (na + lane < tA * G && slot_of(1, na + lane) < total) dst[slot_of(1, na + lane)] = kTlPad;
     if (nbb + lane < tB * G && slot_of(2, nbb + lane) < total) dst[slot_of(2, nbb + lane)] = kTlPad;
   }
+  const int ragged = (p.N % p.C != 0) ? p.nKb - 1 : -1;  // the key block in which the sequence ends
   int rb = 0, ra = 0, rbb = 0;  // entries of each class emitted by earlier windows
   for (int w0 = 0; w0 < W; w0 += 32) {
     const int wi = w0 + lane;
@@ -1965,7 +1971,8 @@ __global__ void __launch_bounds__(32 * NB) build_tile_lists_kernel(const Params 
 #pragma unroll
         for (int n = 0; n < NB; ++n) memb |= ((m[n] >> bit) & 1u) << n;
         const int pos = (k == 0) ? r : slot_of(k, r);
-        if (pos < p.tl_cap) dst[pos] = (uint32_t)(wi * 32 + bit) | (memb << 16);
+        const int j = wi * 32 + bit;
+        if (pos < p.tl_cap) dst[pos] = (uint32_t)j | (memb << 16) | (j == ragged ? kTlRagged : 0u);
         ++r;
       }
     }
@@ -1973,7 +1980,9 @@ __global__ void __launch_bounds__(32 * NB) build_tile_lists_kernel(const Params 
     ra += tot[1];
     rbb += tot[2];
   }
-  if (lane == 0) p.tl_count[unit] = total;
+  if (lane == 0)
+    p.tl_count[unit] = (int32_t)((uint32_t)(total / G) | ((nb + na > 0) ? kHdrHas : 0u) |
+                                 ((nb + nbb > 0) ? 2u * kHdrHas : 0u) | ((nb == 0 && tmin > 0) ? kHdrLate : 0u));
 }
 
 // ---------------------------------------------------------------------------- host side
@@ -2319,6 +2328,7 @@ int launch_attn(AttnMode mode, const Geometry& g, const void* q, const void* k, 
   prm.B = g.B;
   prm.H = g.H;
   prm.N = g.N;
+  prm.C = g.C;
   prm.nQb = g.nQb;
   prm.nKb = g.nKb;
   prm.nQt = g.nQt;

@@ -37,12 +37,14 @@ struct PairControl {
   uint64_t v_full[kPairNV], v_empty[kPairNV];
   uint64_t s_full[3], p_ready[3], pv_done[3];  // per score buffer
   uint64_t o_done, o_free;
+  uint64_t hdr_full[2], hdr_empty[2], hdr_next;
   uint64_t tl_full[kTlChunks], tl_empty[kTlChunks];
   uint64_t pair_bar[8];    // per (group, lane quarter): the two halves of a row
   uint64_t ref_full[2], ref_empty[2];
   uint64_t item_bar;       // all softmax warps of the CTA, at the end of an item
   uint64_t fold_bar;       // ... and after the fused step's masses are folded out of the table
   uint64_t drain;
+  uint2 hdr[2];
   alignas(16) uint32_t tl[kTlChunks * 32];  // (read in groups of up to four entries with one vector load)
   float ref[2][128];       // the rows' reference, from the group that met the first tile to the other
   float xch[2][8][128];    // the rows' partial sums at the end of an item (two sets, used in turn):
@@ -51,6 +53,14 @@ struct PairControl {
   int abort_flag;
   int ovf_unit;
 };
+
+// Key blocks of a unit in the dense modes.
+__device__ __forceinline__ void pair_key_range(const Params& p, uint32_t ent, int& jlo, int& jhi) {
+  const int part = (ent & kTlPartial) ? (int)((ent >> 24) & 7u) : 0;
+  const int parts = (ent & kTlPartial) ? p.split_parts : 1;
+  jlo = (int)(((int64_t)p.nKb * part) / parts);
+  jhi = (int)(((int64_t)p.nKb * (part + 1)) / parts);
+}
 
 #define PAIR_WAIT_CL(bar, parity)                                                          \
   do {                                                                                     \
@@ -61,69 +71,54 @@ struct PairControl {
     }                                                                                      \
   } while (0)
 
-// The pair kernel's tile list is made of GROUPS of kG = 128 / C entries, each aligned to its size:
-// a K/V tile's key blocks, or an item header / end marker followed by filler.  A group is read
-// with one vector load (whole warp); a consumed chunk of 32 entries is handed back to the
-// scheduler of the first CTA.
-#define PAIR_TL_NEXT_TILE(grp, more)                                                       \
+// What the roles are told.  Per work unit the scheduler of the first CTA publishes a header in both
+// CTAs: the item, and a word with the number of K/V tiles (kHdrTiles), which of the two query tiles
+// lists any (kHdrHas), and whether query tile 1 lists its first one in the unit's second tile instead
+// of its first (kHdrLate).  The dense modes need no more: a unit's tiles follow from its share of the
+// key range.  In the sparse mode the unit's tile list follows in chunks of 32 entries - GROUPS of
+// kG = 128 / C, one per K/V tile, a unit beginning with a chunk of its own - which only the producers
+// and the softmax warps read, the latter only the tiles they work on.  (When every warp walked one
+// list of headers and tiles entry by entry, in the dense modes too, that took more instructions per
+// tile than the exponentials: 529 warp instructions per 64 scores of a warp, 224 of them arithmetic.)
+//
+// Next header (whole warp); `nu` is the warp's unit counter.
+#define PAIR_HDR_NEXT(ent, word)                                                           \
   do {                                                                                     \
-    const uint32_t c_ = (te >> 5) & (kTlChunks - 1);                                       \
-    if ((te & 31) == 0) PAIR_WAIT_CL(&ctl->tl_full[c_], (te / (kTlChunks * 32)) & 1);      \
-    ptx::ld_shared_volatile_vec<kG>(&ctl->tl[te & (kTlChunks * 32 - 1)], (grp));           \
-    if ((te & 31) == 32 - kG) {                                                            \
-      __syncwarp();                                                                        \
-      if (lane == 0) ptx::mbar_arrive_cluster(tl_empty0 + 8u * c_);                        \
-    }                                                                                      \
-    te += kG;                                                                              \
-    (more) = ((grp)[0] >> 28) == 0;                                                        \
-  } while (0)
-
-// ... the first group of the list or of an item: its header
-#define PAIR_TL_NEXT(ent)                                                                  \
-  do {                                                                                     \
-    uint32_t hdr_[kG];                                                                     \
-    bool more_;                                                                            \
-    PAIR_TL_NEXT_TILE(hdr_, more_);                                                        \
-    (void)more_;                                                                           \
-    (ent) = hdr_[0];                                                                       \
-  } while (0)
-
-// Scheduler of the first CTA: publish a chunk in both CTAs.
-#define PAIR_TL_PUBLISH(chunk)                                                             \
-  do {                                                                                     \
-    ptx::mbar_arrive(&ctl->tl_full[(chunk)]);                                              \
-    ptx::mbar_arrive_cluster(tl_full1 + 8u * (chunk));                                     \
-  } while (0)
-
-// ... append n <= 32 entries at once, lane i holding entry i (whole warp)
-#define PAIR_TL_PUT_BULK(ent, n)                                                           \
-  do {                                                                                     \
-    const uint32_t first_ = te, last_ = te + (uint32_t)(n) - 1;                            \
-    if ((first_ & 31) == 0)                                                                \
-      LOSA_WAIT_RELAXED(&ctl->tl_empty[(first_ >> 5) & (kTlChunks - 1)],                \
-                           ((first_ / (kTlChunks * 32)) & 1) ^ 1);                         \
-    if ((last_ >> 5) != (first_ >> 5))                                                     \
-      LOSA_WAIT_RELAXED(&ctl->tl_empty[(last_ >> 5) & (kTlChunks - 1)],                 \
-                           ((last_ / (kTlChunks * 32)) & 1) ^ 1);                          \
-    if (lane < (n)) {                                                                      \
-      const uint32_t i_ = (first_ + lane) & (kTlChunks * 32 - 1);                          \
-      ctl->tl[i_] = (ent);                                                                 \
-      ptx::st_cluster_u32(tl1 + 4u * i_, (ent));                                           \
-    }                                                                                      \
-    ptx::fence_acq_rel_cluster();                                                          \
+    const uint32_t s_ = nu & 1u;                                                           \
+    PAIR_WAIT_CL(&ctl->hdr_full[s_], (nu >> 1) & 1u);                                      \
+    uint32_t h_[2];                                                                        \
+    ptx::ld_shared_volatile_vec<2>(&ctl->hdr[s_].x, h_);                                   \
     __syncwarp();                                                                          \
-    if (lane == 0) {                                                                       \
-      if ((last_ >> 5) != (first_ >> 5)) PAIR_TL_PUBLISH((first_ >> 5) & (kTlChunks - 1)); \
-      if ((last_ & 31) == 31) PAIR_TL_PUBLISH((last_ >> 5) & (kTlChunks - 1));             \
-    }                                                                                      \
-    te += (uint32_t)(n);                                                                   \
+    if (lane == 0) ptx::mbar_arrive_cluster(hdr_empty0 + 8u * s_);                         \
+    (ent) = h_[0];                                                                         \
+    (word) = h_[1];                                                                        \
+    ++nu;                                                                                  \
   } while (0)
 
-// ... append an item header or the end marker: a group of its own, filled up with padding entries
-#define PAIR_TL_PUT(ent)                                                                   \
+// Chunk `nc` of the tile lists: wait for it, hand it back (whole warp).
+#define PAIR_CHUNK_WAIT() PAIR_WAIT_CL(&ctl->tl_full[nc & (kTlChunks - 1)], (nc / kTlChunks) & 1u)
+#define PAIR_CHUNK_DONE()                                                                  \
   do {                                                                                     \
-    const uint32_t e_ = (lane == 0) ? (uint32_t)(ent) : kTlPad;                            \
-    PAIR_TL_PUT_BULK(e_, kG);                                                              \
+    __syncwarp();                                                                          \
+    if (lane == 0) ptx::mbar_arrive_cluster(tl_empty0 + 8u * (nc & (kTlChunks - 1)));      \
+    ++nc;                                                                                  \
+  } while (0)
+
+// Scheduler of the first CTA: publish a header in both CTAs.
+#define PAIR_HDR_PUT(ent, word)                                                            \
+  do {                                                                                     \
+    const uint32_t s_ = nu & 1u;                                                           \
+    LOSA_WAIT_RELAXED(&ctl->hdr_empty[s_], ((nu >> 1) & 1u) ^ 1u);                         \
+    if (lane == 0) {                                                                       \
+      ctl->hdr[s_] = make_uint2((ent), (word));                                            \
+      ptx::st_cluster_u32(hdr1 + 8u * s_, (ent));                                          \
+      ptx::st_cluster_u32(hdr1 + 8u * s_ + 4u, (word));                                    \
+      ptx::fence_acq_rel_cluster();                                                        \
+      ptx::mbar_arrive(&ctl->hdr_full[s_]);                                                \
+      ptx::mbar_arrive_cluster(hdr_full1 + 8u * s_);                                       \
+    }                                                                                      \
+    __syncwarp();                                                                          \
+    ++nu;                                                                                  \
   } while (0)
 
 template <int C_, int MODE>
@@ -142,6 +137,7 @@ losa_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   constexpr bool kWantMass = (MODE == kFused || MODE == kMass);  // the block masses (Eq. 1) are wanted
   // the mass pass alone has no V, no P and no O: its score buffers go back as soon as they are read
   constexpr bool kHasV = (MODE != kMass);
+  constexpr int kChunkTiles = (MODE == kSparse) ? 32 / kG : (1 << 28);  // K/V tiles per chunk of the list
   static_assert(offsetof(PairControl, tl) % 16 == 0, "the tile list is read with 16-byte loads");
 
   extern __shared__ __align__(1024) uint8_t smem_raw[];
@@ -165,6 +161,9 @@ losa_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   const uint32_t o_free0 = ptx::mapa(ptx::smem_u32(&ctl->o_free), 0);
   const uint32_t tl_empty0 = ptx::mapa(ptx::smem_u32(&ctl->tl_empty[0]), 0);
   const uint32_t tl_full1 = ptx::mapa(ptx::smem_u32(&ctl->tl_full[0]), 1);
+  const uint32_t hdr_empty0 = ptx::mapa(ptx::smem_u32(&ctl->hdr_empty[0]), 0);
+  const uint32_t hdr_full1 = ptx::mapa(ptx::smem_u32(&ctl->hdr_full[0]), 1);
+  const uint32_t hdr1 = ptx::mapa(ptx::smem_u32(&ctl->hdr[0]), 1);
   const uint32_t tl1 = ptx::mapa(ptx::smem_u32(&ctl->tl[0]), 1);
   const uint32_t abort_peer = ptx::mapa(ptx::smem_u32(&ctl->abort_flag), rank ^ 1u);
 
@@ -188,9 +187,13 @@ losa_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     ptx::mbar_init(&ctl->o_free, 32);  // every softmax warp of both CTAs reads a quarter of its rows' O
     for (int i = 0; i < kTlChunks; ++i) {
       ptx::mbar_init(&ctl->tl_full[i], 1);
-      // readers: first CTA producer, two issuers, 16 softmax warps; second CTA producer, 16 softmax warps
-      ptx::mbar_init(&ctl->tl_empty[i], 19 + 17);
+      ptx::mbar_init(&ctl->tl_empty[i], 2 * 17);  // readers: each CTA's producer and 16 softmax warps
     }
+    for (int i = 0; i < 2; ++i) {
+      ptx::mbar_init(&ctl->hdr_full[i], 1);
+      ptx::mbar_init(&ctl->hdr_empty[i], 2 * 17 + 2);  // ... and the two issuers
+    }
+    ptx::mbar_init(&ctl->hdr_next, 1);  // the first CTA's producer, near the end of a unit
     for (int i = 0; i < 8; ++i) ptx::mbar_init(&ctl->pair_bar[i], 2);
     for (int i = 0; i < 2; ++i) {
       ptx::mbar_init(&ctl->ref_full[i], 4);   // the first halves' warps of the group that sets it
@@ -241,10 +244,11 @@ losa_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     if (ctl->abort_flag) goto teardown;
     if (warp == kProducerWarp) {
       // ------------------------------------------------------------------ TMA producer (both CTAs)
-      uint32_t nq = 0, nk = 0, nv = 0, te = 0, ent;
+      uint32_t nq = 0, nk = 0, nv = 0, nu = 0, nc = 0, ent, word;
       int problem = -1;  // batched launch: whose tensor maps this warp has acquired
-      PAIR_TL_NEXT(ent);
-      while ((ent >> 28) == 1) {
+      for (;;) {
+        PAIR_HDR_NEXT(ent, word);
+        if ((ent >> 28) != 1) break;
         const int w = (int)(ent & kTlItemMask);
         const int pbh = w / p.nPairs, pr = w % p.nPairs;
         const int bh = pbh % (p.B * p.H);
@@ -272,13 +276,23 @@ losa_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           ptx::tma_load_4d_pair(sQ + 16384, mq, q_full0, 64, T * 128, h, b);
         }
         ++nq;
-        for (;;) {
+        const int tiles = (int)(word & kHdrTiles);
+        int jlo, jhi;  // dense modes: the unit's key blocks
+        pair_key_range(p, ent, jlo, jhi);
+        // the scheduler draws the next unit when this one is 16 tiles from its end
+        const int call_at = max(0, tiles - 16);
+        if (tiles == 0 && rank == 0 && lane == 0) ptx::mbar_arrive(&ctl->hdr_next);
+        for (int base = 0; base < tiles; base += kChunkTiles) {
+        if (MODE == kSparse) PAIR_CHUNK_WAIT();
+        const int end = min(tiles, base + kChunkTiles);
+        for (int i = base; i < end; ++i) {
+          if (i == call_at && rank == 0 && lane == 0) ptx::mbar_arrive(&ctl->hdr_next);
           uint32_t grp[kG];
-          bool more;
-          PAIR_TL_NEXT_TILE(grp, more);
-          if (!more) {
-            ent = grp[0];
-            break;
+          if (MODE == kSparse) {
+            ptx::ld_shared_volatile_vec<kG>(&ctl->tl[(nc & (kTlChunks - 1)) * 32 + (i - base) * kG], grp);
+          } else {
+#pragma unroll
+            for (int g = 0; g < kG; ++g) grp[g] = (jlo + i * kG + g < jhi) ? (uint32_t)(jlo + i * kG + g) : kTlPad;
           }
           // K: keys 64 * rank ... + 63 of the tile, all 128 head-dimension columns (two slabs)
           const uint32_t ks = nk % kPairNK;
@@ -336,6 +350,8 @@ losa_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           }
           ++nv;
         }
+        if (MODE == kSparse) PAIR_CHUNK_DONE();
+        }
       }
     } else if (warp == kIssuerWarp && rank == 0) {
       // ------------------------------------------------------------------ S = Q K^T of the pair
@@ -348,18 +364,12 @@ losa_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
 #pragma unroll
       for (int kk = 0; kk < D / 16; ++kk)
         qd[kk] = ptx::smem_desc_lo(ptx::smem_u32(sQ), 16) + (((kk >> 2) * 16384 + (kk & 3) * 32) >> 4);
-      uint32_t nq = 0, nt = 0, te = 0, ent;
-      PAIR_TL_NEXT(ent);
-      while ((ent >> 28) == 1) {
+      uint32_t nq = 0, nt = 0, nu = 0, ent, word;
+      for (;;) {
+        PAIR_HDR_NEXT(ent, word);
+        if ((ent >> 28) != 1) break;
         bool q_ready = false;
-        for (;;) {
-          uint32_t grp[kG];
-          bool more;
-          PAIR_TL_NEXT_TILE(grp, more);
-          if (!more) {
-            ent = grp[0];
-            break;
-          }
+        for (int i = (int)(word & kHdrTiles); i > 0; --i) {
           const uint32_t ks = nt % kPairNK;
           LOSA_WAIT(&ctl->k_full[ks], (nt / kPairNK) & 1);
           if (!q_ready) {
@@ -398,19 +408,12 @@ losa_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       constexpr uint32_t kDescHi = ptx::smem_desc_hi_sw128(1024);
       const uint32_t v_lo = ptx::smem_desc_lo(ptx::smem_u32(sV), kPairStage);
       const uint32_t tO = tmem_base + 384;
-      uint32_t nof = 0, nt = 0, te = 0, ent;
-      PAIR_TL_NEXT(ent);
-      while ((ent >> 28) == 1) {
+      uint32_t nof = 0, nt = 0, nu = 0, ent, word;
+      for (;;) {
+        PAIR_HDR_NEXT(ent, word);
+        if ((ent >> 28) != 1) break;
         uint32_t pv_item = 0;
-        for (;;) {
-          uint32_t grp[kG];
-          bool more;
-          PAIR_TL_NEXT_TILE(grp, more);
-          if (!more) {
-            ent = grp[0];
-            break;
-          }
-          if (!kHasV) continue;  // (mass pass: this warp only hands the list's chunks back)
+        for (int i = kHasV ? (int)(word & kHdrTiles) : 0; i > 0; --i) {  // (the mass pass has no products)
           const uint32_t vs = nt % kPairNV;
           LOSA_WAIT(&ctl->v_full[vs], (nt / kPairNV) & 1);
           const uint32_t bsel = nt % 3u;
@@ -438,7 +441,7 @@ losa_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       }
     } else if (warp == kSchedulerWarp && rank == 0) {
       // ------------------------------------------------------------------ scheduler of the pair
-      uint32_t te = 0;
+      uint32_t nu = 0, nc = 0;
       bool first_item = true;
       for (;;) {
         if (p.stall) break;  // diagnostic launch: nothing is published and every wait runs out
@@ -460,38 +463,35 @@ losa_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         }
         const int unit = (flags != 0) ? p.split_first + (w - p.split_first) * parts + part : w;
         const int pr = w % p.nPairs;
-        PAIR_TL_PUT(kTlItem | flags | (uint32_t)w);
         if (MODE == kSparse) {
-          const int cnt = LOSA_IN_RANGE(unit, p.cap_units) ? min(__ldcg(p.tl_count + unit), p.tl_cap) : 0;
+          const uint32_t word = LOSA_IN_RANGE(unit, p.cap_units) ? (uint32_t)__ldcg(p.tl_count + unit) : 0u;
+          const int cnt = min((int)(word & kHdrTiles) * kG, p.tl_cap);
+          PAIR_HDR_PUT(kTlItem | flags | (uint32_t)w, (word & ~kHdrTiles) | (uint32_t)(cnt / kG));
           const uint32_t* src = p.tl_entries + (int64_t)unit * p.tl_cap;
           for (int base = 0; base < cnt; base += 32) {
-            const int n = min(32, cnt - base);
-            const uint32_t e = (lane < n) ? __ldcg(src + base + lane) : 0u;
-            PAIR_TL_PUT_BULK(e, n);
+            const uint32_t e = (base + lane < cnt) ? __ldcg(src + base + lane) : 0u;
+            const uint32_t c = nc & (kTlChunks - 1);
+            LOSA_WAIT_RELAXED(&ctl->tl_empty[c], ((nc / kTlChunks) & 1u) ^ 1u);
+            ctl->tl[c * 32 + lane] = e;
+            ptx::st_cluster_u32(tl1 + 4u * (c * 32 + lane), e);
+            ptx::fence_acq_rel_cluster();
+            __syncwarp();
+            if (lane == 0) {
+              ptx::mbar_arrive(&ctl->tl_full[c]);
+              ptx::mbar_arrive_cluster(tl_full1 + 8u * c);
+            }
+            ++nc;
           }
-          continue;
+        } else {
+          const uint32_t ent = kTlItem | flags | (uint32_t)w;
+          int jlo, jhi;
+          pair_key_range(p, ent, jlo, jhi);
+          const uint32_t has = (2 * pr + 1 < p.nQb) ? 3u * kHdrHas : kHdrHas;
+          PAIR_HDR_PUT(ent, has | (uint32_t)((jhi - jlo + kG - 1) / kG));
         }
-        uint32_t memb = 0;
-#pragma unroll
-        for (int n = 0; n < 2; ++n)
-          if (2 * pr + n < p.nQb) memb |= 1u << n;
-        const int jlo = (int)(((int64_t)p.nKb * part) / parts);
-        const int jhi = (int)(((int64_t)p.nKb * (part + 1)) / parts);
-        const int cnt = (jhi - jlo + kG - 1) / kG * kG;
-        for (int base = 0; base < cnt; base += 32) {
-          const int n = min(32, cnt - base);
-          const int j = jlo + base + lane;
-          const uint32_t e = (j < jhi) ? ((uint32_t)j | (memb << 16)) : kTlPad;
-          PAIR_TL_PUT_BULK(e, n);
-        }
+        LOSA_WAIT_RELAXED(&ctl->hdr_next, (nu - 1u) & 1u);
       }
-      if (!p.stall) {
-        PAIR_TL_PUT(kTlEnd);
-        if ((te & 31) != 0) {  // publish the last, partly filled chunk
-          __syncwarp();
-          if (lane == 0) PAIR_TL_PUBLISH(((te - 1) >> 5) & (kTlChunks - 1));
-        }
-      }
+      if (!p.stall) PAIR_HDR_PUT(kTlEnd, 0u);
     }
   } else {
     // ------------------------------------------------------------------ softmax warps (both CTAs)
@@ -507,7 +507,7 @@ losa_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     constexpr int kBW = 64 / kHB;                // columns per such block
     uint64_t* const pair_bar = &ctl->pair_bar[grpi * 4 + wl];
     const int quarter = grpi * 2 + half;         // which 32 columns of O this thread writes out
-    uint32_t kq = 0, nod = 0, npair = 0, nitem = 0, nref = 0, nfold = 0, te = 0, ent;
+    uint32_t kq = 0, nod = 0, npair = 0, nitem = 0, nref = 0, nfold = 0, nu = 0, nc = 0, ent, word;
     // fused step: this row's column of the CTA's table of per-block sums of the unrounded
     // exponentials (one float per row and 64-column half of a key tile when a key block fills the
     // tile, else one per row and key block)
@@ -515,8 +515,9 @@ losa_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
                                         (int64_t)blockIdx.x * 2 * (int64_t)p.nKb * 256 + row
                                   : nullptr;
 
-    PAIR_TL_NEXT(ent);
-    while ((ent >> 28) == 1) {
+    for (;;) {
+      PAIR_HDR_NEXT(ent, word);
+      if ((ent >> 28) != 1) break;
       const int w = (int)(ent & kTlItemMask);
       const bool partial = (ent & kTlPartial) != 0;
       const int part = (int)((ent >> 24) & 7u);
@@ -527,104 +528,113 @@ losa_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       const int T = 2 * pr + (int)rank;
       const int grow = T * 128 + row;
       float m_ref = 0.f, l = 0.f, le = 0.f;  // le: row sum of the unrounded exponentials (masses, LSE)
-      // the reference of the item: set by the group that meets the first key tile this query tile
-      // lists, taken over by the other group at its own first such tile (or dropped at the item's end)
-      bool item_ref = false, have_ref = false, ref_mine = false, ovf = false;
-      uint32_t pv_item = 0;
-      for (;;) {
-        uint32_t grp[kG];
-        bool more;
-        PAIR_TL_NEXT_TILE(grp, more);
-        if (!more) {
-          ent = grp[0];
-          break;
-        }
-        bool member = false;
+      bool ovf = false;
+      const int tiles = (int)(word & kHdrTiles);
+      const uint32_t pv_item = (uint32_t)tiles;
+      // does this query tile list any of the unit's tiles?  (R = 128: a query tile is a query block)
+      const bool has = (word & (kHdrHas << my_bit)) != 0;
+      // dense modes: the unit's key blocks, the end of its keys
+      int jlo, jhi;
+      pair_key_range(p, ent, jlo, jhi);
+      const int kend = min(p.N, jhi * kC);
+      // Score k of the launch (kq: of the unit's first tile) is worked on by group k % 2 and lies in
+      // buffer k % 3, in that buffer's use k / 3.
+      const int first = (grpi ^ (int)kq) & 1;
+      uint32_t bsel = (kq + (uint32_t)first) % 3u, sph = ((kq + (uint32_t)first) / 3u) & 1u;
+      // ---- the reference of the unit: the rows' maximum over the first key tile this query tile
+      // lists, from the group that works on that tile - it is that group's first tile - to the other
+      if (has) {
+        const int late = (my_bit == 1 && (word & kHdrLate)) ? 1 : 0;
+        const uint32_t rs = nref & 1u;
+        if (first == late) {
+          if (MODE == kSparse) PAIR_CHUNK_WAIT();
+          uint32_t grp[kG];
+          if (MODE == kSparse) ptx::ld_shared_volatile_vec<kG>(&ctl->tl[(nc & (kTlChunks - 1)) * 32 + first * kG], grp);
+          LOSA_WAIT(&ctl->s_full[bsel], sph);
+          ptx::tc_fence_after_sync();
+          const uint32_t tSrow = tmem_base + lane_base + bsel * 128;
+          float mx = -INFINITY;
 #pragma unroll
-        for (int g = 0; g < kG; ++g) member = member || ((grp[g] >> (16 + my_bit)) & 1u);
-        const bool first_member = member && !item_ref;
-        if (first_member) {
-          item_ref = true;
-          ref_mine = ((int)(kq & 1u) == grpi);
-        }
-        const uint32_t bsel = kq % 3u, sph = (kq / 3u) & 1u;
-        const bool my_tile = ((int)(kq & 1u) == grpi);
-        ++kq;
-        ++pv_item;
-        if (!my_tile) continue;
-        // hv[i]: how many columns of block i of this half the row attends to
-        int hv[kHB];
-        bool mine = false, whole = true;
+          for (int c0 = 0; c0 < kW; c0 += 32) {
+            uint32_t r[32];
+            ptx::tmem_ld32(tSrow + c0, r);
+            ptx::tmem_wait_ld();
 #pragma unroll
-        for (int i = 0; i < kHB; ++i) {
-          const int g = (kG >= 2) ? half * kHB + i : 0;
-          const int jg = (int)(grp[g] & 0xffffu);
-          const int valid = ((grp[g] >> (16 + my_bit)) & 1u) ? min(kC, p.N - jg * kC) : 0;
-          hv[i] = (kG >= 2) ? valid : max(0, min(64, valid - 64 * half));
-          mine = mine || hv[i] > 0;
-          whole = whole && hv[i] == kBW;
+            for (int c = 0; c < 32; ++c) {
+              const int cc = c0 + c;
+              int valid;  // of the key block's columns
+              if (MODE == kSparse)
+                valid = ((grp[cc / kC] >> (16 + my_bit)) & 1u) ? p.N - (int)(grp[cc / kC] & 0xffffu) * kC : 0;
+              else
+                valid = kend - (jlo + first * kG + cc / kC) * kC;
+              if ((cc % kC) < valid) mx = fmaxf(mx, __uint_as_float(r[c]));
+            }
+          }
+          m_ref = mx * p.scale_log2;
+          // the other half reads the whole row too: nobody packs P over it before both are done
+          ptx::tc_fence_before_sync();
+          __syncwarp();
+          if (lane == 0) ptx::mbar_arrive(pair_bar);
+          LOSA_WAIT(pair_bar, npair & 1);
+          ++npair;
+          ptx::tc_fence_after_sync();
+          if (half == 0) {
+            // (the slot's last readers, two units with a reference ago, are done with it)
+            if (nref >= 2u) LOSA_WAIT(&ctl->ref_empty[rs], ((nref >> 1) - 1u) & 1);
+            ctl->ref[rs][row] = m_ref;
+            __syncwarp();
+            if (lane == 0) ptx::mbar_arrive(&ctl->ref_full[rs]);
+          }
+        } else {
+          LOSA_WAIT(&ctl->ref_full[rs], (nref >> 1) & 1);
+          m_ref = ctl->ref[rs][row];
+          __syncwarp();
+          if (lane == 0) ptx::mbar_arrive(&ctl->ref_empty[rs]);
         }
-        const uint32_t tSrow = tmem_base + lane_base + bsel * 128;
-        const uint32_t tS = tSrow + half * 64;
+        ++nref;
+      }
+      const float2 sc2 = make_float2(p.scale_log2, p.scale_log2);
+      for (int base = 0; base < tiles; base += kChunkTiles) {
+      if (MODE == kSparse) PAIR_CHUNK_WAIT();
+      const int end = min(tiles, base + kChunkTiles);
+      for (int i = base + first; i < end; i += 2) {
+        // the key blocks of this half of the tile: a half block (C = 128), one block, or two (C = 32)
+        uint32_t own[kHB];
+        bool mine, ragged;  // the row attends to some of the half's keys; not all of them exist
+        if (MODE == kSparse) {
+          const uint32_t* e = &ctl->tl[(nc & (kTlChunks - 1)) * 32 + (i - base) * kG + ((kG >= 2) ? half * kHB : 0)];
+          ptx::ld_shared_volatile_vec<kHB>(e, own);
+          uint32_t any = 0u;
+#pragma unroll
+          for (int j = 0; j < kHB; ++j) any |= ((own[j] >> (16 + my_bit)) & 1u) ? own[j] : 0u;
+          ragged = (any & kTlRagged) != 0u;
+          mine = any != 0u;
+          if (kG == 1 && ragged) mine = p.N - (int)(own[0] & 0xffffu) * kC > 64 * half;
+        } else {
+          const int key0 = (jlo + i * kG) * kC + 64 * half;
+          mine = has && key0 < kend;
+          ragged = key0 + 64 > kend;
+        }
+        const uint32_t tS = tmem_base + lane_base + bsel * 128 + half * 64;
         LOSA_WAIT(&ctl->s_full[bsel], sph);
         ptx::tc_fence_after_sync();
-        if (member && !have_ref) {
-          const uint32_t rs = nref & 1u;
-          if (first_member) {
-            // the row's maximum over the keys it attends to in this tile, computed by both halves
-            float mx = -INFINITY;
-#pragma unroll
-            for (int c0 = 0; c0 < kW; c0 += 32) {
-              uint32_t r[32];
-              ptx::tmem_ld32(tSrow + c0, r);
-              ptx::tmem_wait_ld();
-#pragma unroll
-              for (int c = 0; c < 32; ++c) {
-                const int cc = c0 + c;
-                const int jg = (int)(grp[cc / kC] & 0xffffu);
-                const int valid = ((grp[cc / kC] >> (16 + my_bit)) & 1u) ? min(kC, p.N - jg * kC) : 0;
-                if ((cc % kC) < valid) mx = fmaxf(mx, __uint_as_float(r[c]));
-              }
-            }
-            m_ref = mx * p.scale_log2;
-            // the other half reads the whole row too: nobody packs P over it before both are done
-            ptx::tc_fence_before_sync();
-            __syncwarp();
-            if (lane == 0) ptx::mbar_arrive(pair_bar);
-            LOSA_WAIT(pair_bar, npair & 1);
-            ++npair;
-            ptx::tc_fence_after_sync();
-            if (half == 0) {
-              // (the slot's last readers, two items with a reference ago, are done with it)
-              if (nref >= 2u) LOSA_WAIT(&ctl->ref_empty[rs], ((nref >> 1) - 1u) & 1);
-              ctl->ref[rs][row] = m_ref;
-              __syncwarp();
-              if (lane == 0) ptx::mbar_arrive(&ctl->ref_full[rs]);
-            }
-          } else {
-            LOSA_WAIT(&ctl->ref_full[rs], (nref >> 1) & 1);
-            m_ref = ctl->ref[rs][row];
-            __syncwarp();
-            if (lane == 0) ptx::mbar_arrive(&ctl->ref_empty[rs]);
-          }
-          have_ref = true;
-        }
         uint32_t sr[64];
         if (mine) {
           ptx::tmem_ld32(tS, &sr[0]);
-          if (whole) ptx::tmem_wait_ld();
+          ptx::tmem_wait_ld();
           ptx::tmem_ld32(tS + 32, &sr[32]);
-          if (!whole) {
+          if (ragged) {
             // keys that do not exist (>= N, in the sequence's last key block): -inf column by column
             ptx::tmem_wait_ld();
-            bool ragged = false;
+            int hv[kHB];
 #pragma unroll
-            for (int i = 0; i < kHB; ++i) ragged = ragged || (hv[i] > 0 && hv[i] < kBW);
-            if (ragged) {
-#pragma unroll
-              for (int c = 0; c < 64; ++c)
-                if ((c % kBW) >= hv[c / kBW]) sr[c] = 0xff800000u;
+            for (int j = 0; j < kHB; ++j) {
+              if (MODE == kSparse) hv[j] = p.N - (int)(own[j] & 0xffffu) * kC - ((kG == 1) ? 64 * half : 0);
+              else hv[j] = kend - (jlo + i * kG) * kC - 64 * half - j * kBW;
             }
+#pragma unroll
+            for (int c = 0; c < 64; ++c)
+              if ((c % kBW) >= hv[c / kBW]) sr[c] = 0xff800000u;
           }
           if (!kHasV) {
             // mass pass: the scores are in registers and nothing is packed over them
@@ -634,22 +644,23 @@ losa_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
             if (lane == 0) ptx::mbar_arrive_cluster(p_ready0 + 8u * bsel);
           }
           // key blocks the row's query block does not list get -inf as the addend of the scaling FMA
-          const float2 sc2 = make_float2(p.scale_log2, p.scale_log2);
+          // (one block per half or less: the half would not be here)
           float2 nm2[kHB];
 #pragma unroll
-          for (int i = 0; i < kHB; ++i) {
-            const float a = (hv[i] > 0) ? -m_ref : -INFINITY;
-            nm2[i] = make_float2(a, a);
+          for (int j = 0; j < kHB; ++j) {
+            const bool listed = MODE != kSparse || kHB == 1 || ((own[j] >> (16 + my_bit)) & 1u);
+            const float a = listed ? -m_ref : -INFINITY;
+            nm2[j] = make_float2(a, a);
           }
           // The output is normalised by the sum of the weights the tensor core multiplies with V -
           // P as rounded to bf16 - so that o is a weighted mean of V whatever the rounding does.
           float2 racc[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
           float2 eacc[kHB];  // fused step: sums of the unrounded exponentials, per block of this half
 #pragma unroll
-          for (int i = 0; i < kHB; ++i) eacc[i] = make_float2(0.f, 0.f);
+          for (int j = 0; j < kHB; ++j) eacc[j] = make_float2(0.f, 0.f);
 #pragma unroll
           for (int c = 0; c < 64; c += 4) {
-            if (kHasV && whole && c == 32) ptx::tmem_wait_ld();
+            if (kHasV && c == 32) ptx::tmem_wait_ld();
             float2 x0 = ptx::fma2(make_float2(__uint_as_float(sr[c]), __uint_as_float(sr[c + 1])), sc2,
                                   nm2[c / kBW]);
             float2 x1 = ptx::fma2(make_float2(__uint_as_float(sr[c + 2]), __uint_as_float(sr[c + 3])), sc2,
@@ -672,19 +683,20 @@ losa_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           float tsum = (racc[0].x + racc[0].y) + (racc[1].x + racc[1].y);
           if (!kHasV) {
 #pragma unroll
-            for (int i = 0; i < kHB; ++i) tsum += eacc[i].x + eacc[i].y;
+            for (int j = 0; j < kHB; ++j) tsum += eacc[j].x + eacc[j].y;
           }
           ovf = ovf || __any_sync(0xffffffffu, !(tsum <= kSplitSafeSum));
           l += tsum;
           if (kHasV) ptx::tmem_st32(tS, &sr[0]);
           if (kWantMass) {
 #pragma unroll
-            for (int i = 0; i < kHB; ++i) {
-              const float es = eacc[i].x + eacc[i].y;
+            for (int j = 0; j < kHB; ++j) {
+              const float es = eacc[j].x + eacc[j].y;
               le += es;
-              const int g = (kG >= 2) ? half * kHB + i : 0;
-              const int64_t sb = (kG >= 2) ? (int64_t)(grp[g] & 0xffffu) : (int64_t)(grp[0] & 0xffffu) * 2 + half;
-              if (hv[i] > 0 && LOSA_IN_RANGE(sb * 128 + row, p.cap_table_floats)) tabf[sb * 128] = es;
+              // (kG = 1: entry of this half of the key block; else of the key block)
+              const int sb = (kG >= 2) ? jlo + i * kG + half * kHB + j : (jlo + i) * 2 + half;
+              const bool exists = kHB == 1 || sb < jhi;
+              if (exists && LOSA_IN_RANGE((int64_t)sb * 128 + row, p.cap_table_floats)) tabf[(int64_t)sb * 128] = es;
             }
           }
         } else {
@@ -701,9 +713,9 @@ losa_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
             if (lane == 0) ptx::mbar_arrive_cluster(p_ready0 + 8u * bsel);
           }
           // (a key block that fills the tile but ends before this half: its entry of the table is 0)
-          if (kWantMass && kG == 1 && member &&
-              LOSA_IN_RANGE(((int64_t)(grp[0] & 0xffffu) * 2 + half) * 128 + row, p.cap_table_floats))
-            tabf[((int64_t)(grp[0] & 0xffffu) * 2 + half) * 128] = 0.f;
+          if (kWantMass && kG == 1 && has &&
+              LOSA_IN_RANGE(((int64_t)(jlo + i) * 2 + half) * 128 + row, p.cap_table_floats))
+            tabf[((int64_t)(jlo + i) * 2 + half) * 128] = 0.f;
         }
         if (kHasV) {
           ptx::tmem_wait_st();
@@ -711,21 +723,19 @@ losa_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           __syncwarp();
           if (lane == 0) ptx::mbar_arrive_cluster(p_ready0 + 8u * bsel);
         }
+        // two scores on: k + 2 lies in the buffer before k's, in that buffer's next use, or in the last one
+        if (bsel == 0u) {
+          bsel = 2u;
+        } else {
+          bsel -= 1u;
+          sph ^= 1u;
+        }
       }
+      if (MODE == kSparse) PAIR_CHUNK_DONE();
+      }
+      kq += (uint32_t)tiles;
 
       // ---- end of the item
-      if (item_ref) {
-        if (!ref_mine && !have_ref) {
-          // this group met none of the tiles the query tile lists: it takes the reference here
-          // (a partial unit records it) and hands the slot back
-          const uint32_t rs = nref & 1u;
-          LOSA_WAIT(&ctl->ref_full[rs], (nref >> 1) & 1);
-          m_ref = ctl->ref[rs][row];
-          __syncwarp();
-          if (lane == 0) ptx::mbar_arrive(&ctl->ref_empty[rs]);
-        }
-        ++nref;
-      }
       // the four partial sums of a row (two groups, two halves) meet in shared memory
       float* const xset = &ctl->xch[nitem & 1][0][0];
       xset[quarter * 128 + row] = l;
@@ -868,9 +878,8 @@ teardown:
   }
 }
 
-#undef PAIR_TL_PUT
-#undef PAIR_TL_PUT_BULK
-#undef PAIR_TL_PUBLISH
-#undef PAIR_TL_NEXT_TILE
-#undef PAIR_TL_NEXT
+#undef PAIR_HDR_PUT
+#undef PAIR_HDR_NEXT
+#undef PAIR_CHUNK_WAIT
+#undef PAIR_CHUNK_DONE
 #undef PAIR_WAIT_CL

@@ -150,3 +150,25 @@ def test_two_streams_with_their_own_workspaces_do_not_disturb_each_other(Dh, Rq,
     for i in range(2):
         for o_s, o_d in results[i]:
             assert torch.equal(o_s, alone[i][0]) and torch.equal(o_d, alone[i][1])
+
+
+@pytest.mark.parametrize("C", [128, 64, 32])
+def test_tile_lists_that_end_around_a_chunk_of_the_list(C):
+    """A unit's tile list reaches the kernel in chunks of 32 entries (32 C / 128 K/V tiles), which its
+    two softmax groups read tile about: list lengths around one and two chunks, next to units of a
+    single tile, whole and (one head) cut into parts."""
+    losa = lib()
+    N = 128 * 70 - 37
+    nQb, nKb = -(-N // R), -(-N // C)
+    chunk = 32  # entries
+    lengths = [chunk - 1, chunk, chunk + 1, 1, 2 * chunk, 2 * chunk + 1, 2, 2 * chunk - 1, 3, chunk + 2]
+    for H in (2, 1):
+        lists = [range(g % 5, min(nKb, g % 5 + lengths[(g // 2 + g % 2) % len(lengths)])) for g in range(H * nQb)]
+        off, idx = csr_from(lists)
+        q, k, v = (util.rand_bf16((1, H, N, D), 950 + i, 1.0 if i == 2 else 2.0) for i in range(3))
+        o = losa.losa_sparse_attn(q.cuda(), k.cuda(), v.cuda(), torch.from_numpy(off).cuda(),
+                                  torch.from_numpy(idx).cuda(), R, C, out_dtype=torch.float32)
+        assert losa.losa_async_status() == 0
+        ref = orc.blocks_to_tokens(
+            orc.sparse_attn(util.to_np(q), util.to_np(k), util.to_np(v), R, C, off, idx), 1, H, N)
+        util.assert_output_close(o, ref, f"C={C} H={H}")
