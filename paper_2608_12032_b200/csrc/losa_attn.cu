@@ -20,12 +20,10 @@
 // partly filled wave of the persistent grid are cut into parts of their lists, merged by
 // the fallback launch.
 //
-// One S = Q K^T covers a whole K/V tile (128-wide MMAs).  At head dimension 128 TMEM holds exactly
-// S and O of both query tiles, P overwrites S, and per query tile the steps S -> softmax ->
-// O += P V -> next S form a serial chain; the two tiles run that chain half a period apart, one
-// issuer each, under a lock that keeps their bursts of MMAs from interleaving.  At head dimension
-// 64 a third S buffer fits and the tiles take the three buffers in turn (one issuer for all
-// S = Q K^T, one for all O += P V).  No mode keeps a running maximum on its common path: the
+// One S = Q K^T covers a whole K/V tile (128-wide MMAs).  TMEM holds exactly S and O of both query
+// tiles, P overwrites S, and per query tile the steps S -> softmax -> O += P V -> next S form a serial
+// chain; the two tiles run that chain half a period apart, one issuer each, under a lock that keeps
+// their bursts of MMAs from interleaving.  No mode keeps a running maximum on its common path: the
 // exponentials are taken against a reference that moves only when a tile's row sums leave the safe
 // range (one thread per row), or never within a work unit (two threads per row; units whose scores
 // outgrow it are recomputed by a second launch of the one-thread-per-row kernel).
@@ -33,10 +31,8 @@
 // Every wait is bounded; a wait that expires raises the CTA's abort flag, records
 // LOSA_ERR_TIMEOUT, and all roles leave through the common teardown that frees TMEM.
 //
-// The dense and sparse forward and the fused step at head dimension 128 with 128-row query blocks and
-// key blocks of 64 or 128 keys run in a second kernel, losa_pair_kernel (losa_attn_pair.cuh, included below): pairs
-// of CTAs that multiply together (tcgen05.mma.cta_group::2), one query tile and three S buffers per
-// CTA.  This kernel serves every other shape and mode and the fallback launch of all of them.
+// Head dimension 64, and head dimension 128 with 128-row query blocks, run in a second kernel,
+// losa_tile_kernel (losa_attn_tile.cuh, included below): one query tile and three S buffers per CTA.  This kernel serves the rest and the fallback launch of all.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <math.h>
@@ -53,16 +49,6 @@ namespace {
 #ifndef LOSA_USE_PAIR
 #define LOSA_USE_PAIR 1
 #endif
-#ifndef LOSA_PAIR_FUSED
-#define LOSA_PAIR_FUSED 1
-#endif
-#ifndef LOSA_PAIR_MASS
-#define LOSA_PAIR_MASS 1
-#endif
-#ifndef LOSA_PAIR_MIN_C
-#define LOSA_PAIR_MIN_C 32
-#endif
-
 std::atomic<uint32_t> g_stall_polls{0u};  // > 0: the next attention launch is a diagnostic one
 
 // Thread layout.  Warps 0-3 are the utility warpgroup (TMA, 2 MMA issuers, scheduler); the softmax
@@ -114,7 +100,11 @@ constexpr uint32_t kTlPad = 0xffffu;
 constexpr uint32_t kTlRagged = 1u << 20;  // tile entry: the sequence ends inside this key block
 // What is said of a unit's tile list: how many K/V tiles, which query tiles list any (kHdrHas << query
 // tile), and whether query tile 1 lists its first in the second K/V tile
-constexpr uint32_t kHdrTiles = 0x1fffffffu, kHdrLate = 1u << 29, kHdrHas = 1u << 30;
+// (a unit that is one query tile: bit kHdrHas alone, and which of the item's two it is, kHdrOdd)
+constexpr uint32_t kHdrTiles = 0x0fffffffu, kHdrOdd = 1u << 28, kHdrLate = 1u << 29, kHdrHas = 1u << 30;
+// Tile lists per work unit: one for its pair of query tiles, or (head dimension 64, where a CTA works on
+// one query tile at a time) one for each.
+__host__ __device__ constexpr int tile_lists_per_unit(int D) { return D == 64 ? 2 : 1; }
 constexpr int kMaxParts = 8;
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLn2 = 0.6931471805599453f;
@@ -123,7 +113,7 @@ constexpr float kSafeRowSum = 1.099511627776e12f;  // 2^40: a tile's row sum bey
 // two threads per row: a tile's half-row sum beyond 2^60 (or NaN) sends the work unit to the fallback
 constexpr float kSplitSafeSum = 1.152921504606846976e18f;
 
-template <int D, int R, int C_, int MODE, int KT, bool ROT = false>
+template <int D, int R, int C_, int MODE, int KT>
 struct Cfg {
   static constexpr int kC = C_;                       // keys per key block
   static constexpr int kT = KT;                       // keys per K/V tile: one S = Q K^T per tile
@@ -146,11 +136,9 @@ struct Cfg {
   static constexpr int kRingBudget = (kHasV ? 160 : 128) * 1024;  // K + V rings
   // a V tile stays in use about one tile longer than a K tile (its product is issued after the
   // tile's softmax), so V gets the deeper ring
-  // (rotating score buffers, head dimension 64: O += P V trails S = Q K^T by up to three steps, so
-  // a V tile is held that much longer while a K tile goes back at once: 7 V and 4 K stages of 16 KB)
-  static constexpr int kNV = ROT ? 7 : kHasV ? ((kKVBytes >= 32768) ? 3 : 4) : 0;
+  static constexpr int kNV = kHasV ? ((kKVBytes >= 32768) ? 3 : 4) : 0;
   static constexpr int kNK0 = (kRingBudget - kNV * kKVBytes) / kKVBytes;
-  static constexpr int kNK = ROT ? 4 : kNK0 > 6 ? 6 : kNK0;
+  static constexpr int kNK = kNK0 > 6 ? 6 : kNK0;
   static constexpr uint32_t kIdescQK = ptx::idesc_bf16_f32(128, kW, false, false);
   static constexpr uint32_t kIdescPV = ptx::idesc_bf16_f32(128, D, false, true);
 };
@@ -212,7 +200,7 @@ struct Params {
   int stall;            // diagnostic launch: the scheduler publishes nothing, so that every wait runs out
 };
 
-template <int NK, int NV, bool SPLIT, bool ROT>
+template <int NK, int NV, bool SPLIT>
 struct Control {
   uint64_t q_full[2], q_empty[2];
   uint64_t k_full[NK], k_empty[NK];
@@ -233,12 +221,6 @@ struct Control {
   uint64_t pair_bar[SPLIT ? 8 : 1];
   float xch[SPLIT ? 2 * 2 * 128 : 1];
   int ovf_unit;
-  // head dimension 64, two threads per row: three score buffers used in turn by both query tiles.
-  // One barrier per (query tile, buffer): a barrier's phases then follow one query tile's own
-  // sequence of tiles, so that its warps are never more than one phase away from it (they may be
-  // whole work units ahead of, or behind, the other query tile's warps).
-  uint64_t rot_s_full[ROT ? 6 : 1], rot_p_ready[ROT ? 6 : 1];
-  uint64_t pv_done[ROT ? 3 : 1];  // per buffer: the product that read its P has run
 };
 
 // Checked build (-DLOSA_CHECKED=1, a substitute for a memory checker): every index the kernels
@@ -427,17 +409,9 @@ __global__ void __launch_bounds__(Lay<SPLIT>::kThreads, 1)
 losa_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                  const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_kw,
                  const __grid_constant__ CUtensorMap map_vw, const Params p) {
-  using C = Cfg<D, R, C_, MODE, KT, SPLIT && D == 64 && MODE != kMass>;
+  using C = Cfg<D, R, C_, MODE, KT>;
   using L = Lay<SPLIT>;
-  using Ctl = Control<C::kNK, C::kNV, SPLIT, SPLIT && D == 64 && MODE != kMass>;
-  // Head dimension 64 leaves 128 tensor-memory columns unused (O takes 64 per query tile), enough
-  // for a third score buffer.  The two query tiles then take the three buffers in turn, in the
-  // order in which their S = Q K^T are issued, so that the S of a query tile's next key tile is
-  // computed while its current one is still being exponentiated: the softmax warps never wait for
-  // the tensor core.  One issuer warp issues every S = Q K^T of the CTA in that fixed order, the
-  // other every O += P V; a buffer is written again only after the product that read its P has
-  // completed (a barrier between the two issuers).
-  constexpr bool kRot = SPLIT && D == 64 && C::kHasV;
+  using Ctl = Control<C::kNK, C::kNV, SPLIT>;
   constexpr int kC = C::kC, kG = C::kG, kQBT = C::kQBT, kNB = C::kNB, kW = C::kW, kNS = C::kNS;
   constexpr uint32_t kSStride = C::kSStride, kNVs = C::kNV > 0 ? C::kNV : 1;
   constexpr uint32_t kQMask = (1u << kQBT) - 1u;
@@ -447,20 +421,6 @@ losa_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   // is slower, 5.6 and 5.8 ms: the loop turns issue-bound).  Not in the attention modes, which
   // wait on the chain of their steps, not on that unit (tried twice, slower each time).
   constexpr int kPolyEvery = (MODE == kMass) ? 4 : 0;
-#ifndef LOSA_SPLIT_POLY
-#define LOSA_SPLIT_POLY 1
-#endif
-#ifndef LOSA_SPLIT_POLY_OF
-#define LOSA_SPLIT_POLY_OF 8
-#endif
-  // Two threads per row, head dimension 64, modes with an attention output: one group of four
-  // scores in every eight (12.5 %) takes its exponentials from a polynomial on the FMA pipe.
-  // Measured at the CogVideoX shape: dense 5.57 -> 4.95 ms, sparse 4.96 -> 4.54 ms (6.25 % gives
-  // 5.02 / 4.58, 18.75 % 5.13 / 4.62, 25 % 5.35 / 4.81, 50 % 6.26 / 5.55), fused step 6.52 -> 6.38.
-  // At head dimension 128 the fused step gets 3 % slower with it, and has none.
-  constexpr int kSplitPoly = (SPLIT && C::kHasV && D == 64) ? LOSA_SPLIT_POLY : 0;
-  constexpr int kSplitPolyOf = LOSA_SPLIT_POLY_OF;
-
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   // (the swizzled tiles need 1024-byte alignment; the one-thread-per-row layout has room for the
   // slack, the other relies on the declared alignment and checks it)
@@ -517,13 +477,6 @@ losa_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     if (SPLIT) {
       for (int i = 0; i < 8; ++i) ptx::mbar_init(&ctl->pair_bar[i], 2);
       ctl->ovf_unit = -1;
-    }
-    if (kRot) {
-      for (int i = 0; i < 3; ++i) ptx::mbar_init(&ctl->pv_done[i], 1);
-      for (int i = 0; i < 6; ++i) {
-        ptx::mbar_init(&ctl->rot_s_full[i], 1);
-        ptx::mbar_init(&ctl->rot_p_ready[i], L::kSoftmaxWarps / 2);
-      }
     }
     ptx::mbar_init(&ctl->drain, 2);  // the MMA issuers arrive on the abort path
     ctl->mma_lock = 0;
@@ -655,135 +608,6 @@ losa_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
                                &ctl->v_full[vs], s * 64, r0, h, b);
             }
             ++nv;
-          }
-        }
-      }
-    }
-  } else if (kRot && warp == kIssuerWarp) {
-    // ------------------------------------------------------------------ rotating score buffers: the S = Q K^T issuer
-    // For every K/V tile of the list, for each query tile that lists it (query tile 0 first): the
-    // next score, number k, goes into buffer k % 3.  That buffer still holds the P of score
-    // k - 3 until its O += P V has run, which the other issuer warp signals (pv_done).
-    {
-      const bool leader = ptx::elect_one();
-      constexpr uint32_t kDescHi = ptx::smem_desc_hi_sw128(1024);
-      const uint32_t k_lo = ptx::smem_desc_lo(ptx::smem_u32(sK), 16);
-      const uint32_t q_lo = ptx::smem_desc_lo(ptx::smem_u32(sQ), 16);
-      uint32_t nq[2] = {0, 0}, nt = 0, te = 0, ent, kq = 0;
-      LOSA_TL_NEXT(ent);
-      while ((ent >> 28) == 1) {
-        bool q_ready[2] = {false, false};
-        const int pr_ = (int)(ent & kTlItemMask) % p.nPairs;
-        for (;;) {
-          uint32_t grp[kG];
-          bool more;
-          LOSA_TL_NEXT_TILE(grp, more);
-          if (!more) {
-            ent = grp[0];
-            break;
-          }
-          uint32_t memb = 0;
-#pragma unroll
-          for (int g = 0; g < kG; ++g) memb |= (grp[g] >> 16) & 0xfu;
-          const uint32_t ks = nt % C::kNK, kph = (nt / C::kNK) & 1;
-          LOSA_WAIT(&ctl->k_full[ks], kph);
-#pragma unroll
-          for (int qt = 0; qt < 2; ++qt) {
-            if (((memb >> (qt * kQBT)) & kQMask) != 0) {
-              if (!q_ready[qt]) {
-                LOSA_WAIT(&ctl->q_full[qt], nq[qt] & 1);
-                ++nq[qt];
-                q_ready[qt] = true;
-              }
-              const uint32_t b = kq % 3u;
-              if (kq >= 3u) LOSA_WAIT(&ctl->pv_done[b], (kq / 3u - 1u) & 1);
-              ptx::tc_fence_after_sync();
-              if (leader) {
-                const uint32_t qd0 = q_lo + qt * (C::kQBytes >> 4), kd0 = k_lo + ks * (C::kKVBytes >> 4);
-#pragma unroll
-                for (int kk = 0; kk < D / 16; ++kk)
-                  ptx::mma_ss_lo(tmem_base + b * 128, qd0 + (((kk >> 2) * C::kQSlab + (kk & 3) * 32) >> 4),
-                                 kd0 + (((kk >> 2) * C::kKVSlab + (kk & 3) * 32) >> 4), kDescHi,
-                                 C::kIdescQK, kk > 0 ? 1u : 0u);
-                ptx::mma_commit(&ctl->rot_s_full[qt * 3 + b]);
-                ptx::mma_commit(&ctl->k_empty[ks]);
-              }
-              ++kq;
-            } else {
-              if (leader) ptx::mbar_arrive(&ctl->k_empty[ks]);
-            }
-          }
-          ++nt;
-        }
-#pragma unroll
-        for (int qt = 0; qt < 2; ++qt) {
-          if (q_ready[qt]) {
-            if (leader) ptx::mma_commit(&ctl->q_empty[qt]);
-          } else if (2 * pr_ + qt < p.nQt) {
-            // no key tile of this unit was listed by the query tile: its buffer goes back unused
-            LOSA_WAIT(&ctl->q_full[qt], nq[qt] & 1);
-            ++nq[qt];
-            if (leader) ptx::mbar_arrive(&ctl->q_empty[qt]);
-          }
-        }
-      }
-    }
-  } else if (kRot && warp == kIssuerWarp + 1) {
-    // ------------------------------------------------------------------ rotating score buffers: the O += P V issuer
-    // Walks the same list in the same order; product k reads P from buffer k % 3 once the softmax
-    // warps of its query tile have packed it.
-    {
-      const bool leader = ptx::elect_one();
-      constexpr uint32_t kDescHi = ptx::smem_desc_hi_sw128(1024);
-      const uint32_t v_lo = ptx::smem_desc_lo(ptx::smem_u32(sV), C::kKVSlab);
-      uint32_t nof[2] = {0, 0}, uses[6] = {0, 0, 0, 0, 0, 0}, nt = 0, te = 0, ent, kp = 0;
-      LOSA_TL_NEXT(ent);
-      while ((ent >> 28) == 1) {
-        uint32_t pv_item[2] = {0, 0};
-        for (;;) {
-          uint32_t grp[kG];
-          bool more;
-          LOSA_TL_NEXT_TILE(grp, more);
-          if (!more) {
-            ent = grp[0];
-            break;
-          }
-          uint32_t memb = 0;
-#pragma unroll
-          for (int g = 0; g < kG; ++g) memb |= (grp[g] >> 16) & 0xfu;
-          const uint32_t vs = nt % kNVs, vph = (nt / kNVs) & 1;
-          LOSA_WAIT(&ctl->v_full[vs], vph);
-#pragma unroll
-          for (int qt = 0; qt < 2; ++qt) {
-            if (((memb >> (qt * kQBT)) & kQMask) != 0) {
-              const uint32_t b = kp % 3u;
-              if (pv_item[qt] == 0 && nof[qt] > 0) LOSA_WAIT(&ctl->o_free[qt], (nof[qt] - 1) & 1);
-              LOSA_WAIT(&ctl->rot_p_ready[qt * 3 + b], uses[qt * 3 + b] & 1);
-              ++uses[qt * 3 + b];
-              ptx::tc_fence_after_sync();
-              if (leader) {
-                const uint32_t tP = tmem_base + b * 128, tO = tmem_base + 384 + qt * 64;
-                const uint32_t vd0 = v_lo + vs * (C::kKVBytes >> 4);
-#pragma unroll
-                for (int kk = 0; kk < kW / 16; ++kk)
-                  ptx::mma_ts_lo(tO, tP + (kk & 3) * 8 + (kk >> 2) * 64, vd0 + kk * (2048 >> 4), kDescHi,
-                                 C::kIdescPV, (kk > 0 || pv_item[qt] > 0) ? 1u : 0u);
-                ptx::mma_commit(&ctl->pv_done[b]);
-                ptx::mma_commit(&ctl->v_empty[vs]);
-              }
-              ++pv_item[qt];
-              ++kp;
-            } else {
-              if (leader) ptx::mbar_arrive(&ctl->v_empty[vs]);
-            }
-          }
-          ++nt;
-        }
-#pragma unroll
-        for (int qt = 0; qt < 2; ++qt) {
-          if (pv_item[qt] > 0) {
-            if (leader) ptx::mma_commit(&ctl->o_done[qt]);  // every product of the item is done
-            ++nof[qt];
           }
         }
       }
@@ -1009,13 +833,18 @@ losa_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         // the unit's merged tile list was built before the launch: stream it into the ring,
         // 32 entries per step, so that this warp takes next to no issue slots from the softmax
         // warps of its scheduler partition
-        const int cnt = LOSA_IN_RANGE(unit, p.cap_units)
-                            ? min((int)((uint32_t)__ldcg(p.tl_count + unit) & kHdrTiles) * kG, p.tl_cap) : 0;
-        const uint32_t* src = p.tl_entries + (int64_t)unit * p.tl_cap;
-        for (int base = 0; base < cnt; base += 32) {
-          const int n = min(32, cnt - base);
-          const uint32_t e = (lane < n) ? __ldcg(src + base + lane) : 0u;
-          LOSA_TL_PUT_BULK(e, n);
+        // (head dimension 64: a list per query tile, one after the other)
+        constexpr int kLists = tile_lists_per_unit(D);
+        for (int t = 0; t < kLists; ++t) {
+          const int list = unit * kLists + t;
+          const int cnt = LOSA_IN_RANGE(list, p.cap_units)
+                              ? min((int)((uint32_t)__ldcg(p.tl_count + list) & kHdrTiles) * kG, p.tl_cap) : 0;
+          const uint32_t* src = p.tl_entries + (int64_t)list * p.tl_cap;
+          for (int base = 0; base < cnt; base += 32) {
+            const int n = min(32, cnt - base);
+            const uint32_t e = (lane < n) ? __ldcg(src + base + lane) : 0u;
+            LOSA_TL_PUT_BULK(e, n);
+          }
         }
         continue;
       }
@@ -1423,11 +1252,10 @@ losa_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     const int qt = sw >> 3, half = (sw >> 2) & 1, wl = sw & 3;  // TMEM lanes 32 * (warp % 4) .. + 31
     const int row = wl * 32 + lane;
     const uint32_t lane_base = (uint32_t)(wl * 32) << 16;
-    // the row's 128 score columns, and this half's 64 of them (its P goes over their first 32);
-    // with rotating buffers (head dimension 64) they change from tile to tile
+    // the row's 128 score columns, and this half's 64 of them (its P goes over their first 32)
     uint32_t tSrow = tmem_base + lane_base + qt * kSStride;
     uint32_t tS = tSrow + half * 64;
-    const uint32_t tO = tmem_base + lane_base + (kRot ? 384 + qt * 64 : 256 + qt * 128);
+    const uint32_t tO = tmem_base + lane_base + 256 + qt * 128;
     // fused construction step: this row's column of the CTA's table of per-block sums of the
     // unrounded exponentials, one float per row and 64-column half of a key tile when a key block
     // fills the tile (the halves' entries are added at the end), else one per row and key block
@@ -1435,8 +1263,6 @@ losa_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
                                            ((int64_t)blockIdx.x * 2 + qt) * (int64_t)p.nKb * 256 + row
                                      : nullptr;
     uint32_t nwg = 0;
-    uint32_t kq = 0;  // rotating buffers: scores issued so far, counted as the issuer counts them
-    uint32_t uses[3] = {0, 0, 0};  // ... and how many of them, per buffer, were this query tile's
     const int sub = (R == 64) ? (wl >> 1) : 0;
     const int my_bit = qt * kQBT + sub;
     constexpr int kHB = (kG >= 2) ? kG / 2 : 1;   // key blocks of a half (a half block when C = 128)
@@ -1485,33 +1311,15 @@ losa_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           mine = mine || hv[i] > 0;
           whole = whole && hv[i] == kBW;
         }
-        uint32_t rot_b = 0;
-        if (kRot) {
-          // the buffer follows from the tile's place in the issue order: per K/V tile, query tile 0
-          // first, then query tile 1, each only if it lists the tile
-          const bool m0 = (memb & kQMask) != 0, m1 = ((memb >> kQBT) & kQMask) != 0;
-          const uint32_t kmine = kq + ((qt == 1 && m0) ? 1u : 0u);
-          kq += (m0 ? 1u : 0u) + (m1 ? 1u : 0u);
-          if (!(qt == 0 ? m0 : m1)) continue;
-          rot_b = kmine % 3u;
-          tSrow = tmem_base + lane_base + rot_b * 128;
+        if (((memb >> (qt * kQBT)) & kQMask) == 0) continue;
+        // S of this key tile is complete, and so is every earlier product into O
+        // (the mass pass has two S buffers per query tile and no O)
+        const uint32_t buf = nsub % kNS;
+        if (!C::kHasV) {
+          tSrow = tmem_base + lane_base + qt * kSStride + buf * 128;
           tS = tSrow + half * 64;
-          const uint32_t par = (rot_b == 0 ? uses[0] : rot_b == 1 ? uses[1] : uses[2]) & 1;
-          uses[0] += (rot_b == 0);
-          uses[1] += (rot_b == 1);
-          uses[2] += (rot_b == 2);
-          LOSA_WAIT(&ctl->rot_s_full[qt * 3 + rot_b], par);
-        } else {
-          if (((memb >> (qt * kQBT)) & kQMask) == 0) continue;
-          // S of this key tile is complete, and so is every earlier product into O
-          // (the mass pass has two S buffers per query tile and no O)
-          const uint32_t buf = nsub % kNS;
-          if (!C::kHasV) {
-            tSrow = tmem_base + lane_base + qt * kSStride + buf * 128;
-            tS = tSrow + half * 64;
-          }
-          LOSA_WAIT(&ctl->s_full[qt][buf], (nsub / kNS) & 1);
         }
+        LOSA_WAIT(&ctl->s_full[qt][buf], (nsub / kNS) & 1);
         ptx::tc_fence_after_sync();
         if (!have_ref && pair_mine) {
           // the item's first tile for this row: the reference is the maximum of the row's scores
@@ -1585,15 +1393,10 @@ losa_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
                 make_float2(__uint_as_float(sr[c]), __uint_as_float(sr[c + 1])), sc2, nm2[c / kBW]);
             float2 x1 = ptx::fma2(
                 make_float2(__uint_as_float(sr[c + 2]), __uint_as_float(sr[c + 3])), sc2, nm2[c / kBW]);
-            if (kSplitPoly > 0 && (c >> 2) % kSplitPolyOf < kSplitPoly) {
-              x0 = ptx::ex2_poly2(x0);
-              x1 = ptx::ex2_poly2(x1);
-            } else {
-              x0.x = ptx::ex2_approx(x0.x);
-              x0.y = ptx::ex2_approx(x0.y);
-              x1.x = ptx::ex2_approx(x1.x);
-              x1.y = ptx::ex2_approx(x1.y);
-            }
+            x0.x = ptx::ex2_approx(x0.x);
+            x0.y = ptx::ex2_approx(x0.y);
+            x1.x = ptx::ex2_approx(x1.x);
+            x1.y = ptx::ex2_approx(x1.y);
             if (C::kHasV) {
               const uint32_t u0 = ptx::pack_bf16x2(x0.x, x0.y), u1 = ptx::pack_bf16x2(x1.x, x1.y);
               sr[c >> 1] = u0;
@@ -1644,7 +1447,7 @@ losa_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           ++pv_item;
           ptx::tc_fence_before_sync();
           __syncwarp();
-          if (lane == 0) ptx::mbar_arrive(kRot ? &ctl->rot_p_ready[qt * 3 + rot_b] : &ctl->p_ready[qt]);
+          if (lane == 0) ptx::mbar_arrive(&ctl->p_ready[qt]);
         }
         ++nsub;
       }
@@ -1823,7 +1626,7 @@ teardown:
   }
 }
 
-#include "losa_attn_pair.cuh"
+#include "losa_attn_tile.cuh"
 
 #undef LOSA_TL_PUT_BULK
 #undef LOSA_TL_NEXT_TILE
@@ -1845,13 +1648,16 @@ teardown:
 // One warp per list fills its bitmap (a list of a small layer is nothing but the latency of its two
 // dependent loads), then the first warp writes the tile list.  The first CTA also zeroes the
 // launch's counters.
-template <int NB, int G>
+// ONE: a list is that of one query tile of the unit (its NB query blocks), in ascending order.
+template <int NB, int G, bool ONE>
 __global__ void __launch_bounds__(32 * NB) build_tile_lists_kernel(const Params p) {
   extern __shared__ uint32_t bm[];  // [NB][W] bitmaps
   ptx::grid_launch_dependents();
   ptx::grid_dependency_wait();  // (batched launch: the table of the problems)
-  const int lane = threadIdx.x & 31, n = threadIdx.x >> 5, unit = blockIdx.x;
-  if (unit == 0 && threadIdx.x < kCounters) p.work_counter[threadIdx.x] = 0;
+  const int lane = threadIdx.x & 31, n = threadIdx.x >> 5;
+  const int list = blockIdx.x, unit = ONE ? list >> 1 : list;
+  const int bit0 = ONE ? (list & 1) * NB : 0;  // membership bit of the first query block
+  if (list == 0 && threadIdx.x < kCounters) p.work_counter[threadIdx.x] = 0;
   int w = unit, part = 0, parts = 1;
   if (unit >= p.split_first) {
     const int r = unit - p.split_first;
@@ -1870,7 +1676,7 @@ __global__ void __launch_bounds__(32 * NB) build_tile_lists_kernel(const Params 
   }
   const int W = (p.nKb + 31) >> 5;
   uint32_t* const mine = bm + n * W;
-  const int g = pr * NB + n;
+  const int g = pr * (ONE ? 2 * NB : NB) + bit0 + n;
   int b = 0, e = 0;
   if (g < p.nQb) {
     const int64_t row = (int64_t)bh * p.nQb + g;
@@ -1903,7 +1709,7 @@ __global__ void __launch_bounds__(32 * NB) build_tile_lists_kernel(const Params 
   // (K/V tile by K/V tile; a class that does not fill its last K/V tile pads it), then what is
   // left of the longer class.  Within a class the blocks ascend.  Correctness does not depend on
   // the order of the key blocks.
-  uint32_t* dst = p.tl_entries + (int64_t)unit * p.tl_cap;
+  uint32_t* dst = p.tl_entries + (int64_t)list * p.tl_cap;
   int nb = 0, na = 0, nbb = 0;  // both, tile 0 only, tile 1 only
   for (int w0 = 0; w0 < W; w0 += 32) {
     const int wi = w0 + lane;
@@ -1911,7 +1717,9 @@ __global__ void __launch_bounds__(32 * NB) build_tile_lists_kernel(const Params 
 #pragma unroll
     for (int n = 0; n < NB; ++n) {
       const uint32_t m = (wi < W) ? bm[n * W + wi] : 0u;
-      if (n < NB / 2) ta |= m; else tb |= m;
+      if (ONE) ta |= m, tb |= m;
+      else if (n < NB / 2) ta |= m;
+      else tb |= m;
     }
     nb += __popc(ta & tb);
     na += __popc(ta & ~tb);
@@ -1945,7 +1753,9 @@ __global__ void __launch_bounds__(32 * NB) build_tile_lists_kernel(const Params 
 #pragma unroll
     for (int n = 0; n < NB; ++n) {
       m[n] = (wi < W) ? bm[n * W + wi] : 0u;
-      if (n < NB / 2) ta |= m[n]; else tb |= m[n];
+      if (ONE) ta |= m[n], tb |= m[n];
+      else if (n < NB / 2) ta |= m[n];
+      else tb |= m[n];
     }
     uint32_t cls[3] = {ta & tb, ta & ~tb, tb & ~ta};
     int incl[3], tot[3];
@@ -1969,7 +1779,7 @@ __global__ void __launch_bounds__(32 * NB) build_tile_lists_kernel(const Params 
         u &= u - 1;
         uint32_t memb = 0;
 #pragma unroll
-        for (int n = 0; n < NB; ++n) memb |= ((m[n] >> bit) & 1u) << n;
+        for (int n = 0; n < NB; ++n) memb |= ((m[n] >> bit) & 1u) << (bit0 + n);
         const int pos = (k == 0) ? r : slot_of(k, r);
         const int j = wi * 32 + bit;
         if (pos < p.tl_cap) dst[pos] = (uint32_t)j | (memb << 16) | (j == ragged ? kTlRagged : 0u);
@@ -1981,7 +1791,7 @@ __global__ void __launch_bounds__(32 * NB) build_tile_lists_kernel(const Params 
     rbb += tot[2];
   }
   if (lane == 0)
-    p.tl_count[unit] = (int32_t)((uint32_t)(total / G) | ((nb + na > 0) ? kHdrHas : 0u) |
+    p.tl_count[list] = (int32_t)((uint32_t)(total / G) | ((nb + na > 0) ? kHdrHas : 0u) |
                                  ((nb + nbb > 0) ? 2u * kHdrHas : 0u) | ((nb == 0 && tmin > 0) ? kHdrLate : 0u));
 }
 
@@ -2090,9 +1900,9 @@ int launch(void (*kern)(P...), dim3 grid, int threads, size_t smem, cudaStream_t
 template <int D, int R, int C_, int MODE, int KT, bool SPLIT>
 int launch_kernel(const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv, const CUtensorMap& mkw,
                   const CUtensorMap& mvw, const Params& prm, int grid, cudaStream_t st) {
-  using C = Cfg<D, R, C_, MODE, KT, SPLIT && D == 64 && MODE != kMass>;
+  using C = Cfg<D, R, C_, MODE, KT>;
   using L = Lay<SPLIT>;
-  using Ctl = Control<C::kNK, C::kNV, SPLIT, SPLIT && D == 64 && MODE != kMass>;
+  using Ctl = Control<C::kNK, C::kNV, SPLIT>;
   // (one thread per row: 1024 bytes of slack to align the tiles; two threads per row: none left,
   // the kernel checks the alignment of its shared memory instead)
   const size_t smem = (SPLIT ? 0 : 1024) + 2 * C::kQBytes +
@@ -2119,44 +1929,49 @@ int launch_kernel(const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMa
   return launch(kern, dim3(grid), L::kThreads, smem, st, true, mq, mk, mv, mkw, mvw, prm);
 }
 
-// Configures (once per device) and launches the CTA-pair kernel on `clusters` pairs; *max_clusters
-// (if not null) receives how many pairs the device can hold at once.
-template <int C_, int MODE>
-int launch_pair(const CUtensorMap& mq, const CUtensorMap& mkh, const CUtensorMap& mv, const CUtensorMap& mk64,
+// Configures (once per device) and launches the tile kernel on `clusters` pairs of CTAs, or (PAIR =
+// false) as many CTAs; *max_clusters (if not null) receives how many the device can hold at once.
+template <int D, int R, int C_, int MODE, bool PAIR>
+int launch_tile(const CUtensorMap& mq, const CUtensorMap& mkh, const CUtensorMap& mv, const CUtensorMap& mk64,
                 const CUtensorMap& mv128, const Params& prm, int clusters, cudaStream_t st, int* max_clusters) {
   using L = Lay<true>;
-  constexpr size_t smem = kPairQBytes + (size_t)(kPairNK + kPairNV) * kPairStage + sizeof(PairControl);
+  constexpr size_t smem = 256 * D + (size_t)(kTileNK + kTileNV) * kTileStage + sizeof(TileControl);
   static_assert(smem <= 227 * 1024, "shared memory of one CTA");
-  auto kern = losa_pair_kernel<C_, MODE>;
+  auto kern = losa_tile_kernel<D, R, C_, MODE, PAIR>;
   static int max_on[kMaxDevices] = {};
   int dev = 0;
   LOSA_CUDA_TRY(cudaGetDevice(&dev));
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[2];
-  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[1].val.programmaticStreamSerializationAllowed = 1;
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = 2;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = 2;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
   cfg.blockDim = dim3(L::kThreads, 1, 1);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = PAIR ? 2 : 1;
   if (max_on[dev] == 0) {
     cudaFuncAttributes fa;
     LOSA_CUDA_TRY(cudaFuncGetAttributes(&fa, kern));
     if (fa.numRegs * L::kThreads < 128 * L::kRegsUtility + 32 * L::kSoftmaxWarps * L::kRegsSoftmax) {
-      set_cuda_error(cudaErrorLaunchOutOfResources, "register budget of losa_pair_kernel");
+      set_cuda_error(cudaErrorLaunchOutOfResources, "register budget of losa_tile_kernel");
       return LOSA_ERR_UNSUPPORTED;
     }
     LOSA_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     cfg.gridDim = dim3(2 * kMaxPersistentCtas, 1, 1);
-    int n = 0;
-    LOSA_CUDA_TRY(cudaOccupancyMaxActiveClusters(&n, kern, &cfg));
+    int n = 1;
+    if (PAIR) {
+      cudaLaunchConfig_t ask = cfg;
+      ask.attrs = attr + 1;
+      ask.numAttrs = 1;
+      LOSA_CUDA_TRY(cudaOccupancyMaxActiveClusters(&n, kern, &ask));
+    }
     if (n < 1) {
-      set_cuda_error(cudaErrorLaunchOutOfResources, "no resident CTA pair of losa_pair_kernel");
+      set_cuda_error(cudaErrorLaunchOutOfResources, "no resident CTA pair of losa_tile_kernel");
       return LOSA_ERR_UNSUPPORTED;
     }
     max_on[dev] = n;
@@ -2165,8 +1980,7 @@ int launch_pair(const CUtensorMap& mq, const CUtensorMap& mkh, const CUtensorMap
     *max_clusters = max_on[dev];
     return LOSA_OK;
   }
-  cfg.gridDim = dim3(2 * clusters, 1, 1);
-  cfg.numAttrs = 2;
+  cfg.gridDim = dim3((PAIR ? 2 : 1) * clusters, 1, 1);
   LOSA_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, mq, mkh, mv, mk64, mv128, prm));
   return LOSA_OK;
 }
@@ -2180,24 +1994,24 @@ int launch_t(const Geometry& g, const void* q, const void* k, const void* v, Par
   if ((rc = make_maps(&maps, g, q, k, C::kHasV ? v : nullptr)) != LOSA_OK) return rc;
   const CUtensorMap &mq = maps.map_q, &mk = maps.map_k, &mv = maps.map_v;
   int ctas = min(sms, kMaxPersistentCtas);
-  // Head dimension 128 with 128-row query blocks, modes with an attention output: pairs of CTAs,
-  // one work item per pair at a time (see losa_attn_pair.cuh); the single-CTA kernels stay the
-  // fallback.  (With 32-key blocks the pair kernel was slower than the single-CTA kernel until
-  // tiles of consecutive key blocks were copied whole: dense forward 6.3 against 5.9 ms before,
-  // 5.56 against 6.20 ms after.)  The mass pass alone runs on pairs only with 32-key blocks (5.65 -> 5.16
-  // ms at the Wan shape; with 64- and 128-key blocks it measured the same or 2 % slower on pairs: the
-  // exponential unit bounds it either way).
-  constexpr bool kPairMode = LOSA_USE_PAIR && D == 128 && R == 128 && C_ >= LOSA_PAIR_MIN_C &&
-                             (MODE == kDense || MODE == kSparse || (LOSA_PAIR_FUSED && MODE == kFused) ||
-                              (LOSA_PAIR_MASS && MODE == kMass && C_ < 64));
-  bool pair = false;  // (a device that cannot hold a pair of these CTAs runs the single-CTA kernel)
+  // Which kernel.  The tile kernel (losa_attn_tile.cuh): head dimension 128 with 128-row query blocks on
+  // pairs of CTAs, head dimension 64 on single CTAs.  (The mass pass alone gained least from pairs as
+  // long as every warp walked the tile lists: 32-key blocks 5.65 -> 5.16 ms at the Wan shape, with 64-
+  // and 128-key blocks nothing; without the lists 4.35 -> 3.78 ms and 4.06 -> 3.94 ms.)  Everything
+  // else, the fallback launch of all, and a device that cannot hold a pair: losa_attn_kernel.
+  constexpr bool kPairMode = LOSA_USE_PAIR && D == 128 && R == 128;
+  constexpr bool kTileMode = D == 64;
+  bool pair = kTileMode;
   if constexpr (kPairMode) {
     int fit = 0;
-    if (launch_pair<C_, MODE>(mq, maps.map_kh, mv, maps.map_k64, maps.map_v128, prm, 0, st, &fit) == LOSA_OK && fit >= 1 && sms >= 2) {
+    if (launch_tile<D, R, C_, MODE, true>(mq, maps.map_kh, mv, maps.map_k64, maps.map_v128, prm, 0, st, &fit) == LOSA_OK &&
+        fit >= 1 && sms >= 2) {
       pair = true;
       ctas = min(min(sms / 2, fit), kMaxPersistentCtas);
     }
   }
+  // (head dimension 64: a work item's two query tiles run on two CTAs)
+  if (kTileMode) ctas = max(1, min(sms, kMaxPersistentCtas) / 2);
   // The items of the last, partly filled wave of the persistent grid (all items, if there are
   // fewer than CTAs) are cut into parts of the key range, so that the wave ends after 1/parts of
   // an item; their partial results are merged by a second, small kernel.  Attention output
@@ -2220,7 +2034,10 @@ int launch_t(const Geometry& g, const void* q, const void* k, const void* v, Par
   // Every kernel after the first is launched as a dependent of the one before.
   if (MODE == kSparse) {
     const size_t bm_bytes = (size_t)C::kNB * ((prm.nKb + 31) / 32) * sizeof(uint32_t);  // <= 32 KB
-    rc = launch(build_tile_lists_kernel<C::kNB, C::kG>, dim3(prm.nUnits), 32 * C::kNB, bm_bytes, st, prm.nProb > 1, prm);
+    constexpr bool kOne = tile_lists_per_unit(D) == 2;
+    constexpr int kBlocks = kOne ? C::kNB / 2 : C::kNB;  // query blocks of a list
+    rc = launch(build_tile_lists_kernel<kBlocks, C::kG, kOne>, dim3(prm.nUnits * tile_lists_per_unit(D)), 32 * kBlocks,
+                bm_bytes, st, prm.nProb > 1, prm);
   } else {
     rc = launch(init_counters_kernel, dim3(1), 32, 0, st, false, prm.work_counter);
   }
@@ -2228,18 +2045,16 @@ int launch_t(const Geometry& g, const void* q, const void* k, const void* v, Par
   // All modes run with two threads per query row and a reference that never moves; the units whose
   // scores outgrew it (none, on ordinary inputs) are listed, and a second launch of the
   // one-thread-per-row kernel recomputes them with a moving reference and merges the partial units.
-  bool launched = false;
-  if constexpr (kPairMode) {
-    if (pair) {
-      if ((rc = launch_pair<C_, MODE>(mq, maps.map_kh, mv, maps.map_k64, maps.map_v128, prm, grid, st, nullptr)) != LOSA_OK)
-        return rc;
-      launched = true;
+  if constexpr (kTileMode) {
+    rc = launch_tile<D, R, C_, MODE, false>(mq, mk, mv, maps.map_k128, maps.map_v128, prm,
+                                            min(2 * ctas, 2 * prm.nUnits), st, nullptr);
+  } else {
+    if constexpr (kPairMode) {
+      if (pair) rc = launch_tile<D, R, C_, MODE, true>(mq, maps.map_kh, mv, maps.map_k64, maps.map_v128, prm, grid, st, nullptr);
     }
+    if (!pair) rc = launch_kernel<D, R, C_, MODE, KT, true>(mq, mk, mv, maps.map_k128, maps.map_v128, prm, grid, st);
   }
-  if (!launched) {
-    rc = launch_kernel<D, R, C_, MODE, KT, true>(mq, mk, mv, maps.map_k128, maps.map_v128, prm, grid, st);
-    if (rc != LOSA_OK) return rc;
-  }
+  if (rc != LOSA_OK) return rc;
   if (prm.stall) return LOSA_OK;
   prm.work_counter += 2;  // the second launch's own counter
   // (as many CTAs as SMs, whichever kernel ran first, where there is something to merge)
@@ -2278,11 +2093,15 @@ int64_t max_units(const Geometry& g, int n_prob) {
   return (int64_t)n_prob * g.B * g.H * g.nPairs + kMaxPersistentCtas;
 }
 int tile_list_cap(const Geometry& g) { return (g.nKb + 16 + 31) / 32 * 32; }  // union <= nKb, + padding of three sections
+int64_t max_lists(const Geometry& g, int n_prob) { return max_units(g, n_prob) * tile_lists_per_unit(g.D); }
+size_t redo_list_bytes(const Geometry& g, int n_prob) {
+  return ((size_t)max_units(g, n_prob) * 2 * sizeof(int32_t) + 255) / 256 * 256;
+}
 size_t tl_count_bytes(const Geometry& g, int n_prob) {
-  return ((size_t)max_units(g, n_prob) * sizeof(int32_t) + 255) / 256 * 256;
+  return ((size_t)max_lists(g, n_prob) * sizeof(int32_t) + 255) / 256 * 256;
 }
 size_t tl_entries_bytes(const Geometry& g, int n_prob) {
-  return ((size_t)max_units(g, n_prob) * tile_list_cap(g) * sizeof(uint32_t) + 255) / 256 * 256;
+  return ((size_t)max_lists(g, n_prob) * tile_list_cap(g) * sizeof(uint32_t) + 255) / 256 * 256;
 }
 }  // namespace
 
@@ -2293,10 +2112,8 @@ void arm_stalled_launch(uint32_t polls) { g_stall_polls.store(polls); }
 // work items are spread (which of them the last wave cuts into parts).
 int attn_work_slots(AttnMode mode, const Geometry& g, int sms) {
   const int ctas = sms < kMaxPersistentCtas ? sms : kMaxPersistentCtas;
-  const bool pair = LOSA_USE_PAIR && g.D == 128 && g.R == 128 && g.C >= LOSA_PAIR_MIN_C &&
-                    (mode == kDense || mode == kSparse || (LOSA_PAIR_FUSED && mode == kFused) ||
-                     (LOSA_PAIR_MASS && mode == kMass && g.C < 64)) && sms >= 2;
-  return pair ? ctas / 2 : ctas;
+  const bool pair = LOSA_USE_PAIR && g.D == 128 && g.R == 128 && sms >= 2;
+  return (pair || g.D == 64) ? (ctas > 1 ? ctas / 2 : 1) : ctas;
 }
 
 size_t attn_workspace_bytes(AttnMode mode, const Geometry& g, int n_prob) {
@@ -2308,15 +2125,15 @@ size_t attn_workspace_bytes(AttnMode mode, const Geometry& g, int n_prob) {
     if (mode == kSparse) bytes += tl_count_bytes(g, n_prob) + tl_entries_bytes(g, n_prob);
     // batched launch: the table of the problems' tensor maps and pointers
     if (n_prob > 1) bytes += (size_t)n_prob * sizeof(ProblemEntry);
-    // the work units handed to the fallback launch (each CTA of a pair may list a unit)
-    bytes += 2 * tl_count_bytes(g, n_prob);
+    // the work units handed to the fallback launch (each of a unit's query tiles may list it)
+    bytes += redo_list_bytes(g, n_prob);
     return bytes;
   }
   // counter, per-CTA row statistics (three times as many for the fused step with two threads per
   // row: two sets of the halves' row sums, and the rows' weights), per-CTA table of one entry per
   // row and key tile, and the fused step's list of units for the fallback launch
   return kCounterBytes + 5 * kRowstatBytes +
-         (size_t)kMaxPersistentCtas * 2 * (size_t)g.nKb * 128 * sizeof(float2) + 2 * tl_count_bytes(g, 1);
+         (size_t)kMaxPersistentCtas * 2 * (size_t)g.nKb * 128 * sizeof(float2) + redo_list_bytes(g, 1);
 }
 
 // Batched launch (n_prob > 1, attention-only modes): `layers` is a host array of n_prob problems of
@@ -2397,7 +2214,7 @@ int launch_attn(AttnMode mode, const Geometry& g, const void* q, const void* k, 
   prm.cap_table_floats = (long long)g.nKb * 256;
   prm.cap_mass = (long long)g.B * g.H * g.nQb * g.nKb;
   prm.cap_lse = (long long)g.B * g.H * g.N;
-  prm.cap_units = (long long)max_units(g, n_prob);
+  prm.cap_units = (long long)max_lists(g, n_prob);
   prm.scale_log2 = g.scale * kLog2e;
   int rc = LOSA_OK;
   const DeviceState* dev = device_state(&rc);

@@ -1,46 +1,60 @@
-// Dense and block-sparse forward (Eq. 4) and the fused construction step (dense forward plus the
-// block masses of Eq. 1) at head dimension 128 with 128-row query blocks, run by PAIRS of CTAs
-// (clusters of two, one SM each).  Included by losa_attn.cu, inside its namespace.
+// The tile kernel: one query tile per CTA, for dense and block-sparse forward (Eq. 4), the fused
+// construction step (dense forward plus the block masses of Eq. 1) and the mass pass.  Included by
+// losa_attn.cu, inside its namespace.
 //
-// A work item is the same pair of consecutive query tiles as in the single-CTA kernel, but each
-// CTA of the pair owns ONE of the two tiles, and the two SMs multiply together: every MMA is a
-// tcgen05.mma.cta_group::2 over 256 rows (128 per CTA), issued by one thread of the first CTA,
-// whose B operand is split between the two CTAs' shared memories - for S = Q K^T each CTA loads 64
-// of the tile's 128 keys, for O += P V each loads the 64 head-dimension columns of V that it
-// accumulates into.  A K/V tile is thus still fetched once for both query tiles, each SM reads
-// 96 B per clock from shared memory instead of 128 (the limit), half as many MMAs are issued, and
-// each CTA's tensor memory holds one O (128 columns) and THREE S buffers used in turn, so that the
-// chain S -> softmax -> O += P V of one key tile overlaps the chains of the next two.
+// Each CTA's tensor memory holds one O and THREE S buffers used in turn, so that the chain
+// S -> softmax -> O += P V of one key tile overlaps the chains of the next two.
 //
-// Per CTA: warp 0 copies (its query tile, its half of every K and V tile), warp 3 of the first CTA
-// publishes the tile list into both CTAs' rings, warps 1 and 2 of the first CTA issue every
-// S = Q K^T and every O += P V of the pair, and 16 softmax warps turn S into P: two threads per query
+// Head dimension 128 with 128-row query blocks (PAIR): a work item is a pair of consecutive query
+// tiles, run by a PAIR of CTAs (a cluster of two, one SM each) that own one of the two tiles each and
+// multiply together: every MMA is a tcgen05.mma.cta_group::2 over 256 rows (128 per CTA), issued by one
+// thread of the first CTA, whose B operand is split between the two CTAs' shared memories - for
+// S = Q K^T each CTA loads 64 of the tile's 128 keys, for O += P V each loads the 64 head-dimension
+// columns of V that it accumulates into.  A K/V tile is thus fetched once for both query tiles, each
+// SM reads 96 B per clock from shared memory instead of 128 (the limit), and half as many MMAs are
+// issued.  A key tile that only one of the two query tiles lists is multiplied for both and masked to
+// P = 0 for the other.
+//
+// Head dimension 64: the two query tiles of an item are two units, drawn one by one by single CTAs.
+// K and V stages are 16 KB there too (128 keys of 64 columns), L2 delivers the second copy of each, and
+// a query tile's list holds only what its own query blocks list.  Against two query tiles per CTA with
+// rotating score buffers (every warp walking one list, 3344 cycles per key tile and two query tiles
+// against 2048 of the special-function unit): 17776 tokens, 8 heads 893 -> 736 us dense, 1118 -> 887 us
+// with the masses, 833 -> 761 us masses alone.
+//
+// Per CTA: warp 0 copies (its query tile, its share of every K and V tile), warp 3 of the (first) CTA
+// publishes the work, warps 1 and 2 of the first CTA issue every S = Q K^T and every O += P V, and 16 softmax warps turn S into P: two threads per query
 // row (64 columns each), key tiles taken alternately by two groups of eight warps, so that each
 // group has two tile periods for one tile.  The exponentials are taken against a reference that
 // never moves within a work unit (the row maximum over the first key tile the row attends to,
 // handed from the group that meets that tile to the other); units whose scores outgrow it are
-// listed for the fallback launch, as in the single-CTA kernel.  A key tile that only one of the
-// two query tiles lists is multiplied for both and masked to P = 0 for the other.
+// listed for the fallback launch.
 //
 // Barriers that both CTAs feed (operands landed, P written, O read out, tile-list chunk consumed)
 // live in the first CTA; barriers that the MMAs' completion feeds in both CTAs are reached with a
 // commit to both.  Every wait is bounded; on the way out both CTAs meet at the cluster's barrier,
 // so that neither leaves while the other may still signal into its shared memory.
 
-constexpr int kPairNK = 4, kPairNV = 7;      // K and V stages of 16 KB per CTA
-constexpr int kPairStage = 16384;
-constexpr int kPairQBytes = 32768;
+constexpr int kTileNK = 4, kTileNV = 7;      // K and V stages of 16 KB per CTA
+constexpr int kTileStage = 16384;
+#ifndef LOSA_POLY_OF
+#define LOSA_POLY_OF 8
+#endif
+#ifndef LOSA_POLY_OF_MASS
+#define LOSA_POLY_OF_MASS 4
+#endif
+constexpr float kTileSafeLow = 8.6736173798840355e-19f;  // 2^-60
 
-struct PairControl {
+struct TileControl {
   uint64_t q_full, q_empty;
-  uint64_t k_full[kPairNK], k_empty[kPairNK];
-  uint64_t v_full[kPairNV], v_empty[kPairNV];
+  uint64_t k_full[kTileNK], k_empty[kTileNK];
+  uint64_t v_full[kTileNV], v_empty[kTileNV];
   uint64_t s_full[3], p_ready[3], pv_done[3];  // per score buffer
   uint64_t o_done, o_free;
   uint64_t hdr_full[2], hdr_empty[2], hdr_next;
   uint64_t tl_full[kTlChunks], tl_empty[kTlChunks];
   uint64_t pair_bar[8];    // per (group, lane quarter): the two halves of a row
-  uint64_t ref_full[2], ref_empty[2];
+  uint64_t ref_full[2][2], ref_empty[2][2];  // [set][query block of the query tile]
   uint64_t item_bar;       // all softmax warps of the CTA, at the end of an item
   uint64_t fold_bar;       // ... and after the fused step's masses are folded out of the table
   uint64_t drain;
@@ -55,16 +69,18 @@ struct PairControl {
 };
 
 // Key blocks of a unit in the dense modes.
-__device__ __forceinline__ void pair_key_range(const Params& p, uint32_t ent, int& jlo, int& jhi) {
+__device__ __forceinline__ void tile_key_range(const Params& p, uint32_t ent, int& jlo, int& jhi) {
   const int part = (ent & kTlPartial) ? (int)((ent >> 24) & 7u) : 0;
   const int parts = (ent & kTlPartial) ? p.split_parts : 1;
   jlo = (int)(((int64_t)p.nKb * part) / parts);
   jhi = (int)(((int64_t)p.nKb * (part + 1)) / parts);
 }
 
-#define PAIR_WAIT_CL(bar, parity)                                                          \
+// (a barrier whose data the other CTA of a pair may have written)
+#define TILE_WAIT(bar, parity)                                                             \
   do {                                                                                     \
-    if (!ptx::mbar_wait_cluster((bar), (parity), &ctl->abort_flag, p.wait_polls)) {        \
+    if (!(PAIR ? ptx::mbar_wait_cluster((bar), (parity), &ctl->abort_flag, p.wait_polls)   \
+               : ptx::mbar_wait((bar), (parity), &ctl->abort_flag, p.wait_polls))) {       \
       ctl->abort_flag = 1;                                                                 \
       report_error(p.status, LOSA_ERR_TIMEOUT);                                            \
       goto teardown;                                                                       \
@@ -82,122 +98,167 @@ __device__ __forceinline__ void pair_key_range(const Params& p, uint32_t ent, in
 // tile than the exponentials: 529 warp instructions per 64 scores of a warp, 224 of them arithmetic.)
 //
 // Next header (whole warp); `nu` is the warp's unit counter.
-#define PAIR_HDR_NEXT(ent, word)                                                           \
+#define TILE_HDR_NEXT(ent, word)                                                           \
   do {                                                                                     \
     const uint32_t s_ = nu & 1u;                                                           \
-    PAIR_WAIT_CL(&ctl->hdr_full[s_], (nu >> 1) & 1u);                                      \
+    TILE_WAIT(&ctl->hdr_full[s_], (nu >> 1) & 1u);                                      \
     uint32_t h_[2];                                                                        \
     ptx::ld_shared_volatile_vec<2>(&ctl->hdr[s_].x, h_);                                   \
     __syncwarp();                                                                          \
-    if (lane == 0) ptx::mbar_arrive_cluster(hdr_empty0 + 8u * s_);                         \
+    if (lane == 0) arrive0<PAIR>(hdr_empty0 + 8u * s_);                                    \
     (ent) = h_[0];                                                                         \
     (word) = h_[1];                                                                        \
     ++nu;                                                                                  \
   } while (0)
 
 // Chunk `nc` of the tile lists: wait for it, hand it back (whole warp).
-#define PAIR_CHUNK_WAIT() PAIR_WAIT_CL(&ctl->tl_full[nc & (kTlChunks - 1)], (nc / kTlChunks) & 1u)
-#define PAIR_CHUNK_DONE()                                                                  \
+#define TILE_CHUNK_WAIT() TILE_WAIT(&ctl->tl_full[nc & (kTlChunks - 1)], (nc / kTlChunks) & 1u)
+#define TILE_CHUNK_DONE()                                                                  \
   do {                                                                                     \
     __syncwarp();                                                                          \
-    if (lane == 0) ptx::mbar_arrive_cluster(tl_empty0 + 8u * (nc & (kTlChunks - 1)));      \
+    if (lane == 0) arrive0<PAIR>(tl_empty0 + 8u * (nc & (kTlChunks - 1)));                 \
     ++nc;                                                                                  \
   } while (0)
 
 // Scheduler of the first CTA: publish a header in both CTAs.
-#define PAIR_HDR_PUT(ent, word)                                                            \
+#define TILE_HDR_PUT(ent, word)                                                            \
   do {                                                                                     \
     const uint32_t s_ = nu & 1u;                                                           \
     LOSA_WAIT_RELAXED(&ctl->hdr_empty[s_], ((nu >> 1) & 1u) ^ 1u);                         \
     if (lane == 0) {                                                                       \
       ctl->hdr[s_] = make_uint2((ent), (word));                                            \
-      ptx::st_cluster_u32(hdr1 + 8u * s_, (ent));                                          \
-      ptx::st_cluster_u32(hdr1 + 8u * s_ + 4u, (word));                                    \
-      ptx::fence_acq_rel_cluster();                                                        \
+      if (PAIR) {                                                                          \
+        ptx::st_cluster_u32(hdr1 + 8u * s_, (ent));                                        \
+        ptx::st_cluster_u32(hdr1 + 8u * s_ + 4u, (word));                                  \
+        ptx::fence_acq_rel_cluster();                                                      \
+      }                                                                                    \
       ptx::mbar_arrive(&ctl->hdr_full[s_]);                                                \
-      ptx::mbar_arrive_cluster(hdr_full1 + 8u * s_);                                       \
+      if (PAIR) ptx::mbar_arrive_cluster(hdr_full1 + 8u * s_);                             \
     }                                                                                      \
     __syncwarp();                                                                          \
     ++nu;                                                                                  \
   } while (0)
 
-template <int C_, int MODE>
+// Arrivals on, and copies counted by, a barrier of the first CTA (of the only one, without pairs).
+template <bool PAIR>
+__device__ __forceinline__ void arrive0(uint32_t bar0) {
+  if (PAIR) ptx::mbar_arrive_cluster(bar0);
+  else ptx::mbar_arrive_u32(bar0);
+}
+template <bool PAIR>
+__device__ __forceinline__ void expect0(uint32_t bar0, uint32_t bytes) {
+  if (PAIR) ptx::mbar_arrive_expect_tx_cluster(bar0, bytes);
+  else ptx::mbar_arrive_expect_tx_u32(bar0, bytes);
+}
+template <bool PAIR>
+__device__ __forceinline__ void load0(void* dst, const CUtensorMap* map, uint32_t bar0, int c0, int c1, int c2, int c3) {
+  if (PAIR) ptx::tma_load_4d_pair(dst, map, bar0, c0, c1, c2, c3);
+  else ptx::tma_load_4d_u32(dst, map, bar0, c0, c1, c2, c3);
+}
+// Signals a barrier when the MMAs issued so far are complete: in the first CTA, or in both.
+template <bool PAIR>
+__device__ __forceinline__ void commit0(uint64_t* bar) {
+  if (PAIR) ptx::mma2_commit(bar);
+  else ptx::mma_commit(bar);
+}
+template <bool PAIR>
+__device__ __forceinline__ void commit_all(uint64_t* bar) {
+  if (PAIR) ptx::mma2_commit_both(bar);
+  else ptx::mma_commit(bar);
+}
+
+template <int D, int R, int C_, int MODE, bool PAIR>
 __global__ void __launch_bounds__(Lay<true>::kThreads, 1)
-losa_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
+losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                  const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_kw,
                  const __grid_constant__ CUtensorMap map_vw, const Params p) {
   using L = Lay<true>;
-  constexpr int D = 128, R = 128;
+  static_assert(PAIR ? (D == 128 && R == 128) : D == 64, "pairs at head dimension 128, one CTA at 64");
+  constexpr int kQB = 128 / R;  // query blocks of the query tile
   constexpr int kC = C_, kG = 128 / C_, kW = 128;
-  constexpr int kKBox = (C_ < 64) ? C_ : 64;  // key rows per copy of this CTA's half of a K tile
-  constexpr int kKCopies = 64 / kKBox;        // ... and copies per 64-column slab
-  constexpr uint32_t kIdescQK = ptx::idesc_bf16_f32(256, 128, false, false);
-  constexpr uint32_t kIdescPV = ptx::idesc_bf16_f32(256, 128, false, true);
-  using Ctl = PairControl;
+  constexpr int kQBytes = 128 * D * 2;
+  constexpr int kKRows = PAIR ? 64 : 128;             // keys of a K tile that this CTA copies
+  constexpr int kKBox = (C_ < kKRows) ? C_ : kKRows;  // ... per copy
+  constexpr int kKCopies = kKRows / kKBox;            // ... and copies per 64-column slab
+  constexpr int kSlabs = D / 64;                      // slabs of a K tile
+  constexpr uint32_t kIdescQK = ptx::idesc_bf16_f32(PAIR ? 256 : 128, 128, false, false);
+  constexpr uint32_t kIdescPV = ptx::idesc_bf16_f32(PAIR ? 256 : 128, D, false, true);
+  // Head dimension 64: a key tile needs 1024 cycles of the special-function unit against 512 of the
+  // tensor cores, so one group of four scores in every kPolyOf takes its exponentials from a
+  // polynomial on the FMA pipe.  17776 tokens, 8 heads: dense 735 us with one in 8, 742 in 16, 763 in 6,
+  // 805 in 4.  The mass pass (no P to pack and to sum) takes one in 4: 735 us, 759 in 8, 786 in 6; at head
+  // dimension 128 (Wan shape) 3635 us, 3750 in 8, 3937 without.
+  constexpr int kPolyOf = (MODE == kMass) ? LOSA_POLY_OF_MASS : (D == 64) ? LOSA_POLY_OF : 0;
+  using Ctl = TileControl;
   constexpr bool kWantMass = (MODE == kFused || MODE == kMass);  // the block masses (Eq. 1) are wanted
   // the mass pass alone has no V, no P and no O: its score buffers go back as soon as they are read
   constexpr bool kHasV = (MODE != kMass);
   constexpr int kChunkTiles = (MODE == kSparse) ? 32 / kG : (1 << 28);  // K/V tiles per chunk of the list
-  static_assert(offsetof(PairControl, tl) % 16 == 0, "the tile list is read with 16-byte loads");
+  static_assert(offsetof(TileControl, tl) % 16 == 0, "the tile list is read with 16-byte loads");
 
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* const sQ = smem_raw;
-  uint8_t* const sK = sQ + kPairQBytes;
-  uint8_t* const sV = sK + kPairNK * kPairStage;
-  Ctl* const ctl = reinterpret_cast<Ctl*>(sV + kPairNV * kPairStage);
+  uint8_t* const sK = sQ + kQBytes;
+  uint8_t* const sV = sK + kTileNK * kTileStage;
+  Ctl* const ctl = reinterpret_cast<Ctl*>(sV + kTileNV * kTileStage);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint32_t rank = ptx::cluster_ctarank();  // 0: the CTA that issues the MMAs; also the query tile of the pair
+  const uint32_t rank = PAIR ? ptx::cluster_ctarank() : 0u;  // 0: the CTA that issues the MMAs; also the query tile
   ptx::grid_launch_dependents();
   // (the swizzled tiles rely on the declared alignment of the dynamic shared memory)
   const bool misaligned = (ptx::smem_u32(smem_raw) & 1023u) != 0;
 
   // shared::cluster addresses of the first CTA's barriers that both CTAs arrive on, and of the
   // second CTA's copy of the tile list (used by the first CTA's scheduler)
-  const uint32_t q_full0 = ptx::mapa(ptx::smem_u32(&ctl->q_full), 0);
-  const uint32_t k_full0 = ptx::mapa(ptx::smem_u32(&ctl->k_full[0]), 0);
-  const uint32_t v_full0 = ptx::mapa(ptx::smem_u32(&ctl->v_full[0]), 0);
-  const uint32_t p_ready0 = ptx::mapa(ptx::smem_u32(&ctl->p_ready[0]), 0);
-  const uint32_t o_free0 = ptx::mapa(ptx::smem_u32(&ctl->o_free), 0);
-  const uint32_t tl_empty0 = ptx::mapa(ptx::smem_u32(&ctl->tl_empty[0]), 0);
-  const uint32_t tl_full1 = ptx::mapa(ptx::smem_u32(&ctl->tl_full[0]), 1);
-  const uint32_t hdr_empty0 = ptx::mapa(ptx::smem_u32(&ctl->hdr_empty[0]), 0);
-  const uint32_t hdr_full1 = ptx::mapa(ptx::smem_u32(&ctl->hdr_full[0]), 1);
-  const uint32_t hdr1 = ptx::mapa(ptx::smem_u32(&ctl->hdr[0]), 1);
-  const uint32_t tl1 = ptx::mapa(ptx::smem_u32(&ctl->tl[0]), 1);
-  const uint32_t abort_peer = ptx::mapa(ptx::smem_u32(&ctl->abort_flag), rank ^ 1u);
+  auto at0 = [](const void* x) { return PAIR ? ptx::mapa(ptx::smem_u32(x), 0) : ptx::smem_u32(x); };
+  auto at1 = [](const void* x) { return PAIR ? ptx::mapa(ptx::smem_u32(x), 1) : 0u; };
+  const uint32_t q_full0 = at0(&ctl->q_full);
+  const uint32_t k_full0 = at0(&ctl->k_full[0]);
+  const uint32_t v_full0 = at0(&ctl->v_full[0]);
+  const uint32_t p_ready0 = at0(&ctl->p_ready[0]);
+  const uint32_t o_free0 = at0(&ctl->o_free);
+  const uint32_t tl_empty0 = at0(&ctl->tl_empty[0]);
+  const uint32_t tl_full1 = at1(&ctl->tl_full[0]);
+  const uint32_t hdr_empty0 = at0(&ctl->hdr_empty[0]);
+  const uint32_t hdr_full1 = at1(&ctl->hdr_full[0]);
+  const uint32_t hdr1 = at1(&ctl->hdr[0]);
+  const uint32_t tl1 = at1(&ctl->tl[0]);
+  const uint32_t abort_peer = PAIR ? ptx::mapa(ptx::smem_u32(&ctl->abort_flag), rank ^ 1u) : 0u;
 
   if (threadIdx.x == 0) {
-    ptx::mbar_init(&ctl->q_full, 2);   // one arrival (with its byte count) per CTA's producer
+    constexpr int kCtas = PAIR ? 2 : 1;
+    ptx::mbar_init(&ctl->q_full, kCtas);   // one arrival (with its byte count) per CTA's producer
     ptx::mbar_init(&ctl->q_empty, 1);
-    for (int i = 0; i < kPairNK; ++i) {
-      ptx::mbar_init(&ctl->k_full[i], 2);
+    for (int i = 0; i < kTileNK; ++i) {
+      ptx::mbar_init(&ctl->k_full[i], kCtas);
       ptx::mbar_init(&ctl->k_empty[i], 1);
     }
-    for (int i = 0; i < kPairNV; ++i) {
-      ptx::mbar_init(&ctl->v_full[i], 2);
+    for (int i = 0; i < kTileNV; ++i) {
+      ptx::mbar_init(&ctl->v_full[i], kCtas);
       ptx::mbar_init(&ctl->v_empty[i], 1);
     }
     for (int i = 0; i < 3; ++i) {
       ptx::mbar_init(&ctl->s_full[i], 1);
-      ptx::mbar_init(&ctl->p_ready[i], 16);  // the eight warps of a group, in both CTAs
+      ptx::mbar_init(&ctl->p_ready[i], 8 * kCtas);  // the eight warps of a group, in both CTAs
       ptx::mbar_init(&ctl->pv_done[i], 1);
     }
     ptx::mbar_init(&ctl->o_done, 1);
-    ptx::mbar_init(&ctl->o_free, 32);  // every softmax warp of both CTAs reads a quarter of its rows' O
+    ptx::mbar_init(&ctl->o_free, 16 * kCtas);  // every softmax warp of both CTAs reads a quarter of its rows' O
     for (int i = 0; i < kTlChunks; ++i) {
       ptx::mbar_init(&ctl->tl_full[i], 1);
-      ptx::mbar_init(&ctl->tl_empty[i], 2 * 17);  // readers: each CTA's producer and 16 softmax warps
+      ptx::mbar_init(&ctl->tl_empty[i], 17 * kCtas);  // readers: each CTA's producer and 16 softmax warps
     }
     for (int i = 0; i < 2; ++i) {
       ptx::mbar_init(&ctl->hdr_full[i], 1);
-      ptx::mbar_init(&ctl->hdr_empty[i], 2 * 17 + 2);  // ... and the two issuers
+      ptx::mbar_init(&ctl->hdr_empty[i], 17 * kCtas + 2);  // ... and the two issuers
     }
     ptx::mbar_init(&ctl->hdr_next, 1);  // the first CTA's producer, near the end of a unit
     for (int i = 0; i < 8; ++i) ptx::mbar_init(&ctl->pair_bar[i], 2);
     for (int i = 0; i < 2; ++i) {
-      ptx::mbar_init(&ctl->ref_full[i], 4);   // the first halves' warps of the group that sets it
-      ptx::mbar_init(&ctl->ref_empty[i], 8);  // the warps of the other group
+      for (int q = 0; q < kQB; ++q) {
+        ptx::mbar_init(&ctl->ref_full[i][q], 4 / kQB);   // the first halves' warps of the group that sets it
+        ptx::mbar_init(&ctl->ref_empty[i][q], 8 / kQB);  // the warps of the other group
+      }
     }
     ptx::mbar_init(&ctl->item_bar, 16);
     ptx::mbar_init(&ctl->fold_bar, 16);
@@ -208,8 +269,13 @@ losa_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   }
   if (warp == kIssuerWarp) {
     // (one warp of each CTA of the pair)
-    ptx::tmem_alloc2(&ctl->tmem_base, kTmemCols);
-    ptx::tmem_relinquish_alloc_permit2();
+    if (PAIR) {
+      ptx::tmem_alloc2(&ctl->tmem_base, kTmemCols);
+      ptx::tmem_relinquish_alloc_permit2();
+    } else {
+      ptx::tmem_alloc(&ctl->tmem_base, kTmemCols);
+      ptx::tmem_relinquish_alloc_permit();
+    }
   }
   if (warp == kProducerWarp && lane == 0) {
     ptx::prefetch_tensormap(&map_q);
@@ -222,12 +288,13 @@ losa_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   }
   ptx::tc_fence_before_sync();
   __syncthreads();
-  ptx::cluster_sync();  // both CTAs' barriers are initialised before either signals the other
+  if (PAIR) ptx::cluster_sync();  // both CTAs' barriers are initialised before either signals the other
   ptx::tc_fence_after_sync();
   const uint32_t tmem_base = ctl->tmem_base;
   {
     // the MMAs address both CTAs' tensor memory with one address
-    const uint32_t other = ptx::ld_cluster_u32(ptx::mapa(ptx::smem_u32(&ctl->tmem_base), rank ^ 1u));
+    const uint32_t other =
+        PAIR ? ptx::ld_cluster_u32(ptx::mapa(ptx::smem_u32(&ctl->tmem_base), rank ^ 1u)) : tmem_base;
     if (misaligned || other != tmem_base) {
       if (threadIdx.x == 0) {
         ctl->abort_flag = 1;
@@ -247,7 +314,7 @@ losa_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       uint32_t nq = 0, nk = 0, nv = 0, nu = 0, nc = 0, ent, word;
       int problem = -1;  // batched launch: whose tensor maps this warp has acquired
       for (;;) {
-        PAIR_HDR_NEXT(ent, word);
+        TILE_HDR_NEXT(ent, word);
         if ((ent >> 28) != 1) break;
         const int w = (int)(ent & kTlItemMask);
         const int pbh = w / p.nPairs, pr = w % p.nPairs;
@@ -258,9 +325,9 @@ losa_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         if (p.problems != nullptr) {
           const ProblemEntry* pe = p.problems + pbh / (p.B * p.H);
           mq = &pe->map_q;
-          mk = &pe->map_kh;
+          mk = PAIR ? &pe->map_kh : &pe->map_k;
           mv = &pe->map_v;
-          mkw = &pe->map_k64;
+          mkw = PAIR ? &pe->map_k64 : &pe->map_k128;
           mvw = &pe->map_v128;
           if (pbh / (p.B * p.H) != problem) {
             problem = pbh / (p.B * p.H);
@@ -268,22 +335,22 @@ losa_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           }
         }
         // this CTA's query tile (rows past the end of the sequence are filled with zeros)
-        const int T = 2 * pr + (int)rank;
+        const int T = 2 * pr + (PAIR ? (int)rank : (int)((word & kHdrOdd) != 0u));
         LOSA_WAIT_RELAXED(&ctl->q_empty, (nq & 1) ^ 1);
         if (lane == 0) {
-          ptx::mbar_arrive_expect_tx_cluster(q_full0, kPairQBytes);
-          ptx::tma_load_4d_pair(sQ, mq, q_full0, 0, T * 128, h, b);
-          ptx::tma_load_4d_pair(sQ + 16384, mq, q_full0, 64, T * 128, h, b);
+          expect0<PAIR>(q_full0, kQBytes);
+#pragma unroll
+          for (int s = 0; s < kSlabs; ++s) load0<PAIR>(sQ + s * 16384, mq, q_full0, s * 64, T * 128, h, b);
         }
         ++nq;
         const int tiles = (int)(word & kHdrTiles);
         int jlo, jhi;  // dense modes: the unit's key blocks
-        pair_key_range(p, ent, jlo, jhi);
+        tile_key_range(p, ent, jlo, jhi);
         // the scheduler draws the next unit when this one is 16 tiles from its end
         const int call_at = max(0, tiles - 16);
         if (tiles == 0 && rank == 0 && lane == 0) ptx::mbar_arrive(&ctl->hdr_next);
         for (int base = 0; base < tiles; base += kChunkTiles) {
-        if (MODE == kSparse) PAIR_CHUNK_WAIT();
+        if (MODE == kSparse) TILE_CHUNK_WAIT();
         const int end = min(tiles, base + kChunkTiles);
         for (int i = base; i < end; ++i) {
           if (i == call_at && rank == 0 && lane == 0) ptx::mbar_arrive(&ctl->hdr_next);
@@ -294,26 +361,30 @@ losa_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
 #pragma unroll
             for (int g = 0; g < kG; ++g) grp[g] = (jlo + i * kG + g < jhi) ? (uint32_t)(jlo + i * kG + g) : kTlPad;
           }
-          // K: keys 64 * rank ... + 63 of the tile, all 128 head-dimension columns (two slabs)
-          const uint32_t ks = nk % kPairNK;
-          LOSA_WAIT_RELAXED(&ctl->k_empty[ks], ((nk / kPairNK) & 1) ^ 1);
-          if (lane == 0) ptx::mbar_arrive_expect_tx_cluster(k_full0 + 8u * ks, kPairStage);
+          // K: a pair's CTAs keys 64 * rank ... + 63 of the tile each; all head-dimension columns, per slab of 64
+          const uint32_t ks = nk % kTileNK;
+          LOSA_WAIT_RELAXED(&ctl->k_empty[ks], ((nk / kTileNK) & 1) ^ 1);
+          if (lane == 0) expect0<PAIR>(k_full0 + 8u * ks, kTileStage);
           __syncwarp();
-          // 32-key blocks: this CTA's two key blocks, if consecutive, are one copy per slab
-          bool wide_k = false;
+          // 32-key blocks: this CTA's key blocks, if consecutive, are one copy per slab
+          constexpr int kKBlocks = (kKRows / kC > 0) ? kKRows / kC : 1;  // key blocks of this CTA's rows
+          bool wide_k = kG > 2;
           uint32_t first_k = grp[0];
-          if constexpr (kKCopies == 2) {
-            const uint32_t e0 = (rank == 0) ? grp[0] : grp[kG / 2], e1 = (rank == 0) ? grp[1] : grp[kG / 2 + 1];
-            wide_k = (e1 & 0xffffu) == (e0 & 0xffffu) + 1u;
-            first_k = e0;
+          if constexpr (kG > 2) {
+            first_k = (rank == 0) ? grp[0] : grp[kG / 2];
+#pragma unroll
+            for (int j = 1; j < kKBlocks; ++j) {
+              const uint32_t ej = (rank == 0) ? grp[j] : grp[kG / 2 + (PAIR ? j : 0)];
+              wide_k = wide_k && (ej & 0xffffu) == (first_k & 0xffffu) + j;
+            }
           }
           if (wide_k) {
-            if (lane < 2)
-              ptx::tma_load_4d_pair(sK + ks * kPairStage + lane * 8192, mkw, k_full0 + 8u * ks, lane * 64,
-                                    (int)(first_k & 0xffffu) * kC, h, b);
-          } else if (lane < 2 * kKCopies) {
-            const int i = lane >> 1, s = lane & 1;
-            const int keyoff = 64 * (int)rank + i * kKBox;  // within the tile
+            if (lane < kSlabs)
+              load0<PAIR>(sK + ks * kTileStage + lane * (kKRows * 128), mkw, k_full0 + 8u * ks, lane * 64,
+                          (int)(first_k & 0xffffu) * kC, h, b);
+          } else if (lane < kSlabs * kKCopies) {
+            const int j = lane / kSlabs, s = lane % kSlabs;
+            const int keyoff = 64 * (int)rank + j * kKBox;  // within the tile
             const int g = keyoff / kC, inb = keyoff % kC;
             uint32_t eg = grp[0];
 #pragma unroll
@@ -321,23 +392,22 @@ losa_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
               if (g == gg) eg = grp[gg];
             const int jg = (int)(eg & 0xffffu);
             const int r0 = (jg == (int)kTlPad) ? p.nKb * kC : jg * kC + inb;
-            ptx::tma_load_4d_pair(sK + ks * kPairStage + s * 8192 + i * kKBox * 128, mk, k_full0 + 8u * ks,
-                                  s * 64, r0, h, b);
+            load0<PAIR>(sK + ks * kTileStage + s * (kKRows * 128) + j * kKBox * 128, mk, k_full0 + 8u * ks, s * 64, r0,
+                        h, b);
           }
           ++nk;
           if (!kHasV) continue;
-          // V: all 128 keys of the tile, head-dimension columns 64 * rank ... + 63 (one slab)
-          const uint32_t vs = nv % kPairNV;
-          LOSA_WAIT_RELAXED(&ctl->v_empty[vs], ((nv / kPairNV) & 1) ^ 1);
-          if (lane == 0) ptx::mbar_arrive_expect_tx_cluster(v_full0 + 8u * vs, kPairStage);
+          // V: all 128 keys of the tile, (a pair: of each CTA) 64 of the head-dimension columns, one slab
+          const uint32_t vs = nv % kTileNV;
+          LOSA_WAIT_RELAXED(&ctl->v_empty[vs], ((nv / kTileNV) & 1) ^ 1);
+          if (lane == 0) expect0<PAIR>(v_full0 + 8u * vs, kTileStage);
           __syncwarp();
           bool wide_v = kG > 2;
 #pragma unroll
           for (int gg = 1; gg < kG; ++gg) wide_v = wide_v && (grp[gg] & 0xffffu) == (grp[0] & 0xffffu) + gg;
           if (wide_v) {
             if (lane == 0)
-              ptx::tma_load_4d_pair(sV + vs * kPairStage, mvw, v_full0 + 8u * vs, (int)rank * 64,
-                                    (int)(grp[0] & 0xffffu) * kC, h, b);
+              load0<PAIR>(sV + vs * kTileStage, mvw, v_full0 + 8u * vs, (int)rank * 64, (int)(grp[0] & 0xffffu) * kC, h, b);
           } else if (lane < kG) {
             uint32_t eg = grp[0];
 #pragma unroll
@@ -345,12 +415,11 @@ losa_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
               if (lane == gg) eg = grp[gg];
             const int jg = (int)(eg & 0xffffu);
             const int r0 = (jg == (int)kTlPad) ? p.nKb * kC : jg * kC;
-            ptx::tma_load_4d_pair(sV + vs * kPairStage + lane * kC * 128, mv, v_full0 + 8u * vs,
-                                  (int)rank * 64, r0, h, b);
+            load0<PAIR>(sV + vs * kTileStage + lane * kC * 128, mv, v_full0 + 8u * vs, (int)rank * 64, r0, h, b);
           }
           ++nv;
         }
-        if (MODE == kSparse) PAIR_CHUNK_DONE();
+        if (MODE == kSparse) TILE_CHUNK_DONE();
         }
       }
     } else if (warp == kIssuerWarp && rank == 0) {
@@ -366,12 +435,12 @@ losa_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         qd[kk] = ptx::smem_desc_lo(ptx::smem_u32(sQ), 16) + (((kk >> 2) * 16384 + (kk & 3) * 32) >> 4);
       uint32_t nq = 0, nt = 0, nu = 0, ent, word;
       for (;;) {
-        PAIR_HDR_NEXT(ent, word);
+        TILE_HDR_NEXT(ent, word);
         if ((ent >> 28) != 1) break;
         bool q_ready = false;
         for (int i = (int)(word & kHdrTiles); i > 0; --i) {
-          const uint32_t ks = nt % kPairNK;
-          LOSA_WAIT(&ctl->k_full[ks], (nt / kPairNK) & 1);
+          const uint32_t ks = nt % kTileNK;
+          LOSA_WAIT(&ctl->k_full[ks], (nt / kTileNK) & 1);
           if (!q_ready) {
             LOSA_WAIT(&ctl->q_full, nq & 1);
             ++nq;
@@ -385,13 +454,17 @@ losa_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           }
           ptx::tc_fence_after_sync();
           if (leader) {
-            const uint32_t kd0 = k_lo + ks * (kPairStage >> 4);
+            const uint32_t kd0 = k_lo + ks * (kTileStage >> 4);
 #pragma unroll
             for (int kk = 0; kk < D / 16; ++kk)
-              ptx::mma2_ss_lo(tmem_base + bsel * 128, qd[kk], kd0 + (((kk >> 2) * 8192 + (kk & 3) * 32) >> 4),
-                              kDescHi, kIdescQK, kk > 0 ? 1u : 0u);
-            ptx::mma2_commit_both(&ctl->s_full[bsel]);
-            ptx::mma2_commit_both(&ctl->k_empty[ks]);
+              if (PAIR)
+                ptx::mma2_ss_lo(tmem_base + bsel * 128, qd[kk], kd0 + (((kk >> 2) * 8192 + (kk & 3) * 32) >> 4),
+                                kDescHi, kIdescQK, kk > 0 ? 1u : 0u);
+              else
+                ptx::mma_ss_lo(tmem_base + bsel * 128, qd[kk], kd0 + (((kk & 3) * 32) >> 4), kDescHi, kIdescQK,
+                               kk > 0 ? 1u : 0u);
+            commit_all<PAIR>(&ctl->s_full[bsel]);
+            commit_all<PAIR>(&ctl->k_empty[ks]);
           }
           ++nt;
         }
@@ -400,42 +473,46 @@ losa_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           LOSA_WAIT(&ctl->q_full, nq & 1);
           ++nq;
         }
-        if (leader) ptx::mma2_commit_both(&ctl->q_empty);
+        if (leader) commit_all<PAIR>(&ctl->q_empty);
       }
     } else if (warp == kIssuerWarp + 1 && rank == 0) {
       // ------------------------------------------------------------------ O += P V of the pair
       const bool leader = ptx::elect_one();
       constexpr uint32_t kDescHi = ptx::smem_desc_hi_sw128(1024);
-      const uint32_t v_lo = ptx::smem_desc_lo(ptx::smem_u32(sV), kPairStage);
+      const uint32_t v_lo = ptx::smem_desc_lo(ptx::smem_u32(sV), kTileStage);
       const uint32_t tO = tmem_base + 384;
       uint32_t nof = 0, nt = 0, nu = 0, ent, word;
       for (;;) {
-        PAIR_HDR_NEXT(ent, word);
+        TILE_HDR_NEXT(ent, word);
         if ((ent >> 28) != 1) break;
         uint32_t pv_item = 0;
         for (int i = kHasV ? (int)(word & kHdrTiles) : 0; i > 0; --i) {  // (the mass pass has no products)
-          const uint32_t vs = nt % kPairNV;
-          LOSA_WAIT(&ctl->v_full[vs], (nt / kPairNV) & 1);
+          const uint32_t vs = nt % kTileNV;
+          LOSA_WAIT(&ctl->v_full[vs], (nt / kTileNV) & 1);
           const uint32_t bsel = nt % 3u;
           if (pv_item == 0 && nof > 0) LOSA_WAIT(&ctl->o_free, (nof - 1) & 1);
           LOSA_WAIT(&ctl->p_ready[bsel], (nt / 3u) & 1);
           ptx::tc_fence_after_sync();
           if (leader) {
             const uint32_t tP = tmem_base + bsel * 128;
-            const uint32_t vd0 = v_lo + vs * (kPairStage >> 4);
+            const uint32_t vd0 = v_lo + vs * (kTileStage >> 4);
             // (each half of a row packs its P over the head of its own 64 score columns)
 #pragma unroll
             for (int kk = 0; kk < kW / 16; ++kk)
-              ptx::mma2_ts_lo(tO, tP + (kk & 3) * 8 + (kk >> 2) * 64, vd0 + kk * (2048 >> 4), kDescHi, kIdescPV,
-                              (kk > 0 || pv_item > 0) ? 1u : 0u);
-            ptx::mma2_commit(&ctl->pv_done[bsel]);
-            ptx::mma2_commit_both(&ctl->v_empty[vs]);
+              if (PAIR)
+                ptx::mma2_ts_lo(tO, tP + (kk & 3) * 8 + (kk >> 2) * 64, vd0 + kk * (2048 >> 4), kDescHi, kIdescPV,
+                                (kk > 0 || pv_item > 0) ? 1u : 0u);
+              else
+                ptx::mma_ts_lo(tO, tP + (kk & 3) * 8 + (kk >> 2) * 64, vd0 + kk * (2048 >> 4), kDescHi, kIdescPV,
+                               (kk > 0 || pv_item > 0) ? 1u : 0u);
+            commit0<PAIR>(&ctl->pv_done[bsel]);
+            commit_all<PAIR>(&ctl->v_empty[vs]);
           }
           ++pv_item;
           ++nt;
         }
         if (pv_item > 0) {
-          if (leader) ptx::mma2_commit_both(&ctl->o_done);  // every product of the item is done
+          if (leader) commit_all<PAIR>(&ctl->o_done);  // every product of the item is done
           ++nof;
         }
       }
@@ -445,53 +522,60 @@ losa_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       bool first_item = true;
       for (;;) {
         if (p.stall) break;  // diagnostic launch: nothing is published and every wait runs out
-        int w = (int)(blockIdx.x >> 1);  // a first item by position, then from the counter
+        // a first unit by position, then from the counter; without pairs of CTAs a unit's two query
+        // tiles are drawn one by one
+        int w = (int)(PAIR ? blockIdx.x >> 1 : blockIdx.x);
         if (!first_item) {
-          if (lane == 0) w = (int)(gridDim.x >> 1) + atomicAdd(p.work_counter, 1);
+          if (lane == 0) w = (int)(PAIR ? gridDim.x >> 1 : gridDim.x) + atomicAdd(p.work_counter, 1);
           w = __shfl_sync(0xffffffffu, w, 0);
         }
         first_item = false;
+        const int list = w;  // its tile list
+        const uint32_t odd = (!PAIR && (w & 1)) ? kHdrOdd : 0u;
+        if (!PAIR) w >>= 1;
         if (w >= p.nUnits) break;
-        int part = 0, parts = 1;
         uint32_t flags = 0;
         if (w >= p.split_first) {
           const int r = w - p.split_first;
-          parts = p.split_parts;
-          part = r % parts;
-          w = p.split_first + r / parts;
-          flags = kTlPartial | ((uint32_t)part << 24);
+          flags = kTlPartial | ((uint32_t)(r % p.split_parts) << 24);
+          w = p.split_first + r / p.split_parts;
         }
-        const int unit = (flags != 0) ? p.split_first + (w - p.split_first) * parts + part : w;
-        const int pr = w % p.nPairs;
         if (MODE == kSparse) {
-          const uint32_t word = LOSA_IN_RANGE(unit, p.cap_units) ? (uint32_t)__ldcg(p.tl_count + unit) : 0u;
+          const uint32_t word = LOSA_IN_RANGE(list, p.cap_units) ? (uint32_t)__ldcg(p.tl_count + list) : 0u;
           const int cnt = min((int)(word & kHdrTiles) * kG, p.tl_cap);
-          PAIR_HDR_PUT(kTlItem | flags | (uint32_t)w, (word & ~kHdrTiles) | (uint32_t)(cnt / kG));
-          const uint32_t* src = p.tl_entries + (int64_t)unit * p.tl_cap;
+          TILE_HDR_PUT(kTlItem | flags | (uint32_t)w, (word & ~kHdrTiles) | odd | (uint32_t)(cnt / kG));
+          const uint32_t* src = p.tl_entries + (int64_t)list * p.tl_cap;
           for (int base = 0; base < cnt; base += 32) {
             const uint32_t e = (base + lane < cnt) ? __ldcg(src + base + lane) : 0u;
             const uint32_t c = nc & (kTlChunks - 1);
             LOSA_WAIT_RELAXED(&ctl->tl_empty[c], ((nc / kTlChunks) & 1u) ^ 1u);
             ctl->tl[c * 32 + lane] = e;
-            ptx::st_cluster_u32(tl1 + 4u * (c * 32 + lane), e);
-            ptx::fence_acq_rel_cluster();
+            if (PAIR) {
+              ptx::st_cluster_u32(tl1 + 4u * (c * 32 + lane), e);
+              ptx::fence_acq_rel_cluster();
+            }
             __syncwarp();
             if (lane == 0) {
               ptx::mbar_arrive(&ctl->tl_full[c]);
-              ptx::mbar_arrive_cluster(tl_full1 + 8u * c);
+              if (PAIR) ptx::mbar_arrive_cluster(tl_full1 + 8u * c);
             }
             ++nc;
           }
         } else {
           const uint32_t ent = kTlItem | flags | (uint32_t)w;
           int jlo, jhi;
-          pair_key_range(p, ent, jlo, jhi);
-          const uint32_t has = (2 * pr + 1 < p.nQb) ? 3u * kHdrHas : kHdrHas;
-          PAIR_HDR_PUT(ent, has | (uint32_t)((jhi - jlo + kG - 1) / kG));
+          tile_key_range(p, ent, jlo, jhi);
+          const bool two = 2 * (w % p.nPairs) + 1 < p.nQt;  // the pair's second query tile exists
+          if (PAIR) {
+            TILE_HDR_PUT(ent, (two ? 3u : 1u) * kHdrHas | (uint32_t)((jhi - jlo + kG - 1) / kG));
+          } else {
+            // (a query tile that does not exist is a unit without tiles)
+            TILE_HDR_PUT(ent, odd | ((two || !odd) ? kHdrHas | (uint32_t)((jhi - jlo + kG - 1) / kG) : 0u));
+          }
         }
         LOSA_WAIT_RELAXED(&ctl->hdr_next, (nu - 1u) & 1u);
       }
-      if (!p.stall) PAIR_HDR_PUT(kTlEnd, 0u);
+      if (!p.stall) TILE_HDR_PUT(kTlEnd, 0u);
     }
   } else {
     // ------------------------------------------------------------------ softmax warps (both CTAs)
@@ -502,7 +586,7 @@ losa_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     const int row = wl * 32 + lane;
     const uint32_t lane_base = (uint32_t)(wl * 32) << 16;
     const uint32_t tO = tmem_base + lane_base + 384;
-    const int my_bit = (int)rank;
+    const int sub = (R == 64) ? (wl >> 1) : 0;   // query block of the query tile
     constexpr int kHB = (kG >= 2) ? kG / 2 : 1;  // key blocks of a half (a half block when C = 128)
     constexpr int kBW = 64 / kHB;                // columns per such block
     uint64_t* const pair_bar = &ctl->pair_bar[grpi * 4 + wl];
@@ -516,7 +600,7 @@ losa_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
                                   : nullptr;
 
     for (;;) {
-      PAIR_HDR_NEXT(ent, word);
+      TILE_HDR_NEXT(ent, word);
       if ((ent >> 28) != 1) break;
       const int w = (int)(ent & kTlItemMask);
       const bool partial = (ent & kTlPartial) != 0;
@@ -525,77 +609,108 @@ losa_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       const int bh = pbh % (p.B * p.H);
       const int b = bh / p.H, h = bh % p.H;
       void* const o_base = (p.problems != nullptr) ? p.problems[pbh / (p.B * p.H)].o : p.o;
-      const int T = 2 * pr + (int)rank;
+      const int tile = PAIR ? (int)rank : (int)((word & kHdrOdd) != 0u);  // of the item's two query tiles
+      const int my_bit = tile * kQB + sub;
+      const int T = 2 * pr + tile;
       const int grow = T * 128 + row;
       float m_ref = 0.f, l = 0.f, le = 0.f;  // le: row sum of the unrounded exponentials (masses, LSE)
-      bool ovf = false;
+      bool ovf = false, seen = false;  // (seen: this warp met keys that its rows attend to)
       const int tiles = (int)(word & kHdrTiles);
       const uint32_t pv_item = (uint32_t)tiles;
-      // does this query tile list any of the unit's tiles?  (R = 128: a query tile is a query block)
-      const bool has = (word & (kHdrHas << my_bit)) != 0;
+      // does this query tile list any of the unit's tiles?
+      const bool has = (word & (PAIR ? kHdrHas << tile : kHdrHas)) != 0;
       // dense modes: the unit's key blocks, the end of its keys
       int jlo, jhi;
-      pair_key_range(p, ent, jlo, jhi);
+      tile_key_range(p, ent, jlo, jhi);
       const int kend = min(p.N, jhi * kC);
       // Score k of the launch (kq: of the unit's first tile) is worked on by group k % 2 and lies in
       // buffer k % 3, in that buffer's use k / 3.
       const int first = (grpi ^ (int)kq) & 1;
       uint32_t bsel = (kq + (uint32_t)first) % 3u, sph = ((kq + (uint32_t)first) / 3u) & 1u;
-      // ---- the reference of the unit: the rows' maximum over the first key tile this query tile
-      // lists, from the group that works on that tile - it is that group's first tile - to the other
-      if (has) {
-        const int late = (my_bit == 1 && (word & kHdrLate)) ? 1 : 0;
-        const uint32_t rs = nref & 1u;
-        if (first == late) {
-          if (MODE == kSparse) PAIR_CHUNK_WAIT();
-          uint32_t grp[kG];
-          if (MODE == kSparse) ptx::ld_shared_volatile_vec<kG>(&ctl->tl[(nc & (kTlChunks - 1)) * 32 + first * kG], grp);
-          LOSA_WAIT(&ctl->s_full[bsel], sph);
-          ptx::tc_fence_after_sync();
-          const uint32_t tSrow = tmem_base + lane_base + bsel * 128;
-          float mx = -INFINITY;
+      // ---- the reference of the unit: the rows' maximum over the first key tile their query block
+      // lists, from the group that works on that tile to the other.  Where the query tile is a query
+      // block that tile is one of the unit's first two, the first of the group that works on it, and
+      // the reference is exchanged here; with two query blocks (R = 64) and a list it may be any tile
+      // and is exchanged when the loop below comes to it.
+      constexpr bool kLazyRef = kQB > 1 && MODE == kSparse;
+      const uint32_t rs = nref & 1u;
+      bool have_ref = !has;
+      int ref_tile = (PAIR && tile == 1 && (word & kHdrLate)) ? 1 : 0;
+      bool listed_only = true;  // the maximum is over the keys the row attends to
+      auto row_max = [&](int i, uint32_t chunk, int at) {  // tile i of the unit, its group at `at` in the list
+        const uint32_t tSrow = tmem_base + lane_base + bsel * 128;
+        uint32_t grp[kG];
+        if (MODE == kSparse) ptx::ld_shared_volatile_vec<kG>(&ctl->tl[(chunk & (kTlChunks - 1)) * 32 + at], grp);
+        float mx = -INFINITY;
 #pragma unroll
-          for (int c0 = 0; c0 < kW; c0 += 32) {
-            uint32_t r[32];
-            ptx::tmem_ld32(tSrow + c0, r);
-            ptx::tmem_wait_ld();
+        for (int c0 = 0; c0 < kW; c0 += 32) {
+          uint32_t r[32];
+          ptx::tmem_ld32(tSrow + c0, r);
+          ptx::tmem_wait_ld();
 #pragma unroll
-            for (int c = 0; c < 32; ++c) {
-              const int cc = c0 + c;
-              int valid;  // of the key block's columns
-              if (MODE == kSparse)
-                valid = ((grp[cc / kC] >> (16 + my_bit)) & 1u) ? p.N - (int)(grp[cc / kC] & 0xffffu) * kC : 0;
-              else
-                valid = kend - (jlo + first * kG + cc / kC) * kC;
-              if ((cc % kC) < valid) mx = fmaxf(mx, __uint_as_float(r[c]));
-            }
+          for (int c = 0; c < 32; ++c) {
+            const int cc = c0 + c;
+            int valid;  // of the key block's columns
+            if (MODE == kSparse)
+              valid = (!listed_only || ((grp[cc / kC] >> (16 + my_bit)) & 1u))
+                          ? p.N - (int)(grp[cc / kC] & 0xffffu) * kC : 0;
+            else
+              valid = kend - (jlo + i * kG + cc / kC) * kC;
+            if ((cc % kC) < valid) mx = fmaxf(mx, __uint_as_float(r[c]));
           }
-          m_ref = mx * p.scale_log2;
-          // the other half reads the whole row too: nobody packs P over it before both are done
-          ptx::tc_fence_before_sync();
-          __syncwarp();
-          if (lane == 0) ptx::mbar_arrive(pair_bar);
-          LOSA_WAIT(pair_bar, npair & 1);
-          ++npair;
-          ptx::tc_fence_after_sync();
-          if (half == 0) {
-            // (the slot's last readers, two units with a reference ago, are done with it)
-            if (nref >= 2u) LOSA_WAIT(&ctl->ref_empty[rs], ((nref >> 1) - 1u) & 1);
-            ctl->ref[rs][row] = m_ref;
-            __syncwarp();
-            if (lane == 0) ptx::mbar_arrive(&ctl->ref_full[rs]);
-          }
-        } else {
-          LOSA_WAIT(&ctl->ref_full[rs], (nref >> 1) & 1);
-          m_ref = ctl->ref[rs][row];
-          __syncwarp();
-          if (lane == 0) ptx::mbar_arrive(&ctl->ref_empty[rs]);
         }
-        ++nref;
+        return mx * p.scale_log2;
+      };
+      // (m_ref of the group that has it; both halves read the whole row first, so that neither packs P
+      // over it before the other is done)
+#define TILE_REF_GIVE()                                                                             \
+  do {                                                                                              \
+    ptx::tc_fence_before_sync();                                                                    \
+    __syncwarp();                                                                                   \
+    if (lane == 0) ptx::mbar_arrive(pair_bar);                                                      \
+    LOSA_WAIT(pair_bar, npair & 1);                                                                 \
+    ++npair;                                                                                        \
+    ptx::tc_fence_after_sync();                                                                     \
+    if (half == 0) {                                                                                \
+      /* (the slot's last readers, two units with a reference ago, are done with it) */             \
+      if (nref >= 2u) LOSA_WAIT(&ctl->ref_empty[rs][sub], ((nref >> 1) - 1u) & 1);                  \
+      ctl->ref[rs][row] = m_ref;                                                                    \
+      __syncwarp();                                                                                 \
+      if (lane == 0) ptx::mbar_arrive(&ctl->ref_full[rs][sub]);                                     \
+    }                                                                                               \
+  } while (0)
+#define TILE_REF_TAKE()                                                                             \
+  do {                                                                                              \
+    LOSA_WAIT(&ctl->ref_full[rs][sub], (nref >> 1) & 1);                                            \
+    m_ref = ctl->ref[rs][row];                                                                      \
+    __syncwarp();                                                                                   \
+    if (lane == 0) ptx::mbar_arrive(&ctl->ref_empty[rs][sub]);                                      \
+  } while (0)
+      if (has) {
+        if (kLazyRef) {
+          // a query block that lists none of the first chunk's entries takes the maximum over all keys
+          // of the first tile
+          TILE_CHUNK_WAIT();
+          const uint32_t e = *reinterpret_cast<volatile uint32_t*>(&ctl->tl[(nc & (kTlChunks - 1)) * 32 + lane]);
+          const uint32_t mine = __ballot_sync(0xffffffffu, lane < tiles * kG && ((e >> (16 + my_bit)) & 1u));
+          listed_only = mine != 0u;
+          ref_tile = listed_only ? (__ffs(mine) - 1) / kG : 0;
+        } else {
+          if (first == ref_tile) {
+            if (MODE == kSparse) TILE_CHUNK_WAIT();
+            LOSA_WAIT(&ctl->s_full[bsel], sph);
+            ptx::tc_fence_after_sync();
+            m_ref = row_max(first, nc, first * kG);
+            TILE_REF_GIVE();
+          } else {
+            TILE_REF_TAKE();
+          }
+          have_ref = true;
+        }
       }
       const float2 sc2 = make_float2(p.scale_log2, p.scale_log2);
       for (int base = 0; base < tiles; base += kChunkTiles) {
-      if (MODE == kSparse) PAIR_CHUNK_WAIT();
+      if (MODE == kSparse) TILE_CHUNK_WAIT();
       const int end = min(tiles, base + kChunkTiles);
       for (int i = base + first; i < end; i += 2) {
         // the key blocks of this half of the tile: a half block (C = 128), one block, or two (C = 32)
@@ -618,7 +733,17 @@ losa_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         const uint32_t tS = tmem_base + lane_base + bsel * 128 + half * 64;
         LOSA_WAIT(&ctl->s_full[bsel], sph);
         ptx::tc_fence_after_sync();
+        if (kLazyRef && !have_ref && i >= ref_tile) {
+          if (i == ref_tile) {
+            m_ref = row_max(i, nc, (i - base) * kG);
+            TILE_REF_GIVE();
+          } else {
+            TILE_REF_TAKE();
+          }
+          have_ref = true;
+        }
         uint32_t sr[64];
+        if (kQB > 1) seen = seen || mine;
         if (mine) {
           ptx::tmem_ld32(tS, &sr[0]);
           ptx::tmem_wait_ld();
@@ -641,7 +766,7 @@ losa_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
             ptx::tmem_wait_ld();
             ptx::tc_fence_before_sync();
             __syncwarp();
-            if (lane == 0) ptx::mbar_arrive_cluster(p_ready0 + 8u * bsel);
+            if (lane == 0) arrive0<PAIR>(p_ready0 + 8u * bsel);
           }
           // key blocks the row's query block does not list get -inf as the addend of the scaling FMA
           // (one block per half or less: the half would not be here)
@@ -665,12 +790,16 @@ losa_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
                                   nm2[c / kBW]);
             float2 x1 = ptx::fma2(make_float2(__uint_as_float(sr[c + 2]), __uint_as_float(sr[c + 3])), sc2,
                                   nm2[c / kBW]);
-            // (a share of these on the FMA pipe, as at head dimension 64, measured -1 % at 12.5 %
-            // and +5 % at 25 % here: none)
-            x0.x = ptx::ex2_approx(x0.x);
-            x0.y = ptx::ex2_approx(x0.y);
-            x1.x = ptx::ex2_approx(x1.x);
-            x1.y = ptx::ex2_approx(x1.y);
+            // (at head dimension 128 a share of these on the FMA pipe measured -1 % at 12.5 % and +5 % at 25 %)
+            if (kPolyOf > 0 && (c >> 2) % (kPolyOf > 0 ? kPolyOf : 1) == 0) {
+              x0 = ptx::ex2_poly2(x0);
+              x1 = ptx::ex2_poly2(x1);
+            } else {
+              x0.x = ptx::ex2_approx(x0.x);
+              x0.y = ptx::ex2_approx(x0.y);
+              x1.x = ptx::ex2_approx(x1.x);
+              x1.y = ptx::ex2_approx(x1.y);
+            }
             if (kHasV) {
               const uint32_t u0 = ptx::pack_bf16x2(x0.x, x0.y), u1 = ptx::pack_bf16x2(x1.x, x1.y);
               sr[c >> 1] = u0;
@@ -710,7 +839,7 @@ losa_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
             // mass pass: the buffer goes back untouched
             ptx::tc_fence_before_sync();
             __syncwarp();
-            if (lane == 0) ptx::mbar_arrive_cluster(p_ready0 + 8u * bsel);
+            if (lane == 0) arrive0<PAIR>(p_ready0 + 8u * bsel);
           }
           // (a key block that fills the tile but ends before this half: its entry of the table is 0)
           if (kWantMass && kG == 1 && has &&
@@ -721,7 +850,7 @@ losa_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           ptx::tmem_wait_st();
           ptx::tc_fence_before_sync();
           __syncwarp();
-          if (lane == 0) ptx::mbar_arrive_cluster(p_ready0 + 8u * bsel);
+          if (lane == 0) arrive0<PAIR>(p_ready0 + 8u * bsel);
         }
         // two scores on: k + 2 lies in the buffer before k's, in that buffer's next use, or in the last one
         if (bsel == 0u) {
@@ -731,55 +860,66 @@ losa_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           sph ^= 1u;
         }
       }
-      if (MODE == kSparse) PAIR_CHUNK_DONE();
+      if (MODE == kSparse) TILE_CHUNK_DONE();
       }
       kq += (uint32_t)tiles;
 
       // ---- end of the item
+      if (kLazyRef && !have_ref) TILE_REF_TAKE();  // (this group met no tile from the reference's on)
+      if (has) ++nref;
+#undef TILE_REF_GIVE
+#undef TILE_REF_TAKE
       // the four partial sums of a row (two groups, two halves) meet in shared memory
       float* const xset = &ctl->xch[nitem & 1][0][0];
       xset[quarter * 128 + row] = l;
       if (kWantMass) xset[(4 + quarter) * 128 + row] = le;
-      if (ovf && lane == 0) {
+      auto hand_over = [&]() {
         const int unit = partial ? p.split_first + (w - p.split_first) * p.split_parts + part : w;
+        // (once per CTA: its two query tiles of one unit may come one after the other)
         if (atomicExch(&ctl->ovf_unit, unit) != unit) {
           const int slot = atomicAdd(p.redo_count, 1);
-          if (slot < 2 * p.nUnits) p.redo_list[slot] = unit;  // (each CTA of the pair may list it)
+          if (slot < 2 * p.nUnits) p.redo_list[slot] = unit;  // (each query tile may list it)
         }
-      }
+      };
+      if (ovf && lane == 0) hand_over();
       __syncwarp();
       if (lane == 0) ptx::mbar_arrive(&ctl->item_bar);
       LOSA_WAIT(&ctl->item_bar, nitem & 1);
       ++nitem;
       l = (xset[row] + xset[128 + row]) + (xset[256 + row] + xset[384 + row]);
+      // rows whose own keys lie 40 nats below a reference taken over other keys: their weights may have
+      // lost their tail
+      if (kQB > 1 && __any_sync(0xffffffffu, seen && l < kTileSafeLow) && lane == 0) hand_over();
       if (kHasV) {
-        // every thread writes out a quarter (32 columns) of its row of O
+        // every thread writes out a quarter of its row of O
         const bool valid = (T < p.nQt) && grow < p.N;
         const float inv = (l > 0.f) ? 1.f / l : 0.f;
         const int64_t off = (int64_t)b * p.sb + (int64_t)h * p.sh + (int64_t)grow * p.sn;
-        const int64_t pslot = ((((int64_t)(w - p.split_first) * p.split_parts + part) * 2 + (int)rank) * 128 + row);
+        const int64_t pslot = ((((int64_t)(w - p.split_first) * p.split_parts + part) * 2 + tile) * 128 + row);
         if (partial && quarter == 0 && T < p.nQt && LOSA_IN_RANGE(pslot, p.cap_part_rows)) p.part_ml[pslot] = make_float2(m_ref, l);
-        const int c0 = quarter * 32;
-        uint32_t r[32];
+        constexpr int kOC = D / 4;
+        const int c0 = quarter * kOC;
+        uint32_t r[kOC];
         if (pv_item > 0) {
           LOSA_WAIT(&ctl->o_done, nod & 1);
           ++nod;
           ptx::tc_fence_after_sync();
-          ptx::tmem_ld32(tO + c0, r);
+          if constexpr (kOC == 32) ptx::tmem_ld32(tO + c0, r);
+          else ptx::tmem_ld16(tO + c0, r);
           ptx::tmem_wait_ld();
           // (O is in registers: the next item's first product may overwrite it)
           ptx::tc_fence_before_sync();
           __syncwarp();
-          if (lane == 0) ptx::mbar_arrive_cluster(o_free0);
+          if (lane == 0) arrive0<PAIR>(o_free0);
         } else {
 #pragma unroll
-          for (int c = 0; c < 32; ++c) r[c] = 0u;
+          for (int c = 0; c < kOC; ++c) r[c] = 0u;
         }
         if (partial) {
           if (T < p.nQt) {
             float4* dst = reinterpret_cast<float4*>(p.part_o + (LOSA_IN_RANGE(pslot, p.cap_part_rows) ? pslot : 0) * D + c0);
 #pragma unroll
-            for (int c = 0; c < 32; c += 4)
+            for (int c = 0; c < kOC; c += 4)
               dst[c >> 2] = make_float4(__uint_as_float(r[c]), __uint_as_float(r[c + 1]),
                                         __uint_as_float(r[c + 2]), __uint_as_float(r[c + 3]));
           }
@@ -787,13 +927,13 @@ losa_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           if (p.o_f32) {
             float4* dst = reinterpret_cast<float4*>(static_cast<float*>(o_base) + off + c0);
 #pragma unroll
-            for (int c = 0; c < 32; c += 4)
+            for (int c = 0; c < kOC; c += 4)
               dst[c >> 2] = make_float4(__uint_as_float(r[c]) * inv, __uint_as_float(r[c + 1]) * inv,
                                         __uint_as_float(r[c + 2]) * inv, __uint_as_float(r[c + 3]) * inv);
           } else {
             uint4* dst = reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(o_base) + off + c0);
 #pragma unroll
-            for (int c = 0; c < 32; c += 8) {
+            for (int c = 0; c < kOC; c += 8) {
               uint4 v;
               v.x = ptx::pack_bf16x2(__uint_as_float(r[c]) * inv, __uint_as_float(r[c + 1]) * inv);
               v.y = ptx::pack_bf16x2(__uint_as_float(r[c + 2]) * inv, __uint_as_float(r[c + 3]) * inv);
@@ -824,22 +964,28 @@ losa_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
             const float le_r = (xset[512 + r] + xset[640 + r]) + (xset[768 + r] + xset[896 + r]);
             iv[rr] = (T * 128 + r < p.N && le_r > 0.f) ? 1.f / le_r : 0.f;
           }
-          const int nvalid = min(R, p.N - T * R);
           for (int u = sw; u < p.nKb; u += 16) {
-            float acc = 0.f;
+            float acc[kQB];
+#pragma unroll
+            for (int q = 0; q < kQB; ++q) acc[q] = 0.f;
 #pragma unroll
             for (int rr = 0; rr < 4; ++rr) {
               const int r = rr * 32 + lane;
               if (iv[rr] > 0.f) {
                 const float sum = (kG >= 2) ? tb[(int64_t)u * 128 + r]
                                             : tb[(int64_t)u * 256 + r] + tb[(int64_t)u * 256 + 128 + r];
-                acc += sum * iv[rr];
+                acc[(rr * 32) / R] += sum * iv[rr];
               }
             }
 #pragma unroll
-            for (int d = 16; d > 0; d >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, d);
-            const int64_t mi = ((int64_t)bh * p.nQb + T) * p.nKb + u;
-            if (lane == 0 && LOSA_IN_RANGE(mi, p.cap_mass)) p.mass[mi] = acc / (float)nvalid;
+            for (int q = 0; q < kQB; ++q) {
+#pragma unroll
+              for (int d = 16; d > 0; d >>= 1) acc[q] += __shfl_xor_sync(0xffffffffu, acc[q], d);
+              const int g = T * kQB + q;
+              const int64_t mi = ((int64_t)bh * p.nQb + g) * p.nKb + u;
+              if (lane == 0 && g < p.nQb && LOSA_IN_RANGE(mi, p.cap_mass))
+                p.mass[mi] = acc[q] / (float)min(R, p.N - g * R);
+            }
           }
         }
         // (the table is written again by the next item)
@@ -854,11 +1000,11 @@ losa_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
 teardown:
   if (ctl->abort_flag) {
     // the other CTA's waits give up at their next look at the flag
-    if (lane == 0) ptx::st_cluster_u32(abort_peer, 1u);
+    if (PAIR && lane == 0) ptx::st_cluster_u32(abort_peer, 1u);
     // give MMAs and bulk copies still in flight a bounded time to land before shared memory and
     // tensor memory are released
     if (rank == 0 && (warp == kIssuerWarp || warp == kIssuerWarp + 1) && ptx::elect_one()) {
-      ptx::mma2_commit(&ctl->drain);
+      commit0<PAIR>(&ctl->drain);
       for (uint32_t it = 0; it < (1u << 16); ++it) {
         if (ptx::mbar_try_wait(&ctl->drain, 0)) break;
         __nanosleep(128);
@@ -871,15 +1017,16 @@ teardown:
   ptx::tc_fence_before_sync();
   __syncthreads();
   // neither CTA leaves, or frees its tensor memory, while the other may still signal into it
-  ptx::cluster_sync();
+  if (PAIR) ptx::cluster_sync();
   if (warp == kIssuerWarp) {
     ptx::tc_fence_after_sync();
-    ptx::tmem_dealloc2(tmem_base, kTmemCols);
+    if (PAIR) ptx::tmem_dealloc2(tmem_base, kTmemCols);
+    else ptx::tmem_dealloc(tmem_base, kTmemCols);
   }
 }
 
-#undef PAIR_HDR_PUT
-#undef PAIR_HDR_NEXT
-#undef PAIR_CHUNK_WAIT
-#undef PAIR_CHUNK_DONE
-#undef PAIR_WAIT_CL
+#undef TILE_HDR_PUT
+#undef TILE_HDR_NEXT
+#undef TILE_CHUNK_WAIT
+#undef TILE_CHUNK_DONE
+#undef TILE_WAIT

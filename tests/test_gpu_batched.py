@@ -139,3 +139,9 @@ def test_batched_call_replays_from_a_graph(L):
     torch.cuda.synchronize()
     assert losa.losa_async_status() == 0
     assert all(torch.equal(a, b) for a, b in zip(ref, outs))
+
+
+@pytest.mark.parametrize("R,C", [(64, 64), (128, 32), (128, 128)])
+def test_layers_of_head_dimension_64_equal_the_single_calls_bit_for_bit(R, C):
+    """74 items: whole work units, alone and three layers at once, on a GPU with 148 SMs."""
+    test_three_layers_in_one_launch_equal_the_single_calls_bit_for_bit(1, 37, 128 * 4 - 9, 64, R, C)

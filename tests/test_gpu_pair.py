@@ -172,3 +172,24 @@ def test_tile_lists_that_end_around_a_chunk_of_the_list(C):
         ref = orc.blocks_to_tokens(
             orc.sparse_attn(util.to_np(q), util.to_np(k), util.to_np(v), R, C, off, idx), 1, H, N)
         util.assert_output_close(o, ref, f"C={C} H={H}")
+
+
+@pytest.mark.parametrize("R,C", [(64, 64), (128, 64), (128, 32), (128, 128)])
+@pytest.mark.parametrize("kind", ["disjoint_singletons", "late_only_tile", "odd_position_first", "interleaved", "random"])
+def test_crafted_patterns_at_head_dimension_64(R, C, kind):
+    """One query tile per CTA and a list per query tile; with 64-row blocks a query tile's two blocks
+    meet their first listed tile at different places, in either softmax group, or past the first chunk
+    of the list (2560 keys here), where the reference falls back to the tile's own maximum."""
+    losa = lib()
+    H, N = 2, 128 * 41 - 37
+    nQb, nKb = -(-N // R), -(-N // C)
+    lists = []
+    for h in range(H):
+        lists += patterns(nQb, nKb, kind, 31 + h)
+    off, idx = csr_from(lists)
+    q, k, v = (util.rand_bf16((1, H, N, 64), 970 + i, 1.0 if i == 2 else 2.0) for i in range(3))
+    o = losa.losa_sparse_attn(q.cuda(), k.cuda(), v.cuda(), torch.from_numpy(off).cuda(),
+                              torch.from_numpy(idx).cuda(), R, C, out_dtype=torch.float32)
+    assert losa.losa_async_status() == 0
+    ref = orc.blocks_to_tokens(orc.sparse_attn(util.to_np(q), util.to_np(k), util.to_np(v), R, C, off, idx), 1, H, N)
+    util.assert_output_close(o, ref, f"{kind} R={R} C={C}")
