@@ -1878,24 +1878,6 @@ write_problems_kernel(const __grid_constant__ ProblemChunk chunk, ProblemEntry* 
   for (int i = threadIdx.x; i < n * (int)(sizeof(ProblemEntry) / sizeof(uint4)); i += blockDim.x) dst[i] = src[i];
 }
 
-// Launches `kern`; `dependent`: it may be scheduled before the kernel ahead of it in the stream has
-// finished, and waits for it itself (grid_dependency_wait).
-template <typename... P, typename... A>
-int launch(void (*kern)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st, bool dependent, const A&... args) {
-  cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.gridDim = grid;
-  cfg.blockDim = dim3(threads, 1, 1);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cfg.attrs = attr;
-  cfg.numAttrs = dependent ? 1 : 0;
-  LOSA_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, args...));
-  return LOSA_OK;
-}
-
 // Configures (once per device) and launches one layout of the attention kernel.
 template <int D, int R, int C_, int MODE, int KT, bool SPLIT>
 int launch_kernel(const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv, const CUtensorMap& mkw,

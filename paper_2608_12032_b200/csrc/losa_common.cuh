@@ -54,6 +54,24 @@ int make_geometry(const losa_problem_t* p, Geometry* g);  // LOSA_OK or an error
     }                                                              \
   } while (0)
 
+// Launches `kern`; `dependent`: it may be scheduled before the kernel ahead of it in the stream has
+// finished, and waits for it itself (grid_dependency_wait).
+template <typename... P, typename... A>
+int launch(void (*kern)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st, bool dependent, const A&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads, 1, 1);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = attr;
+  cfg.numAttrs = dependent ? 1 : 0;
+  LOSA_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, args...));
+  return LOSA_OK;
+}
+
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 // ---- entry points of the kernel translation units (host launchers) -------------------

@@ -12,6 +12,7 @@
 #include <limits.h>
 
 #include "losa_common.cuh"
+#include "losa_ptx.cuh"
 
 namespace losa {
 namespace {
@@ -37,7 +38,8 @@ namespace {
 // every value about 70 times: 22296 rows of 3713 blocks took 5.48 ms, of 929 blocks 0.33 ms.
 constexpr int kBins = 608;   // per lane of one warp 19, an odd number: the scan has no bank conflicts
 constexpr int kTauShift = 19, kCountShift = 22;
-constexpr int kTopBin = 0x41000000 >> kTauShift;  // of the largest mass, 8.0
+constexpr uint32_t kMaxMassBits = 0x41000000u;       // the largest mass, 8.0
+constexpr int kTopBin = kMaxMassBits >> kTauShift;
 constexpr int kListCap = 256;
 constexpr double kFixedOne = 1152921504606846976.0;  // 2^60
 
@@ -47,10 +49,8 @@ struct RowShared {
   unsigned long long total[8];   // per warp of the row
   unsigned long long above;      // weight of the bins heavier than the one of v*
   double sum[8];
-  int bin, cnt_above, list_len;
-  uint32_t v;
-  int need, s, eq_total;
-  int eq[8];
+  int bin, list_len;
+  int part[8];
 };
 
 // (cap: see `tiny` below)
@@ -86,38 +86,98 @@ __device__ __forceinline__ unsigned long long row_sum_u64(unsigned long long a, 
   return t;
 }
 
+// What a list of m values (low bits x) is searched for: the largest v with weight(values >= v) >= missing,
+// and how many of the values equal to v are needed.  A value weighs lead + x, or 1 if COUNT.  Whole warp.
+template <bool COUNT>
+__device__ __forceinline__ void search_list(const uint32_t* list, int m, int bits, uint32_t lead,
+                                            unsigned long long missing, int lane, uint32_t* v_out, int* need_out,
+                                            int* eq_out) {
+  uint32_t v = 0u;
+  int n_ge = m, n_eq = 0;
+  unsigned long long ge = 0ull;  // weight of the values >= v
+  if (m <= 32) {
+    // every lane adds up the values at or above its own
+    const uint32_t x = (lane < m) ? list[lane] : 0u;
+    uint32_t n = 0u, l = 0u;
+    for (int j = 0; j < m; ++j) {
+      const uint32_t y = __shfl_sync(0xffffffffu, x, j);
+      n += (y >= x) ? 1u : 0u;
+      l += (y >= x) ? y : 0u;
+    }
+    const unsigned long long w = COUNT ? n : (unsigned long long)n * lead + l;
+    const bool ok = lane < m && w >= missing;
+    v = __reduce_max_sync(0xffffffffu, ok ? x : 0u);
+    const uint32_t eq = __ballot_sync(0xffffffffu, lane < m && x == v);
+    n_eq = __popc(eq);
+    const int src = __ffs(eq) - 1;
+    n_ge = (int)__shfl_sync(0xffffffffu, n, src);
+    ge = __shfl_sync(0xffffffffu, w, src);
+  } else {
+    // bit by bit
+    auto measure = [&](uint32_t from, int* n_out) -> unsigned long long {
+      uint32_t n = 0u, l = 0u;
+      for (int i = lane; i < m; i += 32) {
+        const uint32_t x = list[i];
+        n += (x >= from) ? 1u : 0u;
+        l += (x >= from) ? x : 0u;
+      }
+      n = __reduce_add_sync(0xffffffffu, n);
+      *n_out = (int)n;
+      if (COUNT) return n;
+      l = __reduce_add_sync(0xffffffffu, l);
+      return (unsigned long long)n * lead + l;
+    };
+    for (int b = bits - 1; b >= 0; --b) {
+      int n;
+      if (measure(v | (1u << b), &n) >= missing) v |= 1u << b;
+    }
+    ge = measure(v, &n_ge);
+    int n_gt;
+    measure(v + 1u, &n_gt);
+    n_eq = n_ge - n_gt;
+  }
+  int need = n_eq;
+  if (n_eq > 1) {
+    const unsigned long long each = COUNT ? 1ull : (unsigned long long)lead + v;
+    const unsigned long long gt = ge - (unsigned long long)n_eq * each;  // weight of the values > v
+    need = (int)min((missing - gt + each - 1ull) / each, (unsigned long long)n_eq);
+  }
+  *v_out = v;
+  *need_out = need;
+  *eq_out = n_eq;
+}
+
 // W warps per row, K blocks per lane: warp w of the row owns blocks [w * 32 K, (w + 1) * 32 K), its
 // lane l the blocks l, l + 32, ... of those, so that a ballot is a bitmap word.  One row per CTA, or
-// four at W = 1.
-template <int W, int K>
-__global__ void __launch_bounds__(W == 1 ? 128 : 32 * W)
+// four at W = 1.  COUNT: the fixed-ratio rule.
+template <int W, int K, bool COUNT>
+__global__ void __launch_bounds__(W == 1 ? 128 : 32 * W, W == 1 ? 7 : 28 / W)
 select_rows_kernel(const float* __restrict__ mass, int rows, int nKb, double tau, int fixed_count,
                    int32_t* __restrict__ counts, uint32_t* __restrict__ bitmaps, int* status) {
   constexpr int kRowsPerCta = (W == 1) ? 4 : 1;
   constexpr int T = 32 * W;
+  constexpr int kShift = COUNT ? kCountShift : kTauShift;
+  constexpr int kBase = COUNT ? 0 : kTopBin - (kBins - 1);
+  constexpr uint32_t kLowMask = (1u << kShift) - 1u;
   __shared__ RowShared shared[kRowsPerCta];
   const int lane = threadIdx.x & 31;
   const int warp = (W == 1) ? 0 : threadIdx.x >> 5;     // of the row
   const int t = warp * 32 + lane;                       // thread of the row
   RowShared* const rs = &shared[(W == 1) ? threadIdx.x >> 5 : 0];
   const int64_t row = (int64_t)blockIdx.x * kRowsPerCta + ((W == 1) ? threadIdx.x >> 5 : 0);
+  ptx::grid_launch_dependents();
   if (row >= rows) return;
   const int words = (nKb + 31) >> 5;
-  const float* mrow = mass + row * nKb;
-  const int first = warp * 32 * K + lane;
-  const bool counting = fixed_count > 0;
-  const int shift = counting ? kCountShift : kTauShift;
-  const int base = counting ? 0 : kTopBin - (kBins - 1);
+  const int mine = min(32 * K, nKb - warp * 32 * K);    // blocks of this warp (may be none)
+  const float* src = mass + row * nKb + warp * 32 * K + lane;
 
+  // (blocks past the row's end weigh nothing; they are told apart by their index where they could count)
   uint32_t bits[K];
 #pragma unroll
-  for (int k = 0; k < K; ++k) {
-    const int i = first + k * 32;
-    bits[k] = (i < nKb) ? __float_as_uint(__ldg(mrow + i)) : 0u;
-  }
+  for (int k = 0; k < K; ++k) bits[k] = (k * 32 + lane < mine) ? __float_as_uint(__ldg(src + k * 32)) : 0u;
   for (int i = t; i < kBins; i += T) {
     rs->cnt[i] = 0u;
-    rs->low[i] = 0u;
+    if (!COUNT) rs->low[i] = 0u;
   }
   if (t == 0) {
     rs->list_len = 0;
@@ -126,20 +186,18 @@ select_rows_kernel(const float* __restrict__ mass, int rows, int nKb, double tau
   row_sync<W>();
   bool bad = false;
   float sum = 0.0f;
-  const uint32_t low_mask = (1u << shift) - 1u;
 #pragma unroll
   for (int k = 0; k < K; ++k) {
-    const float m = __uint_as_float(bits[k]);
-    if (!(m >= 0.0f) || m > 8.0f) {  // negative, NaN, or far beyond any mass
-      bad = true;
+    if (bits[k] > kMaxMassBits) {  // negative, NaN, or far beyond any mass; -0 becomes +0
+      bad = bad || bits[k] != 0x80000000u;
       bits[k] = 0u;
     }
-    if (bits[k] == 0x80000000u) bits[k] = 0u;  // -0 becomes +0
     sum += __uint_as_float(bits[k]);
-    if (first + k * 32 < nKb) {
-      const int bin = max((int)(bits[k] >> shift) - base, 0);
+    // (a mass of zero changes no sum: only the fixed-ratio rule counts it)
+    if (COUNT ? k * 32 + lane < mine : bits[k] != 0u) {
+      const int bin = max((int)(bits[k] >> kShift) - kBase, 0);
       atomicAdd(&rs->cnt[bin], 1u);
-      if (!counting) atomicAdd(&rs->low[bin], bits[k] & low_mask);
+      if (!COUNT) atomicAdd(&rs->low[bin], bits[k] & kLowMask);
     }
   }
   // The fixed-point sums hold at most 16: a row whose masses add up to more than 8 (a mass row sums
@@ -155,37 +213,38 @@ select_rows_kernel(const float* __restrict__ mass, int rows, int nKb, double tau
     for (int w = 0; w < W; ++w) row_sum += rs->sum[w];
   }
   const bool too_heavy = row_sum > 8.0;
-  if (bad || (t == 0 && too_heavy && (!counting || W > 1))) report_error(status, LOSA_ERR_BAD_MASS);
+  if (bad || (t == 0 && too_heavy && (!COUNT || W > 1))) report_error(status, LOSA_ERR_BAD_MASS);
 
   // A tau far below any useful threshold would be lost in units of 2^-60: its rows are searched over
   // the registers in units of about 2^-50 tau, with every weight cut off at tau (a block of that mass
   // reaches the threshold alone), so that sums still fit.  (Every positive float is above 2^-200.)
-  const bool tiny = !counting && tau < 0x1p-20;
+  const bool tiny = !COUNT && tau < 0x1p-20;
   double scale = kFixedOne, cap = 8.0;
   if (tiny) {
     cap = fmax(tau, 0x1p-200);
     scale = __hiloint2double((1023 + 49 - (((__double2hiint(cap) >> 20) & 0x7ff) - 1023)) << 20, 0);
   }
-  const unsigned long long target = counting ? (unsigned long long)min(fixed_count, nKb)
-                                             : (unsigned long long)(fmin(tiny ? cap : tau, 1.0) * scale);
-  bool all = !counting && (tau >= 1.0 || too_heavy);  // (too heavy: keeps every block)
+  const unsigned long long target = COUNT ? (unsigned long long)min(fixed_count, nKb)
+                                          : (unsigned long long)(fmin(tiny ? cap : tau, 1.0) * scale);
+  bool all = !COUNT && (tau >= 1.0 || too_heavy);  // (too heavy: keeps every block)
   uint32_t v = 0u;   // kept: bits > v, and the first `need` (by index) with bits == v
-  int need = 0, s = nKb, eq_total = 0;
+  int need = 0, eq_total = 0;
   if (!all) {
     // ---- the bin of v*: thread t owns bins [hi - kPer + 1, hi], heaviest bins first
     constexpr int kPer = (kBins + T - 1) / T;
     const int hi = kBins - 1 - t * kPer;
     auto bin_weight = [&](int b) -> unsigned long long {
       const uint32_t c = rs->cnt[b];
-      if (counting) return c;
-      if (c == 0u || b == 0) return 0ull;
-      const uint32_t lead = (uint32_t)(b + base);  // exponent and four mantissa bits
+      if (COUNT) return c;
+      const uint32_t lead = (uint32_t)(b + kBase);  // exponent and four mantissa bits
       const unsigned long long mant = (unsigned long long)c * ((16u | (lead & 15u)) << kTauShift) + rs->low[b];
-      return mant << ((lead >> 4) - 90u);  // the mantissa's unit is 2^(e - 150); e >= 92 here
+      return (b == 0) ? 0ull : mant << ((lead >> 4) - 90u);  // the mantissa's unit is 2^(e - 150); e >= 92 here
     };
-    unsigned long long mine = 0ull;
-    for (int b = hi; b > hi - kPer && b >= 0; --b) mine += bin_weight(b);
-    unsigned long long incl = mine;
+    unsigned long long own = 0ull;
+#pragma unroll
+    for (int j = 0; j < kPer; ++j)
+      if (hi - j >= 0) own += bin_weight(hi - j);
+    unsigned long long incl = own;
 #pragma unroll
     for (int d = 1; d < 32; d <<= 1) {
       const unsigned long long up = __shfl_up_sync(0xffffffffu, incl, d);
@@ -198,7 +257,7 @@ select_rows_kernel(const float* __restrict__ mass, int rows, int nKb, double tau
       for (int w = 0; w < W; ++w)
         if (w < warp) incl += rs->total[w];
     }
-    unsigned long long acc = incl - mine;
+    unsigned long long acc = incl - own;
     if (acc < target && incl >= target) {  // exactly one thread, or none
       for (int b = hi; b > hi - kPer && b >= 0; --b) {
         const unsigned long long w = bin_weight(b);
@@ -211,87 +270,41 @@ select_rows_kernel(const float* __restrict__ mass, int rows, int nKb, double tau
       }
     }
     row_sync<W>();
-    const int bin = tiny ? -1 : rs->bin;
-    const uint32_t lead = (uint32_t)(bin + base);
     // ---- v* within the bin
-    bool listed = false;
-    if (bin >= 0) {
-      const uint32_t m = rs->cnt[bin];
-      listed = m <= (uint32_t)kListCap;
-      if (listed) {
+    const int bin = tiny ? -1 : rs->bin;
+    const uint32_t lead = (uint32_t)(bin + kBase);
+    const int m = (bin >= 0) ? (int)rs->cnt[bin] : 0;
+    if (bin >= 0 && m <= kListCap) {
 #pragma unroll
-        for (int k = 0; k < K; ++k) {
-          const bool in = (first + k * 32 < nKb) && (bits[k] >> shift) == lead;
-          const uint32_t mask = __ballot_sync(0xffffffffu, in);
-          if (mask != 0u) {
-            int at = 0;
-            if (lane == 0) at = atomicAdd(&rs->list_len, __popc(mask));
-            at = __shfl_sync(0xffffffffu, at, 0) + __popc(mask & ((1u << lane) - 1u));
-            if (in) rs->list[at] = bits[k] & low_mask;
-          }
+      for (int k = 0; k < K; ++k) {
+        const bool in = (bits[k] >> kShift) == lead && (!COUNT || k * 32 + lane < mine);
+        const uint32_t mask = __ballot_sync(0xffffffffu, in);
+        if (mask != 0u) {
+          int at = 0;
+          if (lane == 0) at = atomicAdd(&rs->list_len, __popc(mask));
+          at = __shfl_sync(0xffffffffu, at, 0) + __popc(mask & ((1u << lane) - 1u));
+          if (in) rs->list[at] = bits[k] & kLowMask;
         }
-        row_sync<W>();
-        if (warp == 0) {
-          // what the bin has to add, in units of the bin's mantissas: rounded up, the sums below are whole
-          const uint32_t lift = counting ? 0u : (lead >> 4) - 90u;
-          const unsigned long long missing =
-              (target - rs->above + ((1ull << lift) - 1ull)) >> lift;
-          const unsigned long long lead_mant = counting ? 1ull : (unsigned long long)((16u | (lead & 15u)) << kTauShift);
-          const int groups = ((int)m + 31) >> 5;
-          uint32_t lv = 0u;
-          auto measure = [&](uint32_t from, int* n_out) -> unsigned long long {
-            uint32_t n = 0u, l = 0u;
-            for (int g = 0; g < groups; ++g) {
-              const int i = g * 32 + lane;
-              const uint32_t x = (i < (int)m) ? rs->list[i] : 0u;
-              const bool ge = (i < (int)m) && x >= from;
-              n += ge ? 1u : 0u;
-              l += ge ? x : 0u;
-            }
-            n = __reduce_add_sync(0xffffffffu, n);
-            *n_out = (int)n;
-            if (counting) return n;
-            l = __reduce_add_sync(0xffffffffu, l);
-            return n * lead_mant + l;
-          };
-          int n_ge = (int)m;  // of the bin's values, those >= lv
-          for (int b = shift - 1; b >= 0; --b) {
-            int n;
-            if (measure(lv | (1u << b), &n) >= missing) {
-              lv |= 1u << b;
-              n_ge = n;
-            }
-          }
-          int n_gt;
-          const unsigned long long gt = measure(lv + 1u, &n_gt);
-          const unsigned long long each = counting ? 1ull : lead_mant + lv;
-          const int n_eq = n_ge - n_gt;
-          const int take = (int)min((missing - gt + each - 1ull) / each, (unsigned long long)n_eq);
-          // blocks of the bins above
-          int c_above = 0;
-          for (int b = bin + 1 + lane; b < kBins; b += 32) c_above += (int)rs->cnt[b];
-          c_above = __reduce_add_sync(0xffffffffu, c_above);
-          if (lane == 0) {
-            rs->v = (lead << shift) | lv;
-            rs->need = take;
-            rs->eq_total = n_eq;
-            rs->s = c_above + n_gt + take;
-          }
-        }
-        row_sync<W>();
-        v = rs->v;
-        need = rs->need;
-        s = rs->s;
-        eq_total = rs->eq_total;
       }
-    }
-    if (!listed) {
-      // ---- bit by bit over the row: masked sums (or counts) of the blocks with bits >= v
+      row_sync<W>();
+      // what the bin has to add, in units of the bin's mantissas: rounded up, its sums are whole (every
+      // warp searches the list for itself: no hand-over)
+      const uint32_t lift = COUNT ? 0u : (lead >> 4) - 90u;
+      const unsigned long long missing = (target - rs->above + ((1ull << lift) - 1ull)) >> lift;
+      search_list<COUNT>(rs->list, m, kShift, (16u | (lead & 15u)) << kTauShift, missing, lane, &v, &need, &eq_total);
+      v |= lead << kShift;
+    } else {
+      // ---- bit by bit over the row: masked sums (or counts) of the blocks with bits >= v (read again, so
+      // that this path takes no registers from the other)
       auto measure_ge = [&](uint32_t from) -> unsigned long long {
         unsigned long long a = 0ull;
-#pragma unroll
-        for (int k = 0; k < K; ++k)
-          if (bits[k] >= from && first + k * 32 < nKb) a += counting ? 1ull : fixed_weight(bits[k], scale, cap);
+#pragma unroll 1
+        for (int k = 0; k * 32 + lane < mine; ++k) {
+          uint32_t x = __float_as_uint(__ldg(src + k * 32));
+          if (x > kMaxMassBits) x = 0u;
+          if (x >= from) a += COUNT ? 1ull : fixed_weight(x, scale, cap);
+        }
+        __syncwarp();
         return row_sum_u64<W>(a, rs, warp, lane);
       };
       all = measure_ge(0u) < target;  // never reaches tau
@@ -301,54 +314,65 @@ select_rows_kernel(const float* __restrict__ mass, int rows, int nKb, double tau
           if (measure_ge(cand) >= target) v = cand;
         }
         const unsigned long long gt = measure_ge(v + 1u);
-        unsigned long long n = 0ull;  // how many are above v, and how many equal it
+        unsigned long long n = 0ull;
 #pragma unroll
-        for (int k = 0; k < K; ++k) {
-          const bool valid = first + k * 32 < nKb;
-          if (valid && bits[k] > v) n += 1ull;
-          if (valid && bits[k] == v) n += 1ull << 20;
-        }
-        n = row_sum_u64<W>(n, rs, warp, lane);
-        const int n_gt = (int)(n & 0xfffffull);
-        eq_total = (int)(n >> 20);
-        const unsigned long long fv = counting ? 1ull : fixed_weight(v, scale, cap);
+        for (int k = 0; k < K; ++k) n += (k * 32 + lane < mine && bits[k] == v) ? 1ull : 0ull;
+        eq_total = (int)row_sum_u64<W>(n, rs, warp, lane);
+        const unsigned long long fv = COUNT ? 1ull : fixed_weight(v, scale, cap);
         const unsigned long long need64 = (fv == 0ull) ? (unsigned long long)eq_total : (target - gt + fv - 1ull) / fv;
         need = (int)min(need64, (unsigned long long)eq_total);
-        s = n_gt + need;
       }
     }
   }
-  // ---- bitmap words; of the blocks equal to v the first `need` by index
-  int seen = 0;  // ties at lower indices
-  if (!all && need < eq_total) {  // (otherwise all ties are kept and their order does not matter)
-    int n = 0;
+  // ---- bitmap words
+  uint32_t out = 0u;  // lane k: word k of this warp's K
+  if (all || need >= eq_total) {
+    // (all ties are kept: their order does not matter)
+    const uint32_t from = all ? 0u : v;
 #pragma unroll
-    for (int k = 0; k < K; ++k) n += (first + k * 32 < nKb && bits[k] == v) ? 1 : 0;
-    n = __reduce_add_sync(0xffffffffu, n);
+    for (int k = 0; k < K; ++k) {
+      const uint32_t word = __ballot_sync(0xffffffffu, bits[k] >= from);
+      if (lane == k) out = word;
+    }
+  } else {
+    // of the blocks equal to v the first `need` by index
+    int seen = 0;  // ties at lower indices
     if (W > 1) {
-      if (lane == 0) rs->eq[warp] = n;
+      int n = 0;
+#pragma unroll
+      for (int k = 0; k < K; ++k) n += (k * 32 + lane < mine && bits[k] == v) ? 1 : 0;
+      n = __reduce_add_sync(0xffffffffu, n);
+      if (lane == 0) rs->part[warp] = n;
       __syncthreads();
 #pragma unroll
       for (int w = 0; w < W; ++w)
-        if (w < warp) seen += rs->eq[w];
+        if (w < warp) seen += rs->part[w];
+      __syncthreads();
     }
-  }
-  uint32_t out = 0u;  // lane k: word k of this warp's K
 #pragma unroll
-  for (int k = 0; k < K; ++k) {
-    const bool valid = first + k * 32 < nKb;
-    bool keep = valid && (all || bits[k] > v);
-    if (!all) {
-      const bool eq = valid && bits[k] == v;
+    for (int k = 0; k < K; ++k) {
+      const bool eq = k * 32 + lane < mine && bits[k] == v;
       const uint32_t eqm = __ballot_sync(0xffffffffu, eq);
-      keep = keep || (eq && seen + __popc(eqm & ((1u << lane) - 1u)) < need);
+      const uint32_t word =
+          __ballot_sync(0xffffffffu, bits[k] > v || (eq && seen + __popc(eqm & ((1u << lane) - 1u)) < need));
       seen += __popc(eqm);
+      if (lane == k) out = word;
     }
-    const uint32_t word = __ballot_sync(0xffffffffu, keep);
-    if (lane == k) out = word;
   }
+  // (bits of blocks past the end of the row)
+  const int valid = mine - lane * 32;
+  if (lane >= K || valid <= 0) out = 0u;
+  else if (valid < 32) out &= (1u << valid) - 1u;
   if (lane < K && warp * K + lane < words) bitmaps[row * words + warp * K + lane] = out;
-  if (t == 0) counts[row] = s;
+  int kept = __reduce_add_sync(0xffffffffu, __popc(out));
+  if (W > 1) {
+    if (lane == 0) rs->part[warp] = kept;
+    __syncthreads();
+    kept = 0;
+#pragma unroll
+    for (int w = 0; w < W; ++w) kept += rs->part[w];
+  }
+  if (t == 0) counts[row] = kept;
 }
 
 // Bitmaps -> ascending indices, `per_cta` consecutive rows per CTA.  The CTA first adds up the sizes
@@ -367,12 +391,13 @@ expand_rows_kernel(const int32_t* __restrict__ counts, const uint32_t* __restric
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int row0 = blockIdx.x * per_cta, row1 = min(rows, row0 + per_cta);
   const int words = (nKb + 31) >> 5;
+  ptx::grid_dependency_wait();
   int before = 0;
   for (int i = threadIdx.x; i < (row0 >> 2); i += kExpandThreads) {
-    const int4 c = __ldg(reinterpret_cast<const int4*>(counts) + i);
+    const int4 c = __ldcg(reinterpret_cast<const int4*>(counts) + i);
     before += (c.x + c.y) + (c.z + c.w);
   }
-  if (threadIdx.x < (row0 & 3)) before += __ldg(counts + (row0 & ~3) + threadIdx.x);
+  if (threadIdx.x < (row0 & 3)) before += __ldcg(counts + (row0 & ~3) + threadIdx.x);
   before = __reduce_add_sync(0xffffffffu, before);
   if (lane == 0) warp_total[warp] = before;
   __syncthreads();
@@ -382,7 +407,7 @@ expand_rows_kernel(const int32_t* __restrict__ counts, const uint32_t* __restric
   for (int r0 = row0; r0 < row1; r0 += 32) {
     // 32 rows: every warp scans their sizes and expands its share of them
     const int r = r0 + lane;
-    const int c = (r < row1) ? __ldg(counts + r) : 0;
+    const int c = (r < row1) ? __ldcg(counts + r) : 0;
     int incl = c;
 #pragma unroll
     for (int d = 1; d < 32; d <<= 1) {
@@ -395,8 +420,9 @@ expand_rows_kernel(const int32_t* __restrict__ counts, const uint32_t* __restric
       int at = pos + __shfl_sync(0xffffffffu, incl - c, j);
       const uint32_t* bm = bitmaps + (int64_t)(r0 + j) * words;
       for (int w0 = 0; w0 < words; w0 += 32) {
-        const uint32_t mine = (w0 + lane < words) ? __ldg(bm + w0 + lane) : 0u;
+        const uint32_t mine = (w0 + lane < words) ? __ldcg(bm + w0 + lane) : 0u;
         const int m = min(32, words - w0);
+#pragma unroll 4
         for (int i = 0; i < m; ++i) {
           const uint32_t word = __shfl_sync(0xffffffffu, mine, i);
           const int to = at + __popc(word & ((1u << lane) - 1u));
@@ -479,9 +505,14 @@ int launch_select(int rows, int nKb, const float* mass, double tau, int fixed_co
   uint32_t* bitmaps = reinterpret_cast<uint32_t*>(static_cast<char*>(ws) +
                                                   align_up((size_t)rows * sizeof(int32_t), 256));
   // (registers hold 32 blocks per lane at most: longer rows take more warps)
-#define LOSA_SELECT_ROWS(w, k) \
-  select_rows_kernel<w, k><<<(w) == 1 ? (rows + 3) / 4 : rows, (w) == 1 ? 128 : 32 * (w), 0, st>>>( \
-      mass, rows, nKb, tau, fixed_count, counts, bitmaps, status)
+#define LOSA_SELECT_ROWS(w, k)                                                                                 \
+  do {                                                                                                         \
+    const int ctas = (w) == 1 ? (rows + 3) / 4 : rows, threads = (w) == 1 ? 128 : 32 * (w);                    \
+    if (fixed_count > 0)                                                                                       \
+      select_rows_kernel<w, k, true><<<ctas, threads, 0, st>>>(mass, rows, nKb, tau, fixed_count, counts, bitmaps, status); \
+    else                                                                                                       \
+      select_rows_kernel<w, k, false><<<ctas, threads, 0, st>>>(mass, rows, nKb, tau, 0, counts, bitmaps, status); \
+  } while (0)
   if (nKb <= 256) LOSA_SELECT_ROWS(1, 8);
   else if (nKb <= 512) LOSA_SELECT_ROWS(1, 16);
   else if (nKb <= 1024) LOSA_SELECT_ROWS(1, 32);
@@ -492,10 +523,9 @@ int launch_select(int rows, int nKb, const float* mass, double tau, int fixed_co
   // four CTAs per SM at most (but no fewer rows than warps): adding up the sizes of the rows before
   // costs every CTA the same, so more of them only read more
   const int per_cta = max(kExpandThreads / 32, (rows + 591) / 592);
-  expand_rows_kernel<<<(rows + per_cta - 1) / per_cta, kExpandThreads, 0, st>>>(
-      counts, bitmaps, rows, nKb, per_cta, offsets, kv_idx, kv_capacity, status);
   LOSA_CUDA_TRY(cudaGetLastError());
-  return LOSA_OK;
+  return launch(expand_rows_kernel, dim3((rows + per_cta - 1) / per_cta), kExpandThreads, 0, st, true, counts, bitmaps, rows,
+                nKb, per_cta, offsets, kv_idx, kv_capacity, status);
 }
 
 // ---- allocation-free variant ----------------------------------------------------------
