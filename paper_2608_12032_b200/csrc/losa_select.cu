@@ -50,6 +50,8 @@ struct RowShared {
   unsigned long long above;      // weight of the bins heavier than the one of v*
   double sum[8];
   int bin, list_len;
+  uint32_t v;
+  int need, eq_total;
   int part[8];
 };
 
@@ -88,12 +90,52 @@ __device__ __forceinline__ unsigned long long row_sum_u64(unsigned long long a, 
 
 // What a list of m values (low bits x) is searched for: the largest v with weight(values >= v) >= missing,
 // and how many of the values equal to v are needed.  A value weighs lead + x, or 1 if COUNT.  Whole warp.
+// A list of more than eight values is first split by its five leading bits, 32 bins again (in cnt and
+// low), and the values of the threshold's bin are put into `few`.
 template <bool COUNT>
 __device__ __forceinline__ void search_list(const uint32_t* list, int m, int bits, uint32_t lead,
-                                            unsigned long long missing, int lane, uint32_t* v_out, int* need_out,
-                                            int* eq_out) {
+                                            unsigned long long missing, int lane, uint32_t* cnt, uint32_t* low,
+                                            uint32_t* few, uint32_t* v_out, int* need_out, int* eq_out) {
+  if (m > 8) {
+    cnt[lane] = 0u;
+    low[lane] = 0u;
+    __syncwarp();
+    const int shift = bits - 5;
+    for (int i = lane; i < m; i += 32) {
+      const uint32_t x = list[i];
+      atomicAdd(&cnt[x >> shift], 1u);
+      if (!COUNT) atomicAdd(&low[x >> shift], x);
+    }
+    __syncwarp();
+    uint32_t n = cnt[31 - lane], l = low[31 - lane];  // heaviest first
+    const uint32_t n0 = n, l0 = l;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const uint32_t un = __shfl_up_sync(0xffffffffu, n, d), ul = __shfl_up_sync(0xffffffffu, l, d);
+      if (lane >= d) {
+        n += un;
+        l += ul;
+      }
+    }
+    const unsigned long long w = COUNT ? n : (unsigned long long)n * lead + l;
+    const int at = __ffs(__ballot_sync(0xffffffffu, w >= missing)) - 1;
+    const uint32_t n_before = __shfl_sync(0xffffffffu, n - n0, at), l_before = __shfl_sync(0xffffffffu, l - l0, at);
+    missing -= COUNT ? n_before : (unsigned long long)n_before * lead + l_before;
+    const uint32_t bin = 31u - (uint32_t)at;
+    int len = 0;
+    for (int i0 = 0; i0 < m; i0 += 32) {
+      const uint32_t x = (i0 + lane < m) ? list[i0 + lane] : 0u;
+      const bool in = i0 + lane < m && (x >> shift) == bin;
+      const uint32_t mask = __ballot_sync(0xffffffffu, in);
+      if (in) few[len + __popc(mask & ((1u << lane) - 1u))] = x;
+      len += __popc(mask);
+    }
+    __syncwarp();
+    list = few;
+    m = len;
+  }
   uint32_t v = 0u;
-  int n_ge = m, n_eq = 0;
+  int n_eq = 0;
   unsigned long long ge = 0ull;  // weight of the values >= v
   if (m <= 32) {
     // every lane adds up the values at or above its own
@@ -101,19 +143,19 @@ __device__ __forceinline__ void search_list(const uint32_t* list, int m, int bit
     uint32_t n = 0u, l = 0u;
     for (int j = 0; j < m; ++j) {
       const uint32_t y = __shfl_sync(0xffffffffu, x, j);
-      n += (y >= x) ? 1u : 0u;
-      l += (y >= x) ? y : 0u;
+      if (y >= x) {
+        n += 1u;
+        l += y;
+      }
     }
     const unsigned long long w = COUNT ? n : (unsigned long long)n * lead + l;
     const bool ok = lane < m && w >= missing;
     v = __reduce_max_sync(0xffffffffu, ok ? x : 0u);
     const uint32_t eq = __ballot_sync(0xffffffffu, lane < m && x == v);
     n_eq = __popc(eq);
-    const int src = __ffs(eq) - 1;
-    n_ge = (int)__shfl_sync(0xffffffffu, n, src);
-    ge = __shfl_sync(0xffffffffu, w, src);
+    ge = __shfl_sync(0xffffffffu, w, __ffs(eq) - 1);
   } else {
-    // bit by bit
+    // (many nearly equal values) bit by bit
     auto measure = [&](uint32_t from, int* n_out) -> unsigned long long {
       uint32_t n = 0u, l = 0u;
       for (int i = lane; i < m; i += 32) {
@@ -127,14 +169,14 @@ __device__ __forceinline__ void search_list(const uint32_t* list, int m, int bit
       l = __reduce_add_sync(0xffffffffu, l);
       return (unsigned long long)n * lead + l;
     };
+    int n;
     for (int b = bits - 1; b >= 0; --b) {
-      int n;
       if (measure(v | (1u << b), &n) >= missing) v |= 1u << b;
     }
-    ge = measure(v, &n_ge);
     int n_gt;
+    ge = measure(v, &n);
     measure(v + 1u, &n_gt);
-    n_eq = n_ge - n_gt;
+    n_eq = n - n_gt;
   }
   int need = n_eq;
   if (n_eq > 1) {
@@ -189,7 +231,7 @@ select_rows_kernel(const float* __restrict__ mass, int rows, int nKb, double tau
 #pragma unroll
   for (int k = 0; k < K; ++k) {
     if (bits[k] > kMaxMassBits) {  // negative, NaN, or far beyond any mass; -0 becomes +0
-      bad = bad || bits[k] != 0x80000000u;
+      bad |= bits[k] != 0x80000000u;
       bits[k] = 0u;
     }
     sum += __uint_as_float(bits[k]);
@@ -275,24 +317,41 @@ select_rows_kernel(const float* __restrict__ mass, int rows, int nKb, double tau
     const uint32_t lead = (uint32_t)(bin + kBase);
     const int m = (bin >= 0) ? (int)rs->cnt[bin] : 0;
     if (bin >= 0 && m <= kListCap) {
+      uint32_t in = 0u;  // bit k: this lane's block k is in the bin
 #pragma unroll
-      for (int k = 0; k < K; ++k) {
-        const bool in = (bits[k] >> kShift) == lead && (!COUNT || k * 32 + lane < mine);
-        const uint32_t mask = __ballot_sync(0xffffffffu, in);
-        if (mask != 0u) {
-          int at = 0;
-          if (lane == 0) at = atomicAdd(&rs->list_len, __popc(mask));
-          at = __shfl_sync(0xffffffffu, at, 0) + __popc(mask & ((1u << lane) - 1u));
-          if (in) rs->list[at] = bits[k] & kLowMask;
-        }
+      for (int k = 0; k < K; ++k) in |= ((bits[k] >> kShift) == lead) ? 1u << k : 0u;
+      if (COUNT) {
+        const int mine_k = (mine - lane + 31) >> 5;  // this lane's blocks that exist
+        in &= (mine_k >= 32) ? 0xffffffffu : (1u << max(mine_k, 0)) - 1u;
+      }
+      // (a lane has one or two of them: their values are read again instead of picked out of registers)
+      while (in != 0u) {
+        const int k = __ffs(in) - 1;
+        in &= in - 1u;
+        uint32_t x = __float_as_uint(__ldg(src + k * 32));
+        if (x > kMaxMassBits) x = 0u;
+        rs->list[atomicAdd(&rs->list_len, 1)] = x & kLowMask;
       }
       row_sync<W>();
-      // what the bin has to add, in units of the bin's mantissas: rounded up, its sums are whole (every
-      // warp searches the list for itself: no hand-over)
-      const uint32_t lift = COUNT ? 0u : (lead >> 4) - 90u;
-      const unsigned long long missing = (target - rs->above + ((1ull << lift) - 1ull)) >> lift;
-      search_list<COUNT>(rs->list, m, kShift, (16u | (lead & 15u)) << kTauShift, missing, lane, &v, &need, &eq_total);
-      v |= lead << kShift;
+      if (warp == 0) {
+        // what the bin has to add, in units of the bin's mantissas: rounded up, its sums are whole
+        const uint32_t lift = COUNT ? 0u : (lead >> 4) - 90u;
+        const unsigned long long missing = (target - rs->above + ((1ull << lift) - 1ull)) >> lift;
+        search_list<COUNT>(rs->list, m, kShift, (16u | (lead & 15u)) << kTauShift, missing, lane, rs->cnt, rs->low,
+                           rs->cnt + 32, &v, &need, &eq_total);
+        v |= lead << kShift;
+        if (W > 1 && lane == 0) {
+          rs->v = v;
+          rs->need = need;
+          rs->eq_total = eq_total;
+        }
+      }
+      if (W > 1) {
+        row_sync<W>();
+        v = rs->v;
+        need = rs->need;
+        eq_total = rs->eq_total;
+      }
     } else {
       // ---- bit by bit over the row: masked sums (or counts) of the blocks with bits >= v (read again, so
       // that this path takes no registers from the other)
@@ -418,16 +477,30 @@ expand_rows_kernel(const int32_t* __restrict__ counts, const uint32_t* __restric
     if (warp == 0 && lane < n) offsets[r] = pos + incl - c;
     for (int j = warp; j < n; j += kWarps) {
       int at = pos + __shfl_sync(0xffffffffu, incl - c, j);
+      const bool fits = (int64_t)at + __shfl_sync(0xffffffffu, c, j) <= kv_capacity;
+      const uint32_t below = (1u << lane) - 1u, bit = 1u << lane;
       const uint32_t* bm = bitmaps + (int64_t)(r0 + j) * words;
       for (int w0 = 0; w0 < words; w0 += 32) {
         const uint32_t mine = (w0 + lane < words) ? __ldcg(bm + w0 + lane) : 0u;
         const int m = min(32, words - w0);
-#pragma unroll 4
-        for (int i = 0; i < m; ++i) {
-          const uint32_t word = __shfl_sync(0xffffffffu, mine, i);
-          const int to = at + __popc(word & ((1u << lane) - 1u));
-          if (((word >> lane) & 1u) && to < kv_capacity) kv_idx[to] = (w0 + i) * 32 + lane;
-          at += __popc(word);
+        if (fits) {
+          int* to = kv_idx + at;
+          int value = w0 * 32 + lane;
+#pragma unroll 8
+          for (int i = 0; i < m; ++i) {
+            const uint32_t word = __shfl_sync(0xffffffffu, mine, i);
+            if (word & bit) to[__popc(word & below)] = value;
+            to += __popc(word);
+            value += 32;
+          }
+          at = (int)(to - kv_idx);
+        } else {
+          for (int i = 0; i < m; ++i) {
+            const uint32_t word = __shfl_sync(0xffffffffu, mine, i);
+            const int to = at + __popc(word & below);
+            if ((word & bit) && to < kv_capacity) kv_idx[to] = (w0 + i) * 32 + lane;
+            at += __popc(word);
+          }
         }
       }
     }
