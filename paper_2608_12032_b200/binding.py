@@ -7,6 +7,7 @@ loaded the import of a function from here raises.
 from __future__ import annotations
 
 import ctypes
+import functools
 import math
 import os
 from typing import Optional, Tuple
@@ -107,7 +108,8 @@ def _lib():
 
 
 def _stream() -> int:
-    return torch.cuda.current_stream().cuda_stream
+    # (the current stream's handle without a Stream object around it: 1 us of every call)
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
 
 
 def _check(rc: int, where: str) -> None:
@@ -128,11 +130,28 @@ def make_problem(q: torch.Tensor, R: int, C: int, scale: Optional[float] = None)
 
 
 def _same_layout(ref: torch.Tensor, *others: torch.Tensor) -> None:
+    shape, stride, device = ref.shape, ref.stride(), ref.device
     for t in others:
-        if t.shape != ref.shape or t.stride() != ref.stride():
+        if t.shape != shape or t.stride() != stride:
             raise ValueError("q, k, v (and o) must share shape and strides")
-        if t.device != ref.device:
+        if t.device != device:
             raise ValueError("tensors must live on the same device")
+
+
+@functools.lru_cache(maxsize=512, typed=True)
+def _plan(op: int, shape, stride, R: int, C: int, scale: float, n_layers: int):
+    """(reference to the problem's description, workspace bytes) of a call: both follow from the
+    arguments alone, and on a small layer describing the problem and asking for its workspace took
+    as long as two launches."""
+    if len(shape) != 4 or stride[3] != 1:
+        raise ValueError("expected [B, H, N, D] with a contiguous last dimension")
+    prob = Problem(*shape, R, C, *stride[:3], scale)
+    need = losa_workspace_bytes(op, prob) if n_layers == 0 else losa_workspace_bytes_batched(op, prob, n_layers)
+    return ctypes.byref(prob), need
+
+
+def _problem(op: int, q: torch.Tensor, R: int, C: int, scale: Optional[float], n_layers: int = 0):
+    return _plan(op, q.shape, q.stride(), R, C, 0.0 if scale is None else float(scale), n_layers)
 
 
 def losa_workspace_bytes(op: int, problem: Problem) -> int:
@@ -144,11 +163,10 @@ def losa_work_slots(op: int, problem: Problem) -> int:
     return int(_lib().losa_work_slots(op, ctypes.byref(problem)))
 
 
-def _workspace(op: int, problem: Problem, device, ws: Optional[torch.Tensor]) -> Tuple[Optional[torch.Tensor], int]:
-    need = losa_workspace_bytes(op, problem)
+def _workspace(need: int, device, ws: Optional[torch.Tensor]) -> Tuple[Optional[torch.Tensor], int]:
     if ws is None and need > 0:
         ws = torch.empty(need, dtype=torch.uint8, device=device)
-    return ws, (0 if ws is None else ws.numel() * ws.element_size())
+    return ws, (0 if ws is None else ws.nbytes)
 
 
 def losa_block_mass(q: torch.Tensor, k: torch.Tensor, R: int, C: int, scale: Optional[float] = None,
@@ -156,14 +174,14 @@ def losa_block_mass(q: torch.Tensor, k: torch.Tensor, R: int, C: int, scale: Opt
                     mass: Optional[torch.Tensor] = None):
     """mass[B, H, nQb, nKb] (fp32) of one dense attention step; optionally the rows' log-sum-exp."""
     _same_layout(q, k)
-    prob = make_problem(q, R, C, scale)
+    prob, need = _problem(LOSA_OP_BLOCK_MASS, q, R, C, scale)
     B, H, N, _ = q.shape
     nQb, nKb = -(-N // R), -(-N // C)
     if mass is None:
         mass = torch.empty((B, H, nQb, nKb), dtype=torch.float32, device=q.device)
     lse = torch.empty((B, H, N), dtype=torch.float32, device=q.device) if return_lse else None
-    ws, ws_bytes = _workspace(LOSA_OP_BLOCK_MASS, prob, q.device, ws)
-    _check(_lib().losa_block_mass(ctypes.byref(prob), _ptr(q), _ptr(k), _ptr(mass), _ptr(lse),
+    ws, ws_bytes = _workspace(need, q.device, ws)
+    _check(_lib().losa_block_mass(prob, _ptr(q), _ptr(k), _ptr(mass), _ptr(lse),
                                   _ptr(ws), ws_bytes, _stream()), "losa_block_mass")
     return (mass, lse) if return_lse else mass
 
@@ -236,6 +254,7 @@ def losa_select_noalloc(mass: torch.Tensor, tau: float, offsets: torch.Tensor, k
            "losa_select_noalloc")
 
 
+@functools.lru_cache(maxsize=512, typed=True)
 def _select_workspace_bytes(B: int, H: int, nQb: int, nKb: int) -> int:
     # losa_workspace_bytes(LOSA_OP_SELECT) reads B, H and ceil(N/R), ceil(N/C): describe the
     # mass matrix as N = nQb * nKb tokens with R = nKb and C = nQb.
@@ -249,10 +268,10 @@ def losa_sparse_attn(q: torch.Tensor, k: torch.Tensor, v: torch.Tensor, offsets:
                      ws: Optional[torch.Tensor] = None):
     """Block-sparse attention over the frozen CSR pattern; rows >= N do not exist."""
     _same_layout(q, k, v)
-    prob = make_problem(q, R, C, scale)
+    prob, need = _problem(LOSA_OP_SPARSE_ATTN, q, R, C, scale)
     o = _alloc_out(q, out_dtype, out)
-    ws, ws_bytes = _workspace(LOSA_OP_SPARSE_ATTN, prob, q.device, ws)
-    _check(_lib().losa_sparse_attn(ctypes.byref(prob), _ptr(q), _ptr(k), _ptr(v), _ptr(offsets),
+    ws, ws_bytes = _workspace(need, q.device, ws)
+    _check(_lib().losa_sparse_attn(prob, _ptr(q), _ptr(k), _ptr(v), _ptr(offsets),
                                    _ptr(kv_idx), _ptr(o), _dtype_code(o.dtype), _ptr(ws), ws_bytes,
                                    _stream()),
            "losa_sparse_attn")
@@ -270,7 +289,7 @@ def losa_sparse_attn_batched(layers, R: int, C: int, scale: Optional[float] = No
 
     ``layers`` is a sequence of ``(q, k, v, offsets, kv_idx)``; returns the list of outputs."""
     q0 = layers[0][0]
-    prob = make_problem(q0, R, C, scale)
+    prob, need = _problem(LOSA_OP_SPARSE_ATTN, q0, R, C, scale, len(layers))
     arr = (Layer * len(layers))()
     result = []
     for i, (q, k, v, offsets, kv_idx) in enumerate(layers):
@@ -278,10 +297,9 @@ def losa_sparse_attn_batched(layers, R: int, C: int, scale: Optional[float] = No
         o = _alloc_out(q, out_dtype, None if outs is None else outs[i])
         result.append(o)
         arr[i] = Layer(_ptr(q), _ptr(k), _ptr(v), _ptr(offsets), _ptr(kv_idx), _ptr(o))
-    need = losa_workspace_bytes_batched(LOSA_OP_SPARSE_ATTN, prob, len(layers))
     if ws is None:
         ws = torch.empty(max(need, 1), dtype=torch.uint8, device=q0.device)
-    _check(_lib().losa_sparse_attn_batched(ctypes.byref(prob), len(layers), arr,
+    _check(_lib().losa_sparse_attn_batched(prob, len(layers), arr,
                                            _dtype_code(result[0].dtype), _ptr(ws), ws.numel(), _stream()),
            "losa_sparse_attn_batched")
     return result
@@ -292,10 +310,10 @@ def losa_attn(q: torch.Tensor, k: torch.Tensor, v: torch.Tensor, R: int = 128, C
               out: Optional[torch.Tensor] = None, ws: Optional[torch.Tensor] = None):
     """Dense softmax attention with the library's own kernel."""
     _same_layout(q, k, v)
-    prob = make_problem(q, R, C, scale)
+    prob, need = _problem(LOSA_OP_ATTN, q, R, C, scale)
     o = _alloc_out(q, out_dtype, out)
-    ws, ws_bytes = _workspace(LOSA_OP_ATTN, prob, q.device, ws)
-    _check(_lib().losa_attn(ctypes.byref(prob), _ptr(q), _ptr(k), _ptr(v), _ptr(o),
+    ws, ws_bytes = _workspace(need, q.device, ws)
+    _check(_lib().losa_attn(prob, _ptr(q), _ptr(k), _ptr(v), _ptr(o),
                             _dtype_code(o.dtype), _ptr(ws), ws_bytes, _stream()), "losa_attn")
     return o
 
@@ -306,14 +324,14 @@ def losa_attn_mass(q: torch.Tensor, k: torch.Tensor, v: torch.Tensor, R: int, C:
                    mass: Optional[torch.Tensor] = None, ws: Optional[torch.Tensor] = None):
     """The construction step in one kernel: (o, mass[, lse]) = dense attention + block masses."""
     _same_layout(q, k, v)
-    prob = make_problem(q, R, C, scale)
+    prob, need = _problem(LOSA_OP_ATTN_MASS, q, R, C, scale)
     B, H, N, _ = q.shape
     o = _alloc_out(q, out_dtype, out)
     if mass is None:
         mass = torch.empty((B, H, -(-N // R), -(-N // C)), dtype=torch.float32, device=q.device)
     lse = torch.empty((B, H, N), dtype=torch.float32, device=q.device) if return_lse else None
-    ws, ws_bytes = _workspace(LOSA_OP_ATTN_MASS, prob, q.device, ws)
-    _check(_lib().losa_attn_mass(ctypes.byref(prob), _ptr(q), _ptr(k), _ptr(v), _ptr(o),
+    ws, ws_bytes = _workspace(need, q.device, ws)
+    _check(_lib().losa_attn_mass(prob, _ptr(q), _ptr(k), _ptr(v), _ptr(o),
                                  _dtype_code(o.dtype), _ptr(mass), _ptr(lse), _ptr(ws), ws_bytes,
                                  _stream()), "losa_attn_mass")
     return (o, mass, lse) if return_lse else (o, mass)
