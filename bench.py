@@ -50,26 +50,11 @@ NCU_TRAFFIC_SOURCE = "ncu capture of the sparse forward at the Wan2.1 shape (dra
 FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustained": 1400.0}
 
 
-def merge_kernel_runs(wl) -> bool:
-    """Whether the attention-only calls launch their merge kernel for this shape: the library says how
-    many work slots a call occupies; work items are pairs of 128-row query tiles per head, and the
-    items of a last, partly filled wave are cut into parts (at most 8, at most one per key block)."""
-    from paper_2608_12032_b200 import binding
-    prob = binding.Problem(wl.B, wl.H, wl.N, wl.D, wl.R, wl.C, wl.H * wl.N * wl.D, wl.N * wl.D, wl.D, 0.0)
-    ctas = binding.losa_work_slots(binding.LOSA_OP_SPARSE_ATTN, prob)
-    n_work = wl.B * wl.H * ((-(-wl.N // 128) + 1) // 2)
-    rest = n_work if n_work < ctas else n_work % ctas
-    parts = min(ctas // rest, 8, -(-wl.N // wl.C)) if rest else 1
-    return parts >= 2
-
-
-def launches_per_step(wl, draws: int) -> int:
-    """Kernels of the library launched by one step.  Every attention-shaped call launches its kernel
-    and the fallback kernel behind it (which returns at once when no row outgrew its reference): the
-    mass pass 2; select 3; every sparse call also its tile-list pre-pass, plus the merge kernel when the
-    last wave is cut into parts; the dense call the same without the pre-pass; the fused step 2."""
-    merge = int(merge_kernel_runs(wl))
-    return 2 + 3 + draws * (3 + merge) + (2 + merge) + 2
+def launches_per_step(draws: int) -> int:
+    """Kernels of the library launched by one step.  Every attention-shaped call launches three: the
+    work units' tile lists (sparse) or the launch's counters, its kernel, and the fallback kernel, which
+    merges the partial units and returns when no row outgrew its reference; select launches two."""
+    return 3 + 2 + draws * 3 + 3 + 3
 
 
 def cpu_model() -> str:
@@ -636,7 +621,7 @@ def main():
             "note": "Eq. 2 on the GPU's own block masses of each draw, frozen pattern from step 0",
         },
         "roofline": {
-            "kernel": "losa_attn_kernel<sparse>", "bound": "tensor", "achieved": achieved,
+            "kernel": "losa_tile_kernel<sparse>", "bound": "tensor", "achieved": achieved,
             "peak": burst, "unit": "TFLOP/s", "frac": achieved / burst,
             "peak_source": f"{peaks['_source']} bf16_tflops (cuBLAS burst)",
             "frac_of_sustained": achieved / sustained,
@@ -648,7 +633,7 @@ def main():
             "algorithmic_bytes_per_launch": 4 * q0.numel() * 2,
         },
         "clocks": clocks.summary(),
-        "gpu_launches": args.steps * launches_per_step(wl, args.draws),
+        "gpu_launches": args.steps * launches_per_step(args.draws),
     }
     if batched is not None:
         line["batched"] = batched
