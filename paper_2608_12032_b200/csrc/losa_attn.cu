@@ -190,9 +190,12 @@ struct Params {
   // Work units whose scores outgrew the fixed reference of the two-threads-per-row kernel: it
   // appends them here, and a second launch (one thread per row, moving reference) recomputes them.
   // That second launch, which also merges the partial units, draws redo_list[0 .. *redo_count) instead
-  // of all units.
+  // of all units.  A unit's two query tiles, and the warps of each, may all find it outgrown, at
+  // different times and on different CTAs: its flag (zeroed by the launch before) lets one of them
+  // list it, so that the list never holds more than nUnits entries.
   int* redo_count;
   int* redo_list;
+  int* redo_flag;  // [nUnits]
   int* redo_done;  // how many CTAs of the second launch are done
   // extents of the buffers the kernels index into (elements), for the checked build
   long long cap_part_rows, cap_table_floats, cap_mass, cap_lse, cap_units;
@@ -220,7 +223,6 @@ struct Control {
   // this CTA sent to the fallback
   uint64_t pair_bar[SPLIT ? 8 : 1];
   float xch[SPLIT ? 2 * 2 * 128 : 1];
-  int ovf_unit;
 };
 
 // Checked build (-DLOSA_CHECKED=1, a substitute for a memory checker): every index the kernels
@@ -393,6 +395,12 @@ __device__ __forceinline__ void merge_parts(const Params& p, int cta, int ctas) 
   }
 }
 
+// One thread; see Params::redo_list.
+__device__ __forceinline__ void list_outgrown_unit(const Params& p, int unit) {
+  if (LOSA_IN_RANGE(unit, p.nUnits) && atomicExch(p.redo_flag + unit, 1) == 0)
+    p.redo_list[atomicAdd(p.redo_count, 1)] = unit;
+}
+
 // Tensor maps of a batched launch were written to the workspace by a kernel, over those of an earlier call.
 __device__ __forceinline__ void acquire_maps(const ProblemEntry* pe) {
   ptx::tensormap_acquire(&pe->map_q);
@@ -476,7 +484,6 @@ losa_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     }
     if (SPLIT) {
       for (int i = 0; i < 8; ++i) ptx::mbar_init(&ctl->pair_bar[i], 2);
-      ctl->ovf_unit = -1;
     }
     ptx::mbar_init(&ctl->drain, 2);  // the MMA issuers arrive on the abort path
     ctl->mma_lock = 0;
@@ -1471,12 +1478,7 @@ losa_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         l += other.y;
       }
       if (ovf && lane == 0) {
-        // (the pair's warps may both get here, and so may the other pairs: the unit is listed once)
-        const int unit = partial ? p.split_first + (w - p.split_first) * p.split_parts + part : w;
-        if (atomicExch(&ctl->ovf_unit, unit) != unit) {
-          const int slot = atomicAdd(p.redo_count, 1);
-          if (slot < p.nUnits) p.redo_list[slot] = unit;
-        }
+        list_outgrown_unit(p, partial ? p.split_first + (w - p.split_first) * p.split_parts + part : w);
       }
       if (C::kHasV && half == 0 && T < p.nQt) {
         if (!C::kWantMass) l += xset[row];
@@ -1647,7 +1649,7 @@ teardown:
 //
 // One warp per list fills its bitmap (a list of a small layer is nothing but the latency of its two
 // dependent loads), then the first warp writes the tile list.  The first CTA also zeroes the
-// launch's counters.
+// launch's counters, and every CTA its unit's flag.
 // ONE: a list is that of one query tile of the unit (its NB query blocks), in ascending order.
 template <int NB, int G, bool ONE>
 __global__ void __launch_bounds__(32 * NB) build_tile_lists_kernel(const Params p) {
@@ -1658,6 +1660,7 @@ __global__ void __launch_bounds__(32 * NB) build_tile_lists_kernel(const Params 
   const int list = blockIdx.x, unit = ONE ? list >> 1 : list;
   const int bit0 = ONE ? (list & 1) * NB : 0;  // membership bit of the first query block
   if (list == 0 && threadIdx.x < kCounters) p.work_counter[threadIdx.x] = 0;
+  if (threadIdx.x == 0) p.redo_flag[unit] = 0;
   int w = unit, part = 0, parts = 1;
   if (unit >= p.split_first) {
     const int r = unit - p.split_first;
@@ -1857,11 +1860,15 @@ int make_maps(ProblemEntry* e, const Geometry& g, const void* q, const void* k, 
   return LOSA_OK;
 }
 
-// Zeroes the counters of a launch that no other kernel precedes (a kernel and not a memset, so that
-// the attention kernel can be launched as its dependent: 3 us of that kernel's set-up overlap).
-__global__ void __launch_bounds__(32) init_counters_kernel(int* counters) {
+// Zeroes the counters and the units' flags of a launch that no other kernel precedes (a kernel and
+// not a memset, so that the attention kernel can be launched as its dependent: 3 us of that kernel's
+// set-up overlap).
+constexpr int kInitThreads = 256;
+__global__ void __launch_bounds__(kInitThreads) init_counters_kernel(int* counters, int* flags, int units) {
   ptx::grid_launch_dependents();
-  if (threadIdx.x < kCounters) counters[threadIdx.x] = 0;
+  if (blockIdx.x == 0 && threadIdx.x < kCounters) counters[threadIdx.x] = 0;
+  for (int64_t i = (int64_t)blockIdx.x * kInitThreads + threadIdx.x; i < units; i += (int64_t)gridDim.x * kInitThreads)
+    flags[i] = 0;
 }
 
 // Part of a batched launch's table, carried in the kernel's parameters: the call reads its host
@@ -2021,7 +2028,8 @@ int launch_t(const Geometry& g, const void* q, const void* k, const void* v, Par
     rc = launch(build_tile_lists_kernel<kBlocks, C::kG, kOne>, dim3(prm.nUnits * tile_lists_per_unit(D)), 32 * kBlocks,
                 bm_bytes, st, prm.nProb > 1, prm);
   } else {
-    rc = launch(init_counters_kernel, dim3(1), 32, 0, st, false, prm.work_counter);
+    rc = launch(init_counters_kernel, dim3(min(ctas, (prm.nUnits + 4 * kInitThreads - 1) / (4 * kInitThreads))),
+                kInitThreads, 0, st, false, prm.work_counter, prm.redo_flag, prm.nUnits);
   }
   if (rc != LOSA_OK) return rc;
   // All modes run with two threads per query row and a reference that never moves; the units whose
@@ -2107,13 +2115,13 @@ size_t attn_workspace_bytes(AttnMode mode, const Geometry& g, int n_prob) {
     if (mode == kSparse) bytes += tl_count_bytes(g, n_prob) + tl_entries_bytes(g, n_prob);
     // batched launch: the table of the problems' tensor maps and pointers
     if (n_prob > 1) bytes += (size_t)n_prob * sizeof(ProblemEntry);
-    // the work units handed to the fallback launch (each of a unit's query tiles may list it)
+    // the work units handed to the fallback launch, and their flags
     bytes += redo_list_bytes(g, n_prob);
     return bytes;
   }
   // counter, per-CTA row statistics (three times as many for the fused step with two threads per
   // row: two sets of the halves' row sums, and the rows' weights), per-CTA table of one entry per
-  // row and key tile, and the fused step's list of units for the fallback launch
+  // row and key tile, and the units handed to the fallback launch with their flags
   return kCounterBytes + 5 * kRowstatBytes +
          (size_t)kMaxPersistentCtas * 2 * (size_t)g.nKb * 128 * sizeof(float2) + redo_list_bytes(g, 1);
 }
@@ -2191,6 +2199,7 @@ int launch_attn(AttnMode mode, const Geometry& g, const void* q, const void* k, 
     if (mode == kFused || mode == kMass)  // behind the table
       prm.redo_list = reinterpret_cast<int*>(reinterpret_cast<char*>(prm.table) +
                                              (size_t)kMaxPersistentCtas * 2 * (size_t)g.nKb * 128 * sizeof(float2));
+    prm.redo_flag = prm.redo_list + max_units(g, n_prob);
   }
   prm.cap_part_rows = (long long)kMaxPersistentCtas * 2 * 128;
   prm.cap_table_floats = (long long)g.nKb * 256;

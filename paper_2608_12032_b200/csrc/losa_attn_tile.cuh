@@ -65,7 +65,6 @@ struct TileControl {
                            // four of the rounded weights, four of the unrounded exponentials (fused step)
   uint32_t tmem_base;
   int abort_flag;
-  int ovf_unit;
 };
 
 // Key blocks of a unit in the dense modes.
@@ -264,7 +263,6 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     ptx::mbar_init(&ctl->fold_bar, 16);
     ptx::mbar_init(&ctl->drain, 2);
     ctl->abort_flag = 0;
-    ctl->ovf_unit = -1;
     ptx::fence_barrier_init();
   }
   if (warp == kIssuerWarp) {
@@ -874,12 +872,7 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       xset[quarter * 128 + row] = l;
       if (kWantMass) xset[(4 + quarter) * 128 + row] = le;
       auto hand_over = [&]() {
-        const int unit = partial ? p.split_first + (w - p.split_first) * p.split_parts + part : w;
-        // (once per CTA: its two query tiles of one unit may come one after the other)
-        if (atomicExch(&ctl->ovf_unit, unit) != unit) {
-          const int slot = atomicAdd(p.redo_count, 1);
-          if (slot < 2 * p.nUnits) p.redo_list[slot] = unit;  // (each query tile may list it)
-        }
+        list_outgrown_unit(p, partial ? p.split_first + (w - p.split_first) * p.split_parts + part : w);
       };
       if (ovf && lane == 0) hand_over();
       __syncwarp();

@@ -530,3 +530,41 @@ def test_rows_that_outgrow_their_reference_in_whole_and_cut_work_units(D, BLK):
     util.assert_output_close(o_f, orc.dense_attn(qn, kn, vn), "fused, some heads outgrow the reference")
     ref_m = orc.block_mass(qn, kn, BLK, BLK)
     assert np.abs(mass.cpu().numpy().reshape(ref_m.shape) - ref_m).max() <= util.MASS_TOL
+
+
+@pytest.mark.parametrize("D,R,C", [(128, 64, 64), (64, 64, 64), (64, 128, 32), (128, 128, 64)])
+def test_every_unit_outgrows_its_reference(D, R, C):
+    """Units of two key tiles whose second lies 60 nats above the first, in every head: both query tiles
+    of every unit find it outgrown, several units apart from one another, and the list of the second
+    launch has to hold each unit once."""
+    losa = lib()
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    B, H, N = 1, 2 * sms + 5, 256  # one pair of query tiles per head
+    g = torch.Generator("cpu").manual_seed(78)
+    q = torch.randn(B, H, N, D, generator=g) * 0.3 + 1.0
+    k = torch.randn(B, H, N, D, generator=g) * 0.3
+    k[:, :, 128:] += 60.0 * (D ** 0.5) / D
+    v = torch.randn(B, H, N, D, generator=g)
+    q, k, v = q.bfloat16(), k.bfloat16(), v.bfloat16()
+    qd, kd, vd = q.cuda(), k.cuda(), v.cuda()
+    qn, kn, vn = util.to_np(q), util.to_np(k), util.to_np(v)
+    ref, ref_m = orc.dense_attn(qn, kn, vn), orc.block_mass(qn, kn, R, C)
+    off, idx = util.all_blocks_csr(B * H * (N // R), N // C)
+    o = losa.losa_attn(qd, kd, vd, R, C, out_dtype=torch.float32)
+    o_s = losa.losa_sparse_attn(qd, kd, vd, torch.from_numpy(off).cuda(), torch.from_numpy(idx).cuda(), R, C,
+                                out_dtype=torch.float32)
+    prob = losa.make_problem(qd, R, C)
+    for fused in (False, True):
+        op = losa.binding.LOSA_OP_ATTN_MASS if fused else losa.binding.LOSA_OP_BLOCK_MASS
+        ws = torch.empty(losa.losa_workspace_bytes(op, prob), dtype=torch.uint8, device="cuda")
+        if fused:
+            o_f, mass = losa.losa_attn_mass(qd, kd, vd, R, C, out_dtype=torch.float32, ws=ws)
+            util.assert_output_close(o_f, ref, "fused")
+        else:
+            mass = losa.losa_block_mass(qd, kd, R, C, ws=ws)
+        assert np.abs(mass.cpu().numpy().reshape(ref_m.shape) - ref_m).max() <= util.MASS_TOL
+        # the head of the workspace: work items drawn, units listed
+        assert int(ws[:8].view(torch.int32)[1]) == B * H, "every unit is listed once"
+    assert losa.losa_async_status() == 0
+    util.assert_output_close(o, ref, "dense")
+    util.assert_output_close(o_s, ref, "sparse")
