@@ -355,10 +355,11 @@ __device__ __forceinline__ void merge_parts(const Params& p, int cta, int ctas) 
       for (int s = 0; s < kMaxParts; ++s)
         if (s < parts) load(s, v[s]);
     }
-    float m = (ml.y > 0.f) ? ml.x : -INFINITY;
+    // (a part without keys of the row has the sum 0; one that met NaN has the sum NaN, and so has the row)
+    float m = (ml.y != 0.f) ? ml.x : -INFINITY;
 #pragma unroll
     for (int d = kMaxParts / 2; d > 0; d >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, d));
-    const float mine = (ml.y > 0.f) ? ptx::ex2_approx(ml.x - m) : 0.f;
+    const float mine = (ml.y != 0.f) ? ptx::ex2_approx(ml.x - m) : 0.f;
     float L = 0.f, acc[kCols];
 #pragma unroll
     for (int c = 0; c < kCols; ++c) acc[c] = 0.f;
@@ -374,7 +375,7 @@ __device__ __forceinline__ void merge_parts(const Params& p, int cta, int ctas) 
         }
       }
     }
-    const float inv = (L > 0.f) ? 1.f / L : 0.f;
+    const float inv = (L != 0.f) ? 1.f / L : 0.f;
     const int bh = pbh % (p.B * p.H);
     void* const o_base = (p.problems != nullptr) ? p.problems[pbh / (p.B * p.H)].o : p.o;
     const int64_t off = (int64_t)(bh / p.H) * p.sb + (int64_t)(bh % p.H) * p.sh + (int64_t)grow * p.sn + lane * kCols;

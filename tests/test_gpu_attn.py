@@ -568,3 +568,39 @@ def test_every_unit_outgrows_its_reference(D, R, C):
     assert losa.losa_async_status() == 0
     util.assert_output_close(o, ref, "dense")
     util.assert_output_close(o_s, ref, "sparse")
+
+
+@pytest.mark.parametrize("D,R,C", [(64, 64, 64), (64, 128, 32), (128, 128, 128), (128, 128, 32), (128, 64, 64)])
+def test_a_key_that_is_not_a_number_shows_wherever_it_lies(D, R, C):
+    """One NaN key, in whole and in cut work units: the rows that attend to it have no finite output and no
+    finite log-sum-exp (and weigh nothing in the masses), the rows that do not are untouched."""
+    losa = lib()
+    B, H, N = 1, 2, 512 - 9
+    q, k, v = (util.rand_bf16((B, H, N, D), 880 + i) for i in range(3))
+    nQb, nKb = -(-N // R), -(-N // C)
+    off, idx = util.random_csr(B * H * nQb, nKb, 12, 0.6)
+    qd, vd, offd, idxd = q.cuda(), v.cuda(), torch.from_numpy(off).cuda(), torch.from_numpy(idx).cuda()
+    ref_s = orc.blocks_to_tokens(
+        orc.sparse_attn(util.to_np(q), util.to_np(k), util.to_np(v), R, C, off, idx), B, H, N)
+    ref, ref_m = orc.dense_attn(util.to_np(q), util.to_np(k), util.to_np(v)), orc.block_mass(util.to_np(q), util.to_np(k), R, C)
+    for at in (5, 22, 70, 128 + 6, 256 + 105):
+        kn = k.clone()
+        kn[:, 0, at] = float("nan")
+        kd = kn.cuda()
+        listed = torch.tensor([at // C in idx[off[r]:off[r + 1]] for r in range(nQb)]).repeat_interleave(R)[:N]
+        o = losa.losa_attn(qd, kd, vd, R, C, out_dtype=torch.float32)
+        o_s = losa.losa_sparse_attn(qd, kd, vd, offd, idxd, R, C, out_dtype=torch.float32)
+        o_f, mass_f, lse_f = losa.losa_attn_mass(qd, kd, vd, R, C, return_lse=True, out_dtype=torch.float32)
+        mass, lse = losa.losa_block_mass(qd, kd, R, C, return_lse=True)
+        assert losa.losa_async_status() == 0
+        for name, x in (("dense", o), ("fused", o_f), ("lse", lse), ("fused lse", lse_f)):
+            assert x[:, 0].isnan().all() and x[:, 1].isfinite().all(), (name, at)
+        for name, m in (("mass", mass), ("fused mass", mass_f)):
+            assert (m[:, 0] == 0).all(), (name, at)
+            m = m.cpu().numpy().reshape(H, nQb, nKb)
+            assert np.abs(m[1] - ref_m.reshape(H, nQb, nKb)[1]).max() <= util.MASS_TOL, (name, at)
+        assert o_s[0, 0].cpu()[listed].isnan().all(), at
+        free = torch.cat([~listed, torch.ones(N, dtype=torch.bool)])
+        got, want = o_s[0].cpu().reshape(H * N, D)[free], torch.from_numpy(ref_s[0].reshape(H * N, D))[free]
+        assert (got - want).abs().max() <= util.MAX_ABS_TOL, at
+        assert np.abs(o[0, 1].cpu().numpy() - ref[0, 1]).max() <= util.MAX_ABS_TOL
