@@ -576,10 +576,11 @@ __device__ __forceinline__ float ex2_approx(float x) {
 // Inputs below -127 (masked keys hold -inf) are clamped and come out as zero or a denormal;
 // inputs above 127 are clamped too and come out as 2^127, far beyond the row-sum range the
 // callers accept, so that an overflow shows in the sum instead of wrapping into the sign bit.
-// (NaN also clamps to a finite value: callers that must see NaN look at the other columns.)
+// So does NaN: the upper clamp comes first, and fminf(NaN, 127) is 127.  A caller whose sum has left
+// the range recomputes the row without this function, and NaN comes out as NaN.
 __device__ __forceinline__ float2 ex2_poly2(float2 x) {
-  x.x = fminf(fmaxf(x.x, -127.f), 127.f);
-  x.y = fminf(fmaxf(x.y, -127.f), 127.f);
+  x.x = fmaxf(fminf(x.x, 127.f), -127.f);
+  x.y = fmaxf(fminf(x.y, 127.f), -127.f);
   const float2 t = add2(x, make_float2(12582912.f, 12582912.f));
   const float2 n = add2(t, make_float2(-12582912.f, -12582912.f));
   const float2 f = add2(x, make_float2(-n.x, -n.y));

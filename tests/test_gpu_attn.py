@@ -572,8 +572,9 @@ def test_every_unit_outgrows_its_reference(D, R, C):
 
 @pytest.mark.parametrize("D,R,C", [(64, 64, 64), (64, 128, 32), (128, 128, 128), (128, 128, 32), (128, 64, 64)])
 def test_a_key_that_is_not_a_number_shows_wherever_it_lies(D, R, C):
-    """One NaN key, in whole and in cut work units: the rows that attend to it have no finite output and no
-    finite log-sum-exp (and weigh nothing in the masses), the rows that do not are untouched."""
+    """One NaN key, in whole and in cut work units, at key positions whose exponentials the kernels take in
+    different ways: the rows that attend to it have no finite output and no finite log-sum-exp (and weigh
+    nothing in the masses), the rows that do not are untouched."""
     losa = lib()
     B, H, N = 1, 2, 512 - 9
     q, k, v = (util.rand_bf16((B, H, N, D), 880 + i) for i in range(3))
@@ -583,7 +584,7 @@ def test_a_key_that_is_not_a_number_shows_wherever_it_lies(D, R, C):
     ref_s = orc.blocks_to_tokens(
         orc.sparse_attn(util.to_np(q), util.to_np(k), util.to_np(v), R, C, off, idx), B, H, N)
     ref, ref_m = orc.dense_attn(util.to_np(q), util.to_np(k), util.to_np(v)), orc.block_mass(util.to_np(q), util.to_np(k), R, C)
-    for at in (5, 22, 70, 128 + 6, 256 + 105):
+    for at in (0, 1, 2, 3, 4, 5, 17, 22, 34, 51, 66, 70, 128 + 3, 128 + 6, 256 + 98, 256 + 105):
         kn = k.clone()
         kn[:, 0, at] = float("nan")
         kd = kn.cuda()
