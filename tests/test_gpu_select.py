@@ -76,6 +76,30 @@ def test_select_at_the_edges_of_its_row_lengths(nKb, kind):
     assert np.array_equal(off.cpu().numpy(), ref_off) and np.array_equal(idx.cpu().numpy()[: 5 * k], ref_idx)
 
 
+@pytest.mark.parametrize("nKb", [255, 256, 257, 929, 1024, 1025, 3713, 8192])
+@pytest.mark.parametrize("spread", [22, 18, 12, 9, 6, 4, 1])
+def test_select_where_masses_crowd_one_bin(nKb, spread):
+    """Masses that differ in their `spread` lowest mantissa bits alone (diffuse attention): a bin with more
+    values than the list holds is split by the bits that follow, at most three times (19 bits: 9, 5, 5; the
+    fixed-ratio rule's 22: 9, 8, 5), and what is left may be a list or equal values.  The masses are whole
+    multiples of 2^-41, so that both sides' sums are exact."""
+    rng = np.random.default_rng(nKb * 32 + spread)
+    m = (2 ** 23 + rng.integers(0, 2 ** spread, (5, nKb))) * 2.0 ** -37
+    m[1, ::3] = m[1, 0]              # ties across the row
+    m[2, : nKb // 2] *= 2.0 ** -4    # two crowds
+    m[3, nKb // 2:] = 0.0
+    for share in (0.02, 0.5, 0.97):
+        tau = share * float(m[0].sum())
+        off, idx, status = run_select(m.astype(np.float32), tau)
+        assert status == 0
+        sel = orc.select(m, tau)
+        assert util.csr_rows(off, idx[: off[-1]]) == util.csr_rows(sel.offsets, sel.kv_idx), share
+        k = max(1, int(share * nKb))
+        off, idx = lib().losa_select_topk(torch.from_numpy(m.astype(np.float32)).cuda().reshape(1, 1, 5, nKb), k)
+        ref_off, ref_idx = orc.select_topk(m, k)
+        assert np.array_equal(off.cpu().numpy(), ref_off) and np.array_equal(idx.cpu().numpy()[: 5 * k], ref_idx), k
+
+
 def test_select_ties_uniform_and_zero_masses():
     nKb = 10
     m = np.full((4, nKb), 0.1, dtype=np.float32)
