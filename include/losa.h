@@ -132,8 +132,8 @@ int losa_select(int32_t B, int32_t H, int32_t nQb, int32_t nKb, const float* mas
 
 /* Fixed-ratio selection, the rule the paper's ablation compares Eq. 3 with ("Retained mass versus
  * fixed-ratio top-k selection"): every row keeps its k heaviest blocks (equal masses: lower block
- * index first), 1 <= k <= nKb.  Same outputs, workspace and error behaviour as losa_select;
- * offsets[r] = r * k. */
+ * index first), 1 <= k <= nKb.  Same outputs, workspace and error behaviour as losa_select, except
+ * that a row with a bad sum keeps its k heaviest blocks like any other; offsets[r] = r * k. */
 int losa_select_topk(int32_t B, int32_t H, int32_t nQb, int32_t nKb, const float* mass, int32_t k,
                      int32_t* offsets, int32_t* kv_idx, int64_t kv_capacity, void* ws,
                      size_t ws_bytes, void* cuda_stream);

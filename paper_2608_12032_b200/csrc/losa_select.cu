@@ -290,7 +290,8 @@ select_rows_kernel(const float* __restrict__ mass, int rows, int nKb, double tau
     }
   }
   // The fixed-point sums hold at most 16: a row whose masses add up to more than 8 (a mass row sums
-  // to 1) is reported, and keeps every block, instead of wrapping silently.
+  // to 1) is reported, and keeps every block, instead of wrapping silently.  (The fixed-ratio rule adds
+  // nothing up and keeps its k blocks; it reports such a row too.)
   double row_sum = (double)sum;
 #pragma unroll
   for (int d = 16; d > 0; d >>= 1) row_sum += __shfl_xor_sync(0xffffffffu, row_sum, d);
@@ -302,7 +303,7 @@ select_rows_kernel(const float* __restrict__ mass, int rows, int nKb, double tau
     for (int w = 0; w < W; ++w) row_sum += rs->sum[w];
   }
   const bool too_heavy = row_sum > 8.0;
-  if (bad || (t == 0 && too_heavy && (!COUNT || W > 1))) report_error(status, LOSA_ERR_BAD_MASS);
+  if (bad || (t == 0 && too_heavy)) report_error(status, LOSA_ERR_BAD_MASS);
 
   // A tau far below any useful threshold would be lost in units of 2^-60: its rows are searched over
   // the registers in units of about 2^-50 tau, with every weight cut off at tau (a block of that mass

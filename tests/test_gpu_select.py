@@ -191,6 +191,25 @@ def test_select_flags_rows_whose_masses_do_not_look_like_masses(nKb):
     assert losa.losa_status_string(run_select(m, 0.9)[2]) == "LOSA_ERR_BAD_MASS"
 
 
+@pytest.mark.parametrize("nKb", [40, 1024, 1025, 4097])
+def test_topk_reports_the_rows_that_select_reports(nKb):
+    """A bad value, and a row whose masses add up to more than 8, at every row length; the k heaviest blocks
+    come out all the same."""
+    losa = lib()
+    k = nKb // 3
+    for bad in ("value", "sum"):
+        m = random_mass(4, nKb, 17)
+        if bad == "value":
+            m[1, 7] = 9.0
+        else:
+            m[2] = 1.0
+        off, idx = losa.losa_select_topk(torch.from_numpy(m).cuda().reshape(1, 1, 4, nKb), k)
+        assert losa.losa_status_string(losa.losa_async_status()) == "LOSA_ERR_BAD_MASS", bad
+        m[1, 7] = 0.0 if bad == "value" else m[1, 7]  # (a bad value counts as 0)
+        ref_off, ref_idx = orc.select_topk(m.astype(np.float64), k)
+        assert np.array_equal(off.cpu().numpy(), ref_off) and np.array_equal(idx.cpu().numpy()[: 4 * k], ref_idx)
+
+
 def test_select_host_side_argument_errors():
     losa = lib()
     mass = torch.rand(1, 1, 4, 8, device="cuda")
