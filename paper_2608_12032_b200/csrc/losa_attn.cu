@@ -84,8 +84,8 @@ constexpr int kTmemCols = 512;
 // Tile list ring: the scheduler warp writes one 32-bit entry per work item header, per K/V tile
 // and one end marker; every other warp reads all of them in order.
 constexpr size_t kCounterBytes = 256;  // head of the workspace: the launch's counters
-// work-item counter, length of the fallback list, the fallback launch's item counter, its CTAs that are done
-constexpr int kCounters = 4;
+// work-item counter, length of the fallback list, the fallback launch's item counter
+constexpr int kCounters = 3;
 constexpr size_t kRowstatBytes = (size_t)kMaxPersistentCtas * 2 * 128 * sizeof(float2);
 constexpr size_t kPartMlBytes = kRowstatBytes;  // same shape: [slot][2][128] float2
 constexpr int kTlChunks = 4;
@@ -195,8 +195,7 @@ struct Params {
   // list it, so that the list never holds more than nUnits entries.
   int* redo_count;
   int* redo_list;
-  int* redo_flag;  // [nUnits]
-  int* redo_done;  // how many CTAs of the second launch are done
+  int* redo_flag;  // [nUnits], and a word per split item (merge_redone_rows)
   // extents of the buffers the kernels index into (elements), for the checked build
   long long cap_part_rows, cap_table_floats, cap_mass, cap_lse, cap_units;
   uint32_t wait_polls;  // bound of every device-side wait, in polls (ptx::kWaitPolls)
@@ -316,15 +315,48 @@ struct Control {
     ++te;                                                                            \
   } while (0)
 
-// Merge of the partial units: for every row of the split items, combine the parts' unnormalised
-// O, reference maximum and row sum (the usual log-sum-exp merge) and write the attention output.  A
-// warp per row, its lanes the columns; all parts of a row are read at once, whatever their weights
-// turn out to be, because the merge is nothing but the latency of its loads (as a kernel of its own
-// that read the statistics, then part after part, it took 14 us at D = 64 and 20 us at D = 128 for
-// 8 parts; the attention kernel before it 21 us on a 2048-token layer).  AT_ONCE = false: part after
-// part, for the few registers that are left behind the attention kernel's roles.
-template <int D, bool AT_ONCE>
-__device__ __forceinline__ void merge_parts(const Params& p, int cta, int ctas) {
+// ---- merge of the partial units: for every row of the split items, combine the parts' unnormalised
+// O, reference maximum and row sum (the usual log-sum-exp merge) and write the attention output.
+// (slot0: of part 0; part s of the row lies 256 s slots further.  Lanes are the columns.)
+template <int D>
+__device__ __forceinline__ void load_part_row(const Params& p, int64_t slot, int lane, float* v) {
+  const float* src = p.part_o + slot * D + lane * (D / 32);
+  if constexpr (D == 128) {
+    const float4 x = __ldcg(reinterpret_cast<const float4*>(src));
+    v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
+  } else {
+    const float2 x = __ldcg(reinterpret_cast<const float2*>(src));
+    v[0] = x.x; v[1] = x.y;
+  }
+}
+template <int D>
+__device__ __forceinline__ void store_merged_row(const Params& p, int pbh, int grow, int lane, const float* acc, float inv) {
+  const int bh = pbh % (p.B * p.H);
+  void* const o_base = (p.problems != nullptr) ? p.problems[pbh / (p.B * p.H)].o : p.o;
+  const int64_t off = (int64_t)(bh / p.H) * p.sb + (int64_t)(bh % p.H) * p.sh + (int64_t)grow * p.sn + lane * (D / 32);
+  if (p.o_f32) {
+    float* dst = static_cast<float*>(o_base) + off;
+    if constexpr (D == 128)
+      *reinterpret_cast<float4*>(dst) = make_float4(acc[0] * inv, acc[1] * inv, acc[2] * inv, acc[3] * inv);
+    else
+      *reinterpret_cast<float2*>(dst) = make_float2(acc[0] * inv, acc[1] * inv);
+  } else {
+    __nv_bfloat16* dst = static_cast<__nv_bfloat16*>(o_base) + off;
+    if constexpr (D == 128)
+      *reinterpret_cast<uint2*>(dst) = make_uint2(ptx::pack_bf16x2(acc[0] * inv, acc[1] * inv),
+                                                  ptx::pack_bf16x2(acc[2] * inv, acc[3] * inv));
+    else
+      *reinterpret_cast<uint32_t*>(dst) = ptx::pack_bf16x2(acc[0] * inv, acc[1] * inv);
+  }
+}
+
+// Of all split items, or (skip_redo) of those that hold no unit of the fallback list.  A warp per row; all
+// parts of a row are read at once, whatever their weights turn out to be, because the merge is nothing
+// but the latency of its loads (as a kernel of its own that read the statistics, then part after part, it
+// took 14 us at D = 64 and 20 us at D = 128 for 8 parts; the attention kernel before it 21 us on a
+// 2048-token layer).
+template <int D>
+__device__ __forceinline__ void merge_parts(const Params& p, int cta, int ctas, bool skip_redo) {
   constexpr int kCols = D / 32;
   const int warps = blockDim.x >> 5, lane = threadIdx.x & 31;
   const int parts = p.split_parts;
@@ -336,25 +368,15 @@ __device__ __forceinline__ void merge_parts(const Params& p, int cta, int ctas) 
     const int pbh = w / p.nPairs, pr = w % p.nPairs;
     const int T = 2 * pr + qt, grow = T * 128 + row;
     if (grow >= p.N) continue;
-    const int64_t slot0 = ((int64_t)r * parts * 2 + qt) * 128 + row;  // of part s: slot0 + 256 s
+    if (skip_redo && __any_sync(0xffffffffu, lane < parts && __ldcg(p.redo_flag + p.split_first + r * parts + lane) != 0))
+      continue;
+    const int64_t slot0 = ((int64_t)r * parts * 2 + qt) * 128 + row;
     float2 ml = make_float2(0.f, 0.f);
     if (lane < parts) ml = __ldcg(p.part_ml + slot0 + lane * 256);
-    auto load = [&](int s, float* v) {
-      const float* src = p.part_o + (slot0 + s * 256) * D + lane * kCols;
-      if constexpr (kCols == 4) {
-        const float4 x = __ldcg(reinterpret_cast<const float4*>(src));
-        v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
-      } else {
-        const float2 x = __ldcg(reinterpret_cast<const float2*>(src));
-        v[0] = x.x; v[1] = x.y;
-      }
-    };
-    float v[AT_ONCE ? kMaxParts : 1][kCols];
-    if constexpr (AT_ONCE) {
+    float v[kMaxParts][kCols];
 #pragma unroll
-      for (int s = 0; s < kMaxParts; ++s)
-        if (s < parts) load(s, v[s]);
-    }
+    for (int s = 0; s < kMaxParts; ++s)
+      if (s < parts) load_part_row<D>(p, slot0 + s * 256, lane, v[s]);
     // (a part without keys of the row has the sum 0; one that met NaN has the sum NaN, and so has the row)
     float m = (ml.y != 0.f) ? ml.x : -INFINITY;
 #pragma unroll
@@ -363,35 +385,85 @@ __device__ __forceinline__ void merge_parts(const Params& p, int cta, int ctas) 
     float L = 0.f, acc[kCols];
 #pragma unroll
     for (int c = 0; c < kCols; ++c) acc[c] = 0.f;
-#pragma unroll(AT_ONCE ? kMaxParts : 1)
+#pragma unroll
     for (int s = 0; s < kMaxParts; ++s) {
       if (s < parts) {
         const float sc = __shfl_sync(0xffffffffu, mine, s);
         L += __shfl_sync(0xffffffffu, ml.y, s) * sc;
-        if constexpr (!AT_ONCE) load(s, v[0]);
         if (sc != 0.f) {
 #pragma unroll
-          for (int c = 0; c < kCols; ++c) acc[c] += v[AT_ONCE ? s : 0][c] * sc;
+          for (int c = 0; c < kCols; ++c) acc[c] += v[s][c] * sc;
         }
       }
     }
-    const float inv = (L != 0.f) ? 1.f / L : 0.f;
-    const int bh = pbh % (p.B * p.H);
-    void* const o_base = (p.problems != nullptr) ? p.problems[pbh / (p.B * p.H)].o : p.o;
-    const int64_t off = (int64_t)(bh / p.H) * p.sb + (int64_t)(bh % p.H) * p.sh + (int64_t)grow * p.sn + lane * kCols;
-    if (p.o_f32) {
-      float* dst = static_cast<float*>(o_base) + off;
-      if constexpr (kCols == 4)
-        *reinterpret_cast<float4*>(dst) = make_float4(acc[0] * inv, acc[1] * inv, acc[2] * inv, acc[3] * inv);
-      else
-        *reinterpret_cast<float2*>(dst) = make_float2(acc[0] * inv, acc[1] * inv);
-    } else {
-      __nv_bfloat16* dst = static_cast<__nv_bfloat16*>(o_base) + off;
-      if constexpr (kCols == 4)
-        *reinterpret_cast<uint2*>(dst) = make_uint2(ptx::pack_bf16x2(acc[0] * inv, acc[1] * inv),
-                                                    ptx::pack_bf16x2(acc[2] * inv, acc[3] * inv));
-      else
-        *reinterpret_cast<uint32_t*>(dst) = ptx::pack_bf16x2(acc[0] * inv, acc[1] * inv);
+    store_merged_row<D>(p, pbh, grow, lane, acc, (L != 0.f) ? 1.f / L : 0.f);
+  }
+}
+
+// Fallback launch: a warp has rewritten its 32 rows of one part of split item r.  The last of the item's
+// recomputed parts to get there merges these rows (no other wait for any of them is needed: the parts that
+// are not recomputed come from the launch before).  A lane holds its row's weights; the loads of several
+// rows are in flight at a time.  (When the launch's last CTA merged all rows of all items alone, one
+// row that outgrew its reference made a call on 2048 tokens take 1140 instead of 55 us.)
+template <int D>
+__device__ __forceinline__ void merge_redone_rows(const Params& p, int r, int qt, int warp_rows, int lane) {
+  constexpr int kCols = D / 32;
+  const int parts = p.split_parts;
+  const int redone = __popc(__ballot_sync(
+      0xffffffffu, lane < parts && __ldcg(p.redo_flag + p.split_first + r * parts + lane) != 0));
+  __threadfence();
+  __syncwarp();
+  uint32_t done = 0u;  // of these rows, parts recomputed before this one: a nibble of the item's word
+  const int nibble = 4 * (qt * 4 + warp_rows);
+  if (lane == 0) done = (atomicAdd(reinterpret_cast<uint32_t*>(p.redo_flag) + p.nUnits + r, 1u << nibble) >> nibble) & 15u;
+  done = __shfl_sync(0xffffffffu, done, 0);
+  if ((int)done + 1 != redone) return;
+  __threadfence();
+  const int w = p.split_first + r;
+  const int pbh = w / p.nPairs, T = 2 * (w % p.nPairs) + qt;
+  const int grow0 = T * 128 + warp_rows * 32;
+  const int64_t slot0 = ((int64_t)r * parts * 2 + qt) * 128 + warp_rows * 32;
+  auto stat = [&](int s) { return __ldcg(p.part_ml + slot0 + s * 256 + lane); };
+  auto weight = [](float2 ml, float m) { return (ml.y != 0.f) ? ptx::ex2_approx(ml.x - m) : 0.f; };
+  float m = -INFINITY, L = 0.f;
+#pragma unroll 4
+  for (int s = 0; s < parts; ++s) {
+    const float2 ml = stat(s);
+    m = fmaxf(m, (ml.y != 0.f) ? ml.x : -INFINITY);
+  }
+#pragma unroll 4
+  for (int s = 0; s < parts; ++s) {
+    const float2 ml = stat(s);
+    L += ml.y * weight(ml, m);
+  }
+  const float inv = (L != 0.f) ? 1.f / L : 0.f;
+  constexpr int kRows = 8;
+#pragma unroll 1
+  for (int row0 = 0; row0 < 32; row0 += kRows) {
+    float acc[kRows][kCols];
+#pragma unroll
+    for (int j = 0; j < kRows; ++j)
+#pragma unroll
+      for (int c = 0; c < kCols; ++c) acc[j][c] = 0.f;
+#pragma unroll 1
+    for (int s = 0; s < parts; ++s) {
+      float v[kRows][kCols];
+#pragma unroll
+      for (int j = 0; j < kRows; ++j) load_part_row<D>(p, slot0 + s * 256 + row0 + j, lane, v[j]);
+      const float mine = weight(stat(s), m);
+#pragma unroll
+      for (int j = 0; j < kRows; ++j) {
+        const float sc = __shfl_sync(0xffffffffu, mine, row0 + j);
+        if (sc != 0.f) {
+#pragma unroll
+          for (int c = 0; c < kCols; ++c) acc[j][c] += v[j][c] * sc;
+        }
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < kRows; ++j) {
+      const float row_inv = __shfl_sync(0xffffffffu, inv, row0 + j);
+      if (grow0 + row0 + j < p.N) store_merged_row<D>(p, pbh, grow0 + row0 + j, lane, acc[j], row_inv);
     }
   }
 }
@@ -437,12 +509,16 @@ losa_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     ptx::grid_launch_dependents();
   } else {
     // Fallback launch: on ordinary inputs there is nothing to recompute, and the CTAs only merge the
-    // partial units and leave, before they set anything up.
+    // partial units and leave, before they set anything up.  Otherwise the CTAs that get no unit merge
+    // the items without one (all CTAs, if each gets a unit); the others follow where they are recomputed.
     ptx::grid_dependency_wait();
-    if (*reinterpret_cast<volatile int*>(p.redo_count) == 0) {
-      if (MODE == kDense || MODE == kSparse) merge_parts<D, true>(p, blockIdx.x, gridDim.x);
-      return;
+    const int redo = *reinterpret_cast<volatile int*>(p.redo_count);
+    const int idle = (int)gridDim.x - redo;
+    if (MODE == kDense || MODE == kSparse) {
+      if (idle <= 0) merge_parts<D>(p, blockIdx.x, gridDim.x, true);
+      else if ((int)blockIdx.x >= redo) merge_parts<D>(p, (int)blockIdx.x - redo, idle, redo > 0);
     }
+    if ((int)blockIdx.x >= redo) return;
   }
   uint8_t* sQ = smem;
   uint8_t* sK = sQ + 2 * C::kQBytes;
@@ -1178,6 +1254,7 @@ losa_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
             ptx::tc_fence_before_sync();
             ptx::mbar_arrive(&ctl->o_free[qt]);
           }
+          if ((MODE == kDense || MODE == kSparse) && partial) merge_redone_rows<D>(p, w - p.split_first, qt, wl, lane);
         }
       }
       if (C::kWantMass) {
@@ -1609,15 +1686,6 @@ teardown:
     ptx::tc_fence_after_sync();
     ptx::tmem_dealloc(tmem_base, kTmemCols);
   }
-  if (!SPLIT && (MODE == kDense || MODE == kSparse) && p.split_parts > 1) {
-    // the last CTA that is done recomputing merges the partial units alone
-    __threadfence();
-    __syncthreads();
-    if (__syncthreads_or(threadIdx.x == 0 && atomicAdd(p.redo_done, 1) == (int)gridDim.x - 1)) {
-      __threadfence();
-      merge_parts<D, false>(p, 0, 1);
-    }
-  }
 }
 
 #include "losa_attn_tile.cuh"
@@ -1652,7 +1720,11 @@ __global__ void __launch_bounds__(32 * NB) build_tile_lists_kernel(const Params 
   const int list = blockIdx.x, unit = ONE ? list >> 1 : list;
   const int bit0 = ONE ? (list & 1) * NB : 0;  // membership bit of the first query block
   if (list == 0 && threadIdx.x < kCounters) p.work_counter[threadIdx.x] = 0;
-  if (threadIdx.x == 0) p.redo_flag[unit] = 0;
+  if (threadIdx.x == 0) {
+    p.redo_flag[unit] = 0;
+    if (unit >= p.split_first && (unit - p.split_first) % p.split_parts == 0)
+      p.redo_flag[p.nUnits + (unit - p.split_first) / p.split_parts] = 0;
+  }
   int w = unit, part = 0, parts = 1;
   if (unit >= p.split_first) {
     const int r = unit - p.split_first;
@@ -1856,10 +1928,10 @@ int make_maps(ProblemEntry* e, const Geometry& g, const void* q, const void* k, 
 // not a memset, so that the attention kernel can be launched as its dependent: 3 us of that kernel's
 // set-up overlap).
 constexpr int kInitThreads = 256;
-__global__ void __launch_bounds__(kInitThreads) init_counters_kernel(int* counters, int* flags, int units) {
+__global__ void __launch_bounds__(kInitThreads) init_counters_kernel(int* counters, int* flags, int n) {
   ptx::grid_launch_dependents();
   if (blockIdx.x == 0 && threadIdx.x < kCounters) counters[threadIdx.x] = 0;
-  for (int64_t i = (int64_t)blockIdx.x * kInitThreads + threadIdx.x; i < units; i += (int64_t)gridDim.x * kInitThreads)
+  for (int64_t i = (int64_t)blockIdx.x * kInitThreads + threadIdx.x; i < n; i += (int64_t)gridDim.x * kInitThreads)
     flags[i] = 0;
 }
 
@@ -2021,7 +2093,8 @@ int launch_t(const Geometry& g, const void* q, const void* k, const void* v, Par
                 bm_bytes, st, prm.nProb > 1, prm);
   } else {
     rc = launch(init_counters_kernel, dim3(min(ctas, (prm.nUnits + 4 * kInitThreads - 1) / (4 * kInitThreads))),
-                kInitThreads, 0, st, false, prm.work_counter, prm.redo_flag, prm.nUnits);
+                kInitThreads, 0, st, false, prm.work_counter, prm.redo_flag,
+                prm.nUnits + prm.nWork - prm.split_first);
   }
   if (rc != LOSA_OK) return rc;
   // All modes run with two threads per query row and a reference that never moves; the units whose
@@ -2107,7 +2180,8 @@ size_t attn_workspace_bytes(AttnMode mode, const Geometry& g, int n_prob) {
     if (mode == kSparse) bytes += tl_count_bytes(g, n_prob) + tl_entries_bytes(g, n_prob);
     // batched launch: the table of the problems' tensor maps and pointers
     if (n_prob > 1) bytes += (size_t)n_prob * sizeof(ProblemEntry);
-    // the work units handed to the fallback launch, and their flags
+    // the work units handed to the fallback launch; their flags and the split items' words (whose parts
+    // are kMaxPersistentCtas at most: units and split items together are no more than max_units)
     bytes += redo_list_bytes(g, n_prob);
     return bytes;
   }
@@ -2184,7 +2258,6 @@ int launch_attn(AttnMode mode, const Geometry& g, const void* q, const void* k, 
     }
     // (kCounters)
     prm.redo_count = prm.work_counter + 1;
-    prm.redo_done = prm.work_counter + 3;
     prm.redo_list = reinterpret_cast<int*>(
         tl + (mode == kSparse ? tl_count_bytes(g, n_prob) + tl_entries_bytes(g, n_prob) : 0) +
         (n_prob > 1 ? (size_t)n_prob * sizeof(ProblemEntry) : 0));

@@ -605,3 +605,40 @@ def test_a_key_that_is_not_a_number_shows_wherever_it_lies(D, R, C):
         got, want = o_s[0].cpu().reshape(H * N, D)[free], torch.from_numpy(ref_s[0].reshape(H * N, D))[free]
         assert (got - want).abs().max() <= util.MAX_ABS_TOL, at
         assert np.abs(o[0, 1].cpu().numpy() - ref[0, 1]).max() <= util.MAX_ABS_TOL
+
+
+@pytest.mark.parametrize("D,R,C", [(64, 64, 64), (64, 128, 32), (128, 128, 128), (128, 64, 64)])
+@pytest.mark.parametrize("heads", [(1,), (0, 2), (0, 1, 2, 3)])
+def test_cut_items_of_which_some_parts_outgrow(D, R, C, heads):
+    """A small layer, all of whose work items are cut into parts.  In some heads one row meets a key far
+    above its first ones in one part, another row in several parts: these parts are recomputed and their
+    item is merged behind them, next to items that no part of has to be."""
+    losa = lib()
+    B, H, N = 1, 4, 2048 - 30
+    g = torch.Generator("cpu").manual_seed(79)
+    q, k, v = (torch.randn(B, H, N, D, generator=g) for _ in range(3))
+    far = torch.zeros(D)
+    far[3] = (120.0 * D ** 0.5) ** 0.5  # a score of 120 with itself, of a few with the other rows
+    for h in heads:
+        q[0, h, 700] = far
+        q[0, h, 1100 + h] = far
+        for at in (N - 5,) if h == 2 else (N - 5, 1300, 500):
+            k[0, h, at] = far
+    q, k, v = q.bfloat16(), k.bfloat16(), v.bfloat16()
+    qd, kd, vd = q.cuda(), k.cuda(), v.cuda()
+    qn, kn, vn = util.to_np(q), util.to_np(k), util.to_np(v)
+    nQb, nKb = -(-N // R), -(-N // C)
+    off, idx = util.random_csr(B * H * nQb, nKb, 21, 0.7)
+    offd, idxd = torch.from_numpy(off).cuda(), torch.from_numpy(idx).cuda()
+    ws = torch.empty(losa.losa_workspace_bytes(losa.binding.LOSA_OP_ATTN, losa.make_problem(qd, R, C)),
+                     dtype=torch.uint8, device="cuda")
+    o = losa.losa_attn(qd, kd, vd, R, C, out_dtype=torch.float32, ws=ws)
+    assert int(ws[:8].view(torch.int32)[1]) >= len(heads)  # units were listed
+    again = losa.losa_attn(qd, kd, vd, R, C, out_dtype=torch.float32, ws=ws)
+    o_s = losa.losa_sparse_attn(qd, kd, vd, offd, idxd, R, C, out_dtype=torch.float32)
+    again_s = losa.losa_sparse_attn(qd, kd, vd, offd, idxd, R, C, out_dtype=torch.float32)
+    assert losa.losa_async_status() == 0
+    util.assert_output_close(o, orc.dense_attn(qn, kn, vn), "dense")
+    util.assert_output_close(
+        o_s, orc.blocks_to_tokens(orc.sparse_attn(qn, kn, vn, R, C, off, idx), B, H, N), "sparse")
+    assert torch.equal(o, again) and torch.equal(o_s, again_s)
