@@ -193,3 +193,35 @@ def test_crafted_patterns_at_head_dimension_64(R, C, kind):
     assert losa.losa_async_status() == 0
     ref = orc.blocks_to_tokens(orc.sparse_attn(util.to_np(q), util.to_np(k), util.to_np(v), R, C, off, idx), 1, H, N)
     util.assert_output_close(o, ref, f"{kind} R={R} C={C}")
+
+
+def test_rows_far_below_a_borrowed_reference():
+    """64-row query blocks at head dimension 64: a query block that lists nothing in the first chunk of its
+    query tile's list takes its reference from keys that it does not attend to.  Here these lie 38 to 100
+    nats above its own: row sums (576 keys) of about 2^-49, 2^-56 and 2^-66 (below 2^-60 a unit is recomputed),
+    of next to nothing and of nothing.  Whole items and (of the last heads) cut ones."""
+    losa = lib()
+    Rq, nats, N, Dh = 64, (38.0, 43.0, 49.5, 60.0, 100.0), 64 * 80, 64
+    H = len(nats)
+    nb = N // Rq
+    off, idx = csr_from([range(70) if g % 2 == 0 else range(71, 80) for _ in range(H) for g in range(nb)])
+    q, k, v = (util.rand_bf16((1, H, N, Dh), 990 + i) for i in range(3))
+    odd = (torch.arange(N) // Rq) % 2 == 1
+    q[..., 5] = torch.where(odd, 8.0, 0.0).bfloat16()
+    for h, x in enumerate(nats):
+        k[0, h, :, 5] = torch.where(torch.arange(N) < 70 * 64, x, 0.0).bfloat16()  # 8 x / sqrt(64): x nats
+    prob = losa.make_problem(q.cuda(), Rq, 64)
+    ws = torch.empty(losa.losa_workspace_bytes(losa.binding.LOSA_OP_SPARSE_ATTN, prob), dtype=torch.uint8, device="cuda")
+    slots, items = losa.losa_work_slots(losa.binding.LOSA_OP_SPARSE_ATTN, prob), H * nb // 4
+    rest = items % slots if items > slots else items
+    parts = min(slots // rest, 8) if rest else 1
+    o = losa.losa_sparse_attn(q.cuda(), k.cuda(), v.cuda(), torch.from_numpy(off).cuda(), torch.from_numpy(idx).cuda(),
+                              Rq, 64, out_dtype=torch.float32, ws=ws)
+    assert losa.losa_async_status() == 0
+    if rest <= 3 * nb // 4:  # the units of the last three heads, and no others
+        assert int(ws[:8].view(torch.int32)[1]) == 3 * nb // 4 + rest * (parts - 1)
+    ref = orc.blocks_to_tokens(orc.sparse_attn(util.to_np(q), util.to_np(k), util.to_np(v), Rq, 64, off, idx), 1, H, N)
+    util.assert_output_close(o, ref, "rows below a borrowed reference")
+    for h in range(H):
+        err = (o[0, h].cpu() - torch.from_numpy(ref[0, h])).norm() / np.linalg.norm(ref[0, h])
+        assert err <= 4e-3, (nats[h], err)  # bf16 weights: 2^-9 each, at random
