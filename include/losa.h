@@ -114,9 +114,10 @@ int losa_block_mass(const losa_problem_t* p, const void* q, const void* k, float
                     float* lse, void* ws, size_t ws_bytes, void* cuda_stream);
 
 /* Retained-mass selection (Eq. 3).  For every row r = (b, h, i): sort the nKb masses in
- * decreasing order (equal masses: lower block index first), accumulate them in fp64 and
- * keep the shortest prefix whose sum is >= tau; tau >= 1 keeps every block, and so does a
- * row whose sum never reaches tau.  Each row keeps at least one block.
+ * decreasing order (equal masses: lower block index first), accumulate them and keep the
+ * shortest prefix whose sum is >= tau; tau >= 1 keeps every block, and so does a row whose
+ * sum never reaches tau.  Each row keeps at least one block.  (The sums are taken in integers,
+ * in units of 2^-60: they differ from sequential fp64 sums by less than 1e-14.)
  *   mass        f32 [rows, nKb], rows = B*H*nQb, nKb <= LOSA_SELECT_MAX_KEY_BLOCKS; values in
  *               [0, 8] and row sums <= 8 (a mass row sums to 1), else LOSA_ERR_BAD_MASS is
  *               recorded: a bad value counts as 0, a row with a bad sum keeps every block
@@ -189,9 +190,9 @@ int losa_select_noalloc(int32_t B, int32_t H, int32_t nQb, int32_t nKb, const fl
  *   ws       >= losa_workspace_bytes(LOSA_OP_SPARSE_ATTN, p) bytes (about 21 MB at D = 128
  *            plus the work units' tile lists: the counter the persistent CTAs draw work
  *            items from, the partial results of the last work items, which are processed in
- *            parts and merged by a second kernel on the same stream, and the list of work
- *            units that a fallback launch recomputes because their scores outgrew the
- *            reference of their first tile); not shared between calls that may run
+ *            parts and merged by a second launch on the same stream, and the list of work
+ *            units that this launch recomputes because their scores outgrew the reference
+ *            of their first tile); not shared between calls that may run
  *            concurrently; contents undefined afterwards.  The result does not depend on
  *            timing: the same call on the same GPU gives the same bits.
  * The output is normalised by the sum of the bf16-rounded weights the tensor core multiplies

@@ -167,7 +167,7 @@ int losa_select(int32_t B, int32_t H, int32_t nQb, int32_t nKb, const float* mas
   if (!mass || !offsets || !kv_idx || kv_capacity < 0) return LOSA_ERR_INVALID_ARG;
   const int64_t rows = (int64_t)B * H * nQb;
   if (rows * nKb > INT32_MAX) return LOSA_ERR_UNSUPPORTED;
-  if (nKb > LOSA_SELECT_MAX_KEY_BLOCKS) return LOSA_ERR_UNSUPPORTED;  // one row is sorted in shared memory
+  if (nKb > LOSA_SELECT_MAX_KEY_BLOCKS) return LOSA_ERR_UNSUPPORTED;  // one row is held in the registers of 8 warps
   const size_t need = select_workspace_bytes(rows, nKb);
   if (!ws || ws_bytes < need) return LOSA_ERR_WORKSPACE;
   if (!aligned16(ws)) return LOSA_ERR_INVALID_ARG;

@@ -1,6 +1,9 @@
 // Attention kernels of liblosa for sm_100a: dense attention, block-sparse attention over a
-// frozen CSR pattern (Eq. 4), the exact block-mass pass (Eq. 1) and the fused construction step,
-// as ONE warp-specialised persistent kernel template with two thread layouts.
+// frozen CSR pattern (Eq. 4), the exact block-mass pass (Eq. 1) and the fused construction step.
+// Head dimension 64, and head dimension 128 with 128-row query blocks, run in losa_tile_kernel
+// (losa_attn_tile.cuh, included below): one query tile and three S buffers per CTA.
+// losa_attn_kernel, described here, is one warp-specialised persistent kernel template with two thread
+// layouts; it serves head dimension 128 with 64-row query blocks and the fallback launch of all.
 //
 // Warps 0-3 are utility warps: warp 0 is the TMA producer, which streams the query tiles and the
 // K / V tiles named by the tile list into 128B-swizzled shared-memory rings (a K/V tile is 128
@@ -8,10 +11,10 @@
 // thread each) issue the tcgen05 MMAs: S = Q K^T from shared memory into TMEM, O += P V with P
 // read from TMEM (bf16, written over S) and V from shared memory as the MN-major operand; warp 3
 // publishes the tile list every other warp follows (sparse mode: streamed from lists that
-// build_tile_lists_kernel made before the launch).  The softmax warps follow: two warpgroups, one
-// 128-row query tile each and one thread per query row (mass pass, fused step, fallback), or four
-// warpgroups with two threads per query row (dense and sparse forward); they take their registers
-// from the utility warpgroup.
+// build_tile_lists_kernel made before the launch).  The softmax warps follow: four warpgroups with
+// two threads per query row (the main launch of every mode), or two warpgroups, one 128-row query
+// tile each and one thread per query row (the fallback launch); they take their registers from the
+// utility warpgroup.
 //
 // A work item is a pair of consecutive query tiles of one (batch, head) - of one problem, in a
 // batched launch.  The key blocks the pair visits are the union of the index lists of its query
@@ -30,9 +33,6 @@
 //
 // Every wait is bounded; a wait that expires raises the CTA's abort flag, records
 // LOSA_ERR_TIMEOUT, and all roles leave through the common teardown that frees TMEM.
-//
-// Head dimension 64, and head dimension 128 with 128-row query blocks, run in a second kernel,
-// losa_tile_kernel (losa_attn_tile.cuh, included below): one query tile and three S buffers per CTA.  This kernel serves the rest and the fallback launch of all.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <math.h>
@@ -54,8 +54,7 @@ std::atomic<uint32_t> g_stall_polls{0u};  // > 0: the next attention launch is a
 // Thread layout.  Warps 0-3 are the utility warpgroup (TMA, 2 MMA issuers, scheduler); the softmax
 // warps follow.  Two layouts:
 //   one thread per query row (SPLIT = false): 2 softmax warpgroups, one per query tile, each thread
-//     holding a whole 128-column S row.  Used by the mass pass and the fused construction step,
-//     and as the fallback of the attention-only modes.
+//     holding a whole 128-column S row.  Used by the fallback launch of every mode.
 //   two threads per query row (SPLIT = true): 4 softmax warpgroups, two per query tile, each
 //     thread holding 64 columns.  A warp's ex2 instructions occupy it for 8 issue cycles each and
 //     its other instructions do not overlap them (measured on the loop alone: 1301 cycles per
@@ -2077,7 +2076,7 @@ int launch_t(const Geometry& g, const void* q, const void* k, const void* v, Par
   if (kTileMode) ctas = max(1, min(sms, kMaxPersistentCtas) / 2);
   // The items of the last, partly filled wave of the persistent grid (all items, if there are
   // fewer than CTAs) are cut into parts of the key range, so that the wave ends after 1/parts of
-  // an item; their partial results are merged by a second, small kernel.  Attention output
+  // an item; their partial results are merged by the fallback launch.  Attention output
   // only: the mass epilogue needs a row's final statistics inside the kernel.
   prm.nUnits = prm.nWork;
   prm.split_first = prm.nWork;

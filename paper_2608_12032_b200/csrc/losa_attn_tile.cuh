@@ -186,7 +186,8 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   // tensor cores, so one group of four scores in every kPolyOf takes its exponentials from a
   // polynomial on the FMA pipe.  17776 tokens, 8 heads: dense 735 us with one in 8, 742 in 16, 763 in 6,
   // 805 in 4.  The mass pass (no P to pack and to sum) takes one in 4: 735 us, 759 in 8, 786 in 6; at head
-  // dimension 128 (Wan shape) 3635 us, 3750 in 8, 3937 without.
+  // dimension 128 (32760 tokens, 12 heads, 128-key blocks, unit normal q and k) 3463 us, 3639 in 8, 3924
+  // without (against 64 bits its masses err by 1 % more with it than without, 2e-7).
   constexpr int kPolyOf = (MODE == kMass) ? LOSA_POLY_OF_MASS : (D == 64) ? LOSA_POLY_OF : 0;
   using Ctl = TileControl;
   constexpr bool kWantMass = (MODE == kFused || MODE == kMass);  // the block masses (Eq. 1) are wanted
@@ -952,8 +953,8 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           const float* tb = reinterpret_cast<const float*>(p.table) + (int64_t)blockIdx.x * 2 * (int64_t)p.nKb * 256;
           // Lane l sums rows 4 l .. 4 l + 3 of four key blocks at a time: one 16-byte load per block (two
           // where the halves of a block have entries of their own) and four blocks in flight.  The fold is
-          // the latency of these loads: one block at a time in four 4-byte loads, the mass pass took 4175 us
-          // with 1024 key blocks (Wan shape) and takes 3830, the fused step 5960 and 5440.
+          // the latency of these loads: one block at a time in four 4-byte loads, the mass pass took 4523 us
+          // with 1024 key blocks (32760 tokens, 12 heads) and takes 4250.
           float iv[4];
 #pragma unroll
           for (int rr = 0; rr < 4; ++rr) {

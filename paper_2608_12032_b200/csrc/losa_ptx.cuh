@@ -124,12 +124,12 @@ __device__ __forceinline__ void prefetch_tensormap(const CUtensorMap* m) {
   asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(m)) : "memory");
 }
 
-// 4D tiled load global -> this CTA's shared memory, completion on an mbarrier.
 // Before a copy through a tensor map that a kernel wrote to global memory.
 __device__ __forceinline__ void tensormap_acquire(const CUtensorMap* m) {
   asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(m) : "memory");
 }
 
+// 4D tiled load global -> this CTA's shared memory, completion on an mbarrier.
 __device__ __forceinline__ void tma_load_4d(void* smem_dst, const CUtensorMap* map, uint64_t* bar,
                                             int x, int y, int z, int w) {
   asm volatile(

@@ -179,7 +179,7 @@ def test_tile_lists_that_end_around_a_chunk_of_the_list(C):
 def test_crafted_patterns_at_head_dimension_64(R, C, kind):
     """One query tile per CTA and a list per query tile; with 64-row blocks a query tile's two blocks
     meet their first listed tile at different places, in either softmax group, or past the first chunk
-    of the list (2560 keys here), where the reference falls back to the tile's own maximum."""
+    of the list (32 entries), where the reference is the maximum over all keys of the first tile."""
     losa = lib()
     H, N = 2, 128 * 41 - 37
     nQb, nKb = -(-N // R), -(-N // C)

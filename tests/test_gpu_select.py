@@ -117,7 +117,7 @@ def test_select_ties_uniform_and_zero_masses():
 @pytest.mark.parametrize("nKb", [3, 8, 64, 2048])
 def test_select_threshold_is_inclusive_on_exactly_representable_masses(nKb):
     """A prefix whose mass equals tau exactly already suffices (Eq. 3: >= tau).  Masses are powers
-    of two, so both sides add them without rounding; nKb = 2048 takes the sorting kernel."""
+    of two, so both sides add them without rounding; nKb = 2048 takes two warps per row."""
     m = np.zeros((3, nKb), dtype=np.float32)
     m[0, :3] = (0.5, 0.25, 0.25)
     m[1, :3] = (0.25, 0.25, 0.5)
@@ -173,9 +173,9 @@ def test_select_flags_negative_and_nan_mass():
 
 @pytest.mark.parametrize("nKb", [40, 1500])
 def test_select_flags_rows_whose_masses_do_not_look_like_masses(nKb):
-    """Masses above 8, and rows whose masses add up to more than 8 (beyond the warp kernel's
+    """Masses above 8, and rows whose masses add up to more than 8 (beyond the
     fixed-point range), are reported instead of giving a silently wrong pattern; a row with a bad
-    sum keeps every block.  Both selection kernels (nKb = 1500 takes the sorting one)."""
+    sum keeps every block.  One and (nKb = 1500) two warps per row."""
     losa = lib()
     m = random_mass(4, nKb, 11)
     m[2] = 1.0            # each value passes, the row adds up to nKb

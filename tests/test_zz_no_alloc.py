@@ -7,7 +7,7 @@ scratch array.  This test drives that entry point through the C ABI and checks, 
 row that share the scratch array (with different inputs, so stale contents would show), that it
 returns exactly what losa_select returns and exactly what the fp64 oracle's Eq. 3 gives on the
 same masses.  Integer results: both comparisons are bit-exact.  Rows of 278 and 33 blocks take
-the warp-per-row kernel, rows of 1500 blocks the sorting kernel, as in losa_select.
+one warp each, rows of 1500 blocks two, as in losa_select.
 
 Collected last on purpose, so a run that stops at the first failure has already run the rest.
 """
