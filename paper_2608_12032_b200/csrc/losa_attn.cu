@@ -1729,11 +1729,6 @@ __global__ void __launch_bounds__(32 * NB) build_tile_lists_kernel(const Params 
   const int list = blockIdx.x, unit = ONE ? list >> 1 : list;
   const int bit0 = ONE ? (list & 1) * NB : 0;  // membership bit of the first query block
   if (list == 0 && threadIdx.x < kCounters) p.work_counter[threadIdx.x] = 0;
-  if (threadIdx.x == 0) {
-    p.redo_flag[unit] = 0;
-    if (unit >= p.split_first && (unit - p.split_first) % p.split_parts == 0)
-      p.redo_flag[p.nUnits + (unit - p.split_first) / p.split_parts] = 0;
-  }
   int w = unit, part = 0, parts = 1;
   if (unit >= p.split_first) {
     const int r = unit - p.split_first;
@@ -1866,9 +1861,12 @@ __global__ void __launch_bounds__(32 * NB) build_tile_lists_kernel(const Params 
     ra += tot[1];
     rbb += tot[2];
   }
-  if (lane == 0)
+  if (lane == 0) {
     p.tl_count[list] = (int32_t)((uint32_t)(total / G) | ((nb + na > 0) ? kHdrHas : 0u) |
                                  ((nb + nbb > 0) ? 2u * kHdrHas : 0u) | ((nb == 0 && tmin > 0) ? kHdrLate : 0u));
+    p.redo_flag[unit] = 0;
+    if (parts > 1 && part == 0) p.redo_flag[p.nUnits + w - p.split_first] = 0;
+  }
 }
 
 // ---------------------------------------------------------------------------- host side
