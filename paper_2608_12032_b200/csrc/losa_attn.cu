@@ -349,13 +349,13 @@ __device__ __forceinline__ void store_merged_row(const Params& p, int pbh, int g
   }
 }
 
-// Of all split items, or (skip_redo) of those that hold no unit of the fallback list.  A warp per row; all
+// Of all split items, or (SKIP) of those that hold no unit of the fallback list.  A warp per row; all
 // parts of a row are read at once, whatever their weights turn out to be, because the merge is nothing
 // but the latency of its loads (as a kernel of its own that read the statistics, then part after part, it
 // took 14 us at D = 64 and 20 us at D = 128 for 8 parts; the attention kernel before it 21 us on a
 // 2048-token layer).
-template <int D>
-__device__ __forceinline__ void merge_parts(const Params& p, int cta, int ctas, bool skip_redo) {
+template <int D, bool SKIP>
+__device__ __forceinline__ void merge_parts(const Params& p, int cta, int ctas) {
   constexpr int kCols = D / 32;
   const int warps = blockDim.x >> 5, lane = threadIdx.x & 31;
   const int parts = p.split_parts;
@@ -367,7 +367,7 @@ __device__ __forceinline__ void merge_parts(const Params& p, int cta, int ctas, 
     const int pbh = w / p.nPairs, pr = w % p.nPairs;
     const int T = 2 * pr + qt, grow = T * 128 + row;
     if (grow >= p.N) continue;
-    if (skip_redo && __any_sync(0xffffffffu, lane < parts && __ldcg(p.redo_flag + p.split_first + r * parts + lane) != 0))
+    if (SKIP && __any_sync(0xffffffffu, lane < parts && __ldcg(p.redo_flag + p.split_first + r * parts + lane) != 0))
       continue;
     const int64_t slot0 = ((int64_t)r * parts * 2 + qt) * 128 + row;
     float2 ml = make_float2(0.f, 0.f);
@@ -512,11 +512,13 @@ losa_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     // the items without one (all CTAs, if each gets a unit); the others follow where they are recomputed.
     ptx::grid_dependency_wait();
     const int redo = *reinterpret_cast<volatile int*>(p.redo_count);
-    const int idle = (int)gridDim.x - redo;
-    if (MODE == kDense || MODE == kSparse) {
-      if (idle <= 0) merge_parts<D>(p, blockIdx.x, gridDim.x, true);
-      else if ((int)blockIdx.x >= redo) merge_parts<D>(p, (int)blockIdx.x - redo, idle, redo > 0);
+    if (redo == 0) {
+      if (MODE == kDense || MODE == kSparse) merge_parts<D, false>(p, blockIdx.x, gridDim.x);
+      return;
     }
+    const int idle = (int)gridDim.x - redo;
+    if ((MODE == kDense || MODE == kSparse) && (idle <= 0 || (int)blockIdx.x >= redo))
+      merge_parts<D, true>(p, (int)blockIdx.x - (idle > 0 ? redo : 0), idle > 0 ? idle : (int)gridDim.x);
     if ((int)blockIdx.x >= redo) return;
   }
   uint8_t* sQ = smem;
