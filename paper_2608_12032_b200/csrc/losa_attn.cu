@@ -1,9 +1,9 @@
 // Attention kernels of liblosa for sm_100a: dense attention, block-sparse attention over a
 // frozen CSR pattern (Eq. 4), the exact block-mass pass (Eq. 1) and the fused construction step.
-// Head dimension 64, and head dimension 128 with 128-row query blocks, run in losa_tile_kernel
-// (losa_attn_tile.cuh, included below): one query tile and three S buffers per CTA.
-// losa_attn_kernel, described here, is one warp-specialised persistent kernel template with two thread
-// layouts; it serves head dimension 128 with 64-row query blocks and the fallback launch of all.
+// They run in losa_tile_kernel (losa_attn_tile.cuh, included below): one query tile and three S buffers per CTA,
+// on pairs of CTAs at head dimension 128.  losa_attn_kernel, described here, is one warp-specialised persistent
+// kernel template with two thread layouts; it serves the fallback launch of all, and head dimension 128 on a
+// device (or partition of one) that cannot hold a pair of CTAs.
 //
 // Warps 0-3 are utility warps: warp 0 is the TMA producer, which streams the query tiles and the
 // K / V tiles named by the tile list into 128B-swizzled shared-memory rings (a K/V tile is 128
@@ -12,7 +12,7 @@
 // read from TMEM (bf16, written over S) and V from shared memory as the MN-major operand; warp 3
 // publishes the tile list every other warp follows (sparse mode: streamed from lists that
 // build_tile_lists_kernel made before the launch).  The softmax warps follow: four warpgroups with
-// two threads per query row (the main launch of every mode), or two warpgroups, one 128-row query
+// two threads per query row (a main launch), or two warpgroups, one 128-row query
 // tile each and one thread per query row (the fallback launch); they take their registers from the
 // utility warpgroup.
 //
@@ -2056,12 +2056,14 @@ int launch_t(const Geometry& g, const void* q, const void* k, const void* v, Par
   if ((rc = make_maps(&maps, g, q, k, C::kHasV ? v : nullptr)) != LOSA_OK) return rc;
   const CUtensorMap &mq = maps.map_q, &mk = maps.map_k, &mv = maps.map_v;
   int ctas = min(sms, kMaxPersistentCtas);
-  // Which kernel.  The tile kernel (losa_attn_tile.cuh): head dimension 128 with 128-row query blocks on
-  // pairs of CTAs, head dimension 64 on single CTAs.  (The mass pass alone gained least from pairs as
-  // long as every warp walked the tile lists: 32-key blocks 5.65 -> 5.16 ms at the Wan shape, with 64-
-  // and 128-key blocks nothing; without the lists 4.35 -> 3.78 ms and 4.06 -> 3.94 ms.)  Everything
-  // else, the fallback launch of all, and a device that cannot hold a pair: losa_attn_kernel.
-  constexpr bool kPairMode = LOSA_USE_PAIR && D == 128 && R == 128;
+  // Which kernel.  The tile kernel (losa_attn_tile.cuh): head dimension 128 on pairs of CTAs, head
+  // dimension 64 on single CTAs.  (The mass pass alone gained least from pairs as long as every warp
+  // walked the tile lists: 32-key blocks 5.65 -> 5.16 ms at the Wan shape, with 64- and 128-key blocks
+  // nothing; without the lists 4.35 -> 3.78 ms and 4.06 -> 3.94 ms.  64-row query blocks, 9600 tokens, 12
+  // heads, against two query tiles per CTA: dense 557 -> 487 us, sparse 457 -> 419, masses 474 -> 359,
+  // construction step 703 -> 538.)  The fallback launch of all, and a device that cannot hold a pair:
+  // losa_attn_kernel.
+  constexpr bool kPairMode = LOSA_USE_PAIR && D == 128;
   constexpr bool kTileMode = D == 64;
   bool pair = kTileMode;
   if constexpr (kPairMode) {
@@ -2176,7 +2178,7 @@ void arm_stalled_launch(uint32_t polls) { g_stall_polls.store(polls); }
 // work items are spread (which of them the last wave cuts into parts).
 int attn_work_slots(AttnMode mode, const Geometry& g, int sms) {
   const int ctas = sms < kMaxPersistentCtas ? sms : kMaxPersistentCtas;
-  const bool pair = LOSA_USE_PAIR && g.D == 128 && g.R == 128 && sms >= 2;
+  const bool pair = LOSA_USE_PAIR && g.D == 128 && sms >= 2;
   return (pair || g.D == 64) ? (ctas > 1 ? ctas / 2 : 1) : ctas;
 }
 

@@ -5,7 +5,7 @@
 // Each CTA's tensor memory holds one O and THREE S buffers used in turn, so that the chain
 // S -> softmax -> O += P V of one key tile overlaps the chains of the next two.
 //
-// Head dimension 128 with 128-row query blocks (PAIR): a work item is a pair of consecutive query
+// Head dimension 128 (PAIR): a work item is a pair of consecutive query
 // tiles, run by a PAIR of CTAs (a cluster of two, one SM each) that own one of the two tiles each and
 // multiply together: every MMA is a tcgen05.mma.cta_group::2 over 256 rows (128 per CTA), issued by one
 // thread of the first CTA, whose B operand is split between the two CTAs' shared memories - for
@@ -172,7 +172,7 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
                  const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_kw,
                  const __grid_constant__ CUtensorMap map_vw, const Params p) {
   using L = Lay<true>;
-  static_assert(PAIR ? (D == 128 && R == 128) : D == 64, "pairs at head dimension 128, one CTA at 64");
+  static_assert(PAIR ? D == 128 : D == 64, "pairs at head dimension 128, one CTA at 64");
   constexpr int kQB = 128 / R;  // query blocks of the query tile
   constexpr int kC = C_, kG = 128 / C_, kW = 128;
   constexpr int kQBytes = 128 * D * 2;

@@ -148,3 +148,8 @@ def test_batched_call_replays_from_a_graph(L):
 def test_layers_of_head_dimension_64_equal_the_single_calls_bit_for_bit(R, C):
     """74 items: whole work units, alone and three layers at once, on a GPU with 148 SMs."""
     test_three_layers_in_one_launch_equal_the_single_calls_bit_for_bit(1, 37, 128 * 4 - 9, 64, R, C)
+
+
+def test_layers_of_64_row_query_blocks_on_pairs_equal_the_single_calls_bit_for_bit():
+    """74 items: whole work units on the pairs of CTAs of a GPU with 148 SMs."""
+    test_three_layers_in_one_launch_equal_the_single_calls_bit_for_bit(1, 37, 128 * 4 - 9, 128, 64, 64)

@@ -225,3 +225,20 @@ def test_rows_far_below_a_borrowed_reference():
     for h in range(H):
         err = (o[0, h].cpu() - torch.from_numpy(ref[0, h])).norm() / np.linalg.norm(ref[0, h])
         assert err <= 4e-3, (nats[h], err)  # bf16 weights: 2^-9 each, at random
+
+
+@pytest.mark.parametrize("H", [1, 2])
+@pytest.mark.parametrize("kind", ["disjoint_singletons", "late_only_tile", "odd_position_first", "interleaved", "random"])
+def test_crafted_patterns_of_64_row_query_blocks_on_pairs(kind, H):
+    """Head dimension 128 with 64-row query blocks: four query blocks to a pair of CTAs, each of which meets its
+    first listed tile at a place of its own, or past the first chunk of the list; whole items and cut ones."""
+    losa = lib()
+    Rq, N = 64, 128 * 41 - 37
+    nb = -(-N // Rq)
+    off, idx = csr_from([row for h in range(H) for row in patterns(nb, nb, kind, 47 + h)])
+    q, k, v = (util.rand_bf16((1, H, N, D), 1010 + i, 1.0 if i == 2 else 2.0) for i in range(3))
+    o = losa.losa_sparse_attn(q.cuda(), k.cuda(), v.cuda(), torch.from_numpy(off).cuda(),
+                              torch.from_numpy(idx).cuda(), Rq, Rq, out_dtype=torch.float32)
+    assert losa.losa_async_status() == 0
+    ref = orc.blocks_to_tokens(orc.sparse_attn(util.to_np(q), util.to_np(k), util.to_np(v), Rq, Rq, off, idx), 1, H, N)
+    util.assert_output_close(o, ref, f"{kind} H={H}")
