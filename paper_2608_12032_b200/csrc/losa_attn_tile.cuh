@@ -37,6 +37,12 @@
 
 constexpr int kTileNK = 4, kTileNV = 7;      // K and V stages of 16 KB per CTA
 constexpr int kTileStage = 16384;
+// Head dimension 64: one K step (16 keys) of 64 more columns of V, all ones, behind the V stages.  Every
+// O += P V reads 16 of these columns, so that the row sums of P come out of it as columns of O: 64 x 80
+// instead of 64 x 64 per K step on the tensor cores, which are idle half of the time, and 96 warp instructions per 64
+// scores fewer on the softmax warps (64 adds and the moves that they need, of 405).  At head dimension 128 tensor
+// memory has no columns left.
+constexpr int kTileOnes = 2048;
 #ifndef LOSA_POLY_OF
 #define LOSA_POLY_OF 8
 #endif
@@ -181,7 +187,8 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   constexpr int kKCopies = kKRows / kKBox;            // ... and copies per 64-column slab
   constexpr int kSlabs = D / 64;                      // slabs of a K tile
   constexpr uint32_t kIdescQK = ptx::idesc_bf16_f32(PAIR ? 256 : 128, 128, false, false);
-  constexpr uint32_t kIdescPV = ptx::idesc_bf16_f32(PAIR ? 256 : 128, D, false, true);
+  constexpr uint32_t kIdescPV =
+      ptx::idesc_bf16_f32(PAIR ? 256 : 128, (D == 64 && MODE != kMass) ? D + 16 : D, false, true);
   // Head dimension 64: a key tile needs 1024 cycles of the special-function unit against 512 of the
   // tensor cores, so one group of four scores in every kPolyOf takes its exponentials from a
   // polynomial on the FMA pipe.  17776 tokens, 8 heads: dense 735 us with one in 8, 742 in 16, 763 in 6,
@@ -190,6 +197,13 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   // without (against 64 bits its masses err by 1 % more with it than without, 2e-7).
   constexpr int kPolyOf = (MODE == kMass) ? LOSA_POLY_OF_MASS : (D == 64) ? LOSA_POLY_OF : 0;
   using Ctl = TileControl;
+  // The row sums of P come out of O += P V (see kTileOnes).  The second 32 of a thread's scores are then
+  // fetched while the first are worked on, and P is stored 32 scores at a time: without the sums' chains the
+  // compiler spread the exponentials so far that it spilled.  17776 tokens, 48 heads, against sums in the softmax
+  // warps: dense 4757 us, 4727 with the sums as columns, 4512 with the late fetch, 4470 with the early store as well;
+  // sparse (coverage 0.85) 4510, 4247, 4187, 4157.  A share of 1 in 8 for the polynomial stays the best one (dense
+  // 4531 us without, 4543 in 16, 4564 in 7, 4788 in 4).
+  constexpr bool kSumCol = (D == 64 && MODE != kMass);
   constexpr bool kWantMass = (MODE == kFused || MODE == kMass);  // the block masses (Eq. 1) are wanted
   // the mass pass alone has no V, no P and no O: its score buffers go back as soon as they are read
   constexpr bool kHasV = (MODE != kMass);
@@ -200,7 +214,8 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   uint8_t* const sQ = smem_raw;
   uint8_t* const sK = sQ + kQBytes;
   uint8_t* const sV = sK + kTileNK * kTileStage;
-  Ctl* const ctl = reinterpret_cast<Ctl*>(sV + kTileNV * kTileStage);
+  uint8_t* const sOnes = sV + kTileNV * kTileStage;
+  Ctl* const ctl = reinterpret_cast<Ctl*>(sOnes + (D == 64 ? kTileOnes : 0));
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = PAIR ? ptx::cluster_ctarank() : 0u;  // 0: the CTA that issues the MMAs; also the query tile
@@ -265,6 +280,10 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     ptx::mbar_init(&ctl->drain, 2);
     ctl->abort_flag = 0;
     ptx::fence_barrier_init();
+  }
+  if (kSumCol && threadIdx.x < kTileOnes / 16) {
+    reinterpret_cast<uint4*>(sOnes)[threadIdx.x] = make_uint4(0x3f803f80u, 0x3f803f80u, 0x3f803f80u, 0x3f803f80u);
+    ptx::fence_proxy_async();
   }
   if (warp == kIssuerWarp) {
     // (one warp of each CTA of the pair)
@@ -478,7 +497,10 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       // ------------------------------------------------------------------ O += P V of the pair
       const bool leader = ptx::elect_one();
       constexpr uint32_t kDescHi = ptx::smem_desc_hi_sw128(1024);
-      const uint32_t v_lo = ptx::smem_desc_lo(ptx::smem_u32(sV), kTileStage);
+      // (without pairs of CTAs a product's columns from 64 on, which lie a leading byte offset behind its
+      // first key's row, are the ones: the offset shrinks as the row advances)
+      const uint32_t v_lo = ptx::smem_desc_lo(ptx::smem_u32(sV), kSumCol ? kTileNV * kTileStage : kTileStage);
+      auto v_desc = [&](uint32_t bytes) { return v_lo + (bytes >> 4) - (kSumCol ? (bytes >> 4) << 16 : 0u); };
       const uint32_t tO = tmem_base + 384;
       uint32_t nof = 0, nt = 0, nu = 0, ent, word;
       for (;;) {
@@ -494,7 +516,7 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           ptx::tc_fence_after_sync();
           if (leader) {
             const uint32_t tP = tmem_base + bsel * 128;
-            const uint32_t vd0 = v_lo + vs * (kTileStage >> 4);
+            const uint32_t vd0 = v_desc(vs * kTileStage);
             // (each half of a row packs its P over the head of its own 64 score columns)
 #pragma unroll
             for (int kk = 0; kk < kW / 16; ++kk)
@@ -502,7 +524,8 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
                 ptx::mma2_ts_lo(tO, tP + (kk & 3) * 8 + (kk >> 2) * 64, vd0 + kk * (2048 >> 4), kDescHi, kIdescPV,
                                 (kk > 0 || pv_item > 0) ? 1u : 0u);
               else
-                ptx::mma_ts_lo(tO, tP + (kk & 3) * 8 + (kk >> 2) * 64, vd0 + kk * (2048 >> 4), kDescHi, kIdescPV,
+                ptx::mma_ts_lo(tO, tP + (kk & 3) * 8 + (kk >> 2) * 64,
+                               vd0 + kk * (kSumCol ? (2048u >> 4) - (2048u << 12) : 2048u >> 4), kDescHi, kIdescPV,
                                (kk > 0 || pv_item > 0) ? 1u : 0u);
             commit0<PAIR>(&ctl->pv_done[bsel]);
             commit_all<PAIR>(&ctl->v_empty[vs]);
@@ -746,10 +769,9 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         if (mine) {
           ptx::tmem_ld32(tS, &sr[0]);
           ptx::tmem_wait_ld();
-          ptx::tmem_ld32(tS + 32, &sr[32]);
-          if (ragged) {
-            // keys that do not exist (>= N, in the sequence's last key block): -inf column by column
-            ptx::tmem_wait_ld();
+          if (!kSumCol) ptx::tmem_ld32(tS + 32, &sr[32]);
+          // keys that do not exist (>= N, in the sequence's last key block): -inf column by column
+          auto cut_ragged = [&](int from, int to) {
             int hv[kHB];
 #pragma unroll
             for (int j = 0; j < kHB; ++j) {
@@ -758,7 +780,11 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
             }
 #pragma unroll
             for (int c = 0; c < 64; ++c)
-              if ((c % kBW) >= hv[c / kBW]) sr[c] = 0xff800000u;
+              if (c >= from && c < to && (c % kBW) >= hv[c / kBW]) sr[c] = 0xff800000u;
+          };
+          if (ragged) {
+            if (!kSumCol) ptx::tmem_wait_ld();
+            cut_ragged(0, kSumCol ? 32 : 64);
           }
           if (!kHasV) {
             // mass pass: the scores are in registers and nothing is packed over them
@@ -784,7 +810,12 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           for (int j = 0; j < kHB; ++j) eacc[j] = make_float2(0.f, 0.f);
 #pragma unroll
           for (int c = 0; c < 64; c += 4) {
-            if (kHasV && c == 32) ptx::tmem_wait_ld();
+            if (kSumCol && c == 24) ptx::tmem_ld32(tS + 32, &sr[32]);
+            if (kSumCol && c == 32) ptx::tmem_st16(tS, &sr[0]);
+            if (kHasV && c == 32) {
+              ptx::tmem_wait_ld();
+              if (kSumCol && ragged) cut_ragged(32, 64);
+            }
             float2 x0 = ptx::fma2(make_float2(__uint_as_float(sr[c]), __uint_as_float(sr[c + 1])), sc2,
                                   nm2[c / kBW]);
             float2 x1 = ptx::fma2(make_float2(__uint_as_float(sr[c + 2]), __uint_as_float(sr[c + 3])), sc2,
@@ -803,8 +834,10 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
               const uint32_t u0 = ptx::pack_bf16x2(x0.x, x0.y), u1 = ptx::pack_bf16x2(x1.x, x1.y);
               sr[c >> 1] = u0;
               sr[(c >> 1) + 1] = u1;
-              ptx::add_bf16x2(racc[0], u0);
-              ptx::add_bf16x2(racc[1], u1);
+              if (!kSumCol) {
+                ptx::add_bf16x2(racc[0], u0);
+                ptx::add_bf16x2(racc[1], u1);
+              }
             }
             if (kWantMass) eacc[c / kBW] = ptx::add2(eacc[c / kBW], ptx::add2(x0, x1));
           }
@@ -813,9 +846,12 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
 #pragma unroll
             for (int j = 0; j < kHB; ++j) tsum += eacc[j].x + eacc[j].y;
           }
-          ovf = ovf || __any_sync(0xffffffffu, !(tsum <= kSplitSafeSum));
-          l += tsum;
-          if (kHasV) ptx::tmem_st32(tS, &sr[0]);
+          if (!kSumCol) {
+            ovf = ovf || __any_sync(0xffffffffu, !(tsum <= kSplitSafeSum));
+            l += tsum;
+          }
+          if (kSumCol) ptx::tmem_st16(tS + 16, &sr[16]);
+          else if (kHasV) ptx::tmem_st32(tS, &sr[0]);
           if (kWantMass) {
 #pragma unroll
             for (int j = 0; j < kHB; ++j) {
@@ -870,36 +906,31 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
 #undef TILE_REF_TAKE
       // the four partial sums of a row (two groups, two halves) meet in shared memory
       float* const xset = &ctl->xch[nitem & 1][0][0];
-      xset[quarter * 128 + row] = l;
+      if (!kSumCol) xset[quarter * 128 + row] = l;
       if (kWantMass) xset[(4 + quarter) * 128 + row] = le;
       auto hand_over = [&]() {
         list_outgrown_unit(p, partial ? p.split_first + (w - p.split_first) * p.split_parts + part : w);
       };
-      if (ovf && lane == 0) hand_over();
-      __syncwarp();
-      if (lane == 0) ptx::mbar_arrive(&ctl->item_bar);
-      LOSA_WAIT(&ctl->item_bar, nitem & 1);
-      ++nitem;
-      l = (xset[row] + xset[128 + row]) + (xset[256 + row] + xset[384 + row]);
-      // rows whose own keys lie 40 nats below a reference taken over other keys: their weights may have
-      // lost their tail
-      if (kQB > 1 && __any_sync(0xffffffffu, seen && l < kTileSafeLow) && lane == 0) hand_over();
+      if (!kSumCol && ovf && lane == 0) hand_over();
+      if (!kSumCol || kWantMass) {
+        __syncwarp();
+        if (lane == 0) ptx::mbar_arrive(&ctl->item_bar);
+        LOSA_WAIT(&ctl->item_bar, nitem & 1);
+        ++nitem;
+      }
+      if (!kSumCol) l = (xset[row] + xset[128 + row]) + (xset[256 + row] + xset[384 + row]);
+      // every thread writes out a quarter of its row of O
+      constexpr int kOC = kHasV ? D / 4 : 1;
+      const int c0 = quarter * kOC;
+      uint32_t r[kOC];
       if (kHasV) {
-        // every thread writes out a quarter of its row of O
-        const bool valid = (T < p.nQt) && grow < p.N;
-        const float inv = (l > 0.f) ? 1.f / l : 0.f;
-        const int64_t off = (int64_t)b * p.sb + (int64_t)h * p.sh + (int64_t)grow * p.sn;
-        const int64_t pslot = ((((int64_t)(w - p.split_first) * p.split_parts + part) * 2 + tile) * 128 + row);
-        if (partial && quarter == 0 && T < p.nQt && LOSA_IN_RANGE(pslot, p.cap_part_rows)) p.part_ml[pslot] = make_float2(m_ref, l);
-        constexpr int kOC = D / 4;
-        const int c0 = quarter * kOC;
-        uint32_t r[kOC];
         if (pv_item > 0) {
           LOSA_WAIT(&ctl->o_done, nod & 1);
           ++nod;
           ptx::tc_fence_after_sync();
           if constexpr (kOC == 32) ptx::tmem_ld32(tO + c0, r);
-          else ptx::tmem_ld16(tO + c0, r);
+          else if constexpr (kOC == 16) ptx::tmem_ld16(tO + c0, r);
+          if (kSumCol) l = __uint_as_float(ptx::tmem_ld1(tO + D));
           ptx::tmem_wait_ld();
           // (O is in registers: the next item's first product may overwrite it)
           ptx::tc_fence_before_sync();
@@ -909,6 +940,18 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
 #pragma unroll
           for (int c = 0; c < kOC; ++c) r[c] = 0u;
         }
+      }
+      // rows whose own keys lie 40 nats below a reference taken over other keys: their weights may have
+      // lost their tail
+      const bool low = kQB > 1 && seen && l < kTileSafeLow;
+      if ((kQB > 1 || kSumCol) && __any_sync(0xffffffffu, low || (kSumCol && !(l <= kSplitSafeSum))) && lane == 0)
+        hand_over();
+      if (kHasV) {
+        const bool valid = (T < p.nQt) && grow < p.N;
+        const float inv = (l > 0.f) ? 1.f / l : 0.f;
+        const int64_t off = (int64_t)b * p.sb + (int64_t)h * p.sh + (int64_t)grow * p.sn;
+        const int64_t pslot = ((((int64_t)(w - p.split_first) * p.split_parts + part) * 2 + tile) * 128 + row);
+        if (partial && quarter == 0 && T < p.nQt && LOSA_IN_RANGE(pslot, p.cap_part_rows)) p.part_ml[pslot] = make_float2(m_ref, l);
         if (partial) {
           if (T < p.nQt) {
             float4* dst = reinterpret_cast<float4*>(p.part_o + (LOSA_IN_RANGE(pslot, p.cap_part_rows) ? pslot : 0) * D + c0);
