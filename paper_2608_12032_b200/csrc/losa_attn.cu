@@ -35,10 +35,12 @@
 // LOSA_ERR_TIMEOUT, and all roles leave through the common teardown that frees TMEM.
 #include <cuda.h>
 #include <cuda_bf16.h>
+#include <limits.h>
 #include <math.h>
 
 #include <atomic>
 #include <cstddef>
+#include <type_traits>
 
 #include "losa_common.cuh"
 #include "losa_ptx.cuh"
@@ -88,7 +90,7 @@ constexpr int kCounters = 3;
 constexpr size_t kRowstatBytes = (size_t)kMaxPersistentCtas * 2 * 128 * sizeof(float2);
 constexpr size_t kPartMlBytes = kRowstatBytes;  // same shape: [slot][2][128] float2
 constexpr int kTlChunks = 4;
-constexpr uint32_t kTlItem = 1u << 28, kTlEnd = 2u << 28;  // entry type in bits 31:28 (0 = tile)
+constexpr uint32_t kTlItem = 1u << 28, kTlEnd = 2u << 28, kTlSkip = 3u << 28;  // entry type in bits 31:28 (0 = tile)
 // An item header carries the work item in bits 23:0 and, for a unit that covers only part of the
 // item's key range, the part index in bits 26:24 and a flag in bit 27.
 constexpr uint32_t kTlItemMask = 0x00ffffffu, kTlPartial = 1u << 27;
@@ -100,7 +102,7 @@ constexpr uint32_t kTlRagged = 1u << 20;  // tile entry: the sequence ends insid
 // What is said of a unit's tile list: how many K/V tiles, which query tiles list any (kHdrHas << query
 // tile), and whether query tile 1 lists its first in the second K/V tile
 // (a unit that is one query tile: bit kHdrHas alone, and which of the item's two it is, kHdrOdd)
-constexpr uint32_t kHdrTiles = 0x0fffffffu, kHdrOdd = 1u << 28, kHdrLate = 1u << 29, kHdrHas = 1u << 30;
+constexpr uint32_t kHdrTiles = 0x00ffffffu, kHdrMax = 1u << 26, kHdrRedo = 1u << 27, kHdrOdd = 1u << 28, kHdrLate = 1u << 29, kHdrHas = 1u << 30;
 // Tile lists per work unit: one for its pair of query tiles, or (head dimension 64, where a CTA works on
 // one query tile at a time) one for each.
 __host__ __device__ constexpr int tile_lists_per_unit(int D) { return D == 64 ? 2 : 1; }
@@ -194,7 +196,12 @@ struct Params {
   // list it, so that the list never holds more than nUnits entries.
   int* redo_count;
   int* redo_list;
-  int* redo_flag;  // [nUnits], and a word per split item (merge_redone_rows)
+  int* redo_flag;  // [nUnits]
+  int* redo_word;  // [split items] (merge_redone_rows)
+  // Tile kernel, no more work units than it has slots: each slot takes the one at its position, and needs
+  // nothing prepared for it (counters, flags, tile lists), which saves a launch: the CTAs make their unit's
+  // tile list themselves, and each list's flag says whether its unit was recomputed.
+  int one_wave;
   // extents of the buffers the kernels index into (elements), for the checked build
   long long cap_part_rows, cap_table_floats, cap_mass, cap_lse, cap_units;
   uint32_t wait_polls;  // bound of every device-side wait, in polls (ptx::kWaitPolls)
@@ -414,7 +421,7 @@ __device__ __forceinline__ void merge_redone_rows(const Params& p, int r, int qt
   __syncwarp();
   uint32_t done = 0u;  // of these rows, parts recomputed before this one: a nibble of the item's word
   const int nibble = 4 * (qt * 4 + warp_rows);
-  if (lane == 0) done = (atomicAdd(reinterpret_cast<uint32_t*>(p.redo_flag) + p.nUnits + r, 1u << nibble) >> nibble) & 15u;
+  if (lane == 0) done = (atomicAdd(reinterpret_cast<uint32_t*>(p.redo_word) + r, 1u << nibble) >> nibble) & 15u;
   done = __shfl_sync(0xffffffffu, done, 0);
   if ((int)done + 1 != redone) return;
   __threadfence();
@@ -471,6 +478,195 @@ __device__ __forceinline__ void merge_redone_rows(const Params& p, int r, int qt
 __device__ __forceinline__ void list_outgrown_unit(const Params& p, int unit) {
   if (LOSA_IN_RANGE(unit, p.nUnits) && atomicExch(p.redo_flag + unit, 1) == 0)
     p.redo_list[atomicAdd(p.redo_count, 1)] = unit;
+}
+
+// Sparse mode, before the attention kernel: one warp per work unit merges the index lists of the
+// unit's query blocks into its tile list (entry = key block index | membership bits << 16,
+// padded to whole K/V tiles of G entries; for the order see below).  Every list becomes a bitmap in shared
+// memory (coalesced reads, one atomicOr per index), the union's set bits are enumerated 32 words
+// at a time with a warp scan.  Doing this ahead of the launch keeps the in-kernel scheduler warp,
+// which shares a scheduler partition with two softmax warps and is favoured over them, nearly
+// idle.  A unit that is a part of an item takes the same share, by position, of every list, so
+// each (query block, key block) pair belongs to exactly one part.  Indices out of range are
+// reported and skipped; an unsorted list still gives a valid tile list.
+//
+// One warp per list fills its bitmap (a list of a small layer is nothing but the latency of its two
+// dependent loads), then the first warp writes the tile list.  The first CTA also zeroes the
+// launch's counters, and every CTA its unit's flag.
+// ONE: a list is that of one query tile of the unit (its NB query blocks), in ascending order.
+
+// A list's unit as (item, part of it).
+__device__ __forceinline__ void unit_item(const Params& p, int unit, int& w, int& part, int& parts) {
+  w = unit;
+  part = 0;
+  parts = 1;
+  if (unit >= p.split_first) {
+    const int r = unit - p.split_first;
+    parts = p.split_parts;
+    part = r % parts;
+    w = p.split_first + r / parts;
+  }
+}
+
+// Bitmap of the n-th query block of a list (whole warp).
+template <int NB, bool ONE>
+__device__ __forceinline__ void fill_tile_bitmap(const Params& p, int list, int n, int lane, uint32_t* bm) {
+  const int bit0 = ONE ? (list & 1) * NB : 0;  // membership bit of the first query block
+  int w, part, parts;
+  unit_item(p, ONE ? list >> 1 : list, w, part, parts);
+  const int pbh = w / p.nPairs, pr = w % p.nPairs;
+  const int bh = pbh % (p.B * p.H);
+  const int32_t* offsets = p.offsets;
+  const int32_t* kv_idx = p.kv_idx;
+  if (p.problems != nullptr) {
+    const ProblemEntry* pe = p.problems + pbh / (p.B * p.H);
+    offsets = pe->offsets;
+    kv_idx = pe->kv_idx;
+  }
+  const int W = (p.nKb + 31) >> 5;
+  uint32_t* const mine = bm + n * W;
+  const int g = pr * (ONE ? 2 * NB : NB) + bit0 + n;
+  int b = 0, e = 0;
+  if (g < p.nQb) {
+    const int64_t row = (int64_t)bh * p.nQb + g;
+    const int32_t nnz = __ldg(offsets + (int64_t)p.B * p.H * p.nQb);
+    b = __ldg(offsets + row);
+    e = __ldg(offsets + row + 1);
+    if (b < 0 || e < b || e > nnz || e - b > p.nKb) {
+      report_error(p.status, LOSA_ERR_BAD_INDEX);
+      b = e = 0;
+    }
+  }
+  for (int i = lane; i < W; i += 32) mine[i] = 0u;
+  __syncwarp();
+  {
+    const int b2 = b + (int)(((int64_t)(e - b) * part) / parts);
+    const int e2 = b + (int)(((int64_t)(e - b) * (part + 1)) / parts);
+#pragma unroll 4
+    for (int i = b2 + lane; i < e2; i += 32) {
+      const int v = __ldg(kv_idx + i);
+      if ((unsigned)v < (unsigned)p.nKb) atomicOr(&mine[v >> 5], 1u << (v & 31));
+      else report_error(p.status, LOSA_ERR_BAD_INDEX);  // skipped, never used as an address
+    }
+  }
+}
+
+// The tile list from its query blocks' bitmaps (whole warp).
+template <int NB, int G, bool ONE>
+__device__ __forceinline__ void emit_tile_list(const Params& p, int list, int lane, const uint32_t* bm) {
+  const int W = (p.nKb + 31) >> 5;
+  const int bit0 = ONE ? (list & 1) * NB : 0;
+  // Order of the entries.  A key block that only ONE of the unit's two query tiles lists is
+  // processed by that tile alone, at half the CTA's rate; two such blocks, one of each tile, can
+  // be in flight at the same time (the tiles' chains are independent).  So the list holds first
+  // the blocks both tiles list, then the single-tile blocks of tile 0 and tile 1 in alternation
+  // (K/V tile by K/V tile; a class that does not fill its last K/V tile pads it), then what is
+  // left of the longer class.  Within a class the blocks ascend.  Correctness does not depend on
+  // the order of the key blocks.
+  uint32_t* dst = p.tl_entries + (int64_t)list * p.tl_cap;
+  int nb = 0, na = 0, nbb = 0;  // both, tile 0 only, tile 1 only
+  for (int w0 = 0; w0 < W; w0 += 32) {
+    const int wi = w0 + lane;
+    uint32_t ta = 0, tb = 0;
+#pragma unroll
+    for (int n = 0; n < NB; ++n) {
+      const uint32_t m = (wi < W) ? bm[n * W + wi] : 0u;
+      if (ONE) ta |= m, tb |= m;
+      else if (n < NB / 2) ta |= m;
+      else tb |= m;
+    }
+    nb += __popc(ta & tb);
+    na += __popc(ta & ~tb);
+    nbb += __popc(tb & ~ta);
+  }
+#pragma unroll
+  for (int d = 16; d > 0; d >>= 1) {
+    nb += __shfl_xor_sync(0xffffffffu, nb, d);
+    na += __shfl_xor_sync(0xffffffffu, na, d);
+    nbb += __shfl_xor_sync(0xffffffffu, nbb, d);
+  }
+  const int s1 = (nb + G - 1) / G * G;                       // entries of the first section
+  const int tA = (na + G - 1) / G, tB = (nbb + G - 1) / G;   // K/V tiles of the single-tile classes
+  const int tmin = min(tA, tB);
+  const int total = min(s1 + (tA + tB) * G, p.tl_cap);
+  // padding: the ends of the last K/V tile of each class
+  auto slot_of = [&](int k, int r) {  // position of entry r of class k (1: tile 0 only, 2: tile 1 only)
+    const int t = r / G;
+    return s1 + ((t < tmin) ? 2 * t + (k - 1) : 2 * tmin + (t - tmin)) * G + r % G;
+  };
+  if (lane < G) {
+    if (nb + lane < s1 && nb + lane < total) dst[nb + lane] = kTlPad;
+    if (na + lane < tA * G && slot_of(1, na + lane) < total) dst[slot_of(1, na + lane)] = kTlPad;
+    if (nbb + lane < tB * G && slot_of(2, nbb + lane) < total) dst[slot_of(2, nbb + lane)] = kTlPad;
+  }
+  const int ragged = (p.N % p.C != 0) ? p.nKb - 1 : -1;  // the key block in which the sequence ends
+  int rb = 0, ra = 0, rbb = 0;  // entries of each class emitted by earlier windows
+  for (int w0 = 0; w0 < W; w0 += 32) {
+    const int wi = w0 + lane;
+    uint32_t m[NB], ta = 0, tb = 0;
+#pragma unroll
+    for (int n = 0; n < NB; ++n) {
+      m[n] = (wi < W) ? bm[n * W + wi] : 0u;
+      if (ONE) ta |= m[n], tb |= m[n];
+      else if (n < NB / 2) ta |= m[n];
+      else tb |= m[n];
+    }
+    uint32_t cls[3] = {ta & tb, ta & ~tb, tb & ~ta};
+    int incl[3], tot[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      incl[k] = __popc(cls[k]);
+#pragma unroll
+      for (int d = 1; d < 32; d <<= 1) {
+        const int t = __shfl_up_sync(0xffffffffu, incl[k], d);
+        if (lane >= d) incl[k] += t;
+      }
+      tot[k] = __shfl_sync(0xffffffffu, incl[k], 31);
+    }
+    const int base[3] = {rb, ra, rbb};
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      uint32_t u = cls[k];
+      int r = base[k] + incl[k] - __popc(u);  // rank of this lane's first entry within its class
+      while (u) {
+        const int bit = __ffs(u) - 1;
+        u &= u - 1;
+        uint32_t memb = 0;
+#pragma unroll
+        for (int n = 0; n < NB; ++n) memb |= ((m[n] >> bit) & 1u) << (bit0 + n);
+        const int pos = (k == 0) ? r : slot_of(k, r);
+        const int j = wi * 32 + bit;
+        if (pos < p.tl_cap) dst[pos] = (uint32_t)j | (memb << 16) | (j == ragged ? kTlRagged : 0u);
+        ++r;
+      }
+    }
+    rb += tot[0];
+    ra += tot[1];
+    rbb += tot[2];
+  }
+  if (lane == 0)
+    p.tl_count[list] = (int32_t)((uint32_t)(total / G) | ((nb + na > 0) ? kHdrHas : 0u) |
+                                 ((nb + nbb > 0) ? 2u * kHdrHas : 0u) | ((nb == 0 && tmin > 0) ? kHdrLate : 0u));
+}
+
+template <int NB, int G, bool ONE>
+__global__ void __launch_bounds__(32 * NB) build_tile_lists_kernel(const Params p) {
+  extern __shared__ uint32_t bm[];  // [NB][W] bitmaps
+  ptx::grid_launch_dependents();
+  ptx::grid_dependency_wait();
+  const int lane = threadIdx.x & 31, n = threadIdx.x >> 5;
+  const int list = blockIdx.x, unit = ONE ? list >> 1 : list;
+  if (list == 0 && threadIdx.x < kCounters) p.work_counter[threadIdx.x] = 0;
+  fill_tile_bitmap<NB, ONE>(p, list, n, lane, bm);
+  __syncthreads();
+  if (n != 0) return;
+  emit_tile_list<NB, G, ONE>(p, list, lane, bm);
+  if (lane == 0) {
+    int w, part, parts;
+    unit_item(p, unit, w, part, parts);
+    p.redo_flag[unit] = 0;
+    if (parts > 1 && part == 0) p.redo_word[w - p.split_first] = 0;
+  }
 }
 
 // Tensor maps of a batched launch were written to the workspace by a kernel, over those of an earlier call.
@@ -1708,169 +1904,6 @@ teardown:
 #undef LOSA_WAIT_RELAXED
 #undef LOSA_WAIT
 
-// Sparse mode, before the attention kernel: one warp per work unit merges the index lists of the
-// unit's query blocks into its tile list (entry = key block index | membership bits << 16,
-// padded to whole K/V tiles of G entries; for the order see below).  Every list becomes a bitmap in shared
-// memory (coalesced reads, one atomicOr per index), the union's set bits are enumerated 32 words
-// at a time with a warp scan.  Doing this ahead of the launch keeps the in-kernel scheduler warp,
-// which shares a scheduler partition with two softmax warps and is favoured over them, nearly
-// idle.  A unit that is a part of an item takes the same share, by position, of every list, so
-// each (query block, key block) pair belongs to exactly one part.  Indices out of range are
-// reported and skipped; an unsorted list still gives a valid tile list.
-//
-// One warp per list fills its bitmap (a list of a small layer is nothing but the latency of its two
-// dependent loads), then the first warp writes the tile list.  The first CTA also zeroes the
-// launch's counters, and every CTA its unit's flag.
-// ONE: a list is that of one query tile of the unit (its NB query blocks), in ascending order.
-template <int NB, int G, bool ONE>
-__global__ void __launch_bounds__(32 * NB) build_tile_lists_kernel(const Params p) {
-  extern __shared__ uint32_t bm[];  // [NB][W] bitmaps
-  ptx::grid_launch_dependents();
-  ptx::grid_dependency_wait();  // (batched launch: the table of the problems)
-  const int lane = threadIdx.x & 31, n = threadIdx.x >> 5;
-  const int list = blockIdx.x, unit = ONE ? list >> 1 : list;
-  const int bit0 = ONE ? (list & 1) * NB : 0;  // membership bit of the first query block
-  if (list == 0 && threadIdx.x < kCounters) p.work_counter[threadIdx.x] = 0;
-  int w = unit, part = 0, parts = 1;
-  if (unit >= p.split_first) {
-    const int r = unit - p.split_first;
-    parts = p.split_parts;
-    part = r % parts;
-    w = p.split_first + r / parts;
-  }
-  const int pbh = w / p.nPairs, pr = w % p.nPairs;
-  const int bh = pbh % (p.B * p.H);
-  const int32_t* offsets = p.offsets;
-  const int32_t* kv_idx = p.kv_idx;
-  if (p.problems != nullptr) {
-    const ProblemEntry* pe = p.problems + pbh / (p.B * p.H);
-    offsets = pe->offsets;
-    kv_idx = pe->kv_idx;
-  }
-  const int W = (p.nKb + 31) >> 5;
-  uint32_t* const mine = bm + n * W;
-  const int g = pr * (ONE ? 2 * NB : NB) + bit0 + n;
-  int b = 0, e = 0;
-  if (g < p.nQb) {
-    const int64_t row = (int64_t)bh * p.nQb + g;
-    const int32_t nnz = __ldg(offsets + (int64_t)p.B * p.H * p.nQb);
-    b = __ldg(offsets + row);
-    e = __ldg(offsets + row + 1);
-    if (b < 0 || e < b || e > nnz || e - b > p.nKb) {
-      report_error(p.status, LOSA_ERR_BAD_INDEX);
-      b = e = 0;
-    }
-  }
-  for (int i = lane; i < W; i += 32) mine[i] = 0u;
-  __syncwarp();
-  {
-    const int b2 = b + (int)(((int64_t)(e - b) * part) / parts);
-    const int e2 = b + (int)(((int64_t)(e - b) * (part + 1)) / parts);
-#pragma unroll 4
-    for (int i = b2 + lane; i < e2; i += 32) {
-      const int v = __ldg(kv_idx + i);
-      if ((unsigned)v < (unsigned)p.nKb) atomicOr(&mine[v >> 5], 1u << (v & 31));
-      else report_error(p.status, LOSA_ERR_BAD_INDEX);  // skipped, never used as an address
-    }
-  }
-  __syncthreads();
-  if (n != 0) return;
-  // Order of the entries.  A key block that only ONE of the unit's two query tiles lists is
-  // processed by that tile alone, at half the CTA's rate; two such blocks, one of each tile, can
-  // be in flight at the same time (the tiles' chains are independent).  So the list holds first
-  // the blocks both tiles list, then the single-tile blocks of tile 0 and tile 1 in alternation
-  // (K/V tile by K/V tile; a class that does not fill its last K/V tile pads it), then what is
-  // left of the longer class.  Within a class the blocks ascend.  Correctness does not depend on
-  // the order of the key blocks.
-  uint32_t* dst = p.tl_entries + (int64_t)list * p.tl_cap;
-  int nb = 0, na = 0, nbb = 0;  // both, tile 0 only, tile 1 only
-  for (int w0 = 0; w0 < W; w0 += 32) {
-    const int wi = w0 + lane;
-    uint32_t ta = 0, tb = 0;
-#pragma unroll
-    for (int n = 0; n < NB; ++n) {
-      const uint32_t m = (wi < W) ? bm[n * W + wi] : 0u;
-      if (ONE) ta |= m, tb |= m;
-      else if (n < NB / 2) ta |= m;
-      else tb |= m;
-    }
-    nb += __popc(ta & tb);
-    na += __popc(ta & ~tb);
-    nbb += __popc(tb & ~ta);
-  }
-#pragma unroll
-  for (int d = 16; d > 0; d >>= 1) {
-    nb += __shfl_xor_sync(0xffffffffu, nb, d);
-    na += __shfl_xor_sync(0xffffffffu, na, d);
-    nbb += __shfl_xor_sync(0xffffffffu, nbb, d);
-  }
-  const int s1 = (nb + G - 1) / G * G;                       // entries of the first section
-  const int tA = (na + G - 1) / G, tB = (nbb + G - 1) / G;   // K/V tiles of the single-tile classes
-  const int tmin = min(tA, tB);
-  const int total = min(s1 + (tA + tB) * G, p.tl_cap);
-  // padding: the ends of the last K/V tile of each class
-  auto slot_of = [&](int k, int r) {  // position of entry r of class k (1: tile 0 only, 2: tile 1 only)
-    const int t = r / G;
-    return s1 + ((t < tmin) ? 2 * t + (k - 1) : 2 * tmin + (t - tmin)) * G + r % G;
-  };
-  if (lane < G) {
-    if (nb + lane < s1 && nb + lane < total) dst[nb + lane] = kTlPad;
-    if (na + lane < tA * G && slot_of(1, na + lane) < total) dst[slot_of(1, na + lane)] = kTlPad;
-    if (nbb + lane < tB * G && slot_of(2, nbb + lane) < total) dst[slot_of(2, nbb + lane)] = kTlPad;
-  }
-  const int ragged = (p.N % p.C != 0) ? p.nKb - 1 : -1;  // the key block in which the sequence ends
-  int rb = 0, ra = 0, rbb = 0;  // entries of each class emitted by earlier windows
-  for (int w0 = 0; w0 < W; w0 += 32) {
-    const int wi = w0 + lane;
-    uint32_t m[NB], ta = 0, tb = 0;
-#pragma unroll
-    for (int n = 0; n < NB; ++n) {
-      m[n] = (wi < W) ? bm[n * W + wi] : 0u;
-      if (ONE) ta |= m[n], tb |= m[n];
-      else if (n < NB / 2) ta |= m[n];
-      else tb |= m[n];
-    }
-    uint32_t cls[3] = {ta & tb, ta & ~tb, tb & ~ta};
-    int incl[3], tot[3];
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      incl[k] = __popc(cls[k]);
-#pragma unroll
-      for (int d = 1; d < 32; d <<= 1) {
-        const int t = __shfl_up_sync(0xffffffffu, incl[k], d);
-        if (lane >= d) incl[k] += t;
-      }
-      tot[k] = __shfl_sync(0xffffffffu, incl[k], 31);
-    }
-    const int base[3] = {rb, ra, rbb};
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      uint32_t u = cls[k];
-      int r = base[k] + incl[k] - __popc(u);  // rank of this lane's first entry within its class
-      while (u) {
-        const int bit = __ffs(u) - 1;
-        u &= u - 1;
-        uint32_t memb = 0;
-#pragma unroll
-        for (int n = 0; n < NB; ++n) memb |= ((m[n] >> bit) & 1u) << (bit0 + n);
-        const int pos = (k == 0) ? r : slot_of(k, r);
-        const int j = wi * 32 + bit;
-        if (pos < p.tl_cap) dst[pos] = (uint32_t)j | (memb << 16) | (j == ragged ? kTlRagged : 0u);
-        ++r;
-      }
-    }
-    rb += tot[0];
-    ra += tot[1];
-    rbb += tot[2];
-  }
-  if (lane == 0) {
-    p.tl_count[list] = (int32_t)((uint32_t)(total / G) | ((nb + na > 0) ? kHdrHas : 0u) |
-                                 ((nb + nbb > 0) ? 2u * kHdrHas : 0u) | ((nb == 0 && tmin > 0) ? kHdrLate : 0u));
-    p.redo_flag[unit] = 0;
-    if (parts > 1 && part == 0) p.redo_flag[p.nUnits + w - p.split_first] = 0;
-  }
-}
-
 // ---------------------------------------------------------------------------- host side
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*,
@@ -1933,15 +1966,35 @@ int make_maps(ProblemEntry* e, const Geometry& g, const void* q, const void* k, 
   return LOSA_OK;
 }
 
+// The merge of the partial units as a launch of its own, behind the tile kernel.
+constexpr int kMergeThreads = 128;
+template <int D>
+__global__ void __launch_bounds__(kMergeThreads) merge_parts_kernel(const Params p) {
+  ptx::grid_dependency_wait();
+  merge_parts<D, false>(p, blockIdx.x, gridDim.x);
+  if (p.one_wave && blockIdx.x == 0 && threadIdx.x < 32) {
+    // (how many units were recomputed: elsewhere the tile kernel counts them)
+    constexpr int kLists = tile_lists_per_unit(D);
+    int n = 0;
+    for (int u = threadIdx.x; u < p.nUnits; u += 32)
+      n += (p.redo_flag[u * kLists] | p.redo_flag[u * kLists + kLists - 1]) != 0 ? 1 : 0;
+    n = __reduce_add_sync(0xffffffffu, n);
+    if (threadIdx.x == 0) *p.redo_count = n;
+  }
+}
+
 // Zeroes the counters and the units' flags of a launch that no other kernel precedes (a kernel and
 // not a memset, so that the attention kernel can be launched as its dependent: 3 us of that kernel's
 // set-up overlap).
 constexpr int kInitThreads = 256;
-__global__ void __launch_bounds__(kInitThreads) init_counters_kernel(int* counters, int* flags, int n) {
+__global__ void __launch_bounds__(kInitThreads) init_counters_kernel(int* counters, int* flags, int* words, int n, int n_words) {
   ptx::grid_launch_dependents();
+  ptx::grid_dependency_wait();  // (the stream's call before may still use the workspace)
   if (blockIdx.x == 0 && threadIdx.x < kCounters) counters[threadIdx.x] = 0;
   for (int64_t i = (int64_t)blockIdx.x * kInitThreads + threadIdx.x; i < n; i += (int64_t)gridDim.x * kInitThreads)
     flags[i] = 0;
+  if (blockIdx.x == 0)
+    for (int i = threadIdx.x; i < n_words; i += kInitThreads) words[i] = 0;
 }
 
 // Part of a batched launch's table, carried in the kernel's parameters: the call reads its host
@@ -1953,6 +2006,7 @@ struct ProblemChunk {
 __global__ void __launch_bounds__(256)
 write_problems_kernel(const __grid_constant__ ProblemChunk chunk, ProblemEntry* table, int n) {
   ptx::grid_launch_dependents();
+  ptx::grid_dependency_wait();
   const uint4* src = reinterpret_cast<const uint4*>(&chunk);
   uint4* dst = reinterpret_cast<uint4*>(table);
   for (int i = threadIdx.x; i < n * (int)(sizeof(ProblemEntry) / sizeof(uint4)); i += blockDim.x) dst[i] = src[i];
@@ -2096,38 +2150,49 @@ int launch_t(const Geometry& g, const void* q, const void* k, const void* v, Par
     }
   }
   const int grid = min(ctas, prm.nUnits);
+  prm.one_wave = (pair && prm.nUnits <= ctas) ? 1 : 0;
+  if (prm.one_wave) prm.redo_flag = prm.redo_list;  // (no list; a flag per tile list)
+  prm.redo_word = prm.redo_flag + prm.nUnits;
   // Every kernel after the first is launched as a dependent of the one before.
-  if (MODE == kSparse) {
+  if (prm.one_wave) {
+    rc = LOSA_OK;
+  } else if (MODE == kSparse) {
     const size_t bm_bytes = (size_t)C::kNB * ((prm.nKb + 31) / 32) * sizeof(uint32_t);  // <= 32 KB
     constexpr bool kOne = tile_lists_per_unit(D) == 2;
     constexpr int kBlocks = kOne ? C::kNB / 2 : C::kNB;  // query blocks of a list
     rc = launch(build_tile_lists_kernel<kBlocks, C::kG, kOne>, dim3(prm.nUnits * tile_lists_per_unit(D)), 32 * kBlocks,
-                bm_bytes, st, prm.nProb > 1, prm);
+                bm_bytes, st, true, prm);
   } else {
     rc = launch(init_counters_kernel, dim3(min(ctas, (prm.nUnits + 4 * kInitThreads - 1) / (4 * kInitThreads))),
-                kInitThreads, 0, st, false, prm.work_counter, prm.redo_flag,
-                prm.nUnits + prm.nWork - prm.split_first);
+                kInitThreads, 0, st, true, prm.work_counter, prm.redo_flag, prm.redo_word,
+                prm.nUnits, prm.nWork - prm.split_first);
   }
   if (rc != LOSA_OK) return rc;
-  // All modes run with two threads per query row and a reference that never moves; the units whose
-  // scores outgrew it (none, on ordinary inputs) are listed, and a second launch of the
-  // one-thread-per-row kernel recomputes them with a moving reference and merges the partial units.
-  if constexpr (kTileMode) {
-    rc = launch_tile<D, R, C_, MODE, false>(mq, mk, mv, maps.map_k128, maps.map_v128, prm,
-                                            min(2 * ctas, 2 * prm.nUnits), st, nullptr);
-  } else {
-    if constexpr (kPairMode) {
-      if (pair) rc = launch_tile<D, R, C_, MODE, true>(mq, maps.map_kh, mv, maps.map_k64, maps.map_v128, prm, grid, st, nullptr);
+  if constexpr (kTileMode || kPairMode) {
+    if (pair) {
+      if constexpr (kTileMode)
+        rc = launch_tile<D, R, C_, MODE, false>(mq, mk, mv, maps.map_k128, maps.map_v128, prm,
+                                                min(2 * ctas, 2 * prm.nUnits), st, nullptr);
+      else
+        rc = launch_tile<D, R, C_, MODE, true>(mq, maps.map_kh, mv, maps.map_k64, maps.map_v128, prm, grid, st, nullptr);
+      if (rc != LOSA_OK || prm.stall || prm.split_parts == 1) return rc;
+      constexpr int kRows = kMergeThreads / 32;  // a warp per row
+      return launch(merge_parts_kernel<D>, dim3((prm.nWork - prm.split_first) * (256 / kRows)), kMergeThreads, 0, st, true, prm);
     }
-    if (!pair) rc = launch_kernel<D, R, C_, MODE, KT, true>(mq, mk, mv, maps.map_k128, maps.map_v128, prm, grid, st);
   }
-  if (rc != LOSA_OK) return rc;
-  if (prm.stall) return LOSA_OK;
-  prm.work_counter += 2;  // the second launch's own counter
-  // (as many CTAs as SMs, whichever kernel ran first, where there is something to merge)
-  const int rgrid = min(sms, kMaxPersistentCtas);
-  return launch_kernel<D, R, C_, MODE, KT, false>(mq, mk, mv, maps.map_k128, maps.map_v128, prm,
-                                                  prm.split_parts > 1 ? rgrid : min(rgrid, prm.nUnits), st);
+  if constexpr (!kTileMode) {
+    // Two threads per query row and a reference that never moves; the units whose scores outgrew it (none,
+    // on ordinary inputs) are listed, and a second launch of the one-thread-per-row kernel recomputes them
+    // with a moving reference and merges the partial units.
+    rc = launch_kernel<D, R, C_, MODE, KT, true>(mq, mk, mv, maps.map_k128, maps.map_v128, prm, grid, st);
+    if (rc != LOSA_OK || prm.stall) return rc;
+    prm.work_counter += 2;  // the second launch's own counter
+    // (as many CTAs as SMs, whichever kernel ran first, where there is something to merge)
+    const int rgrid = min(sms, kMaxPersistentCtas);
+    return launch_kernel<D, R, C_, MODE, KT, false>(mq, mk, mv, maps.map_k128, maps.map_v128, prm,
+                                                    prm.split_parts > 1 ? rgrid : min(rgrid, prm.nUnits), st);
+  }
+  return LOSA_ERR_UNSUPPORTED;
 }
 
 template <int MODE>
@@ -2259,7 +2324,7 @@ int launch_attn(AttnMode mode, const Geometry& g, const void* q, const void* k, 
           chunk.e[i].offsets = l.offsets;
           chunk.e[i].kv_idx = l.kv_idx;
         }
-        const int rc = launch(write_problems_kernel, dim3(1), 256, 0, st, false, chunk,
+        const int rc = launch(write_problems_kernel, dim3(1), 256, 0, st, true, chunk,
                               reinterpret_cast<ProblemEntry*>(tab) + i0, n);
         if (rc != LOSA_OK) return rc;
       }

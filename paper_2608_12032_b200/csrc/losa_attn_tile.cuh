@@ -66,6 +66,9 @@ struct TileControl {
   uint64_t drain;
   uint2 hdr[2];
   alignas(16) uint32_t tl[kTlChunks * 32];  // (read in groups of up to four entries with one vector load)
+  uint32_t redo_mark[4];   // per unit (of four in turn): 1 + the tile list of one that outgrew its reference
+  uint32_t redo_queue[4];  // the scheduler's: tile lists of units to be run again
+  float redo_ref[128];     // the rows' maxima, of a unit that is run again
   float ref[2][128];       // the rows' reference, from the group that met the first tile to the other
   float xch[2][8][128];    // the rows' partial sums at the end of an item (two sets, used in turn):
                            // four of the rounded weights, four of the unrounded exponentials (fused step)
@@ -232,6 +235,7 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   const uint32_t v_full0 = at0(&ctl->v_full[0]);
   const uint32_t p_ready0 = at0(&ctl->p_ready[0]);
   const uint32_t o_free0 = at0(&ctl->o_free);
+  const uint32_t redo_mark0 = at0(&ctl->redo_mark[0]);
   const uint32_t tl_empty0 = at0(&ctl->tl_empty[0]);
   const uint32_t tl_full1 = at1(&ctl->tl_full[0]);
   const uint32_t hdr_empty0 = at0(&ctl->hdr_empty[0]);
@@ -278,6 +282,7 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     ptx::mbar_init(&ctl->item_bar, 16);
     ptx::mbar_init(&ctl->fold_bar, 16);
     ptx::mbar_init(&ctl->drain, 2);
+    for (int i = 0; i < 4; ++i) ctl->redo_mark[i] = 0u;
     ctl->abort_flag = 0;
     ptx::fence_barrier_init();
   }
@@ -323,6 +328,19 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   __syncthreads();
   // (the tile lists and the counters come from the kernel before; everything up to here overlaps it)
   ptx::grid_dependency_wait();
+  if (MODE == kSparse && p.one_wave) {
+    // ... or the tile list of this CTA's unit from here
+    constexpr bool kOne = tile_lists_per_unit(D) == 2;
+    constexpr int kNB = (kOne ? 1 : 2) * kQB;  // query blocks of a list
+    const int list = (int)(PAIR ? blockIdx.x >> 1 : blockIdx.x);
+    uint32_t* const bm = reinterpret_cast<uint32_t*>(&ctl->xch[0][0][0]);  // (not in use yet)
+    if (rank == 0 && warp < kNB) fill_tile_bitmap<kNB, kOne>(p, list, warp, lane, bm);
+    __syncthreads();
+    if (rank == 0 && warp == kSchedulerWarp) {
+      emit_tile_list<kNB, kG, kOne>(p, list, lane, bm);
+      __syncwarp();
+    }
+  }
 
   if (warp < 4) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(L::kRegsUtility));
@@ -333,6 +351,10 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       int problem = -1;  // batched launch: whose tensor maps this warp has acquired
       for (;;) {
         TILE_HDR_NEXT(ent, word);
+        if (ent == kTlSkip) {
+          if (rank == 0 && lane == 0) ptx::mbar_arrive(&ctl->hdr_next);
+          continue;
+        }
         if ((ent >> 28) != 1) break;
         const int w = (int)(ent & kTlItemMask);
         const int pbh = w / p.nPairs, pr = w % p.nPairs;
@@ -414,7 +436,7 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
                         h, b);
           }
           ++nk;
-          if (!kHasV) continue;
+          if (!kHasV || (word & kHdrMax)) continue;
           // V: all 128 keys of the tile, (a pair: of each CTA) 64 of the head-dimension columns, one slab
           const uint32_t vs = nv % kTileNV;
           LOSA_WAIT_RELAXED(&ctl->v_empty[vs], ((nv / kTileNV) & 1) ^ 1);
@@ -454,6 +476,7 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       uint32_t nq = 0, nt = 0, nu = 0, ent, word;
       for (;;) {
         TILE_HDR_NEXT(ent, word);
+        if (ent == kTlSkip) continue;
         if ((ent >> 28) != 1) break;
         bool q_ready = false;
         for (int i = (int)(word & kHdrTiles); i > 0; --i) {
@@ -502,14 +525,23 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       const uint32_t v_lo = ptx::smem_desc_lo(ptx::smem_u32(sV), kSumCol ? kTileNV * kTileStage : kTileStage);
       auto v_desc = [&](uint32_t bytes) { return v_lo + (bytes >> 4) - (kSumCol ? (bytes >> 4) << 16 : 0u); };
       const uint32_t tO = tmem_base + 384;
-      uint32_t nof = 0, nt = 0, nu = 0, ent, word;
+      uint32_t nof = 0, nt = 0, nv = 0, nu = 0, ent, word;
       for (;;) {
         TILE_HDR_NEXT(ent, word);
+        if (ent == kTlSkip) continue;
         if ((ent >> 28) != 1) break;
+        if (kHasV && (word & kHdrMax)) {
+          // (no P and no products: the score buffers go back as soon as they are read)
+          for (int i = (int)(word & kHdrTiles); i > 0; --i, ++nt) {
+            LOSA_WAIT(&ctl->p_ready[nt % 3u], (nt / 3u) & 1);
+            if (leader) commit0<PAIR>(&ctl->pv_done[nt % 3u]);
+          }
+          continue;
+        }
         uint32_t pv_item = 0;
         for (int i = kHasV ? (int)(word & kHdrTiles) : 0; i > 0; --i) {  // (the mass pass has no products)
-          const uint32_t vs = nt % kTileNV;
-          LOSA_WAIT(&ctl->v_full[vs], (nt / kTileNV) & 1);
+          const uint32_t vs = nv % kTileNV;
+          LOSA_WAIT(&ctl->v_full[vs], (nv / kTileNV) & 1);
           const uint32_t bsel = nt % 3u;
           if (pv_item == 0 && nof > 0) LOSA_WAIT(&ctl->o_free, (nof - 1) & 1);
           LOSA_WAIT(&ctl->p_ready[bsel], (nt / 3u) & 1);
@@ -532,6 +564,7 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           }
           ++pv_item;
           ++nt;
+          ++nv;
         }
         if (pv_item > 0) {
           if (leader) commit_all<PAIR>(&ctl->o_done);  // every product of the item is done
@@ -540,22 +573,66 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       }
     } else if (warp == kSchedulerWarp && rank == 0) {
       // ------------------------------------------------------------------ scheduler of the pair
-      uint32_t nu = 0, nc = 0;
-      bool first_item = true;
+      // A unit that outgrew its reference is run again: once for its rows' maxima (kHdrMax), once against
+      // these (kHdrRedo).  Every warp marks it before it takes the next header but one, and header nu goes out
+      // when all have taken header nu - 2: the mark of unit nu - 3 is final then.  Before the end come two
+      // headers without work, for the marks of the last two units.
+      uint32_t nu = 0, nc = 0, q_head = 0, q_tail = 0;
+      int again = -1, idle = 0;  // the list whose maxima were taken last
+      bool first_item = true, drawn = false;
+      bool redone = false;
       for (;;) {
         if (p.stall) break;  // diagnostic launch: nothing is published and every wait runs out
-        // a first unit by position, then from the counter; without pairs of CTAs a unit's two query
-        // tiles are drawn one by one
-        int w = (int)(PAIR ? blockIdx.x >> 1 : blockIdx.x);
-        if (!first_item) {
-          if (lane == 0) w = (int)(PAIR ? gridDim.x >> 1 : gridDim.x) + atomicAdd(p.work_counter, 1);
-          w = __shfl_sync(0xffffffffu, w, 0);
+        LOSA_WAIT_RELAXED(&ctl->hdr_empty[nu & 1u], ((nu >> 1) & 1u) ^ 1u);
+        if (PAIR) ptx::fence_acq_rel_cluster();
+        if (nu >= 3u) {
+          const uint32_t mark = *reinterpret_cast<volatile uint32_t*>(&ctl->redo_mark[(nu - 3u) & 3u]);
+          if (mark != 0u) {
+            if (lane == 0) ctl->redo_queue[q_tail & 3u] = mark - 1u;
+            __syncwarp();
+            ++q_tail;
+          }
         }
-        first_item = false;
+        if (lane == 0) ctl->redo_mark[nu & 3u] = 0u;
+        int w = 0;
+        uint32_t mode = 0u;
+        if (again >= 0) {
+          w = again;
+          mode = kHdrRedo;
+          again = -1;
+        } else if (q_head != q_tail) {
+          w = (int)*reinterpret_cast<volatile uint32_t*>(&ctl->redo_queue[q_head & 3u]);
+          ++q_head;
+          mode = kHdrMax;
+          again = w;
+          redone = true;
+        } else if (!drawn) {
+          // a first unit by position, then from the counter; without pairs of CTAs a unit's two query
+          // tiles are drawn one by one
+          w = (int)(PAIR ? blockIdx.x >> 1 : blockIdx.x);
+          if (!first_item) {
+            if (p.one_wave) {
+              w = INT_MAX;
+            } else {
+              if (lane == 0) w = (int)(PAIR ? gridDim.x >> 1 : gridDim.x) + atomicAdd(p.work_counter, 1);
+              w = __shfl_sync(0xffffffffu, w, 0);
+            }
+          }
+          first_item = false;
+          drawn = (PAIR ? w : w >> 1) >= p.nUnits;
+        }
+        if (drawn && mode == 0u) {
+          if (idle == 2) break;
+          ++idle;
+          TILE_HDR_PUT(kTlSkip, 0u);
+          LOSA_WAIT_RELAXED(&ctl->hdr_next, (nu - 1u) & 1u);
+          continue;
+        }
+        idle = 0;
         const int list = w;  // its tile list
-        const uint32_t odd = (!PAIR && (w & 1)) ? kHdrOdd : 0u;
+        const uint32_t odd = ((!PAIR && (w & 1)) ? kHdrOdd : 0u) | mode;
         if (!PAIR) w >>= 1;
-        if (w >= p.nUnits) break;
+        if (mode == kHdrMax && !p.one_wave && lane == 0 && atomicExch(p.redo_flag + w, 1) == 0) atomicAdd(p.redo_count, 1);
         uint32_t flags = 0;
         if (w >= p.split_first) {
           const int r = w - p.split_first;
@@ -589,15 +666,16 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           tile_key_range(p, ent, jlo, jhi);
           const bool two = 2 * (w % p.nPairs) + 1 < p.nQt;  // the pair's second query tile exists
           if (PAIR) {
-            TILE_HDR_PUT(ent, (two ? 3u : 1u) * kHdrHas | (uint32_t)((jhi - jlo + kG - 1) / kG));
+            TILE_HDR_PUT(ent, mode | (two ? 3u : 1u) * kHdrHas | (uint32_t)((jhi - jlo + kG - 1) / kG));
           } else {
             // (a query tile that does not exist is a unit without tiles)
-            TILE_HDR_PUT(ent, odd | ((two || !odd) ? kHdrHas | (uint32_t)((jhi - jlo + kG - 1) / kG) : 0u));
+            TILE_HDR_PUT(ent, odd | ((two || !(odd & kHdrOdd)) ? kHdrHas | (uint32_t)((jhi - jlo + kG - 1) / kG) : 0u));
           }
         }
         LOSA_WAIT_RELAXED(&ctl->hdr_next, (nu - 1u) & 1u);
       }
       if (!p.stall) TILE_HDR_PUT(kTlEnd, 0u);
+      if (p.one_wave && lane == 0) p.redo_flag[PAIR ? blockIdx.x >> 1 : blockIdx.x] = redone ? 1 : 0;
     }
   } else {
     // ------------------------------------------------------------------ softmax warps (both CTAs)
@@ -622,7 +700,9 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
                                   : nullptr;
 
     for (;;) {
+      const uint32_t unit_no = nu;
       TILE_HDR_NEXT(ent, word);
+      if (ent == kTlSkip) continue;
       if ((ent >> 28) != 1) break;
       const int w = (int)(ent & kTlItemMask);
       const bool partial = (ent & kTlPartial) != 0;
@@ -649,6 +729,59 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       // buffer k % 3, in that buffer's use k / 3.
       const int first = (grpi ^ (int)kq) & 1;
       uint32_t bsel = (kq + (uint32_t)first) % 3u, sph = ((kq + (uint32_t)first) / 3u) & 1u;
+      if (word & kHdrMax) {
+        // ---- the rows' maxima over all keys they attend to, for a unit that is run again
+        float mx = -INFINITY;
+        for (int base = 0; base < tiles; base += kChunkTiles) {
+          if (MODE == kSparse) TILE_CHUNK_WAIT();
+          const int end = min(tiles, base + kChunkTiles);
+          for (int i = base + first; i < end; i += 2) {
+            uint32_t own[kHB];
+            if (MODE == kSparse)
+              ptx::ld_shared_volatile_vec<kHB>(
+                  &ctl->tl[(nc & (kTlChunks - 1)) * 32 + (i - base) * kG + ((kG >= 2) ? half * kHB : 0)], own);
+            LOSA_WAIT(&ctl->s_full[bsel], sph);
+            ptx::tc_fence_after_sync();
+#pragma unroll
+            for (int c0 = 0; c0 < 64; c0 += 32) {
+              uint32_t r[32];
+              ptx::tmem_ld32(tmem_base + lane_base + bsel * 128 + half * 64 + c0, r);
+              ptx::tmem_wait_ld();
+#pragma unroll
+              for (int c = 0; c < 32; ++c) {
+                const int j = (c0 + c) / kBW;
+                int valid;  // of the block's columns
+                if (MODE == kSparse)
+                  valid = ((own[j] >> (16 + my_bit)) & 1u)
+                              ? p.N - (int)(own[j] & 0xffffu) * kC - ((kG == 1) ? 64 * half : 0) : 0;
+                else
+                  valid = has ? kend - (jlo + i * kG) * kC - 64 * half - j * kBW : 0;
+                if ((c0 + c) % kBW < valid) mx = fmaxf(mx, __uint_as_float(r[c]));
+              }
+            }
+            ptx::tc_fence_before_sync();
+            __syncwarp();
+            if (lane == 0) arrive0<PAIR>(p_ready0 + 8u * bsel);
+            if (bsel == 0u) {
+              bsel = 2u;
+            } else {
+              bsel -= 1u;
+              sph ^= 1u;
+            }
+          }
+          if (MODE == kSparse) TILE_CHUNK_DONE();
+        }
+        kq += (uint32_t)tiles;
+        float* const xset = &ctl->xch[nitem & 1][0][0];
+        xset[quarter * 128 + row] = mx;
+        __syncwarp();
+        if (lane == 0) ptx::mbar_arrive(&ctl->item_bar);
+        LOSA_WAIT(&ctl->item_bar, nitem & 1);
+        ++nitem;
+        // (every thread of the row finds and leaves the same value)
+        ctl->redo_ref[row] = fmaxf(fmaxf(xset[row], xset[128 + row]), fmaxf(xset[256 + row], xset[384 + row])) * p.scale_log2;
+        continue;
+      }
       // ---- the reference of the unit: the rows' maximum over the first key tile their query block
       // lists, from the group that works on that tile to the other.  Where the query tile is a query
       // block that tile is one of the unit's first two, the first of the group that works on it, and
@@ -656,7 +789,9 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       // and is exchanged when the loop below comes to it.
       constexpr bool kLazyRef = kQB > 1 && MODE == kSparse;
       const uint32_t rs = nref & 1u;
-      bool have_ref = !has;
+      const bool redo = (word & kHdrRedo) != 0;  // against the rows' maxima
+      bool have_ref = !has || redo;
+      if (redo) m_ref = ctl->redo_ref[row];
       int ref_tile = (PAIR && tile == 1 && (word & kHdrLate)) ? 1 : 0;
       bool listed_only = true;  // the maximum is over the keys the row attends to
       auto row_max = [&](int i, uint32_t chunk, int at) {  // tile i of the unit, its group at `at` in the list
@@ -708,7 +843,7 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     __syncwarp();                                                                                   \
     if (lane == 0) ptx::mbar_arrive(&ctl->ref_empty[rs][sub]);                                      \
   } while (0)
-      if (has) {
+      if (has && !redo) {
         if (kLazyRef) {
           // a query block that lists none of the first chunk's entries takes the maximum over all keys
           // of the first tile
@@ -901,7 +1036,7 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
 
       // ---- end of the item
       if (kLazyRef && !have_ref) TILE_REF_TAKE();  // (this group met no tile from the reference's on)
-      if (has) ++nref;
+      if (has && !redo) ++nref;
 #undef TILE_REF_GIVE
 #undef TILE_REF_TAKE
       // the four partial sums of a row (two groups, two halves) meet in shared memory
@@ -909,9 +1044,16 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       if (!kSumCol) xset[quarter * 128 + row] = l;
       if (kWantMass) xset[(4 + quarter) * 128 + row] = le;
       auto hand_over = [&]() {
-        list_outgrown_unit(p, partial ? p.split_first + (w - p.split_first) * p.split_parts + part : w);
+        const int unit = partial ? p.split_first + (w - p.split_first) * p.split_parts + part : w;
+        const uint32_t mark = 1u + (uint32_t)(PAIR ? unit : 2 * unit + tile);
+        if (PAIR) {
+          ptx::st_cluster_u32(redo_mark0 + 4u * (unit_no & 3u), mark);
+          ptx::fence_acq_rel_cluster();
+        } else {
+          *reinterpret_cast<volatile uint32_t*>(&ctl->redo_mark[unit_no & 3u]) = mark;
+        }
       };
-      if (!kSumCol && ovf && lane == 0) hand_over();
+      if (!kSumCol && ovf && !redo && lane == 0) hand_over();
       if (!kSumCol || kWantMass) {
         __syncwarp();
         if (lane == 0) ptx::mbar_arrive(&ctl->item_bar);
@@ -944,11 +1086,13 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       // rows whose own keys lie 40 nats below a reference taken over other keys: their weights may have
       // lost their tail
       const bool low = kQB > 1 && seen && l < kTileSafeLow;
-      if ((kQB > 1 || kSumCol) && __any_sync(0xffffffffu, low || (kSumCol && !(l <= kSplitSafeSum))) && lane == 0)
+      if ((kQB > 1 || kSumCol) && !redo && __any_sync(0xffffffffu, low || (kSumCol && !(l <= kSplitSafeSum))) && lane == 0)
         hand_over();
+      // (against their maxima only rows that met a score that is not a number add up to that much)
+      if (redo && !(l <= kSplitSafeSum)) l = __int_as_float(0x7fc00000);
       if (kHasV) {
         const bool valid = (T < p.nQt) && grow < p.N;
-        const float inv = (l > 0.f) ? 1.f / l : 0.f;
+        const float inv = (l == 0.f) ? 0.f : 1.f / l;
         const int64_t off = (int64_t)b * p.sb + (int64_t)h * p.sh + (int64_t)grow * p.sn;
         const int64_t pslot = ((((int64_t)(w - p.split_first) * p.split_parts + part) * 2 + tile) * 128 + row);
         if (partial && quarter == 0 && T < p.nQt && LOSA_IN_RANGE(pslot, p.cap_part_rows)) p.part_ml[pslot] = make_float2(m_ref, l);
@@ -990,7 +1134,8 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         if (quarter == 0 && T < p.nQt && grow < p.N && p.lse != nullptr &&
             LOSA_IN_RANGE((int64_t)bh * p.N + grow, p.cap_lse)) {
           const float le_row = (xset[512 + row] + xset[640 + row]) + (xset[768 + row] + xset[896 + row]);
-          p.lse[(int64_t)bh * p.N + grow] = (m_ref + log2f(le_row)) * kLn2;
+          p.lse[(int64_t)bh * p.N + grow] =
+              (!redo || le_row <= kSplitSafeSum) ? (m_ref + log2f(le_row)) * kLn2 : __int_as_float(0x7fc00000);
         }
         if (T < p.nQt) {
           const float* tb = reinterpret_cast<const float*>(p.table) + (int64_t)blockIdx.x * 2 * (int64_t)p.nKb * 256;
@@ -1003,7 +1148,7 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           for (int rr = 0; rr < 4; ++rr) {
             const int r = 4 * lane + rr;
             const float le_r = (xset[512 + r] + xset[640 + r]) + (xset[768 + r] + xset[896 + r]);
-            iv[rr] = (T * 128 + r < p.N && le_r > 0.f) ? 1.f / le_r : 0.f;
+            iv[rr] = (T * 128 + r < p.N && le_r > 0.f && (!redo || le_r <= kSplitSafeSum)) ? 1.f / le_r : 0.f;
           }
           constexpr int kFold = 4, kParts = (kG >= 2) ? 1 : 2;
           for (int u0 = sw; u0 < p.nKb; u0 += 16 * kFold) {
