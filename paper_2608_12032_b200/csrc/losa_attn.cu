@@ -2051,8 +2051,8 @@ template <int D, int R, int C_, int MODE, bool PAIR>
 int launch_tile(const CUtensorMap& mq, const CUtensorMap& mkh, const CUtensorMap& mv, const CUtensorMap& mk64,
                 const CUtensorMap& mv128, const Params& prm, int clusters, cudaStream_t st, int* max_clusters) {
   using L = Lay<true>;
-  constexpr size_t smem =
-      256 * D + (size_t)(kTileNK + kTileNV) * kTileStage + (D == 64 ? kTileOnes : 0) + sizeof(TileControl);
+  constexpr size_t smem = (size_t)tile_nq(D) * 256 * D + (size_t)(kTileNK + kTileNV) * kTileStage +
+                          (D == 64 ? kTileOnes : 0) + sizeof(TileControl);
   static_assert(smem <= 227 * 1024, "shared memory of one CTA");
   auto kern = losa_tile_kernel<D, R, C_, MODE, PAIR>;
   static int max_on[kMaxDevices] = {};

@@ -35,7 +35,10 @@
 // commit to both.  Every wait is bounded; on the way out both CTAs meet at the cluster's barrier,
 // so that neither leaves while the other may still signal into its shared memory.
 
-constexpr int kTileNK = 4, kTileNV = 7;      // K and V stages of 16 KB per CTA
+constexpr int kTileNK = 4, kTileNV = 7;      // K and V stages of 16 KB per CTA (at most)
+// Query tiles in shared memory: two where there is room, so that the next unit's keys and its first scores need not
+// wait for this one's last.
+__host__ __device__ constexpr int tile_nq(int D) { return D == 64 ? 2 : 1; }
 constexpr int kTileStage = 16384;
 // Head dimension 64: one K step (16 keys) of 64 more columns of V, all ones, behind the V stages.  Every
 // O += P V reads 16 of these columns, so that the row sums of P come out of it as columns of O: 64 x 80
@@ -52,22 +55,26 @@ constexpr int kTileOnes = 2048;
 constexpr float kTileSafeLow = 8.6736173798840355e-19f;  // 2^-60
 
 struct TileControl {
-  uint64_t q_full, q_empty;
+  uint64_t q_full[2], q_empty[2];
   uint64_t k_full[kTileNK], k_empty[kTileNK];
   uint64_t v_full[kTileNV], v_empty[kTileNV];
   uint64_t s_full[3], p_ready[3], pv_done[3];  // per score buffer
-  uint64_t o_done, o_free;
+  uint64_t o_done[4], o_free;
   uint64_t hdr_full[2], hdr_empty[2], hdr_next;
   uint64_t tl_full[kTlChunks], tl_empty[kTlChunks];
   uint64_t pair_bar[8];    // per (group, lane quarter): the two halves of a row
   uint64_t ref_full[2][2], ref_empty[2][2];  // [set][query block of the query tile]
   uint64_t item_bar;       // all softmax warps of the CTA, at the end of an item
+  uint64_t l_full[4];      // the group that is done with a unit first has left its rows' partial sums
   uint64_t fold_bar;       // ... and after the fused step's masses are folded out of the table
   uint64_t drain;
   uint2 hdr[2];
   alignas(16) uint32_t tl[kTlChunks * 32];  // (read in groups of up to four entries with one vector load)
   uint32_t redo_mark[4];   // per unit (of four in turn): 1 + the tile list of one that outgrew its reference
   uint32_t redo_queue[4];  // the scheduler's: tile lists of units to be run again
+  uint8_t seen[4][16];     // a warp met keys that its rows attend to
+  uint8_t max_uses[16];    // a warp's uses of item_bar, where only units that are run again use it
+  float redo_max[2][4][128];  // ... of each of the row's threads (two sets, used in turn)
   float redo_ref[128];     // the rows' maxima, of a unit that is run again
   float ref[2][128];       // the rows' reference, from the group that met the first tile to the other
   float xch[2][8][128];    // the rows' partial sums at the end of an item (two sets, used in turn):
@@ -185,6 +192,7 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   constexpr int kQB = 128 / R;  // query blocks of the query tile
   constexpr int kC = C_, kG = 128 / C_, kW = 128;
   constexpr int kQBytes = 128 * D * 2;
+  constexpr int kNQ = tile_nq(D), kNV = kTileNV;
   constexpr int kKRows = PAIR ? 64 : 128;             // keys of a K tile that this CTA copies
   constexpr int kKBox = (C_ < kKRows) ? C_ : kKRows;  // ... per copy
   constexpr int kKCopies = kKRows / kKBox;            // ... and copies per 64-column slab
@@ -207,6 +215,8 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   // sparse (coverage 0.85) 4510, 4247, 4187, 4157.  A share of 1 in 8 for the polynomial stays the best one (dense
   // 4531 us without, 4543 in 16, 4564 in 7, 4788 in 4).
   constexpr bool kSumCol = (D == 64 && MODE != kMass);
+  // Who writes O out (and ends the unit): see the end of an item.
+  constexpr bool kOneGroup = (MODE == kDense || MODE == kSparse);
   constexpr bool kWantMass = (MODE == kFused || MODE == kMass);  // the block masses (Eq. 1) are wanted
   // the mass pass alone has no V, no P and no O: its score buffers go back as soon as they are read
   constexpr bool kHasV = (MODE != kMass);
@@ -215,9 +225,9 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
 
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* const sQ = smem_raw;
-  uint8_t* const sK = sQ + kQBytes;
+  uint8_t* const sK = sQ + kNQ * kQBytes;
   uint8_t* const sV = sK + kTileNK * kTileStage;
-  uint8_t* const sOnes = sV + kTileNV * kTileStage;
+  uint8_t* const sOnes = sV + kNV * kTileStage;
   Ctl* const ctl = reinterpret_cast<Ctl*>(sOnes + (D == 64 ? kTileOnes : 0));
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -230,7 +240,7 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   // second CTA's copy of the tile list (used by the first CTA's scheduler)
   auto at0 = [](const void* x) { return PAIR ? ptx::mapa(ptx::smem_u32(x), 0) : ptx::smem_u32(x); };
   auto at1 = [](const void* x) { return PAIR ? ptx::mapa(ptx::smem_u32(x), 1) : 0u; };
-  const uint32_t q_full0 = at0(&ctl->q_full);
+  const uint32_t q_full0 = at0(&ctl->q_full[0]);
   const uint32_t k_full0 = at0(&ctl->k_full[0]);
   const uint32_t v_full0 = at0(&ctl->v_full[0]);
   const uint32_t p_ready0 = at0(&ctl->p_ready[0]);
@@ -246,8 +256,14 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
 
   if (threadIdx.x == 0) {
     constexpr int kCtas = PAIR ? 2 : 1;
-    ptx::mbar_init(&ctl->q_full, kCtas);   // one arrival (with its byte count) per CTA's producer
-    ptx::mbar_init(&ctl->q_empty, 1);
+    for (int i = 0; i < 2; ++i) {
+      ptx::mbar_init(&ctl->q_full[i], kCtas);   // one arrival (with its byte count) per CTA's producer
+      ptx::mbar_init(&ctl->q_empty[i], 1);
+    }
+    for (int i = 0; i < 4; ++i) {
+      ptx::mbar_init(&ctl->o_done[i], 1);
+      ptx::mbar_init(&ctl->l_full[i], 8);
+    }
     for (int i = 0; i < kTileNK; ++i) {
       ptx::mbar_init(&ctl->k_full[i], kCtas);
       ptx::mbar_init(&ctl->k_empty[i], 1);
@@ -261,8 +277,8 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       ptx::mbar_init(&ctl->p_ready[i], 8 * kCtas);  // the eight warps of a group, in both CTAs
       ptx::mbar_init(&ctl->pv_done[i], 1);
     }
-    ptx::mbar_init(&ctl->o_done, 1);
-    ptx::mbar_init(&ctl->o_free, 16 * kCtas);  // every softmax warp of both CTAs reads a quarter of its rows' O
+    // every softmax warp of both CTAs reads a part of its rows' O, or every one of one group
+    ptx::mbar_init(&ctl->o_free, (kOneGroup ? 8 : 16) * kCtas);
     for (int i = 0; i < kTlChunks; ++i) {
       ptx::mbar_init(&ctl->tl_full[i], 1);
       ptx::mbar_init(&ctl->tl_empty[i], 17 * kCtas);  // readers: each CTA's producer and 16 softmax warps
@@ -283,6 +299,7 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     ptx::mbar_init(&ctl->fold_bar, 16);
     ptx::mbar_init(&ctl->drain, 2);
     for (int i = 0; i < 4; ++i) ctl->redo_mark[i] = 0u;
+    for (int i = 0; i < 16; ++i) ctl->max_uses[i] = 0;
     ctl->abort_flag = 0;
     ptx::fence_barrier_init();
   }
@@ -376,11 +393,13 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         }
         // this CTA's query tile (rows past the end of the sequence are filled with zeros)
         const int T = 2 * pr + (PAIR ? (int)rank : (int)((word & kHdrOdd) != 0u));
-        LOSA_WAIT_RELAXED(&ctl->q_empty, (nq & 1) ^ 1);
+        const uint32_t qs = nq % kNQ;
+        LOSA_WAIT_RELAXED(&ctl->q_empty[qs], ((nq / kNQ) & 1) ^ 1);
         if (lane == 0) {
-          expect0<PAIR>(q_full0, kQBytes);
+          expect0<PAIR>(q_full0 + 8u * qs, kQBytes);
 #pragma unroll
-          for (int s = 0; s < kSlabs; ++s) load0<PAIR>(sQ + s * 16384, mq, q_full0, s * 64, T * 128, h, b);
+          for (int s = 0; s < kSlabs; ++s) 
+            load0<PAIR>(sQ + qs * kQBytes + s * 16384, mq, q_full0 + 8u * qs, s * 64, T * 128, h, b);
         }
         ++nq;
         const int tiles = (int)(word & kHdrTiles);
@@ -438,8 +457,8 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           ++nk;
           if (!kHasV || (word & kHdrMax)) continue;
           // V: all 128 keys of the tile, (a pair: of each CTA) 64 of the head-dimension columns, one slab
-          const uint32_t vs = nv % kTileNV;
-          LOSA_WAIT_RELAXED(&ctl->v_empty[vs], ((nv / kTileNV) & 1) ^ 1);
+          const uint32_t vs = nv % kNV;
+          LOSA_WAIT_RELAXED(&ctl->v_empty[vs], ((nv / kNV) & 1) ^ 1);
           if (lane == 0) expect0<PAIR>(v_full0 + 8u * vs, kTileStage);
           __syncwarp();
           bool wide_v = kG > 2;
@@ -483,8 +502,7 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           const uint32_t ks = nt % kTileNK;
           LOSA_WAIT(&ctl->k_full[ks], (nt / kTileNK) & 1);
           if (!q_ready) {
-            LOSA_WAIT(&ctl->q_full, nq & 1);
-            ++nq;
+            LOSA_WAIT(&ctl->q_full[nq % kNQ], (nq / kNQ) & 1);
             q_ready = true;
           }
           const uint32_t bsel = nt % 3u;
@@ -495,14 +513,14 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           }
           ptx::tc_fence_after_sync();
           if (leader) {
-            const uint32_t kd0 = k_lo + ks * (kTileStage >> 4);
+            const uint32_t kd0 = k_lo + ks * (kTileStage >> 4), q0 = (nq % kNQ) * (kQBytes >> 4);
 #pragma unroll
             for (int kk = 0; kk < D / 16; ++kk)
               if (PAIR)
-                ptx::mma2_ss_lo(tmem_base + bsel * 128, qd[kk], kd0 + (((kk >> 2) * 8192 + (kk & 3) * 32) >> 4),
+                ptx::mma2_ss_lo(tmem_base + bsel * 128, qd[kk] + q0, kd0 + (((kk >> 2) * 8192 + (kk & 3) * 32) >> 4),
                                 kDescHi, kIdescQK, kk > 0 ? 1u : 0u);
               else
-                ptx::mma_ss_lo(tmem_base + bsel * 128, qd[kk], kd0 + (((kk & 3) * 32) >> 4), kDescHi, kIdescQK,
+                ptx::mma_ss_lo(tmem_base + bsel * 128, qd[kk] + q0, kd0 + (((kk & 3) * 32) >> 4), kDescHi, kIdescQK,
                                kk > 0 ? 1u : 0u);
             commit_all<PAIR>(&ctl->s_full[bsel]);
             commit_all<PAIR>(&ctl->k_empty[ks]);
@@ -511,10 +529,10 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         }
         if (!q_ready) {
           // a unit without key tiles: the query tiles were loaded all the same
-          LOSA_WAIT(&ctl->q_full, nq & 1);
-          ++nq;
+          LOSA_WAIT(&ctl->q_full[nq % kNQ], (nq / kNQ) & 1);
         }
-        if (leader) commit_all<PAIR>(&ctl->q_empty);
+        if (leader) commit_all<PAIR>(&ctl->q_empty[nq % kNQ]);
+        ++nq;
       }
     } else if (warp == kIssuerWarp + 1 && rank == 0) {
       // ------------------------------------------------------------------ O += P V of the pair
@@ -522,26 +540,27 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       constexpr uint32_t kDescHi = ptx::smem_desc_hi_sw128(1024);
       // (without pairs of CTAs a product's columns from 64 on, which lie a leading byte offset behind its
       // first key's row, are the ones: the offset shrinks as the row advances)
-      const uint32_t v_lo = ptx::smem_desc_lo(ptx::smem_u32(sV), kSumCol ? kTileNV * kTileStage : kTileStage);
+      const uint32_t v_lo = ptx::smem_desc_lo(ptx::smem_u32(sV), kSumCol ? kNV * kTileStage : kTileStage);
       auto v_desc = [&](uint32_t bytes) { return v_lo + (bytes >> 4) - (kSumCol ? (bytes >> 4) << 16 : 0u); };
       const uint32_t tO = tmem_base + 384;
       uint32_t nof = 0, nt = 0, nv = 0, nu = 0, ent, word;
       for (;;) {
         TILE_HDR_NEXT(ent, word);
-        if (ent == kTlSkip) continue;
-        if ((ent >> 28) != 1) break;
-        if (kHasV && (word & kHdrMax)) {
+        if ((ent >> 28) == 2) break;
+        const uint32_t od = (nu - 1u) & 3u;
+        if (ent == kTlSkip || (kHasV && (word & kHdrMax))) {
           // (no P and no products: the score buffers go back as soon as they are read)
           for (int i = (int)(word & kHdrTiles); i > 0; --i, ++nt) {
             LOSA_WAIT(&ctl->p_ready[nt % 3u], (nt / 3u) & 1);
             if (leader) commit0<PAIR>(&ctl->pv_done[nt % 3u]);
           }
+          if (leader) commit_all<PAIR>(&ctl->o_done[od]);
           continue;
         }
         uint32_t pv_item = 0;
         for (int i = kHasV ? (int)(word & kHdrTiles) : 0; i > 0; --i) {  // (the mass pass has no products)
-          const uint32_t vs = nv % kTileNV;
-          LOSA_WAIT(&ctl->v_full[vs], (nv / kTileNV) & 1);
+          const uint32_t vs = nv % kNV;
+          LOSA_WAIT(&ctl->v_full[vs], (nv / kNV) & 1);
           const uint32_t bsel = nt % 3u;
           if (pv_item == 0 && nof > 0) LOSA_WAIT(&ctl->o_free, (nof - 1) & 1);
           LOSA_WAIT(&ctl->p_ready[bsel], (nt / 3u) & 1);
@@ -566,10 +585,8 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           ++nt;
           ++nv;
         }
-        if (pv_item > 0) {
-          if (leader) commit_all<PAIR>(&ctl->o_done);  // every product of the item is done
-          ++nof;
-        }
+        if (leader) commit_all<PAIR>(&ctl->o_done[od]);  // every product of the item is done
+        if (pv_item > 0) ++nof;
       }
     } else if (warp == kSchedulerWarp && rank == 0) {
       // ------------------------------------------------------------------ scheduler of the pair
@@ -691,7 +708,8 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     constexpr int kBW = 64 / kHB;                // columns per such block
     uint64_t* const pair_bar = &ctl->pair_bar[grpi * 4 + wl];
     const int quarter = grpi * 2 + half;         // which 32 columns of O this thread writes out
-    uint32_t kq = 0, nod = 0, npair = 0, nitem = 0, nref = 0, nfold = 0, nu = 0, nc = 0, ent, word;
+    // (cnt: bit 0 the uses of pair_bar, above it the units with a reference)
+    uint32_t kq = 0, cnt = 0, nitem = 0, nfold = 0, nu = 0, nc = 0, ent, word;
     // fused step: this row's column of the CTA's table of per-block sums of the unrounded
     // exponentials (one float per row and 64-column half of a key tile when a key block fills the
     // tile, else one per row and key block)
@@ -700,10 +718,15 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
                                   : nullptr;
 
     for (;;) {
-      const uint32_t unit_no = nu;
       TILE_HDR_NEXT(ent, word);
+      if ((ent >> 28) == 2) break;
+      // Which of the groups is through with the unit first, and leaves its end to the other.
+      constexpr bool kExchange = kOneGroup && (!kSumCol || (kQB > 1 && MODE == kSparse));
+      if (kExchange && (ent == kTlSkip || (word & kHdrMax))) {
+        // (nothing to leave: keeps the phases of these barriers in step with the headers)
+        if (lane == 0 && grpi == 0) ptx::mbar_arrive(&ctl->l_full[(nu - 1u) & 3u]);
+      }
       if (ent == kTlSkip) continue;
-      if ((ent >> 28) != 1) break;
       const int w = (int)(ent & kTlItemMask);
       const bool partial = (ent & kTlPartial) != 0;
       const int part = (int)((ent >> 24) & 7u);
@@ -731,6 +754,10 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       uint32_t bsel = (kq + (uint32_t)first) % 3u, sph = ((kq + (uint32_t)first) / 3u) & 1u;
       if (word & kHdrMax) {
         // ---- the rows' maxima over all keys they attend to, for a unit that is run again
+        if (kOneGroup) {
+          nitem = ctl->max_uses[sw];
+          __syncwarp();
+        }
         float mx = -INFINITY;
         for (int base = 0; base < tiles; base += kChunkTiles) {
           if (MODE == kSparse) TILE_CHUNK_WAIT();
@@ -772,12 +799,13 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           if (MODE == kSparse) TILE_CHUNK_DONE();
         }
         kq += (uint32_t)tiles;
-        float* const xset = &ctl->xch[nitem & 1][0][0];
+        float* const xset = &ctl->redo_max[nitem & 1][0][0];
         xset[quarter * 128 + row] = mx;
+        if (kOneGroup) ctl->max_uses[sw] = (uint8_t)(nitem + 1u);
         __syncwarp();
         if (lane == 0) ptx::mbar_arrive(&ctl->item_bar);
         LOSA_WAIT(&ctl->item_bar, nitem & 1);
-        ++nitem;
+        if (!kOneGroup) ++nitem;
         // (every thread of the row finds and leaves the same value)
         ctl->redo_ref[row] = fmaxf(fmaxf(xset[row], xset[128 + row]), fmaxf(xset[256 + row], xset[384 + row])) * p.scale_log2;
         continue;
@@ -788,7 +816,7 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       // the reference is exchanged here; with two query blocks (R = 64) and a list it may be any tile
       // and is exchanged when the loop below comes to it.
       constexpr bool kLazyRef = kQB > 1 && MODE == kSparse;
-      const uint32_t rs = nref & 1u;
+      const uint32_t rs = (cnt >> 1) & 1u;
       const bool redo = (word & kHdrRedo) != 0;  // against the rows' maxima
       bool have_ref = !has || redo;
       if (redo) m_ref = ctl->redo_ref[row];
@@ -825,12 +853,12 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     ptx::tc_fence_before_sync();                                                                    \
     __syncwarp();                                                                                   \
     if (lane == 0) ptx::mbar_arrive(pair_bar);                                                      \
-    LOSA_WAIT(pair_bar, npair & 1);                                                                 \
-    ++npair;                                                                                        \
+    LOSA_WAIT(pair_bar, cnt & 1u);                                                                  \
+    cnt ^= 1u;                                                                                      \
     ptx::tc_fence_after_sync();                                                                     \
     if (half == 0) {                                                                                \
       /* (the slot's last readers, two units with a reference ago, are done with it) */             \
-      if (nref >= 2u) LOSA_WAIT(&ctl->ref_empty[rs][sub], ((nref >> 1) - 1u) & 1);                  \
+      if (cnt >= 4u) LOSA_WAIT(&ctl->ref_empty[rs][sub], ((cnt >> 2) - 1u) & 1);                    \
       ctl->ref[rs][row] = m_ref;                                                                    \
       __syncwarp();                                                                                 \
       if (lane == 0) ptx::mbar_arrive(&ctl->ref_full[rs][sub]);                                     \
@@ -838,7 +866,7 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   } while (0)
 #define TILE_REF_TAKE()                                                                             \
   do {                                                                                              \
-    LOSA_WAIT(&ctl->ref_full[rs][sub], (nref >> 1) & 1);                                            \
+    LOSA_WAIT(&ctl->ref_full[rs][sub], (cnt >> 2) & 1);                                             \
     m_ref = ctl->ref[rs][row];                                                                      \
     __syncwarp();                                                                                   \
     if (lane == 0) ptx::mbar_arrive(&ctl->ref_empty[rs][sub]);                                      \
@@ -1036,30 +1064,128 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
 
       // ---- end of the item
       if (kLazyRef && !have_ref) TILE_REF_TAKE();  // (this group met no tile from the reference's on)
-      if (has && !redo) ++nref;
+      if (has && !redo) cnt += 2u;
 #undef TILE_REF_GIVE
 #undef TILE_REF_TAKE
-      // the four partial sums of a row (two groups, two halves) meet in shared memory
-      float* const xset = &ctl->xch[nitem & 1][0][0];
-      if (!kSumCol) xset[quarter * 128 + row] = l;
-      if (kWantMass) xset[(4 + quarter) * 128 + row] = le;
       auto hand_over = [&]() {
         const int unit = partial ? p.split_first + (w - p.split_first) * p.split_parts + part : w;
         const uint32_t mark = 1u + (uint32_t)(PAIR ? unit : 2 * unit + tile);
         if (PAIR) {
-          ptx::st_cluster_u32(redo_mark0 + 4u * (unit_no & 3u), mark);
+          ptx::st_cluster_u32(redo_mark0 + 4u * ((nu - 1u) & 3u), mark);
           ptx::fence_acq_rel_cluster();
         } else {
-          *reinterpret_cast<volatile uint32_t*>(&ctl->redo_mark[unit_no & 3u]) = mark;
+          *reinterpret_cast<volatile uint32_t*>(&ctl->redo_mark[(nu - 1u) & 3u]) = mark;
         }
       };
       if (!kSumCol && ovf && !redo && lane == 0) hand_over();
-      if (!kSumCol || kWantMass) {
-        __syncwarp();
-        if (lane == 0) ptx::mbar_arrive(&ctl->item_bar);
-        LOSA_WAIT(&ctl->item_bar, nitem & 1);
-        ++nitem;
+      const int64_t off = (int64_t)b * p.sb + (int64_t)h * p.sh + (int64_t)grow * p.sn;
+      const bool valid = (T < p.nQt) && grow < p.N;
+      // 32 (or 16) columns of a row of O, from `c0` on
+      auto store_o = [&](const uint32_t* r, int c0, float inv, auto cols) {
+        constexpr int kCols = decltype(cols)::value;
+        if (p.o_f32) {
+          float4* dst = reinterpret_cast<float4*>(static_cast<float*>(o_base) + off + c0);
+#pragma unroll
+          for (int c = 0; c < kCols; c += 4)
+            dst[c >> 2] = make_float4(__uint_as_float(r[c]) * inv, __uint_as_float(r[c + 1]) * inv,
+                                      __uint_as_float(r[c + 2]) * inv, __uint_as_float(r[c + 3]) * inv);
+        } else {
+          uint4* dst = reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(o_base) + off + c0);
+#pragma unroll
+          for (int c = 0; c < kCols; c += 8) {
+            uint4 v;
+            v.x = ptx::pack_bf16x2(__uint_as_float(r[c]) * inv, __uint_as_float(r[c + 1]) * inv);
+            v.y = ptx::pack_bf16x2(__uint_as_float(r[c + 2]) * inv, __uint_as_float(r[c + 3]) * inv);
+            v.z = ptx::pack_bf16x2(__uint_as_float(r[c + 4]) * inv, __uint_as_float(r[c + 5]) * inv);
+            v.w = ptx::pack_bf16x2(__uint_as_float(r[c + 6]) * inv, __uint_as_float(r[c + 7]) * inv);
+            dst[c >> 3] = v;
+          }
+        }
+      };
+      if constexpr (kOneGroup) {
+        // The group that worked on the unit's last tile writes O out; the other, whose turn the next tile
+        // is, goes on to the next unit, so that the special-function unit has work while the last product
+        // runs and O is read.  It may be two units ahead before O is free: four sets of partial sums.
+        const uint32_t set = (nu - 1u) & 3u, phase = ((nu - 1u) >> 2) & 1u;
+        float* const xset = &ctl->xch[0][0][0] + set * 512;
+        if (!kSumCol) xset[quarter * 128 + row] = l;
+        if (kLazyRef && lane == 0) ctl->seen[set][sw] = seen ? 1 : 0;
+        const bool last = grpi == (int)((kq - 1u) & 1u);
+        if (kExchange) {
+          __syncwarp();
+          if (last) {
+            if (lane == 0) ptx::mbar_arrive(pair_bar);
+            LOSA_WAIT(pair_bar, cnt & 1u);
+            cnt ^= 1u;
+            LOSA_WAIT(&ctl->l_full[set], phase);
+          } else if (lane == 0) {
+            ptx::mbar_arrive(&ctl->l_full[set]);
+          }
+        }
+        if (!last) continue;
+        if (!kSumCol) l = (xset[row] + xset[128 + row]) + (xset[256 + row] + xset[384 + row]);
+        if (kLazyRef) {
+          const volatile uint8_t* met = ctl->seen[set];
+          seen = (met[wl] | met[4 + wl] | met[8 + wl] | met[12 + wl]) != 0;
+        }
+        constexpr int kOC = D / 2;  // columns of this half
+        float inv = 0.f;
+        const int64_t pslot = ((((int64_t)(w - p.split_first) * p.split_parts + part) * 2 + tile) * 128 + row);
+        if (pv_item > 0) {
+          LOSA_WAIT(&ctl->o_done[set], phase);
+          ptx::tc_fence_after_sync();
+        }
+#pragma unroll
+        for (int c0 = 0; c0 < kOC; c0 += 32) {
+          uint32_t r[32];
+          if (pv_item > 0) {
+            ptx::tmem_ld32(tO + half * kOC + c0, r);
+            if (kSumCol && c0 == 0) l = __uint_as_float(ptx::tmem_ld1(tO + D));
+            ptx::tmem_wait_ld();
+            if (c0 + 32 == kOC) {
+              // (O is in registers: the next item's first product may overwrite it)
+              ptx::tc_fence_before_sync();
+              __syncwarp();
+              if (lane == 0) arrive0<PAIR>(o_free0);
+            }
+          } else {
+#pragma unroll
+            for (int c = 0; c < 32; ++c) r[c] = 0u;
+          }
+          if (c0 == 0) {
+            // rows whose own keys lie 40 nats below a reference taken over other keys: their weights may
+            // have lost their tail
+            const bool low = kLazyRef && seen && l < kTileSafeLow;
+            if ((kLazyRef || kSumCol) && !redo &&
+                __any_sync(0xffffffffu, low || (kSumCol && !(l <= kSplitSafeSum))) && lane == 0)
+              hand_over();
+            // (against their maxima only rows that met a score that is not a number add up to that much)
+            if (redo && !(l <= kSplitSafeSum)) l = __int_as_float(0x7fc00000);
+            inv = (l == 0.f) ? 0.f : 1.f / l;
+            if (partial && half == 0 && T < p.nQt && LOSA_IN_RANGE(pslot, p.cap_part_rows)) p.part_ml[pslot] = make_float2(m_ref, l);
+          }
+          if (partial) {
+            if (T < p.nQt) {
+              float4* dst = reinterpret_cast<float4*>(p.part_o + (LOSA_IN_RANGE(pslot, p.cap_part_rows) ? pslot : 0) * D + half * kOC + c0);
+#pragma unroll
+              for (int c = 0; c < 32; c += 4)
+                dst[c >> 2] = make_float4(__uint_as_float(r[c]), __uint_as_float(r[c + 1]),
+                                          __uint_as_float(r[c + 2]), __uint_as_float(r[c + 3]));
+            }
+          } else if (valid) {
+            store_o(r, half * kOC + c0, inv, std::integral_constant<int, 32>());
+          }
+        }
+        continue;
       }
+      // the four partial sums of a row (two groups, two halves) meet in shared memory
+      float* const xset = &ctl->xch[nitem & 1][0][0];
+      if (!kSumCol) xset[quarter * 128 + row] = l;
+      xset[(4 + quarter) * 128 + row] = le;
+      __syncwarp();
+      if (lane == 0) ptx::mbar_arrive(&ctl->item_bar);
+      LOSA_WAIT(&ctl->item_bar, nitem & 1);
+      ++nitem;
       if (!kSumCol) l = (xset[row] + xset[128 + row]) + (xset[256 + row] + xset[384 + row]);
       // every thread writes out a quarter of its row of O
       constexpr int kOC = kHasV ? D / 4 : 1;
@@ -1067,8 +1193,7 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       uint32_t r[kOC];
       if (kHasV) {
         if (pv_item > 0) {
-          LOSA_WAIT(&ctl->o_done, nod & 1);
-          ++nod;
+          LOSA_WAIT(&ctl->o_done[(nu - 1u) & 3u], ((nu - 1u) >> 2) & 1u);
           ptx::tc_fence_after_sync();
           if constexpr (kOC == 32) ptx::tmem_ld32(tO + c0, r);
           else if constexpr (kOC == 16) ptx::tmem_ld16(tO + c0, r);
@@ -1082,48 +1207,10 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
 #pragma unroll
           for (int c = 0; c < kOC; ++c) r[c] = 0u;
         }
-      }
-      // rows whose own keys lie 40 nats below a reference taken over other keys: their weights may have
-      // lost their tail
-      const bool low = kQB > 1 && seen && l < kTileSafeLow;
-      if ((kQB > 1 || kSumCol) && !redo && __any_sync(0xffffffffu, low || (kSumCol && !(l <= kSplitSafeSum))) && lane == 0)
-        hand_over();
-      // (against their maxima only rows that met a score that is not a number add up to that much)
-      if (redo && !(l <= kSplitSafeSum)) l = __int_as_float(0x7fc00000);
-      if (kHasV) {
-        const bool valid = (T < p.nQt) && grow < p.N;
-        const float inv = (l == 0.f) ? 0.f : 1.f / l;
-        const int64_t off = (int64_t)b * p.sb + (int64_t)h * p.sh + (int64_t)grow * p.sn;
-        const int64_t pslot = ((((int64_t)(w - p.split_first) * p.split_parts + part) * 2 + tile) * 128 + row);
-        if (partial && quarter == 0 && T < p.nQt && LOSA_IN_RANGE(pslot, p.cap_part_rows)) p.part_ml[pslot] = make_float2(m_ref, l);
-        if (partial) {
-          if (T < p.nQt) {
-            float4* dst = reinterpret_cast<float4*>(p.part_o + (LOSA_IN_RANGE(pslot, p.cap_part_rows) ? pslot : 0) * D + c0);
-#pragma unroll
-            for (int c = 0; c < kOC; c += 4)
-              dst[c >> 2] = make_float4(__uint_as_float(r[c]), __uint_as_float(r[c + 1]),
-                                        __uint_as_float(r[c + 2]), __uint_as_float(r[c + 3]));
-          }
-        } else if (valid) {
-          if (p.o_f32) {
-            float4* dst = reinterpret_cast<float4*>(static_cast<float*>(o_base) + off + c0);
-#pragma unroll
-            for (int c = 0; c < kOC; c += 4)
-              dst[c >> 2] = make_float4(__uint_as_float(r[c]) * inv, __uint_as_float(r[c + 1]) * inv,
-                                        __uint_as_float(r[c + 2]) * inv, __uint_as_float(r[c + 3]) * inv);
-          } else {
-            uint4* dst = reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(o_base) + off + c0);
-#pragma unroll
-            for (int c = 0; c < kOC; c += 8) {
-              uint4 v;
-              v.x = ptx::pack_bf16x2(__uint_as_float(r[c]) * inv, __uint_as_float(r[c + 1]) * inv);
-              v.y = ptx::pack_bf16x2(__uint_as_float(r[c + 2]) * inv, __uint_as_float(r[c + 3]) * inv);
-              v.z = ptx::pack_bf16x2(__uint_as_float(r[c + 4]) * inv, __uint_as_float(r[c + 5]) * inv);
-              v.w = ptx::pack_bf16x2(__uint_as_float(r[c + 6]) * inv, __uint_as_float(r[c + 7]) * inv);
-              dst[c >> 3] = v;
-            }
-          }
-        }
+        if (kSumCol && !redo && __any_sync(0xffffffffu, !(l <= kSplitSafeSum)) && lane == 0) hand_over();
+        // (against their maxima only rows that met a score that is not a number add up to that much)
+        if (redo && !(l <= kSplitSafeSum)) l = __int_as_float(0x7fc00000);
+        if (valid) store_o(r, c0, (l == 0.f) ? 0.f : 1.f / l, std::integral_constant<int, kOC>());
       }
       if (kWantMass) {
         // ---- fused construction step: the block masses of this CTA's query tile (Eq. 1).  The
