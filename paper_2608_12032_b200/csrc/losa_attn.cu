@@ -680,6 +680,16 @@ __device__ __forceinline__ void acquire_maps(const ProblemEntry* pe) {
   ptx::tensormap_acquire(&pe->map_v128);
 }
 
+// ... those that the tile kernel uses
+template <int D, int C_, bool HAS_V>
+__device__ __forceinline__ void acquire_tile_maps(const ProblemEntry* pe) {
+  ptx::tensormap_acquire(&pe->map_q);
+  ptx::tensormap_acquire(D == 128 ? &pe->map_kh : &pe->map_k);
+  if (D == 128 ? C_ < 64 : C_ < 128) ptx::tensormap_acquire(D == 128 ? &pe->map_k64 : &pe->map_k128);
+  if (HAS_V) ptx::tensormap_acquire(&pe->map_v);
+  if (HAS_V && C_ < 128) ptx::tensormap_acquire(&pe->map_v128);
+}
+
 template <int D, int R, int C_, int MODE, int KT, bool SPLIT>
 __global__ void __launch_bounds__(Lay<SPLIT>::kThreads, 1)
 losa_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
@@ -1958,11 +1968,9 @@ int make_maps(ProblemEntry* e, const Geometry& g, const void* q, const void* k, 
   e->map_kh = e->map_k64 = e->map_k128 = e->map_k;
   e->map_v128 = e->map_v;
   if (g.C > 64 && (rc = make_map(&e->map_kh, k, g, 64)) != LOSA_OK) return rc;
-  if (g.C < 64) {
-    if ((rc = make_map(&e->map_k64, k, g, 64)) != LOSA_OK) return rc;
-    if ((rc = make_map(&e->map_k128, k, g, 128)) != LOSA_OK) return rc;
-    if (v && (rc = make_map(&e->map_v128, v, g, 128)) != LOSA_OK) return rc;
-  }
+  if (g.C < 64 && (rc = make_map(&e->map_k64, k, g, 64)) != LOSA_OK) return rc;
+  if ((g.C < 64 || (g.C < 128 && g.D == 64)) && (rc = make_map(&e->map_k128, k, g, 128)) != LOSA_OK) return rc;
+  if (g.C < 128 && v && (rc = make_map(&e->map_v128, v, g, 128)) != LOSA_OK) return rc;
   return LOSA_OK;
 }
 

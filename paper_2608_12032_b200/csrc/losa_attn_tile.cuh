@@ -76,6 +76,7 @@ struct TileControl {
   uint8_t max_uses[16];    // a warp's uses of item_bar, where only units that are run again use it
   float redo_max[2][4][128];  // ... of each of the row's threads (two sets, used in turn)
   float redo_ref[128];     // the rows' maxima, of a unit that is run again
+  float half_max[2][2][128];  // ... over each half of the tile it is taken from
   float ref[2][128];       // the rows' reference, from the group that met the first tile to the other
   float xch[2][8][128];    // the rows' partial sums at the end of an item (two sets, used in turn):
                            // four of the rounded weights, four of the unrounded exponentials (fused step)
@@ -321,7 +322,7 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     ptx::prefetch_tensormap(&map_q);
     ptx::prefetch_tensormap(&map_k);
     ptx::prefetch_tensormap(&map_v);
-    if (kG > 2) {
+    if (kG > 1) {
       ptx::prefetch_tensormap(&map_kw);
       ptx::prefetch_tensormap(&map_vw);
     }
@@ -364,12 +365,14 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     if (ctl->abort_flag) goto teardown;
     if (warp == kProducerWarp) {
       // ------------------------------------------------------------------ TMA producer (both CTAs)
-      uint32_t nq = 0, nk = 0, nv = 0, nu = 0, nc = 0, ent, word;
+      // One elected thread makes the copies: from a lane test the compiler cannot tell that there is only one.
+      const bool leader = ptx::elect_one();
+      uint32_t nq = 0, nk = 0, vs = 0, v_par = 1u, nu = 0, nc = 0, ent, word;
       int problem = -1;  // batched launch: whose tensor maps this warp has acquired
       for (;;) {
         TILE_HDR_NEXT(ent, word);
         if (ent == kTlSkip) {
-          if (rank == 0 && lane == 0) ptx::mbar_arrive(&ctl->hdr_next);
+          if (rank == 0 && leader) ptx::mbar_arrive(&ctl->hdr_next);
           continue;
         }
         if ((ent >> 28) != 1) break;
@@ -388,17 +391,17 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           mvw = &pe->map_v128;
           if (pbh / (p.B * p.H) != problem) {
             problem = pbh / (p.B * p.H);
-            acquire_maps(pe);
+            acquire_tile_maps<D, C_, kHasV>(pe);
           }
         }
         // this CTA's query tile (rows past the end of the sequence are filled with zeros)
         const int T = 2 * pr + (PAIR ? (int)rank : (int)((word & kHdrOdd) != 0u));
         const uint32_t qs = nq % kNQ;
         LOSA_WAIT_RELAXED(&ctl->q_empty[qs], ((nq / kNQ) & 1) ^ 1);
-        if (lane == 0) {
+        if (leader) {
           expect0<PAIR>(q_full0 + 8u * qs, kQBytes);
 #pragma unroll
-          for (int s = 0; s < kSlabs; ++s) 
+          for (int s = 0; s < kSlabs; ++s)
             load0<PAIR>(sQ + qs * kQBytes + s * 16384, mq, q_full0 + 8u * qs, s * 64, T * 128, h, b);
         }
         ++nq;
@@ -407,78 +410,84 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         tile_key_range(p, ent, jlo, jhi);
         // the scheduler draws the next unit when this one is 16 tiles from its end
         const int call_at = max(0, tiles - 16);
-        if (tiles == 0 && rank == 0 && lane == 0) ptx::mbar_arrive(&ctl->hdr_next);
+        if (tiles == 0 && rank == 0 && leader) ptx::mbar_arrive(&ctl->hdr_next);
         for (int base = 0; base < tiles; base += kChunkTiles) {
-        if (MODE == kSparse) TILE_CHUNK_WAIT();
-        const int end = min(tiles, base + kChunkTiles);
-        for (int i = base; i < end; ++i) {
-          if (i == call_at && rank == 0 && lane == 0) ptx::mbar_arrive(&ctl->hdr_next);
-          uint32_t grp[kG];
-          if (MODE == kSparse) {
-            ptx::ld_shared_volatile_vec<kG>(&ctl->tl[(nc & (kTlChunks - 1)) * 32 + (i - base) * kG], grp);
-          } else {
+          if (MODE == kSparse) TILE_CHUNK_WAIT();
+          const int end = min(tiles, base + kChunkTiles);
+          if (leader) {
+            bool in_time = true;
+            for (int i = base; i < end; ++i) {
+              if (i == call_at && rank == 0) ptx::mbar_arrive(&ctl->hdr_next);
+              uint32_t grp[kG];
+              if (MODE == kSparse) {
+                ptx::ld_shared_volatile_vec<kG>(&ctl->tl[(nc & (kTlChunks - 1)) * 32 + (i - base) * kG], grp);
 #pragma unroll
-            for (int g = 0; g < kG; ++g) grp[g] = (jlo + i * kG + g < jhi) ? (uint32_t)(jlo + i * kG + g) : kTlPad;
-          }
-          // K: a pair's CTAs keys 64 * rank ... + 63 of the tile each; all head-dimension columns, per slab of 64
-          const uint32_t ks = nk % kTileNK;
-          LOSA_WAIT_RELAXED(&ctl->k_empty[ks], ((nk / kTileNK) & 1) ^ 1);
-          if (lane == 0) expect0<PAIR>(k_full0 + 8u * ks, kTileStage);
-          __syncwarp();
-          // 32-key blocks: this CTA's key blocks, if consecutive, are one copy per slab
-          constexpr int kKBlocks = (kKRows / kC > 0) ? kKRows / kC : 1;  // key blocks of this CTA's rows
-          bool wide_k = kG > 2;
-          uint32_t first_k = grp[0];
-          if constexpr (kG > 2) {
-            first_k = (rank == 0) ? grp[0] : grp[kG / 2];
+                for (int g = 0; g < kG; ++g) grp[g] &= 0xffffu;
+              } else {
 #pragma unroll
-            for (int j = 1; j < kKBlocks; ++j) {
-              const uint32_t ej = (rank == 0) ? grp[j] : grp[kG / 2 + (PAIR ? j : 0)];
-              wide_k = wide_k && (ej & 0xffffu) == (first_k & 0xffffu) + j;
+                for (int g = 0; g < kG; ++g) grp[g] = (jlo + i * kG + g < jhi) ? (uint32_t)(jlo + i * kG + g) : kTlPad;
+              }
+              // K: a pair's CTAs keys 64 * rank ... + 63 of the tile each; all head-dimension columns, per slab of 64
+              const uint32_t ks = nk % kTileNK;
+              in_time = ptx::mbar_wait_relaxed(&ctl->k_empty[ks], ((nk / kTileNK) & 1) ^ 1, &ctl->abort_flag, p.wait_polls);
+              if (!in_time) break;
+              ++nk;
+              expect0<PAIR>(k_full0 + 8u * ks, kTileStage);
+              uint8_t* const k_to = sK + ks * kTileStage;
+              // several key blocks: this CTA's, if consecutive, are one copy per slab (every copy costs its thread
+              // about 70 ns, and at head dimension 64 a tile takes 550)
+              constexpr int kKBlocks = (kKRows / kC > 0) ? kKRows / kC : 1;  // key blocks of this CTA's rows
+              uint32_t mine[kKBlocks];
+              bool wide_k = kKBlocks > 1;
+#pragma unroll
+              for (int j = 0; j < kKBlocks; ++j) {
+                mine[j] = (PAIR && kG > 1 && rank == 1) ? grp[(kG / 2 + j) % kG] : grp[j];
+                if (j > 0) wide_k = wide_k && mine[j] == mine[0] + j;
+              }
+              if (wide_k) {
+#pragma unroll
+                for (int s = 0; s < kSlabs; ++s)
+                  load0<PAIR>(k_to + s * (kKRows * 128), mkw, k_full0 + 8u * ks, s * 64, (int)mine[0] * kC, h, b);
+              } else {
+#pragma unroll
+                for (int j = 0; j < kKCopies; ++j) {
+                  const int inb = (PAIR && kG == 1) ? 64 * (int)rank : 0;  // (half of a 128-key block)
+                  const int r0 = (mine[j] == kTlPad) ? p.nKb * kC : (int)mine[j] * kC + inb;
+#pragma unroll
+                  for (int s = 0; s < kSlabs; ++s)
+                    load0<PAIR>(k_to + s * (kKRows * 128) + j * kKBox * 128, mk, k_full0 + 8u * ks, s * 64, r0, h, b);
+                }
+              }
+              if (!kHasV || (word & kHdrMax)) continue;
+              // V: all 128 keys of the tile, (a pair: of each CTA) 64 of the head-dimension columns, one slab
+              in_time = ptx::mbar_wait_relaxed(&ctl->v_empty[vs], v_par, &ctl->abort_flag, p.wait_polls);
+              if (!in_time) break;
+              expect0<PAIR>(v_full0 + 8u * vs, kTileStage);
+              uint8_t* const v_to = sV + vs * kTileStage;
+              bool wide_v = kG > 1;
+#pragma unroll
+              for (int g = 1; g < kG; ++g) wide_v = wide_v && grp[g] == grp[0] + g;
+              if (wide_v) {
+                load0<PAIR>(v_to, mvw, v_full0 + 8u * vs, (int)rank * 64, (int)grp[0] * kC, h, b);
+              } else {
+#pragma unroll
+                for (int g = 0; g < kG; ++g)
+                  load0<PAIR>(v_to + g * kC * 128, mv, v_full0 + 8u * vs, (int)rank * 64,
+                              (grp[g] == kTlPad) ? p.nKb * kC : (int)grp[g] * kC, h, b);
+              }
+              if (++vs == (uint32_t)kNV) {
+                vs = 0u;
+                v_par ^= 1u;
+              }
+            }
+            if (!in_time) {
+              ctl->abort_flag = 1;
+              report_error(p.status, LOSA_ERR_TIMEOUT);
             }
           }
-          if (wide_k) {
-            if (lane < kSlabs)
-              load0<PAIR>(sK + ks * kTileStage + lane * (kKRows * 128), mkw, k_full0 + 8u * ks, lane * 64,
-                          (int)(first_k & 0xffffu) * kC, h, b);
-          } else if (lane < kSlabs * kKCopies) {
-            const int j = lane / kSlabs, s = lane % kSlabs;
-            const int keyoff = 64 * (int)rank + j * kKBox;  // within the tile
-            const int g = keyoff / kC, inb = keyoff % kC;
-            uint32_t eg = grp[0];
-#pragma unroll
-            for (int gg = 1; gg < kG; ++gg)
-              if (g == gg) eg = grp[gg];
-            const int jg = (int)(eg & 0xffffu);
-            const int r0 = (jg == (int)kTlPad) ? p.nKb * kC : jg * kC + inb;
-            load0<PAIR>(sK + ks * kTileStage + s * (kKRows * 128) + j * kKBox * 128, mk, k_full0 + 8u * ks, s * 64, r0,
-                        h, b);
-          }
-          ++nk;
-          if (!kHasV || (word & kHdrMax)) continue;
-          // V: all 128 keys of the tile, (a pair: of each CTA) 64 of the head-dimension columns, one slab
-          const uint32_t vs = nv % kNV;
-          LOSA_WAIT_RELAXED(&ctl->v_empty[vs], ((nv / kNV) & 1) ^ 1);
-          if (lane == 0) expect0<PAIR>(v_full0 + 8u * vs, kTileStage);
           __syncwarp();
-          bool wide_v = kG > 2;
-#pragma unroll
-          for (int gg = 1; gg < kG; ++gg) wide_v = wide_v && (grp[gg] & 0xffffu) == (grp[0] & 0xffffu) + gg;
-          if (wide_v) {
-            if (lane == 0)
-              load0<PAIR>(sV + vs * kTileStage, mvw, v_full0 + 8u * vs, (int)rank * 64, (int)(grp[0] & 0xffffu) * kC, h, b);
-          } else if (lane < kG) {
-            uint32_t eg = grp[0];
-#pragma unroll
-            for (int gg = 1; gg < kG; ++gg)
-              if (lane == gg) eg = grp[gg];
-            const int jg = (int)(eg & 0xffffu);
-            const int r0 = (jg == (int)kTlPad) ? p.nKb * kC : jg * kC;
-            load0<PAIR>(sV + vs * kTileStage + lane * kC * 128, mv, v_full0 + 8u * vs, (int)rank * 64, r0, h, b);
-          }
-          ++nv;
-        }
-        if (MODE == kSparse) TILE_CHUNK_DONE();
+          if (*reinterpret_cast<volatile int*>(&ctl->abort_flag)) goto teardown;
+          if (MODE == kSparse) TILE_CHUNK_DONE();
         }
       }
     } else if (warp == kIssuerWarp && rank == 0) {
@@ -822,40 +831,49 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       if (redo) m_ref = ctl->redo_ref[row];
       int ref_tile = (PAIR && tile == 1 && (word & kHdrLate)) ? 1 : 0;
       bool listed_only = true;  // the maximum is over the keys the row attends to
-      auto row_max = [&](int i, uint32_t chunk, int at) {  // tile i of the unit, its group at `at` in the list
-        const uint32_t tSrow = tmem_base + lane_base + bsel * 128;
-        uint32_t grp[kG];
-        if (MODE == kSparse) ptx::ld_shared_volatile_vec<kG>(&ctl->tl[(chunk & (kTlChunks - 1)) * 32 + at], grp);
-        float mx = -INFINITY;
+      // The maximum of this half's 64 columns of tile i of the unit, whose group lies at `at` in the list's
+      // chunk; the halves exchange theirs.  (Over all 128 columns by each half, column by column, it took a unit's
+      // first softmax group 1.1 us, for which the other group waits.)
+      auto half_max = [&](int i, uint32_t chunk, int at) {
+        const uint32_t tSh = tmem_base + lane_base + bsel * 128 + half * 64;
+        int hv[kHB];  // columns of each block that count
+        bool whole = true;
+        uint32_t e[kHB];
+        if (MODE == kSparse)
+          ptx::ld_shared_volatile_vec<kHB>(&ctl->tl[(chunk & (kTlChunks - 1)) * 32 + at + ((kG >= 2) ? half * kHB : 0)], e);
 #pragma unroll
-        for (int c0 = 0; c0 < kW; c0 += 32) {
-          uint32_t r[32];
-          ptx::tmem_ld32(tSrow + c0, r);
-          ptx::tmem_wait_ld();
-#pragma unroll
-          for (int c = 0; c < 32; ++c) {
-            const int cc = c0 + c;
-            int valid;  // of the key block's columns
-            if (MODE == kSparse)
-              valid = (!listed_only || ((grp[cc / kC] >> (16 + my_bit)) & 1u))
-                          ? p.N - (int)(grp[cc / kC] & 0xffffu) * kC : 0;
-            else
-              valid = kend - (jlo + i * kG + cc / kC) * kC;
-            if ((cc % kC) < valid) mx = fmaxf(mx, __uint_as_float(r[c]));
-          }
+        for (int j = 0; j < kHB; ++j) {
+          if (MODE == kSparse)
+            hv[j] = (!listed_only || ((e[j] >> (16 + my_bit)) & 1u))
+                        ? p.N - (int)(e[j] & 0xffffu) * kC - ((kG == 1) ? 64 * half : 0) : 0;
+          else
+            hv[j] = kend - (jlo + i * kG) * kC - 64 * half - j * kBW;
+          whole = whole && hv[j] >= kBW;
         }
-        return mx * p.scale_log2;
+        uint32_t r[64];
+        ptx::tmem_ld32(tSh, &r[0]);
+        ptx::tmem_ld32(tSh + 32, &r[32]);
+        ptx::tmem_wait_ld();
+        if (!whole) {
+#pragma unroll
+          for (int c = 0; c < 64; ++c)
+            if ((c % kBW) >= hv[c / kBW]) r[c] = 0xff800000u;
+        }
+        float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll
+        for (int c = 0; c < 64; c += 2) mx[(c >> 1) & 3] = ptx::max3(mx[(c >> 1) & 3], __uint_as_float(r[c]), __uint_as_float(r[c + 1]));
+        return fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])) * p.scale_log2;
       };
-      // (m_ref of the group that has it; both halves read the whole row first, so that neither packs P
-      // over it before the other is done)
-#define TILE_REF_GIVE()                                                                             \
+      // (m_ref of the group that has it)
+#define TILE_REF_GIVE(half_mx)                                                                      \
   do {                                                                                              \
-    ptx::tc_fence_before_sync();                                                                    \
+    const float mx_ = (half_mx);                                                                    \
+    ctl->half_max[rs][half][row] = mx_;                                                             \
     __syncwarp();                                                                                   \
     if (lane == 0) ptx::mbar_arrive(pair_bar);                                                      \
     LOSA_WAIT(pair_bar, cnt & 1u);                                                                  \
     cnt ^= 1u;                                                                                      \
-    ptx::tc_fence_after_sync();                                                                     \
+    m_ref = fmaxf(mx_, ctl->half_max[rs][half ^ 1][row]);                                           \
     if (half == 0) {                                                                                \
       /* (the slot's last readers, two units with a reference ago, are done with it) */             \
       if (cnt >= 4u) LOSA_WAIT(&ctl->ref_empty[rs][sub], ((cnt >> 2) - 1u) & 1);                    \
@@ -885,8 +903,7 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
             if (MODE == kSparse) TILE_CHUNK_WAIT();
             LOSA_WAIT(&ctl->s_full[bsel], sph);
             ptx::tc_fence_after_sync();
-            m_ref = row_max(first, nc, first * kG);
-            TILE_REF_GIVE();
+            TILE_REF_GIVE(half_max(first, nc, first * kG));
           } else {
             TILE_REF_TAKE();
           }
@@ -920,8 +937,7 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         ptx::tc_fence_after_sync();
         if (kLazyRef && !have_ref && i >= ref_tile) {
           if (i == ref_tile) {
-            m_ref = row_max(i, nc, (i - base) * kG);
-            TILE_REF_GIVE();
+            TILE_REF_GIVE(half_max(i, nc, (i - base) * kG));
           } else {
             TILE_REF_TAKE();
           }
