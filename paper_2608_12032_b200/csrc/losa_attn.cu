@@ -680,14 +680,15 @@ __device__ __forceinline__ void acquire_maps(const ProblemEntry* pe) {
   ptx::tensormap_acquire(&pe->map_v128);
 }
 
-// ... those that the tile kernel uses
+// ... those that the tile kernel uses, a lane each (whole warp)
 template <int D, int C_, bool HAS_V>
-__device__ __forceinline__ void acquire_tile_maps(const ProblemEntry* pe) {
-  ptx::tensormap_acquire(&pe->map_q);
-  ptx::tensormap_acquire(D == 128 ? &pe->map_kh : &pe->map_k);
-  if (D == 128 ? C_ < 64 : C_ < 128) ptx::tensormap_acquire(D == 128 ? &pe->map_k64 : &pe->map_k128);
-  if (HAS_V) ptx::tensormap_acquire(&pe->map_v);
-  if (HAS_V && C_ < 128) ptx::tensormap_acquire(&pe->map_v128);
+__device__ __forceinline__ void acquire_tile_maps(const ProblemEntry* pe, int lane) {
+  const CUtensorMap* m = &pe->map_q;
+  if (lane == 1) m = (D == 128) ? &pe->map_kh : &pe->map_k;
+  if (lane == 2) m = (D == 128) ? &pe->map_k64 : &pe->map_k128;  // (equal to map_k where there is no such box)
+  if (lane == 3) m = &pe->map_v;
+  if (lane == 4) m = &pe->map_v128;
+  if (lane < (HAS_V ? 5 : 3)) ptx::tensormap_acquire(m);
 }
 
 template <int D, int R, int C_, int MODE, int KT, bool SPLIT>

@@ -68,7 +68,7 @@ struct TileControl {
   uint64_t l_full[4];      // the group that is done with a unit first has left its rows' partial sums
   uint64_t fold_bar;       // ... and after the fused step's masses are folded out of the table
   uint64_t drain;
-  uint2 hdr[2];
+  alignas(16) uint32_t hdr[4][12];  // (TILE_HDR_PUT)
   alignas(16) uint32_t tl[kTlChunks * 32];  // (read in groups of up to four entries with one vector load)
   uint32_t redo_mark[4];   // per unit (of four in turn): 1 + the tile list of one that outgrew its reference
   uint32_t redo_queue[4];  // the scheduler's: tile lists of units to be run again
@@ -113,17 +113,16 @@ __device__ __forceinline__ void tile_key_range(const Params& p, uint32_t ent, in
 // list of headers and tiles entry by entry, in the dense modes too, that took more instructions per
 // tile than the exponentials: 529 warp instructions per 64 scores of a warp, 224 of them arithmetic.)
 //
-// Next header (whole warp); `nu` is the warp's unit counter.
-#define TILE_HDR_NEXT(ent, word)                                                           \
+// Next header (whole warp); `nu` is the warp's unit counter.  N: how much of it the role reads, in groups of
+// four words.
+#define TILE_HDR_NEXT(hdr_, N)                                                             \
   do {                                                                                     \
     const uint32_t s_ = nu & 1u;                                                           \
-    TILE_WAIT(&ctl->hdr_full[s_], (nu >> 1) & 1u);                                      \
-    uint32_t h_[2];                                                                        \
-    ptx::ld_shared_volatile_vec<2>(&ctl->hdr[s_].x, h_);                                   \
+    TILE_WAIT(&ctl->hdr_full[s_], (nu >> 1) & 1u);                                         \
+    _Pragma("unroll") for (int i_ = 0; i_ < (N); ++i_)                                     \
+        ptx::ld_shared_volatile_vec<4>(&ctl->hdr[nu & 3u][4 * i_], (hdr_) + 4 * i_);       \
     __syncwarp();                                                                          \
     if (lane == 0) arrive0<PAIR>(hdr_empty0 + 8u * s_);                                    \
-    (ent) = h_[0];                                                                         \
-    (word) = h_[1];                                                                        \
     ++nu;                                                                                  \
   } while (0)
 
@@ -136,18 +135,27 @@ __device__ __forceinline__ void tile_key_range(const Params& p, uint32_t ent, in
     ++nc;                                                                                  \
   } while (0)
 
-// Scheduler of the first CTA: publish a header in both CTAs.
-#define TILE_HDR_PUT(ent, word)                                                            \
+// Scheduler of the first CTA: publish a header in both CTAs, a lane per word.  It says where the unit lies, so
+// that not every warp has to divide the item's number up again (five divisions, between two units).  A header
+// lies in one of four places in turn: it is there until its readers are done with the unit.
+#define TILE_HDR_PUT(ent, word, pr, bh, b, h, o, problem)                                  \
   do {                                                                                     \
     const uint32_t s_ = nu & 1u;                                                           \
     LOSA_WAIT_RELAXED(&ctl->hdr_empty[s_], ((nu >> 1) & 1u) ^ 1u);                         \
-    if (lane == 0) {                                                                       \
-      ctl->hdr[s_] = make_uint2((ent), (word));                                            \
+    const uint64_t o_ = (uint64_t)reinterpret_cast<uintptr_t>(o);                          \
+    const uint32_t all_[9] = {(ent), (word), (uint32_t)(pr), (uint32_t)(bh), (uint32_t)(b), (uint32_t)(h), \
+                              (uint32_t)o_, (uint32_t)(o_ >> 32), (uint32_t)(problem)};    \
+    uint32_t mine_ = 0u;                                                                   \
+    _Pragma("unroll") for (int i_ = 0; i_ < 9; ++i_) if (lane == i_) mine_ = all_[i_];     \
+    if (lane < 9) {                                                                        \
+      ctl->hdr[nu & 3u][lane] = mine_;                                                     \
       if (PAIR) {                                                                          \
-        ptx::st_cluster_u32(hdr1 + 8u * s_, (ent));                                        \
-        ptx::st_cluster_u32(hdr1 + 8u * s_ + 4u, (word));                                  \
+        ptx::st_cluster_u32(hdr1 + 48u * (nu & 3u) + 4u * lane, mine_);                    \
         ptx::fence_acq_rel_cluster();                                                      \
       }                                                                                    \
+    }                                                                                      \
+    __syncwarp();                                                                          \
+    if (lane == 0) {                                                                       \
       ptx::mbar_arrive(&ctl->hdr_full[s_]);                                                \
       if (PAIR) ptx::mbar_arrive_cluster(hdr_full1 + 8u * s_);                             \
     }                                                                                      \
@@ -167,7 +175,7 @@ __device__ __forceinline__ void expect0(uint32_t bar0, uint32_t bytes) {
   else ptx::mbar_arrive_expect_tx_u32(bar0, bytes);
 }
 template <bool PAIR>
-__device__ __forceinline__ void load0(void* dst, const CUtensorMap* map, uint32_t bar0, int c0, int c1, int c2, int c3) {
+__device__ __forceinline__ void load0(uint32_t dst, const CUtensorMap* map, uint32_t bar0, int c0, int c1, int c2, int c3) {
   if (PAIR) ptx::tma_load_4d_pair(dst, map, bar0, c0, c1, c2, c3);
   else ptx::tma_load_4d_u32(dst, map, bar0, c0, c1, c2, c3);
 }
@@ -251,7 +259,7 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   const uint32_t tl_full1 = at1(&ctl->tl_full[0]);
   const uint32_t hdr_empty0 = at0(&ctl->hdr_empty[0]);
   const uint32_t hdr_full1 = at1(&ctl->hdr_full[0]);
-  const uint32_t hdr1 = at1(&ctl->hdr[0]);
+  const uint32_t hdr1 = at1(&ctl->hdr[0][0]);
   const uint32_t tl1 = at1(&ctl->tl[0]);
   const uint32_t abort_peer = PAIR ? ptx::mapa(ptx::smem_u32(&ctl->abort_flag), rank ^ 1u) : 0u;
 
@@ -367,31 +375,33 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       // ------------------------------------------------------------------ TMA producer (both CTAs)
       // One elected thread makes the copies: from a lane test the compiler cannot tell that there is only one.
       const bool leader = ptx::elect_one();
-      uint32_t nq = 0, nk = 0, vs = 0, v_par = 1u, nu = 0, nc = 0, ent, word;
+      const uint32_t sQ_a = ptx::smem_u32(sQ), sK_a = ptx::smem_u32(sK), sV_a = ptx::smem_u32(sV);
+      const uint32_t k_empty_a = ptx::smem_u32(&ctl->k_empty[0]), v_empty_a = ptx::smem_u32(&ctl->v_empty[0]);
+      const uint32_t tl_a = ptx::smem_u32(&ctl->tl[0]);
+      uint32_t nq = 0, nk = 0, vs = 0, v_par = 1u, nu = 0, nc = 0, hdr[12];
       int problem = -1;  // batched launch: whose tensor maps this warp has acquired
       for (;;) {
-        TILE_HDR_NEXT(ent, word);
+        TILE_HDR_NEXT(hdr, 3);
+        const uint32_t ent = hdr[0], word = hdr[1];
         if (ent == kTlSkip) {
           if (rank == 0 && leader) ptx::mbar_arrive(&ctl->hdr_next);
           continue;
         }
         if ((ent >> 28) != 1) break;
-        const int w = (int)(ent & kTlItemMask);
-        const int pbh = w / p.nPairs, pr = w % p.nPairs;
-        const int bh = pbh % (p.B * p.H);
-        const int b = bh / p.H, h = bh % p.H;
+        const int pr = (int)hdr[2], b = (int)hdr[4], h = (int)hdr[5];
         // (map_kw: K in boxes of 64 keys, map_vw: V in boxes of 128 keys, for consecutive key blocks)
         const CUtensorMap *mq = &map_q, *mk = &map_k, *mv = &map_v, *mkw = &map_kw, *mvw = &map_vw;
         if (p.problems != nullptr) {
-          const ProblemEntry* pe = p.problems + pbh / (p.B * p.H);
+          const ProblemEntry* pe = p.problems + hdr[8];
           mq = &pe->map_q;
           mk = PAIR ? &pe->map_kh : &pe->map_k;
           mv = &pe->map_v;
           mkw = PAIR ? &pe->map_k64 : &pe->map_k128;
           mvw = &pe->map_v128;
-          if (pbh / (p.B * p.H) != problem) {
-            problem = pbh / (p.B * p.H);
-            acquire_tile_maps<D, C_, kHasV>(pe);
+          if (PAIR && (int)hdr[8] != problem) {
+            problem = (int)hdr[8];
+            acquire_tile_maps<D, C_, kHasV>(pe, lane);
+            __syncwarp();
           }
         }
         // this CTA's query tile (rows past the end of the sequence are filled with zeros)
@@ -402,7 +412,7 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           expect0<PAIR>(q_full0 + 8u * qs, kQBytes);
 #pragma unroll
           for (int s = 0; s < kSlabs; ++s)
-            load0<PAIR>(sQ + qs * kQBytes + s * 16384, mq, q_full0 + 8u * qs, s * 64, T * 128, h, b);
+            load0<PAIR>(sQ_a + qs * kQBytes + s * 16384, mq, q_full0 + 8u * qs, s * 64, T * 128, h, b);
         }
         ++nq;
         const int tiles = (int)(word & kHdrTiles);
@@ -420,7 +430,7 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
               if (i == call_at && rank == 0) ptx::mbar_arrive(&ctl->hdr_next);
               uint32_t grp[kG];
               if (MODE == kSparse) {
-                ptx::ld_shared_volatile_vec<kG>(&ctl->tl[(nc & (kTlChunks - 1)) * 32 + (i - base) * kG], grp);
+                ptx::ld_shared_volatile_vec_u32<kG>(tl_a + 4u * ((nc & (kTlChunks - 1)) * 32 + (i - base) * kG), grp);
 #pragma unroll
                 for (int g = 0; g < kG; ++g) grp[g] &= 0xffffu;
               } else {
@@ -429,11 +439,11 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
               }
               // K: a pair's CTAs keys 64 * rank ... + 63 of the tile each; all head-dimension columns, per slab of 64
               const uint32_t ks = nk % kTileNK;
-              in_time = ptx::mbar_wait_relaxed(&ctl->k_empty[ks], ((nk / kTileNK) & 1) ^ 1, &ctl->abort_flag, p.wait_polls);
+              in_time = ptx::mbar_wait_relaxed_u32(k_empty_a + 8u * ks, ((nk / kTileNK) & 1) ^ 1, &ctl->abort_flag, p.wait_polls);
               if (!in_time) break;
               ++nk;
               expect0<PAIR>(k_full0 + 8u * ks, kTileStage);
-              uint8_t* const k_to = sK + ks * kTileStage;
+              const uint32_t k_to = sK_a + ks * kTileStage;
               // several key blocks: this CTA's, if consecutive, are one copy per slab (every copy costs its thread
               // about 70 ns, and at head dimension 64 a tile takes 550)
               constexpr int kKBlocks = (kKRows / kC > 0) ? kKRows / kC : 1;  // key blocks of this CTA's rows
@@ -460,10 +470,10 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
               }
               if (!kHasV || (word & kHdrMax)) continue;
               // V: all 128 keys of the tile, (a pair: of each CTA) 64 of the head-dimension columns, one slab
-              in_time = ptx::mbar_wait_relaxed(&ctl->v_empty[vs], v_par, &ctl->abort_flag, p.wait_polls);
+              in_time = ptx::mbar_wait_relaxed_u32(v_empty_a + 8u * vs, v_par, &ctl->abort_flag, p.wait_polls);
               if (!in_time) break;
               expect0<PAIR>(v_full0 + 8u * vs, kTileStage);
-              uint8_t* const v_to = sV + vs * kTileStage;
+              const uint32_t v_to = sV_a + vs * kTileStage;
               bool wide_v = kG > 1;
 #pragma unroll
               for (int g = 1; g < kG; ++g) wide_v = wide_v && grp[g] == grp[0] + g;
@@ -501,9 +511,10 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
 #pragma unroll
       for (int kk = 0; kk < D / 16; ++kk)
         qd[kk] = ptx::smem_desc_lo(ptx::smem_u32(sQ), 16) + (((kk >> 2) * 16384 + (kk & 3) * 32) >> 4);
-      uint32_t nq = 0, nt = 0, nu = 0, ent, word;
+      uint32_t nq = 0, nt = 0, nu = 0, hdr[4];
       for (;;) {
-        TILE_HDR_NEXT(ent, word);
+        TILE_HDR_NEXT(hdr, 1);
+        const uint32_t ent = hdr[0], word = hdr[1];
         if (ent == kTlSkip) continue;
         if ((ent >> 28) != 1) break;
         bool q_ready = false;
@@ -552,9 +563,10 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       const uint32_t v_lo = ptx::smem_desc_lo(ptx::smem_u32(sV), kSumCol ? kNV * kTileStage : kTileStage);
       auto v_desc = [&](uint32_t bytes) { return v_lo + (bytes >> 4) - (kSumCol ? (bytes >> 4) << 16 : 0u); };
       const uint32_t tO = tmem_base + 384;
-      uint32_t nof = 0, nt = 0, nv = 0, nu = 0, ent, word;
+      uint32_t nof = 0, nt = 0, nv = 0, nu = 0, hdr[4];
       for (;;) {
-        TILE_HDR_NEXT(ent, word);
+        TILE_HDR_NEXT(hdr, 1);
+        const uint32_t ent = hdr[0], word = hdr[1];
         if ((ent >> 28) == 2) break;
         const uint32_t od = (nu - 1u) & 3u;
         if (ent == kTlSkip || (kHasV && (word & kHdrMax))) {
@@ -605,6 +617,7 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       // headers without work, for the marks of the last two units.
       uint32_t nu = 0, nc = 0, q_head = 0, q_tail = 0;
       int again = -1, idle = 0;  // the list whose maxima were taken last
+      int acquired = -1;         // batched launch: whose tensor maps this warp has acquired
       bool first_item = true, drawn = false;
       bool redone = false;
       for (;;) {
@@ -650,7 +663,7 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         if (drawn && mode == 0u) {
           if (idle == 2) break;
           ++idle;
-          TILE_HDR_PUT(kTlSkip, 0u);
+          TILE_HDR_PUT(kTlSkip, 0u, 0, 0, 0, 0, nullptr, 0);
           LOSA_WAIT_RELAXED(&ctl->hdr_next, (nu - 1u) & 1u);
           continue;
         }
@@ -665,10 +678,23 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           flags = kTlPartial | ((uint32_t)(r % p.split_parts) << 24);
           w = p.split_first + r / p.split_parts;
         }
+        const int pbh = w / p.nPairs, pr = w % p.nPairs;
+        const int problem = pbh / (p.B * p.H), bh = pbh % (p.B * p.H);
+        const int b = bh / p.H, h = bh % p.H;
+        void* o = p.o;
+        if (p.problems != nullptr) {
+          o = p.problems[problem].o;
+          // (without pairs of CTAs the producer's maps, ahead of it: 1 us)
+          if (!PAIR && problem != acquired) {
+            acquired = problem;
+            acquire_tile_maps<D, C_, kHasV>(p.problems + problem, lane);
+            __syncwarp();
+          }
+        }
         if (MODE == kSparse) {
           const uint32_t word = LOSA_IN_RANGE(list, p.cap_units) ? (uint32_t)__ldcg(p.tl_count + list) : 0u;
           const int cnt = min((int)(word & kHdrTiles) * kG, p.tl_cap);
-          TILE_HDR_PUT(kTlItem | flags | (uint32_t)w, (word & ~kHdrTiles) | odd | (uint32_t)(cnt / kG));
+          TILE_HDR_PUT(kTlItem | flags | (uint32_t)w, (word & ~kHdrTiles) | odd | (uint32_t)(cnt / kG), pr, bh, b, h, o, problem);
           const uint32_t* src = p.tl_entries + (int64_t)list * p.tl_cap;
           for (int base = 0; base < cnt; base += 32) {
             const uint32_t e = (base + lane < cnt) ? __ldcg(src + base + lane) : 0u;
@@ -690,17 +716,18 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           const uint32_t ent = kTlItem | flags | (uint32_t)w;
           int jlo, jhi;
           tile_key_range(p, ent, jlo, jhi);
-          const bool two = 2 * (w % p.nPairs) + 1 < p.nQt;  // the pair's second query tile exists
+          const bool two = 2 * pr + 1 < p.nQt;  // the pair's second query tile exists
           if (PAIR) {
-            TILE_HDR_PUT(ent, mode | (two ? 3u : 1u) * kHdrHas | (uint32_t)((jhi - jlo + kG - 1) / kG));
+            TILE_HDR_PUT(ent, mode | (two ? 3u : 1u) * kHdrHas | (uint32_t)((jhi - jlo + kG - 1) / kG), pr, bh, b, h, o, problem);
           } else {
             // (a query tile that does not exist is a unit without tiles)
-            TILE_HDR_PUT(ent, odd | ((two || !(odd & kHdrOdd)) ? kHdrHas | (uint32_t)((jhi - jlo + kG - 1) / kG) : 0u));
+            TILE_HDR_PUT(ent, odd | ((two || !(odd & kHdrOdd)) ? kHdrHas | (uint32_t)((jhi - jlo + kG - 1) / kG) : 0u), pr, bh, b, h, o,
+                         problem);
           }
         }
         LOSA_WAIT_RELAXED(&ctl->hdr_next, (nu - 1u) & 1u);
       }
-      if (!p.stall) TILE_HDR_PUT(kTlEnd, 0u);
+      if (!p.stall) TILE_HDR_PUT(kTlEnd, 0u, 0, 0, 0, 0, nullptr, 0);
       if (p.one_wave && lane == 0) p.redo_flag[PAIR ? blockIdx.x >> 1 : blockIdx.x] = redone ? 1 : 0;
     }
   } else {
@@ -718,7 +745,7 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     uint64_t* const pair_bar = &ctl->pair_bar[grpi * 4 + wl];
     const int quarter = grpi * 2 + half;         // which 32 columns of O this thread writes out
     // (cnt: bit 0 the uses of pair_bar, above it the units with a reference)
-    uint32_t kq = 0, cnt = 0, nitem = 0, nfold = 0, nu = 0, nc = 0, ent, word;
+    uint32_t kq = 0, cnt = 0, nitem = 0, nfold = 0, nu = 0, nc = 0, hdr[4];
     // fused step: this row's column of the CTA's table of per-block sums of the unrounded
     // exponentials (one float per row and 64-column half of a key tile when a key block fills the
     // tile, else one per row and key block)
@@ -727,7 +754,8 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
                                   : nullptr;
 
     for (;;) {
-      TILE_HDR_NEXT(ent, word);
+      TILE_HDR_NEXT(hdr, 1);
+      const uint32_t ent = hdr[0], word = hdr[1];
       if ((ent >> 28) == 2) break;
       // Which of the groups is through with the unit first, and leaves its end to the other.
       constexpr bool kExchange = kOneGroup && (!kSumCol || (kQB > 1 && MODE == kSparse));
@@ -736,17 +764,8 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         if (lane == 0 && grpi == 0) ptx::mbar_arrive(&ctl->l_full[(nu - 1u) & 3u]);
       }
       if (ent == kTlSkip) continue;
-      const int w = (int)(ent & kTlItemMask);
-      const bool partial = (ent & kTlPartial) != 0;
-      const int part = (int)((ent >> 24) & 7u);
-      const int pbh = w / p.nPairs, pr = w % p.nPairs;
-      const int bh = pbh % (p.B * p.H);
-      const int b = bh / p.H, h = bh % p.H;
-      void* const o_base = (p.problems != nullptr) ? p.problems[pbh / (p.B * p.H)].o : p.o;
       const int tile = PAIR ? (int)rank : (int)((word & kHdrOdd) != 0u);  // of the item's two query tiles
       const int my_bit = tile * kQB + sub;
-      const int T = 2 * pr + tile;
-      const int grow = T * 128 + row;
       float m_ref = 0.f, l = 0.f, le = 0.f;  // le: row sum of the unrounded exponentials (masses, LSE)
       bool ovf = false, seen = false;  // (seen: this warp met keys that its rows attend to)
       const int tiles = (int)(word & kHdrTiles);
@@ -1083,6 +1102,17 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       if (has && !redo) cnt += 2u;
 #undef TILE_REF_GIVE
 #undef TILE_REF_TAKE
+      // where the unit lies, and what else of its header only its end needs: read again, not kept in registers
+      uint32_t info[8];
+      ptx::ld_shared_volatile_vec<4>(&ctl->hdr[(nu - 1u) & 3u][0], info);
+      ptx::ld_shared_volatile_vec<4>(&ctl->hdr[(nu - 1u) & 3u][4], info + 4);
+      const int w = (int)(info[0] & kTlItemMask);
+      const bool partial = (info[0] & kTlPartial) != 0;
+      const int part = (int)((info[0] >> 24) & 7u);
+      const int pr = (int)info[2], bh = (int)info[3], b = (int)info[4], h = (int)info[5];
+      void* const o_base = reinterpret_cast<void*>((uint64_t)info[6] | ((uint64_t)info[7] << 32));
+      const int T = 2 * pr + tile;
+      const int grow = T * 128 + row;
       auto hand_over = [&]() {
         const int unit = partial ? p.split_first + (w - p.split_first) * p.split_parts + part : w;
         const uint32_t mark = 1u + (uint32_t)(PAIR ? unit : 2 * unit + tile);

@@ -69,7 +69,7 @@ __device__ __forceinline__ void mbar_arrive_expect_tx_u32(uint32_t saddr, uint32
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(saddr), "r"(bytes) : "memory");
 }
 
-__device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
+__device__ __forceinline__ bool mbar_try_wait_u32(uint32_t saddr, uint32_t parity) {
   uint32_t ok;
   asm volatile(
       "{\n\t"
@@ -78,9 +78,13 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
       "selp.u32 %0, 1, 0, p;\n\t"
       "}"
       : "=r"(ok)
-      : "r"(smem_u32(bar)), "r"(parity)
+      : "r"(saddr), "r"(parity)
       : "memory");
   return ok != 0;
+}
+
+__device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
+  return mbar_try_wait_u32(smem_u32(bar), parity);
 }
 
 // Bounded wait: polls the barrier at most `limit` times (kWaitPolls in ordinary launches: with
@@ -106,10 +110,10 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
 // Same bound, but for roles that run far ahead of the data path (copy producer, tile-list
 // scheduler): they sleep between polls from the start, so that their waiting costs neither issue
 // slots nor power that the softmax and MMA warps of the same SM could use.
-__device__ __forceinline__ bool mbar_wait_relaxed(uint64_t* bar, uint32_t parity,
-                                                  volatile int* abort_flag, uint32_t limit) {
+__device__ __forceinline__ bool mbar_wait_relaxed_u32(uint32_t bar, uint32_t parity,
+                                                      volatile int* abort_flag, uint32_t limit) {
   for (uint32_t it = 0; it < limit; ++it) {
-    if (mbar_try_wait(bar, parity)) return true;
+    if (mbar_try_wait_u32(bar, parity)) return true;
     if (it >= 4) {
       if ((it & 1023u) == 0 && *abort_flag) return false;
       __nanosleep(it < 64 ? 64 : 256);
@@ -121,6 +125,11 @@ __device__ __forceinline__ bool mbar_wait_relaxed(uint64_t* bar, uint32_t parity
 // Makes this thread's writes to shared memory visible to the tensor cores and the copy engine.
 __device__ __forceinline__ void fence_proxy_async() {
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+}
+
+__device__ __forceinline__ bool mbar_wait_relaxed(uint64_t* bar, uint32_t parity,
+                                                  volatile int* abort_flag, uint32_t limit) {
+  return mbar_wait_relaxed_u32(smem_u32(bar), parity, abort_flag, limit);
 }
 
 // ---------------------------------------------------------------- TMA
@@ -144,12 +153,12 @@ __device__ __forceinline__ void tma_load_4d(void* smem_dst, const CUtensorMap* m
       : "memory");
 }
 
-// (the barrier by its shared-memory address)
-__device__ __forceinline__ void tma_load_4d_u32(void* smem_dst, const CUtensorMap* map, uint32_t bar,
+// (barrier and destination by their shared-memory addresses)
+__device__ __forceinline__ void tma_load_4d_u32(uint32_t smem_dst, const CUtensorMap* map, uint32_t bar,
                                             int x, int y, int z, int w) {
   asm volatile(
       "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes"
-      " [%0], [%1, {%3, %4, %5, %6}], [%2];" ::"r"(smem_u32(smem_dst)),
+      " [%0], [%1, {%3, %4, %5, %6}], [%2];" ::"r"(smem_dst),
       "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(x), "r"(y), "r"(z), "r"(w)
       : "memory");
 }
@@ -385,9 +394,8 @@ __device__ __forceinline__ uint32_t ld_cluster_u32(uint32_t caddr) {
 
 // N = 1, 2 or 4 consecutive 32-bit words of shared memory (aligned to their total size), read anew
 template <int N>
-__device__ __forceinline__ void ld_shared_volatile_vec(const uint32_t* p, uint32_t* out) {
+__device__ __forceinline__ void ld_shared_volatile_vec_u32(uint32_t a, uint32_t* out) {
   static_assert(N == 1 || N == 2 || N == 4, "vector width");
-  const uint32_t a = smem_u32(p);
   if constexpr (N == 1) {
     asm volatile("ld.volatile.shared.u32 %0, [%1];" : "=r"(out[0]) : "r"(a) : "memory");
   } else if constexpr (N == 2) {
@@ -398,6 +406,11 @@ __device__ __forceinline__ void ld_shared_volatile_vec(const uint32_t* p, uint32
                  : "r"(a)
                  : "memory");
   }
+}
+
+template <int N>
+__device__ __forceinline__ void ld_shared_volatile_vec(const uint32_t* p, uint32_t* out) {
+  ld_shared_volatile_vec_u32<N>(smem_u32(p), out);
 }
 
 // (default semantics, release at CTA scope: a release at cluster scope on every arrival was measured
@@ -442,11 +455,11 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity
 
 // 4D tiled load into this CTA's shared memory whose completion is counted on a barrier of either
 // CTA of the pair (given by its shared::cluster address).
-__device__ __forceinline__ void tma_load_4d_pair(void* smem_dst, const CUtensorMap* map, uint32_t bar_caddr,
+__device__ __forceinline__ void tma_load_4d_pair(uint32_t smem_dst, const CUtensorMap* map, uint32_t bar_caddr,
                                                  int x, int y, int z, int w) {
   asm volatile(
       "cp.async.bulk.tensor.4d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes"
-      " [%0], [%1, {%3, %4, %5, %6}], [%2];" ::"r"(smem_u32(smem_dst)),
+      " [%0], [%1, {%3, %4, %5, %6}], [%2];" ::"r"(smem_dst),
       "l"(reinterpret_cast<uint64_t>(map)), "r"(bar_caddr), "r"(x), "r"(y), "r"(z), "r"(w)
       : "memory");
 }
