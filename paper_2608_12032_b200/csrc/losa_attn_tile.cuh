@@ -191,6 +191,27 @@ __device__ __forceinline__ void commit_all(uint64_t* bar) {
   else ptx::mma_commit(bar);
 }
 
+// A lane holds N chunks of 16 bytes of a row of its own; afterwards lane j of a group of N holds chunk j of each of
+// the group's rows, that of the group's i-th in place i (whole warp).
+template <int N>
+__device__ __forceinline__ void transpose_chunks(uint32_t* r, int lane) {
+#pragma unroll
+  for (int b = 1; b < N; b <<= 1) {
+    const bool hi = (lane & b) != 0;
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+      if (i & b) continue;
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        uint32_t &x = r[4 * i + e], &y = r[4 * (i | b) + e];
+        const uint32_t other = __shfl_xor_sync(0xffffffffu, hi ? x : y, b);
+        if (hi) x = other;
+        else y = other;
+      }
+    }
+  }
+}
+
 template <int D, int R, int C_, int MODE, bool PAIR>
 __global__ void __launch_bounds__(Lay<true>::kThreads, 1)
 losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
@@ -1124,29 +1145,44 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         }
       };
       if (!kSumCol && ovf && !redo && lane == 0) hand_over();
-      const int64_t off = (int64_t)b * p.sb + (int64_t)h * p.sh + (int64_t)grow * p.sn;
-      const bool valid = (T < p.nQt) && grow < p.N;
-      // 32 (or 16) columns of a row of O, from `c0` on
-      auto store_o = [&](const uint32_t* r, int c0, float inv, auto cols) {
+      // Columns c0 ... of the rows of O of this warp's 32 lanes, a row a lane, to `dst` (rows of `stride` elements of
+      // 4 bytes, or of 2 and rounded); those from `rows` on do not exist.  Groups of lanes write a row's columns
+      // together: with a row a lane every store of 16 bytes went to 32 lines, and the 2048 cycles that took held up
+      // the copies, the next unit's reference and whatever else goes through shared memory.
+      auto store_rows = [&](uint32_t* r, void* dst, int64_t stride, int rows, float by, bool f32, auto cols) {
         constexpr int kCols = decltype(cols)::value;
-        if (p.o_f32) {
-          float4* dst = reinterpret_cast<float4*>(static_cast<float*>(o_base) + off + c0);
 #pragma unroll
-          for (int c = 0; c < kCols; c += 4)
-            dst[c >> 2] = make_float4(__uint_as_float(r[c]) * inv, __uint_as_float(r[c + 1]) * inv,
-                                      __uint_as_float(r[c + 2]) * inv, __uint_as_float(r[c + 3]) * inv);
-        } else {
-          uint4* dst = reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(o_base) + off + c0);
+        for (int c = 0; c < kCols; ++c) r[c] = __float_as_uint(__uint_as_float(r[c]) * by);
+        if (f32) {
 #pragma unroll
-          for (int c = 0; c < kCols; c += 8) {
-            uint4 v;
-            v.x = ptx::pack_bf16x2(__uint_as_float(r[c]) * inv, __uint_as_float(r[c + 1]) * inv);
-            v.y = ptx::pack_bf16x2(__uint_as_float(r[c + 2]) * inv, __uint_as_float(r[c + 3]) * inv);
-            v.z = ptx::pack_bf16x2(__uint_as_float(r[c + 4]) * inv, __uint_as_float(r[c + 5]) * inv);
-            v.w = ptx::pack_bf16x2(__uint_as_float(r[c + 6]) * inv, __uint_as_float(r[c + 7]) * inv);
-            dst[c >> 3] = v;
+          for (int c = 0; c < kCols; c += 16) {
+            transpose_chunks<4>(r + c, lane);
+            float* to = static_cast<float*>(dst) + (int64_t)(lane & ~3) * stride + c + 4 * (lane & 3);
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+              if ((lane & ~3) + i < rows)
+                *reinterpret_cast<uint4*>(to + i * stride) = make_uint4(r[c + 4 * i], r[c + 4 * i + 1], r[c + 4 * i + 2], r[c + 4 * i + 3]);
           }
+        } else {
+          constexpr int kN = kCols / 8;  // chunks of a row
+#pragma unroll
+          for (int c = 0; c < kCols; c += 2) r[c >> 1] = ptx::pack_bf16x2(__uint_as_float(r[c]), __uint_as_float(r[c + 1]));
+          transpose_chunks<kN>(r, lane);
+          __nv_bfloat16* to = static_cast<__nv_bfloat16*>(dst) + (int64_t)(lane & ~(kN - 1)) * stride + 8 * (lane & (kN - 1));
+#pragma unroll
+          for (int i = 0; i < kN; ++i)
+            if ((lane & ~(kN - 1)) + i < rows)
+              *reinterpret_cast<uint4*>(to + i * stride) = make_uint4(r[4 * i], r[4 * i + 1], r[4 * i + 2], r[4 * i + 3]);
         }
+      };
+      const int row0 = T * 128 + wl * 32;  // of this warp
+      const int rows = (T < p.nQt) ? p.N - row0 : 0;
+      // the same to O
+      auto store_o = [&](uint32_t* r, int c0, float inv, auto cols) {
+        const int64_t off = (int64_t)b * p.sb + (int64_t)h * p.sh + (int64_t)row0 * p.sn + c0;
+        store_rows(r, p.o_f32 ? static_cast<void*>(static_cast<float*>(o_base) + off)
+                              : static_cast<void*>(static_cast<__nv_bfloat16*>(o_base) + off),
+                   p.sn, rows, inv, p.o_f32 != 0, cols);
       };
       if constexpr (kOneGroup) {
         // The group that worked on the unit's last tile writes O out; the other, whose turn the next tile
@@ -1211,14 +1247,11 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
             if (partial && half == 0 && T < p.nQt && LOSA_IN_RANGE(pslot, p.cap_part_rows)) p.part_ml[pslot] = make_float2(m_ref, l);
           }
           if (partial) {
-            if (T < p.nQt) {
-              float4* dst = reinterpret_cast<float4*>(p.part_o + (LOSA_IN_RANGE(pslot, p.cap_part_rows) ? pslot : 0) * D + half * kOC + c0);
-#pragma unroll
-              for (int c = 0; c < 32; c += 4)
-                dst[c >> 2] = make_float4(__uint_as_float(r[c]), __uint_as_float(r[c + 1]),
-                                          __uint_as_float(r[c + 2]), __uint_as_float(r[c + 3]));
-            }
-          } else if (valid) {
+            const int64_t slot0 = pslot - lane;  // (of the warp's first row; 32 rows of it exist in any case)
+            if (T < p.nQt)
+              store_rows(r, p.part_o + (LOSA_IN_RANGE(pslot, p.cap_part_rows) ? slot0 : 0) * D + half * kOC + c0, D, 32,
+                         1.f, true, std::integral_constant<int, 32>());
+          } else {
             store_o(r, half * kOC + c0, inv, std::integral_constant<int, 32>());
           }
         }
@@ -1256,7 +1289,7 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         if (kSumCol && !redo && __any_sync(0xffffffffu, !(l <= kSplitSafeSum)) && lane == 0) hand_over();
         // (against their maxima only rows that met a score that is not a number add up to that much)
         if (redo && !(l <= kSplitSafeSum)) l = __int_as_float(0x7fc00000);
-        if (valid) store_o(r, c0, (l == 0.f) ? 0.f : 1.f / l, std::integral_constant<int, kOC>());
+        store_o(r, c0, (l == 0.f) ? 0.f : 1.f / l, std::integral_constant<int, kOC>());
       }
       if (kWantMass) {
         // ---- fused construction step: the block masses of this CTA's query tile (Eq. 1).  The
