@@ -2,8 +2,8 @@
 // frozen CSR pattern (Eq. 4), the exact block-mass pass (Eq. 1) and the fused construction step.
 // They run in losa_tile_kernel (losa_attn_tile.cuh, included below): one query tile and three S buffers per CTA,
 // on pairs of CTAs at head dimension 128.  losa_attn_kernel, described here, is one warp-specialised persistent
-// kernel template with two thread layouts; it serves the fallback launch of all, and head dimension 128 on a
-// device (or partition of one) that cannot hold a pair of CTAs.
+// kernel template with two thread layouts; it serves head dimension 128 on a device (or partition of one) that
+// cannot hold a pair of CTAs: a main launch, and a fallback launch for the units that outgrew their reference.
 //
 // Warps 0-3 are utility warps: warp 0 is the TMA producer, which streams the query tiles and the
 // K / V tiles named by the tile list into 128B-swizzled shared-memory rings (a K/V tile is 128
@@ -20,8 +20,8 @@
 // batched launch.  The key blocks the pair visits are the union of the index lists of its query
 // blocks (two lists, four when R = 64), so a K/V tile needed by both tiles is loaded once, and
 // MMAs are issued only for the query tiles that list one of its blocks.  The items of the last,
-// partly filled wave of the persistent grid are cut into parts of their lists, merged by
-// the fallback launch.
+// partly filled wave of the persistent grid are cut into parts of their lists, merged behind
+// (merge_parts_kernel; here by the fallback launch).
 //
 // One S = Q K^T covers a whole K/V tile (128-wide MMAs).  TMEM holds exactly S and O of both query
 // tiles, P overwrites S, and per query tile the steps S -> softmax -> O += P V -> next S form a serial
@@ -56,7 +56,7 @@ std::atomic<uint32_t> g_stall_polls{0u};  // > 0: the next attention launch is a
 // Thread layout.  Warps 0-3 are the utility warpgroup (TMA, 2 MMA issuers, scheduler); the softmax
 // warps follow.  Two layouts:
 //   one thread per query row (SPLIT = false): 2 softmax warpgroups, one per query tile, each thread
-//     holding a whole 128-column S row.  Used by the fallback launch of every mode.
+//     holding a whole 128-column S row.  Used by the fallback launch.
 //   two threads per query row (SPLIT = true): 4 softmax warpgroups, two per query tile, each
 //     thread holding 64 columns.  A warp's ex2 instructions occupy it for 8 issue cycles each and
 //     its other instructions do not overlap them (measured on the loop alone: 1301 cycles per
@@ -111,7 +111,8 @@ constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLn2 = 0.6931471805599453f;
 constexpr float kRescaleThreshold = 8.0f;
 constexpr float kSafeRowSum = 1.099511627776e12f;  // 2^40: a tile's row sum beyond this re-centres the reference
-// two threads per row: a tile's half-row sum beyond 2^60 (or NaN) sends the work unit to the fallback
+// two threads per row: a tile's half-row sum (or, where it comes out of the product with V, a unit's row sum) beyond
+// 2^60 or NaN has the work unit computed again
 constexpr float kSplitSafeSum = 1.152921504606846976e18f;
 
 template <int D, int R, int C_, int MODE, int KT>
@@ -188,7 +189,8 @@ struct Params {
   float2* table;  // mass modes: [grid][2][nKb][128] (sum of p, reference max) per row and key tile
   float scale_log2;
   int* status;
-  // Work units whose scores outgrew the fixed reference of the two-threads-per-row kernel: it
+  // (losa_attn_kernel; the tile kernel runs such units again itself, and of these uses redo_count and redo_flag, to
+  // count them.)  Work units whose scores outgrew the fixed reference of the two-threads-per-row kernel: it
   // appends them here, and a second launch (one thread per row, moving reference) recomputes them.
   // That second launch, which also merges the partial units, draws redo_list[0 .. *redo_count) instead
   // of all units.  A unit's two query tiles, and the warps of each, may all find it outgrown, at
@@ -552,8 +554,10 @@ __device__ __forceinline__ void fill_tile_bitmap(const Params& p, int list, int 
 }
 
 // The tile list from its query blocks' bitmaps (whole warp).
+// Returns what goes into tl_count; `copy`, if not null, receives the entries as well.
 template <int NB, int G, bool ONE>
-__device__ __forceinline__ void emit_tile_list(const Params& p, int list, int lane, const uint32_t* bm) {
+__device__ __forceinline__ uint32_t emit_tile_list(const Params& p, int list, int lane, const uint32_t* bm,
+                                                   uint32_t* copy) {
   const int W = (p.nKb + 31) >> 5;
   const int bit0 = ONE ? (list & 1) * NB : 0;
   // Order of the entries.  A key block that only ONE of the unit's two query tiles lists is
@@ -564,6 +568,10 @@ __device__ __forceinline__ void emit_tile_list(const Params& p, int list, int la
   // left of the longer class.  Within a class the blocks ascend.  Correctness does not depend on
   // the order of the key blocks.
   uint32_t* dst = p.tl_entries + (int64_t)list * p.tl_cap;
+  auto put = [&](int pos, uint32_t e) {
+    dst[pos] = e;
+    if (copy != nullptr) copy[pos] = e;
+  };
   int nb = 0, na = 0, nbb = 0;  // both, tile 0 only, tile 1 only
   for (int w0 = 0; w0 < W; w0 += 32) {
     const int wi = w0 + lane;
@@ -595,13 +603,40 @@ __device__ __forceinline__ void emit_tile_list(const Params& p, int list, int la
     return s1 + ((t < tmin) ? 2 * t + (k - 1) : 2 * tmin + (t - tmin)) * G + r % G;
   };
   if (lane < G) {
-    if (nb + lane < s1 && nb + lane < total) dst[nb + lane] = kTlPad;
-    if (na + lane < tA * G && slot_of(1, na + lane) < total) dst[slot_of(1, na + lane)] = kTlPad;
-    if (nbb + lane < tB * G && slot_of(2, nbb + lane) < total) dst[slot_of(2, nbb + lane)] = kTlPad;
+    if (nb + lane < s1 && nb + lane < total) put(nb + lane, kTlPad);
+    if (na + lane < tA * G && slot_of(1, na + lane) < total) put(slot_of(1, na + lane), kTlPad);
+    if (nbb + lane < tB * G && slot_of(2, nbb + lane) < total) put(slot_of(2, nbb + lane), kTlPad);
   }
   const int ragged = (p.N % p.C != 0) ? p.nKb - 1 : -1;  // the key block in which the sequence ends
-  int rb = 0, ra = 0, rbb = 0;  // entries of each class emitted by earlier windows
-  for (int w0 = 0; w0 < W; w0 += 32) {
+  int rb = 0, ra = 0, rbb = 0;  // entries of each class emitted by earlier words (windows)
+  // Up to 16 words a lane per bit and word by word (about 40 instructions each); longer ones a lane per word and
+  // bit by bit (up to 32 times 25 for 32 words).  With one word, 32 blocks, the latter is a single lane's work: 1.5 us of
+  // a 20 us call.
+  if (W <= 16) {
+    for (int wi = 0; wi < W; ++wi) {
+      uint32_t memb = 0, ta = 0, tb = 0;
+#pragma unroll
+      for (int n = 0; n < NB; ++n) {
+        const uint32_t m = bm[n * W + wi];
+        if (ONE) ta |= m, tb |= m;
+        else if (n < NB / 2) ta |= m;
+        else tb |= m;
+        memb |= ((m >> lane) & 1u) << (bit0 + n);
+      }
+      const uint32_t both = ta & tb, a = ta & ~tb, b = tb & ~ta, below = (1u << lane) - 1u;
+      if (memb != 0u) {
+        const int pos = ((both >> lane) & 1u) ? rb + __popc(both & below)
+                        : ((a >> lane) & 1u)  ? slot_of(1, ra + __popc(a & below))
+                                              : slot_of(2, rbb + __popc(b & below));
+        const int j = wi * 32 + lane;
+        if (pos < p.tl_cap) put(pos, (uint32_t)j | (memb << 16) | (j == ragged ? kTlRagged : 0u));
+      }
+      rb += __popc(both);
+      ra += __popc(a);
+      rbb += __popc(b);
+    }
+  }
+  for (int w0 = 0; W > 16 && w0 < W; w0 += 32) {
     const int wi = w0 + lane;
     uint32_t m[NB], ta = 0, tb = 0;
 #pragma unroll
@@ -636,7 +671,7 @@ __device__ __forceinline__ void emit_tile_list(const Params& p, int list, int la
         for (int n = 0; n < NB; ++n) memb |= ((m[n] >> bit) & 1u) << (bit0 + n);
         const int pos = (k == 0) ? r : slot_of(k, r);
         const int j = wi * 32 + bit;
-        if (pos < p.tl_cap) dst[pos] = (uint32_t)j | (memb << 16) | (j == ragged ? kTlRagged : 0u);
+        if (pos < p.tl_cap) put(pos, (uint32_t)j | (memb << 16) | (j == ragged ? kTlRagged : 0u));
         ++r;
       }
     }
@@ -644,9 +679,10 @@ __device__ __forceinline__ void emit_tile_list(const Params& p, int list, int la
     ra += tot[1];
     rbb += tot[2];
   }
-  if (lane == 0)
-    p.tl_count[list] = (int32_t)((uint32_t)(total / G) | ((nb + na > 0) ? kHdrHas : 0u) |
-                                 ((nb + nbb > 0) ? 2u * kHdrHas : 0u) | ((nb == 0 && tmin > 0) ? kHdrLate : 0u));
+  const uint32_t word = (uint32_t)(total / G) | ((nb + na > 0) ? kHdrHas : 0u) | ((nb + nbb > 0) ? 2u * kHdrHas : 0u) |
+                        ((nb == 0 && tmin > 0) ? kHdrLate : 0u);
+  if (lane == 0) p.tl_count[list] = (int32_t)word;
+  return word;
 }
 
 template <int NB, int G, bool ONE>
@@ -660,7 +696,7 @@ __global__ void __launch_bounds__(32 * NB) build_tile_lists_kernel(const Params 
   fill_tile_bitmap<NB, ONE>(p, list, n, lane, bm);
   __syncthreads();
   if (n != 0) return;
-  emit_tile_list<NB, G, ONE>(p, list, lane, bm);
+  emit_tile_list<NB, G, ONE>(p, list, lane, bm, nullptr);
   if (lane == 0) {
     int w, part, parts;
     unit_item(p, unit, w, part, parts);
@@ -696,6 +732,7 @@ __global__ void __launch_bounds__(Lay<SPLIT>::kThreads, 1)
 losa_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                  const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_kw,
                  const __grid_constant__ CUtensorMap map_vw, const Params p) {
+  static_assert(D == 128, "head dimension 64 runs in the tile kernel");
   using C = Cfg<D, R, C_, MODE, KT>;
   using L = Lay<SPLIT>;
   using Ctl = Control<C::kNK, C::kNV, SPLIT>;
@@ -1119,27 +1156,12 @@ losa_attn_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         // the unit's merged tile list was built before the launch: stream it into the ring,
         // 32 entries per step, so that this warp takes next to no issue slots from the softmax
         // warps of its scheduler partition
-        // (head dimension 64: a list per query tile; their K/V tiles alternate, so that both query tiles
-        // are at work: one list after the other, a call of 8192 tokens and two heads with one unit here
-        // took 243 us, alternating 211 us; 150 us when a unit had one list)
-        constexpr int kLists = tile_lists_per_unit(D);
-        int tiles[kLists];
-#pragma unroll
-        for (int t = 0; t < kLists; ++t)
-          tiles[t] = LOSA_IN_RANGE(unit * kLists + t, p.cap_units)
-                         ? min((int)((uint32_t)__ldcg(p.tl_count + unit * kLists + t) & kHdrTiles), p.tl_cap / kG) : 0;
-        const int paired = (kLists == 2) ? min(tiles[0], tiles[kLists - 1]) : 0;  // of each list
-        const int cnt = (tiles[0] + (kLists == 2 ? tiles[kLists - 1] : 0)) * kG;
-        const uint32_t* src = p.tl_entries + (int64_t)unit * kLists * p.tl_cap;
+        const int cnt = LOSA_IN_RANGE(unit, p.cap_units)
+                            ? min((int)((uint32_t)__ldcg(p.tl_count + unit) & kHdrTiles) * kG, p.tl_cap) : 0;
+        const uint32_t* src = p.tl_entries + (int64_t)unit * p.tl_cap;
         for (int base = 0; base < cnt; base += 32) {
           const int n = min(32, cnt - base);
-          int at = base + lane;
-          if (kLists == 2) {
-            const int t = at / kG;
-            const int second = (t < 2 * paired) ? (t & 1) : (int)(tiles[kLists - 1] > paired);
-            at = second * p.tl_cap + ((t < 2 * paired) ? t >> 1 : t - paired) * kG + at % kG;
-          }
-          const uint32_t e = (lane < n) ? __ldcg(src + at) : 0u;
+          const uint32_t e = (lane < n) ? __ldcg(src + base + lane) : 0u;
           LOSA_TL_PUT_BULK(e, n);
         }
         continue;
@@ -1975,7 +1997,8 @@ int make_maps(ProblemEntry* e, const Geometry& g, const void* q, const void* k, 
   return LOSA_OK;
 }
 
-// The merge of the partial units as a launch of its own, behind the tile kernel.
+// The merge of the partial units as a launch of its own, behind the tile kernel: 3.5 us, against 6 when it came with the
+// fallback launch, whose CTAs could only start where a tile CTA had given its shared memory back.
 constexpr int kMergeThreads = 128;
 template <int D>
 __global__ void __launch_bounds__(kMergeThreads) merge_parts_kernel(const Params p) {
@@ -2060,7 +2083,7 @@ template <int D, int R, int C_, int MODE, bool PAIR>
 int launch_tile(const CUtensorMap& mq, const CUtensorMap& mkh, const CUtensorMap& mv, const CUtensorMap& mk64,
                 const CUtensorMap& mv128, const Params& prm, int clusters, cudaStream_t st, int* max_clusters) {
   using L = Lay<true>;
-  constexpr size_t smem = (size_t)tile_nq(D) * 256 * D + (size_t)(kTileNK + kTileNV) * kTileStage +
+  constexpr size_t smem = (size_t)tile_nq(D, MODE) * 256 * D + (size_t)(tile_nk(MODE) + tile_nv(MODE)) * kTileStage +
                           (D == 64 ? kTileOnes : 0) + sizeof(TileControl);
   static_assert(smem <= 227 * 1024, "shared memory of one CTA");
   auto kern = losa_tile_kernel<D, R, C_, MODE, PAIR>;
@@ -2125,8 +2148,7 @@ int launch_t(const Geometry& g, const void* q, const void* k, const void* v, Par
   // walked the tile lists: 32-key blocks 5.65 -> 5.16 ms at the Wan shape, with 64- and 128-key blocks
   // nothing; without the lists 4.35 -> 3.78 ms and 4.06 -> 3.94 ms.  64-row query blocks, 9600 tokens, 12
   // heads, against two query tiles per CTA: dense 557 -> 487 us, sparse 457 -> 419, masses 474 -> 359,
-  // construction step 703 -> 538.)  The fallback launch of all, and a device that cannot hold a pair:
-  // losa_attn_kernel.
+  // construction step 703 -> 538.)  A device that cannot hold a pair: losa_attn_kernel.
   constexpr bool kPairMode = LOSA_USE_PAIR && D == 128;
   constexpr bool kTileMode = D == 64;
   bool pair = kTileMode;
@@ -2142,7 +2164,7 @@ int launch_t(const Geometry& g, const void* q, const void* k, const void* v, Par
   if (kTileMode) ctas = max(1, min(sms, kMaxPersistentCtas) / 2);
   // The items of the last, partly filled wave of the persistent grid (all items, if there are
   // fewer than CTAs) are cut into parts of the key range, so that the wave ends after 1/parts of
-  // an item; their partial results are merged by the fallback launch.  Attention output
+  // an item; their partial results are merged by a launch behind.  Attention output
   // only: the mass epilogue needs a row's final statistics inside the kernel.
   prm.nUnits = prm.nWork;
   prm.split_first = prm.nWork;

@@ -27,18 +27,23 @@
 // row (64 columns each), key tiles taken alternately by two groups of eight warps, so that each
 // group has two tile periods for one tile.  The exponentials are taken against a reference that
 // never moves within a work unit (the row maximum over the first key tile the row attends to,
-// handed from the group that meets that tile to the other); units whose scores outgrow it are
-// listed for the fallback launch.
+// handed from the group that meets that tile to the other); a unit whose scores outgrow it is run again
+// by the same CTAs, first for its rows' maxima and then against these.  (A launch of its own for such units
+// cost every call 4 - 6 us and a launch; 2048 tokens, 4 heads, D = 64: 26.9 -> 21.5 us with the launch of the lists
+// gone as well.)
 //
 // Barriers that both CTAs feed (operands landed, P written, O read out, tile-list chunk consumed)
 // live in the first CTA; barriers that the MMAs' completion feeds in both CTAs are reached with a
 // commit to both.  Every wait is bounded; on the way out both CTAs meet at the cluster's barrier,
 // so that neither leaves while the other may still signal into its shared memory.
 
-constexpr int kTileNK = 4, kTileNV = 7;      // K and V stages of 16 KB per CTA (at most)
+constexpr int kTileMaxNK = 8, kTileNV = 7;   // K and V stages of 16 KB per CTA, at most
 // Query tiles in shared memory: two where there is room, so that the next unit's keys and its first scores need not
-// wait for this one's last.
-__host__ __device__ constexpr int tile_nq(int D) { return D == 64 ? 2 : 1; }
+// wait for this one's last.  The mass pass has no V: two query tiles at head dimension 128 too, and more K stages.
+// (Two query tiles and five V stages in the other modes there: within the noise, the construction step 1 % slower.)
+__host__ __device__ constexpr int tile_nq(int D, int mode) { return (D == 64 || mode == kMass) ? 2 : 1; }
+__host__ __device__ constexpr int tile_nk(int mode) { return mode == kMass ? 8 : 4; }
+__host__ __device__ constexpr int tile_nv(int mode) { return mode == kMass ? 0 : kTileNV; }
 constexpr int kTileStage = 16384;
 // Head dimension 64: one K step (16 keys) of 64 more columns of V, all ones, behind the V stages.  Every
 // O += P V reads 16 of these columns, so that the row sums of P come out of it as columns of O: 64 x 80
@@ -56,7 +61,7 @@ constexpr float kTileSafeLow = 8.6736173798840355e-19f;  // 2^-60
 
 struct TileControl {
   uint64_t q_full[2], q_empty[2];
-  uint64_t k_full[kTileNK], k_empty[kTileNK];
+  uint64_t k_full[kTileMaxNK], k_empty[kTileMaxNK];
   uint64_t v_full[kTileNV], v_empty[kTileNV];
   uint64_t s_full[3], p_ready[3], pv_done[3];  // per score buffer
   uint64_t o_done[4], o_free;
@@ -71,7 +76,8 @@ struct TileControl {
   alignas(16) uint32_t hdr[4][12];  // (TILE_HDR_PUT)
   alignas(16) uint32_t tl[kTlChunks * 32];  // (read in groups of up to four entries with one vector load)
   uint32_t redo_mark[4];   // per unit (of four in turn): 1 + the tile list of one that outgrew its reference
-  uint32_t redo_queue[4];  // the scheduler's: tile lists of units to be run again
+  uint32_t redo_queue[4];  // the scheduler's: tile lists of units to be run again, and (1 + the list whose maxima were
+  alignas(16) uint32_t redo_state[4];  // taken last; head and tail of the queue; whether there ever was one)
   uint8_t seen[4][16];     // a warp met keys that its rows attend to
   uint8_t max_uses[16];    // a warp's uses of item_bar, where only units that are run again use it
   float redo_max[2][4][128];  // ... of each of the row's threads (two sets, used in turn)
@@ -222,7 +228,8 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   constexpr int kQB = 128 / R;  // query blocks of the query tile
   constexpr int kC = C_, kG = 128 / C_, kW = 128;
   constexpr int kQBytes = 128 * D * 2;
-  constexpr int kNQ = tile_nq(D), kNV = kTileNV;
+  constexpr int kNQ = tile_nq(D, MODE), kNK = tile_nk(MODE), kNV = tile_nv(MODE);
+  constexpr uint32_t kNVs = kNV > 0 ? kNV : 1;
   constexpr int kKRows = PAIR ? 64 : 128;             // keys of a K tile that this CTA copies
   constexpr int kKBox = (C_ < kKRows) ? C_ : kKRows;  // ... per copy
   constexpr int kKCopies = kKRows / kKBox;            // ... and copies per 64-column slab
@@ -256,7 +263,7 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* const sQ = smem_raw;
   uint8_t* const sK = sQ + kNQ * kQBytes;
-  uint8_t* const sV = sK + kTileNK * kTileStage;
+  uint8_t* const sV = sK + kNK * kTileStage;
   uint8_t* const sOnes = sV + kNV * kTileStage;
   Ctl* const ctl = reinterpret_cast<Ctl*>(sOnes + (D == 64 ? kTileOnes : 0));
 
@@ -294,11 +301,11 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       ptx::mbar_init(&ctl->o_done[i], 1);
       ptx::mbar_init(&ctl->l_full[i], 8);
     }
-    for (int i = 0; i < kTileNK; ++i) {
+    for (int i = 0; i < kNK; ++i) {
       ptx::mbar_init(&ctl->k_full[i], kCtas);
       ptx::mbar_init(&ctl->k_empty[i], 1);
     }
-    for (int i = 0; i < kTileNV; ++i) {
+    for (int i = 0; i < kNV; ++i) {
       ptx::mbar_init(&ctl->v_full[i], kCtas);
       ptx::mbar_init(&ctl->v_empty[i], 1);
     }
@@ -328,7 +335,7 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     ptx::mbar_init(&ctl->item_bar, 16);
     ptx::mbar_init(&ctl->fold_bar, 16);
     ptx::mbar_init(&ctl->drain, 2);
-    for (int i = 0; i < 4; ++i) ctl->redo_mark[i] = 0u;
+    for (int i = 0; i < 4; ++i) ctl->redo_mark[i] = ctl->redo_state[i] = 0u;
     for (int i = 0; i < 16; ++i) ctl->max_uses[i] = 0;
     ctl->abort_flag = 0;
     ptx::fence_barrier_init();
@@ -375,18 +382,18 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   __syncthreads();
   // (the tile lists and the counters come from the kernel before; everything up to here overlaps it)
   ptx::grid_dependency_wait();
+  // (its entries, of which there are few where a slot has 256 tokens or more, are read from shared memory the first
+  // time; they lie behind what the first unit's end uses of that place)
+  constexpr int kListAt = 512;
+  static_assert(sizeof(TileControl::xch) >= 4 * (kListAt + 256 / C_ * (kMaxPersistentCtas / 2) + 48), "room for a list");
+  constexpr bool kOne = tile_lists_per_unit(D) == 2;
+  constexpr int kListBlocks = (kOne ? 1 : 2) * kQB;  // query blocks of a list
   if (MODE == kSparse && p.one_wave) {
-    // ... or the tile list of this CTA's unit from here
-    constexpr bool kOne = tile_lists_per_unit(D) == 2;
-    constexpr int kNB = (kOne ? 1 : 2) * kQB;  // query blocks of a list
+    // ... or the tile list of this CTA's unit from here: the bitmaps of its query blocks, in a place not in use yet
     const int list = (int)(PAIR ? blockIdx.x >> 1 : blockIdx.x);
-    uint32_t* const bm = reinterpret_cast<uint32_t*>(&ctl->xch[0][0][0]);  // (not in use yet)
-    if (rank == 0 && warp < kNB) fill_tile_bitmap<kNB, kOne>(p, list, warp, lane, bm);
+    if (rank == 0 && warp < kListBlocks)
+      fill_tile_bitmap<kListBlocks, kOne>(p, list, warp, lane, reinterpret_cast<uint32_t*>(&ctl->xch[0][0][0]));
     __syncthreads();
-    if (rank == 0 && warp == kSchedulerWarp) {
-      emit_tile_list<kNB, kG, kOne>(p, list, lane, bm);
-      __syncwarp();
-    }
   }
 
   if (warp < 4) {
@@ -459,8 +466,8 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
                 for (int g = 0; g < kG; ++g) grp[g] = (jlo + i * kG + g < jhi) ? (uint32_t)(jlo + i * kG + g) : kTlPad;
               }
               // K: a pair's CTAs keys 64 * rank ... + 63 of the tile each; all head-dimension columns, per slab of 64
-              const uint32_t ks = nk % kTileNK;
-              in_time = ptx::mbar_wait_relaxed_u32(k_empty_a + 8u * ks, ((nk / kTileNK) & 1) ^ 1, &ctl->abort_flag, p.wait_polls);
+              const uint32_t ks = nk % kNK;
+              in_time = ptx::mbar_wait_relaxed_u32(k_empty_a + 8u * ks, ((nk / kNK) & 1) ^ 1, &ctl->abort_flag, p.wait_polls);
               if (!in_time) break;
               ++nk;
               expect0<PAIR>(k_full0 + 8u * ks, kTileStage);
@@ -540,8 +547,8 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         if ((ent >> 28) != 1) break;
         bool q_ready = false;
         for (int i = (int)(word & kHdrTiles); i > 0; --i) {
-          const uint32_t ks = nt % kTileNK;
-          LOSA_WAIT(&ctl->k_full[ks], (nt / kTileNK) & 1);
+          const uint32_t ks = nt % kNK;
+          LOSA_WAIT(&ctl->k_full[ks], (nt / kNK) & 1);
           if (!q_ready) {
             LOSA_WAIT(&ctl->q_full[nq % kNQ], (nq / kNQ) & 1);
             q_ready = true;
@@ -601,8 +608,8 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         }
         uint32_t pv_item = 0;
         for (int i = kHasV ? (int)(word & kHdrTiles) : 0; i > 0; --i) {  // (the mass pass has no products)
-          const uint32_t vs = nv % kNV;
-          LOSA_WAIT(&ctl->v_full[vs], (nv / kNV) & 1);
+          const uint32_t vs = nv % kNVs;
+          LOSA_WAIT(&ctl->v_full[vs], (nv / kNVs) & 1);
           const uint32_t bsel = nt % 3u;
           if (pv_item == 0 && nof > 0) LOSA_WAIT(&ctl->o_free, (nof - 1) & 1);
           LOSA_WAIT(&ctl->p_ready[bsel], (nt / 3u) & 1);
@@ -634,38 +641,54 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       // ------------------------------------------------------------------ scheduler of the pair
       // A unit that outgrew its reference is run again: once for its rows' maxima (kHdrMax), once against
       // these (kHdrRedo).  Every warp marks it before it takes the next header but one, and header nu goes out
-      // when all have taken header nu - 2: the mark of unit nu - 3 is final then.  Before the end come two
-      // headers without work, for the marks of the last two units.
-      uint32_t nu = 0, nc = 0, q_head = 0, q_tail = 0;
-      int again = -1, idle = 0;  // the list whose maxima were taken last
-      int acquired = -1;         // batched launch: whose tensor maps this warp has acquired
+      // when all have taken header nu - 2: the mark of unit nu - 3 is final then.  Before the end comes a header
+      // without work: when that one has been taken, so are the marks of the last two units.
+      uint32_t nu = 0, nc = 0;
+      int idle = 0;
+      int acquired = -1;  // batched launch: whose tensor maps this warp has acquired
       bool first_item = true, drawn = false;
-      bool redone = false;
+      uint32_t own_word = 0u;  // one_wave: what tl_count holds of the CTA's unit
+      if (MODE == kSparse && p.one_wave) {
+        uint32_t* const bm = reinterpret_cast<uint32_t*>(&ctl->xch[0][0][0]);
+        own_word = emit_tile_list<kListBlocks, kG, kOne>(p, (int)(PAIR ? blockIdx.x >> 1 : blockIdx.x), lane, bm, bm + kListAt);
+        __syncwarp();
+      }
       for (;;) {
         if (p.stall) break;  // diagnostic launch: nothing is published and every wait runs out
         LOSA_WAIT_RELAXED(&ctl->hdr_empty[nu & 1u], ((nu >> 1) & 1u) ^ 1u);
         if (PAIR) ptx::fence_acq_rel_cluster();
-        if (nu >= 3u) {
-          const uint32_t mark = *reinterpret_cast<volatile uint32_t*>(&ctl->redo_mark[(nu - 3u) & 3u]);
-          if (mark != 0u) {
-            if (lane == 0) ctl->redo_queue[q_tail & 3u] = mark - 1u;
-            __syncwarp();
-            ++q_tail;
+        auto take_mark = [&](uint32_t unit_no) {
+          volatile uint32_t* const at = &ctl->redo_mark[unit_no & 3u];
+          const uint32_t mark = *at;
+          if (mark == 0u) return false;
+          __syncwarp();
+          if (lane == 0) {
+            *at = 0u;
+            ctl->redo_queue[ctl->redo_state[2]++ & 3u] = mark - 1u;
           }
-        }
+          __syncwarp();
+          return true;
+        };
+        if (nu >= 3u) take_mark(nu - 3u);
         if (lane == 0) ctl->redo_mark[nu & 3u] = 0u;
         int w = 0;
         uint32_t mode = 0u;
-        if (again >= 0) {
-          w = again;
+        uint32_t state[4];
+        ptx::ld_shared_volatile_vec<4>(ctl->redo_state, state);
+        if (state[0] != 0u) {
+          w = (int)state[0] - 1;
           mode = kHdrRedo;
-          again = -1;
-        } else if (q_head != q_tail) {
-          w = (int)*reinterpret_cast<volatile uint32_t*>(&ctl->redo_queue[q_head & 3u]);
-          ++q_head;
+          __syncwarp();
+          if (lane == 0) ctl->redo_state[0] = 0u;
+        } else if (state[1] != state[2]) {
+          w = (int)*reinterpret_cast<volatile uint32_t*>(&ctl->redo_queue[state[1] & 3u]);
           mode = kHdrMax;
-          again = w;
-          redone = true;
+          __syncwarp();
+          if (lane == 0) {
+            ctl->redo_state[0] = (uint32_t)w + 1u;
+            ctl->redo_state[1] = state[1] + 1u;
+            ctl->redo_state[3] = 1u;
+          }
         } else if (!drawn) {
           // a first unit by position, then from the counter; without pairs of CTAs a unit's two query
           // tiles are drawn one by one
@@ -682,7 +705,14 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           drawn = (PAIR ? w : w >> 1) >= p.nUnits;
         }
         if (drawn && mode == 0u) {
-          if (idle == 2) break;
+          if (idle == 1) {
+            // (all have taken the header without work: the last unit's mark is final, too)
+            LOSA_WAIT(&ctl->hdr_empty[(nu - 1u) & 1u], ((nu - 1u) >> 1) & 1u);
+            if (PAIR) ptx::fence_acq_rel_cluster();
+            if (nu < 2u || !take_mark(nu - 2u)) break;
+            idle = 0;
+            continue;
+          }
           ++idle;
           TILE_HDR_PUT(kTlSkip, 0u, 0, 0, 0, 0, nullptr, 0);
           LOSA_WAIT_RELAXED(&ctl->hdr_next, (nu - 1u) & 1u);
@@ -713,12 +743,15 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           }
         }
         if (MODE == kSparse) {
-          const uint32_t word = LOSA_IN_RANGE(list, p.cap_units) ? (uint32_t)__ldcg(p.tl_count + list) : 0u;
+          const bool own = p.one_wave && mode == 0u;  // (made by this CTA)
+          const uint32_t word = own ? own_word : LOSA_IN_RANGE(list, p.cap_units) ? (uint32_t)__ldcg(p.tl_count + list) : 0u;
           const int cnt = min((int)(word & kHdrTiles) * kG, p.tl_cap);
           TILE_HDR_PUT(kTlItem | flags | (uint32_t)w, (word & ~kHdrTiles) | odd | (uint32_t)(cnt / kG), pr, bh, b, h, o, problem);
           const uint32_t* src = p.tl_entries + (int64_t)list * p.tl_cap;
           for (int base = 0; base < cnt; base += 32) {
-            const uint32_t e = (base + lane < cnt) ? __ldcg(src + base + lane) : 0u;
+            const uint32_t e = (base + lane >= cnt) ? 0u
+                               : own ? reinterpret_cast<const uint32_t*>(&ctl->xch[0][0][0])[kListAt + base + lane]
+                                     : __ldcg(src + base + lane);
             const uint32_t c = nc & (kTlChunks - 1);
             LOSA_WAIT_RELAXED(&ctl->tl_empty[c], ((nc / kTlChunks) & 1u) ^ 1u);
             ctl->tl[c * 32 + lane] = e;
@@ -749,7 +782,8 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         LOSA_WAIT_RELAXED(&ctl->hdr_next, (nu - 1u) & 1u);
       }
       if (!p.stall) TILE_HDR_PUT(kTlEnd, 0u, 0, 0, 0, 0, nullptr, 0);
-      if (p.one_wave && lane == 0) p.redo_flag[PAIR ? blockIdx.x >> 1 : blockIdx.x] = redone ? 1 : 0;
+      if (p.one_wave && lane == 0)
+        p.redo_flag[PAIR ? blockIdx.x >> 1 : blockIdx.x] = *reinterpret_cast<volatile int*>(&ctl->redo_state[3]);
     }
   } else {
     // ------------------------------------------------------------------ softmax warps (both CTAs)
