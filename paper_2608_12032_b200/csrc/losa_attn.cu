@@ -107,7 +107,6 @@ constexpr uint32_t kHdrTiles = 0x00ffffffu, kHdrMax = 1u << 26, kHdrRedo = 1u <<
 // one query tile at a time) one for each.
 __host__ __device__ constexpr int tile_lists_per_unit(int D) { return D == 64 ? 2 : 1; }
 constexpr int kMaxParts = 8;
-constexpr int kMinTilesSaved = 8;
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLn2 = 0.6931471805599453f;
 constexpr float kRescaleThreshold = 8.0f;
@@ -2175,10 +2174,7 @@ int launch_t(const Geometry& g, const void* q, const void* k, const void* v, Par
     const int rest = (prm.nWork < ctas) ? prm.nWork : prm.nWork % ctas;
     int parts = rest > 0 ? ctas / rest : 1;
     parts = min(min(parts, kMaxParts), prm.nKb);
-    // (not for less than eight K/V tiles, about 5 us: the merge is a launch of its own, 3.5 us behind the tile kernel and 4
-    // us of the host.  A layer of 256 tokens, cut into parts of one tile, 12 us and the merge; whole, 12 us)
-    const int tiles = (prm.nKb + KT / C_ - 1) / (KT / C_);
-    if (parts >= 2 && tiles - tiles / parts >= kMinTilesSaved) {
+    if (parts >= 2) {
       prm.split_first = prm.nWork - rest;
       prm.split_parts = parts;
       prm.nUnits = prm.split_first + rest * parts;
