@@ -50,11 +50,23 @@ NCU_TRAFFIC_SOURCE = "ncu capture of the sparse forward at the Wan2.1 shape (dra
 FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustained": 1400.0}
 
 
-def launches_per_step(draws: int) -> int:
-    """Kernels of the library launched by one step.  Every attention-shaped call launches three: the
-    work units' tile lists (sparse) or the launch's counters, its kernel, and the fallback kernel, which
-    merges the partial units and returns when no row outgrew its reference; select launches two."""
-    return 3 + 2 + draws * 3 + 3 + 3
+def launches_per_call(wl, slots: int, attention_only: bool) -> int:
+    """Kernels launched by one attention-shaped call: its kernel; before it the work units' tile lists (sparse)
+    or the launch's counters, if there are more units than work slots; behind it the merge of the last wave's
+    units, if they are cut into parts."""
+    items = wl.B * wl.H * ((-(-wl.N // 128) + 1) // 2)
+    rest = items if items < slots else items % slots
+    parts = min(slots // rest if rest else 1, 8, wl.nKb)
+    cut = attention_only and parts >= 2
+    units = items + rest * (parts - 1) if cut else items
+    return 1 + (units > slots) + cut
+
+
+def launches_per_step(wl, slots: int, draws: int) -> int:
+    """Kernels of the library launched by one step: mass pass, selection (two), the sparse draws, the dense and
+    the fused call."""
+    return (launches_per_call(wl, slots, False) + 2 + (draws + 1) * launches_per_call(wl, slots, True)
+            + launches_per_call(wl, slots, False))
 
 
 def cpu_model() -> str:
@@ -633,7 +645,8 @@ def main():
             "algorithmic_bytes_per_launch": 4 * q0.numel() * 2,
         },
         "clocks": clocks.summary(),
-        "gpu_launches": args.steps * launches_per_step(args.draws),
+        "gpu_launches": args.steps * launches_per_step(
+            wl, losa.losa_work_slots(losa.binding.LOSA_OP_SPARSE_ATTN, prob), args.draws),
     }
     if batched is not None:
         line["batched"] = batched

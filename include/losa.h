@@ -103,8 +103,8 @@ size_t losa_workspace_bytes(int op, const losa_problem_t* p);
  * that each row of `mass` sums to 1 and Eq. 3's threshold theta*R becomes tau.
  * One pass over Q K^T: every row keeps a running sum of exponentials against a reference
  * score (the row's maximum over its first key tile; rows whose later scores outgrow the
- * fp32 range around it are recomputed with a running maximum by a second launch on the same
- * stream); the per-key-block sums are taken in the same pass and normalised by the row's
+ * fp32 range around it are recomputed against their maximum over all keys);
+ * the per-key-block sums are taken in the same pass and normalised by the row's
  * final sum at the end.
  *   q, k    bf16 [B,H,N,D] (strides from p)
  *   mass    f32  [B,H,nQb,nKb] contiguous, fully overwritten
@@ -190,8 +190,8 @@ int losa_select_noalloc(int32_t B, int32_t H, int32_t nQb, int32_t nKb, const fl
  *   ws       >= losa_workspace_bytes(LOSA_OP_SPARSE_ATTN, p) bytes (about 21 MB at D = 128
  *            plus the work units' tile lists: the counter the persistent CTAs draw work
  *            items from, the partial results of the last work items, which are processed in
- *            parts and merged by a second launch on the same stream, and the list of work
- *            units that this launch recomputes because their scores outgrew the reference
+ *            parts and merged by a second launch on the same stream, and a word per work
+ *            unit for those that are recomputed because their scores outgrew the reference
  *            of their first tile); not shared between calls that may run
  *            concurrently; contents undefined afterwards.  The result does not depend on
  *            timing: the same call on the same GPU gives the same bits.
