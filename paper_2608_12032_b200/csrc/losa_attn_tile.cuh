@@ -257,6 +257,10 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   constexpr bool kWantMass = (MODE == kFused || MODE == kMass);  // the block masses (Eq. 1) are wanted
   // the mass pass alone has no V, no P and no O: its score buffers go back as soon as they are read
   constexpr bool kHasV = (MODE != kMass);
+  // When a unit's place is read from its header: at its end, but in some of the mass passes, whose registers hold it
+  // and which the compiler orders better around that (16384 tokens, 12 heads, us at the start / at the end: D = 64,
+  // C = 32 957 / 1014, C = 64 828 / 911, C = 128 885 / 870; D = 128, C = 32 2050 / 2070, C = 64 986 / 969, C = 128 998 / 1010).
+  constexpr bool kInfoEarly = MODE == kMass && (D == 64 ? C_ < 128 : C_ != 64);
   constexpr int kChunkTiles = (MODE == kSparse) ? 32 / kG : (1 << 28);  // K/V tiles per chunk of the list
   static_assert(offsetof(TileControl, tl) % 16 == 0, "the tile list is read with 16-byte loads");
 
@@ -821,6 +825,13 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       if (ent == kTlSkip) continue;
       const int tile = PAIR ? (int)rank : (int)((word & kHdrOdd) != 0u);  // of the item's two query tiles
       const int my_bit = tile * kQB + sub;
+      // where the unit lies, and what else of its header only its end needs: read again then, not kept in registers
+      uint32_t info[8];
+      auto read_info = [&]() {
+        ptx::ld_shared_volatile_vec<4>(&ctl->hdr[(nu - 1u) & 3u][0], info);
+        ptx::ld_shared_volatile_vec<4>(&ctl->hdr[(nu - 1u) & 3u][4], info + 4);
+      };
+      if (kInfoEarly) read_info();
       float m_ref = 0.f, l = 0.f, le = 0.f;  // le: row sum of the unrounded exponentials (masses, LSE)
       bool ovf = false, seen = false;  // (seen: this warp met keys that its rows attend to)
       const int tiles = (int)(word & kHdrTiles);
@@ -1157,10 +1168,7 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       if (has && !redo) cnt += 2u;
 #undef TILE_REF_GIVE
 #undef TILE_REF_TAKE
-      // where the unit lies, and what else of its header only its end needs: read again, not kept in registers
-      uint32_t info[8];
-      ptx::ld_shared_volatile_vec<4>(&ctl->hdr[(nu - 1u) & 3u][0], info);
-      ptx::ld_shared_volatile_vec<4>(&ctl->hdr[(nu - 1u) & 3u][4], info + 4);
+      if (!kInfoEarly) read_info();
       const int w = (int)(info[0] & kTlItemMask);
       const bool partial = (info[0] & kTlPartial) != 0;
       const int part = (int)((info[0] >> 24) & 7u);
