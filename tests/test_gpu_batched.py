@@ -44,8 +44,8 @@ def cut_into_parts(n_items, B, H, N, D, R, C):
     return rest > 0 and ctas // rest >= 2
 
 
-# (with 148 SMs 80 and 240 items are whole on 148 slots, 63 and 189 or 74 and 222 on 74; the first two shapes,
-# 80 items on 74 slots, are skipped there)
+# (with 148 SMs every geometry has 74 slots, on which 63 and 189 or 74 and 222 items are whole; the first two shapes and
+# the last one, 80 items, are cut and skipped there)
 @pytest.mark.parametrize("B,H,N,D,R,C", [(1, 5, 128 * 31 + 70, 64, 64, 64), (1, 5, 128 * 32 - 9, 128, 128, 32),
                                          (1, 37, 128 * 4 - 9, 128, 128, 64), (1, 37, 128 * 4 - 9, 128, 128, 128),
                                          (1, 37, 128 * 4 - 9, 128, 128, 32), (1, 3, 128 * 41 + 70, 64, 64, 64),
@@ -153,3 +153,9 @@ def test_layers_of_head_dimension_64_equal_the_single_calls_bit_for_bit(R, C):
 def test_layers_of_64_row_query_blocks_on_pairs_equal_the_single_calls_bit_for_bit():
     """74 items: whole work units on the pairs of CTAs of a GPU with 148 SMs."""
     test_three_layers_in_one_launch_equal_the_single_calls_bit_for_bit(1, 37, 128 * 4 - 9, 128, 64, 64)
+
+
+@pytest.mark.parametrize("D,R,C", [(64, 64, 64), (128, 128, 32), (128, 64, 64)])
+def test_layers_of_more_than_one_wave_equal_the_single_calls_bit_for_bit(D, R, C):
+    """114 items of three batches, 342 together: on 74 slots more than one wave, whose last one is not cut."""
+    test_three_layers_in_one_launch_equal_the_single_calls_bit_for_bit(3, 19, 128 * 3 + 70, D, R, C)
