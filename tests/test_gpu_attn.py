@@ -642,3 +642,30 @@ def test_cut_items_of_which_some_parts_outgrow(D, R, C, heads):
     util.assert_output_close(
         o_s, orc.blocks_to_tokens(orc.sparse_attn(qn, kn, vn, R, C, off, idx), B, H, N), "sparse")
     assert torch.equal(o, again) and torch.equal(o_s, again_s)
+
+
+@pytest.mark.parametrize("mean", [0.0, 1.0])
+def test_row_sums_of_long_rows_lose_no_more_than_the_output_they_divide(mean):
+    """Head dimension 64, 32768 keys in one part, fp32 output.  O and the row sums of P are accumulated alike, 16 keys
+    an addition, each of which may lose an ulp (2^-23) of what it has reached: in V's mean, where neither cancels by
+    chance, the quotient is off by no more than either.  P itself is rounded to bf16: 2^-8 / sqrt(3) of a weight, rms."""
+    losa = lib()
+    N, D, blk = 32768, 64, 64
+    g = torch.Generator("cpu").manual_seed(1500)
+    q, k, v = (torch.randn(1, 1, N, D, generator=g) for _ in range(3))
+    q, k, v = q.bfloat16(), k.bfloat16(), (v + mean).bfloat16()
+    nb = N // blk
+    off, idx = util.all_blocks_csr(nb, nb)
+    qd, kd, vd = q.cuda(), k.cuda(), v.cuda()
+    outs = {"dense": losa.losa_attn(qd, kd, vd, blk, blk, out_dtype=torch.float32),
+            "sparse": losa.losa_sparse_attn(qd, kd, vd, torch.from_numpy(off).cuda(), torch.from_numpy(idx).cuda(), blk, blk,
+                                            out_dtype=torch.float32),
+            "fused": losa.losa_attn_mass(qd, kd, vd, blk, blk, out_dtype=torch.float32)[0]}
+    assert losa.losa_async_status() == 0
+    ids = np.arange(3, nb, 64, dtype=np.int32)
+    ref = orc.sparse_attn(util.to_np(q), util.to_np(k), util.to_np(v), blk, blk, off, idx, row_ids=ids)
+    for name, o in outs.items():
+        d = o[0, 0].cpu().double().numpy().reshape(nb, blk, D)[ids] - ref
+        size = np.sqrt(np.square(ref).mean())
+        assert np.sqrt(np.square(d).mean()) <= 2.0 ** -8 / 3 ** 0.5 * size, name
+        assert abs(d.mean()) <= N / 16 * 2.0 ** -23 * size, (name, d.mean() / size)
