@@ -24,18 +24,23 @@ def problem(H, N, D, seed, heads):
     far[3] = (120.0 * D ** 0.5) ** 0.5  # a score of 120 with itself, of a few with the other rows
     for h in heads:
         q[0, h, 7] = far
-        k[0, h, N - 5] = far
+        k[0, h, N - 2] = far
     return tuple(x.bfloat16() for x in (q, k, v))
 
 
-def check(H, N, D, R, C, heads, seed):
+def check(H, N, D, R, C, heads, seed, again=None):
+    """again: how many units of the dense call are run again (None: not counted, in one uncut wave)"""
     losa = lib()
     q, k, v = problem(H, N, D, seed, heads)
     qd, kd, vd = q.cuda(), k.cuda(), v.cuda()
     qn, kn, vn = (util.to_np(x) for x in (q, k, v))
     nQb, nKb = -(-N // R), -(-N // C)
     off, idx = util.random_csr(H * nQb, nKb, seed, 0.6)
-    o = losa.losa_attn(qd, kd, vd, R, C, out_dtype=torch.float32)
+    ws = torch.empty(losa.losa_workspace_bytes(losa.binding.LOSA_OP_ATTN, losa.make_problem(qd, R, C)), dtype=torch.uint8,
+                     device="cuda")
+    o = losa.losa_attn(qd, kd, vd, R, C, out_dtype=torch.float32, ws=ws)
+    if again is not None:
+        assert int(ws[:8].view(torch.int32)[1]) == again
     o_s = losa.losa_sparse_attn(qd, kd, vd, torch.from_numpy(off).cuda(), torch.from_numpy(idx).cuda(), R, C,
                                 out_dtype=torch.float32)
     mass = losa.losa_block_mass(qd, kd, R, C)
@@ -56,38 +61,51 @@ def test_as_many_units_as_slots_and_one_more_or_less(D, R, C, more):
     losa = lib()
     prob = losa.make_problem(torch.empty((1, 1, 256, D), dtype=torch.bfloat16, device="cuda"), R, C)
     H = losa.losa_work_slots(losa.binding.LOSA_OP_ATTN, prob) + more  # one pair of query tiles per head
-    check(H, 250, D, R, C, (0, H // 2, H - 1), 1200 + more)
+    # (of one more than slots the last is cut into parts of one K/V tile, which takes its reference from all its keys)
+    check(H, 250, D, R, C, (0, H // 2, H - 1), 1200 + more, again=2 if more > 0 else None)
 
 
 @pytest.mark.parametrize("D,R,C", [(64, 64, 64), (64, 128, 128), (128, 128, 32), (128, 64, 64)])
 @pytest.mark.parametrize("tiles", [2, 9])
 def test_short_items_cut_into_as_many_parts_as_there_can_be(D, R, C, tiles):
-    """One or five items of one head: parts of one K/V tile or less, made, run, run again and merged."""
-    check(1, 128 * tiles - 30, D, R, C, (0,), 1300 + tiles)
+    """One item of one head in parts of one key block, which never outgrow their reference; five in parts of two K/V
+    tiles at most, of which the first query block's last part meets its far key in the second and is run again."""
+    check(1, 128 * tiles - 30, D, R, C, (0,), 1300 + tiles, again=1 if tiles == 9 else 0)
 
 
-def test_captured_behind_a_memset_and_behind_another_stream():
+@pytest.mark.parametrize("H", [2, 80])
+@pytest.mark.parametrize("sparse", [False, True])
+def test_captured_behind_a_memset_and_behind_another_stream(H, sparse):
     """The first launch of a call is a dependent of whatever is ahead of it in the stream: a kernel, a memset, a copy
     and the join with another stream, in a captured graph as well."""
     losa = lib()
-    q, k, v = (x.cuda() for x in problem(2, 700, 64, 1400, (0,)))
-    want = losa.losa_attn(q, k, v, 64, 64)
-    o, q2 = torch.empty_like(want), torch.empty_like(q)
-    ws = torch.empty(losa.losa_workspace_bytes(losa.binding.LOSA_OP_ATTN, losa.make_problem(q, 64, 64)), dtype=torch.uint8,
-                     device="cuda")
+    N, blk = 250, 64
+    q, k, v = (x.cuda() for x in problem(H, N, 64, 1400, (0,)))
+    nb = -(-N // blk)
+    csr = tuple(torch.from_numpy(x).cuda() for x in util.random_csr(H * nb, nb, 1401, 0.6)) if sparse else ()
+    call = losa.losa_sparse_attn if sparse else losa.losa_attn
+    op = losa.binding.LOSA_OP_SPARSE_ATTN if sparse else losa.binding.LOSA_OP_ATTN
+    prob = losa.make_problem(q, blk, blk)
+    assert (H > losa.losa_work_slots(op, prob)) == (H == 80)  # 80: a launch ahead of the kernel prepares the units
+    want = call(q, k, v, *csr, blk, blk)
+    outs = [torch.full_like(want, 7.0) for _ in range(3)]
+    q2, v2 = torch.empty_like(q), v.clone()
+    ws = torch.empty(losa.losa_workspace_bytes(op, prob), dtype=torch.uint8, device="cuda")
     torch.cuda.synchronize()
     graph, side = torch.cuda.CUDAGraph(), torch.cuda.Stream()
     with torch.cuda.graph(graph):
-        o.zero_()
-        losa.losa_attn(q, k, v, 64, 64, out=o, ws=ws)
+        q2.zero_()
+        v2.zero_()  # directly ahead of the call that reads it: o is 0
+        call(q, k, v2, *csr, blk, blk, out=outs[0], ws=ws)
+        v2.copy_(v)
+        call(q, k, v2, *csr, blk, blk, out=outs[1], ws=ws)
         side.wait_stream(torch.cuda.current_stream())
         with torch.cuda.stream(side):
-            q2.zero_()
             q2.copy_(q)
         torch.cuda.current_stream().wait_stream(side)
-        losa.losa_attn(q2, k, v, 64, 64, out=o, ws=ws)
+        call(q2, k, v, *csr, blk, blk, out=outs[2], ws=ws)
     for _ in range(3):
         graph.replay()
     torch.cuda.synchronize()
     assert losa.losa_async_status() == 0
-    assert torch.equal(o, want)
+    assert not outs[0].any() and torch.equal(outs[1], want) and torch.equal(outs[2], want)
