@@ -102,6 +102,7 @@ constexpr uint32_t kTlRagged = 1u << 20;  // tile entry: the sequence ends insid
 // What is said of a unit's tile list: how many K/V tiles, which query tiles list any (kHdrHas << query
 // tile), and whether query tile 1 lists its first in the second K/V tile
 // (a unit that is one query tile: bit kHdrHas alone, and which of the item's two it is, kHdrOdd)
+constexpr uint32_t kHdrSetShift = 24;  // (of a unit that is run again)
 constexpr uint32_t kHdrTiles = 0x00ffffffu, kHdrMax = 1u << 26, kHdrRedo = 1u << 27, kHdrOdd = 1u << 28, kHdrLate = 1u << 29, kHdrHas = 1u << 30;
 // Tile lists per work unit: one for its pair of query tiles, or (head dimension 64, where a CTA works on
 // one query tile at a time) one for each.

@@ -28,9 +28,13 @@
 // group has two tile periods for one tile.  The exponentials are taken against a reference that
 // never moves within a work unit (the row maximum over the first key tile the row attends to,
 // handed from the group that meets that tile to the other); a unit whose scores outgrow it is run again
-// by the same CTAs, first for its rows' maxima and then against these.  (A launch of its own for such units
+// by the same CTAs, against the logarithm of the row sums if these are still finite (scores up to about 80 nats above
+// the first tile's) - no row's maximum is above that, nor further below than the logarithm of its keys - and else
+// first for its rows' maxima and then against these.  (A launch of its own for such units
 // cost every call 4 - 6 us and a launch; 2048 tokens, 4 heads, D = 64: 26.9 -> 21.5 us with the launch of the lists
-// gone as well.)
+// gone as well.  16384 tokens, 12 heads, every unit 60 nats above its first tiles from the third on, us with that launch /
+// with a pass for the maxima / without: D = 128 dense 2600 / 3090 / 2390, masses 2040 / 2490 / 1760; D = 64 dense
+// 2130 / 2220 / 1730, masses 2575 / 2140 / 1640.)
 //
 // Barriers that both CTAs feed (operands landed, P written, O read out, tile-list chunk consumed)
 // live in the first CTA; barriers that the MMAs' completion feeds in both CTAs are reached with a
@@ -58,6 +62,9 @@ constexpr int kTileOnes = 2048;
 #define LOSA_POLY_OF_MASS 4
 #endif
 constexpr float kTileSafeLow = 8.6736173798840355e-19f;  // 2^-60
+// A row sum in this range says how high the row's scores go.  (A score that left the exponential's own range counts as
+// infinite or 2^127; one that fell below it as zero.)
+constexpr float kTileKnownLow = 7.8886090522101181e-31f, kTileKnownHigh = 1.3292279957849159e+36f;  // 2^-100, 2^120
 
 struct TileControl {
   uint64_t q_full[2], q_empty[2];
@@ -76,12 +83,12 @@ struct TileControl {
   alignas(16) uint32_t hdr[4][12];  // (TILE_HDR_PUT)
   alignas(16) uint32_t tl[kTlChunks * 32];  // (read in groups of up to four entries with one vector load)
   uint32_t redo_mark[4];   // per unit (of four in turn): 1 + the tile list of one that outgrew its reference
-  uint32_t redo_queue[4];  // the scheduler's: tile lists of units to be run again, and (1 + the list whose maxima were
+  uint32_t redo_need[4];   // ... whether its rows' maxima have to be taken first (directly behind the marks)
+  uint32_t redo_queue[4];  // the scheduler's: units to be run again (kRedoList ...), and (1 + the one whose maxima were
   alignas(16) uint32_t redo_state[4];  // taken last; head and tail of the queue; whether there ever was one)
   uint8_t seen[4][16];     // a warp met keys that its rows attend to
   uint8_t max_uses[16];    // a warp's uses of item_bar, where only units that are run again use it
-  float redo_max[2][4][128];  // ... of each of the row's threads (two sets, used in turn)
-  float redo_ref[128];     // the rows' maxima, of a unit that is run again
+  float redo_ref[4][128];  // per unit (of four in turn): what its rows are run again against
   float half_max[2][2][128];  // ... over each half of the tile it is taken from
   float ref[2][128];       // the rows' reference, from the group that met the first tile to the other
   float xch[2][8][128];    // the rows' partial sums at the end of an item (two sets, used in turn):
@@ -119,6 +126,10 @@ __device__ __forceinline__ void tile_key_range(const Params& p, uint32_t ent, in
 // list of headers and tiles entry by entry, in the dense modes too, that took more instructions per
 // tile than the exponentials: 529 warp instructions per 64 scores of a warp, 224 of them arithmetic.)
 //
+// A unit in the scheduler's queue: its tile list, which of redo_ref is its own, whether its rows' maxima are needed.
+constexpr uint32_t kRedoList = 0x03ffffffu, kRedoSetShift = 28u, kRedoNeed = 1u << 30;
+static_assert(2u * (kTlItemMask + 1u) - 1u <= kRedoList, "a tile list's number");
+
 // Next header (whole warp); `nu` is the warp's unit counter.  N: how much of it the role reads, in groups of
 // four words.
 #define TILE_HDR_NEXT(hdr_, N)                                                             \
@@ -263,6 +274,7 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   constexpr bool kInfoEarly = MODE == kMass && (D == 64 ? C_ < 128 : C_ != 64);
   constexpr int kChunkTiles = (MODE == kSparse) ? 32 / kG : (1 << 28);  // K/V tiles per chunk of the list
   static_assert(offsetof(TileControl, tl) % 16 == 0, "the tile list is read with 16-byte loads");
+  static_assert(offsetof(TileControl, redo_need) == offsetof(TileControl, redo_mark) + 16, "reached from the marks");
 
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* const sQ = smem_raw;
@@ -339,7 +351,7 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     ptx::mbar_init(&ctl->item_bar, 16);
     ptx::mbar_init(&ctl->fold_bar, 16);
     ptx::mbar_init(&ctl->drain, 2);
-    for (int i = 0; i < 4; ++i) ctl->redo_mark[i] = ctl->redo_state[i] = 0u;
+    for (int i = 0; i < 4; ++i) ctl->redo_mark[i] = ctl->redo_need[i] = ctl->redo_state[i] = 0u;
     for (int i = 0; i < 16; ++i) ctl->max_uses[i] = 0;
     ctl->abort_flag = 0;
     ptx::fence_barrier_init();
@@ -643,8 +655,8 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       }
     } else if (warp == kSchedulerWarp && rank == 0) {
       // ------------------------------------------------------------------ scheduler of the pair
-      // A unit that outgrew its reference is run again: once for its rows' maxima (kHdrMax), once against
-      // these (kHdrRedo).  Every warp marks it before it takes the next header but one, and header nu goes out
+      // A unit that outgrew its reference is run again: for its rows' maxima (kHdrMax), where these are needed, and
+      // against what it left or these left in redo_ref (kHdrRedo; which of the four: kHdrSet).  Every warp marks it before it takes the next header but one, and header nu goes out
       // when all have taken header nu - 2: the mark of unit nu - 3 is final then.  Before the end comes a header
       // without work: when that one has been taken, so are the marks of the last two units.
       uint32_t nu = 0, nc = 0;
@@ -665,31 +677,36 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           volatile uint32_t* const at = &ctl->redo_mark[unit_no & 3u];
           const uint32_t mark = *at;
           if (mark == 0u) return false;
+          const uint32_t need = *reinterpret_cast<volatile uint32_t*>(&ctl->redo_need[unit_no & 3u]);
           __syncwarp();
           if (lane == 0) {
             *at = 0u;
-            ctl->redo_queue[ctl->redo_state[2]++ & 3u] = mark - 1u;
+            ctl->redo_queue[ctl->redo_state[2]++ & 3u] =
+                (mark - 1u) | ((unit_no & 3u) << kRedoSetShift) | (need != 0u ? kRedoNeed : 0u);
           }
           __syncwarp();
           return true;
         };
         if (nu >= 3u) take_mark(nu - 3u);
-        if (lane == 0) ctl->redo_mark[nu & 3u] = 0u;
+        if (lane == 0) ctl->redo_mark[nu & 3u] = ctl->redo_need[nu & 3u] = 0u;
         int w = 0;
         uint32_t mode = 0u;
+        bool again = false;  // (a unit's first time again)
         uint32_t state[4];
         ptx::ld_shared_volatile_vec<4>(ctl->redo_state, state);
         if (state[0] != 0u) {
-          w = (int)state[0] - 1;
-          mode = kHdrRedo;
+          w = (int)((state[0] - 1u) & kRedoList);
+          mode = kHdrRedo | (((state[0] - 1u) >> kRedoSetShift & 3u) << kHdrSetShift);
           __syncwarp();
           if (lane == 0) ctl->redo_state[0] = 0u;
         } else if (state[1] != state[2]) {
-          w = (int)*reinterpret_cast<volatile uint32_t*>(&ctl->redo_queue[state[1] & 3u]);
-          mode = kHdrMax;
+          const uint32_t e = *reinterpret_cast<volatile uint32_t*>(&ctl->redo_queue[state[1] & 3u]);
+          w = (int)(e & kRedoList);
+          mode = ((e & kRedoNeed) ? kHdrMax : kHdrRedo) | ((e >> kRedoSetShift & 3u) << kHdrSetShift);
+          again = true;
           __syncwarp();
           if (lane == 0) {
-            ctl->redo_state[0] = (uint32_t)w + 1u;
+            if (e & kRedoNeed) ctl->redo_state[0] = e + 1u;
             ctl->redo_state[1] = state[1] + 1u;
             ctl->redo_state[3] = 1u;
           }
@@ -726,7 +743,7 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         const int list = w;  // its tile list
         const uint32_t odd = ((!PAIR && (w & 1)) ? kHdrOdd : 0u) | mode;
         if (!PAIR) w >>= 1;
-        if (mode == kHdrMax && !p.one_wave && lane == 0 && atomicExch(p.redo_flag + w, 1) == 0) atomicAdd(p.redo_count, 1);
+        if (again && !p.one_wave && lane == 0 && atomicExch(p.redo_flag + w, 1) == 0) atomicAdd(p.redo_count, 1);
         uint32_t flags = 0;
         if (w >= p.split_first) {
           const int r = w - p.split_first;
@@ -893,7 +910,8 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           if (MODE == kSparse) TILE_CHUNK_DONE();
         }
         kq += (uint32_t)tiles;
-        float* const xset = &ctl->redo_max[nitem & 1][0][0];
+        // (where the unit would leave its sums)
+        float* const xset = kOneGroup ? &ctl->xch[0][0][0] + ((nu - 1u) & 3u) * 512 : &ctl->xch[nitem & 1][0][0];
         xset[quarter * 128 + row] = mx;
         if (kOneGroup) ctl->max_uses[sw] = (uint8_t)(nitem + 1u);
         __syncwarp();
@@ -901,7 +919,7 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         LOSA_WAIT(&ctl->item_bar, nitem & 1);
         if (!kOneGroup) ++nitem;
         // (every thread of the row finds and leaves the same value)
-        ctl->redo_ref[row] = fmaxf(fmaxf(xset[row], xset[128 + row]), fmaxf(xset[256 + row], xset[384 + row])) * p.scale_log2;
+        ctl->redo_ref[(word >> kHdrSetShift) & 3u][row] = fmaxf(fmaxf(xset[row], xset[128 + row]), fmaxf(xset[256 + row], xset[384 + row])) * p.scale_log2;
         continue;
       }
       // ---- the reference of the unit: the rows' maximum over the first key tile their query block
@@ -911,9 +929,9 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       // and is exchanged when the loop below comes to it.
       constexpr bool kLazyRef = kQB > 1 && MODE == kSparse;
       const uint32_t rs = (cnt >> 1) & 1u;
-      const bool redo = (word & kHdrRedo) != 0;  // against the rows' maxima
+      const bool redo = (word & kHdrRedo) != 0;  // against what the unit's rows are known to reach
       bool have_ref = !has || redo;
-      if (redo) m_ref = ctl->redo_ref[row];
+      if (redo) m_ref = ctl->redo_ref[(word >> kHdrSetShift) & 3u][row];
       int ref_tile = (PAIR && tile == 1 && (word & kHdrLate)) ? 1 : 0;
       bool listed_only = true;  // the maximum is over the keys the row attends to
       // The maximum of this half's 64 columns of tile i of the unit, whose group lies at `at` in the list's
@@ -1110,6 +1128,8 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
 #pragma unroll
             for (int j = 0; j < kHB; ++j) tsum += eacc[j].x + eacc[j].y;
           }
+          // (in the mass pass l is le once more; without it, and with a vote over the whole sums at the unit's end, the
+          // compiler ordered the exponentials worse: 1024 key blocks 4090 us against 4300)
           if (!kSumCol) {
             ovf = ovf || __any_sync(0xffffffffu, !(tsum <= kSplitSafeSum));
             l += tsum;
@@ -1187,6 +1207,19 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         }
       };
       if (!kSumCol && ovf && !redo && lane == 0) hand_over();
+      // What the row is run again against, should any of the unit's rows have outgrown its reference, from the row's
+      // whole sum (one thread of a row).
+      auto leave_ref = [&](float sum) {
+        ctl->redo_ref[(nu - 1u) & 3u][row] = (sum > 0.f) ? m_ref + __log2f(sum) : m_ref;
+        if (!(sum < kTileKnownHigh) || (kLazyRef && seen && sum < kTileKnownLow)) {
+          if (PAIR) {
+            ptx::st_cluster_u32(redo_mark0 + 16u + 4u * ((nu - 1u) & 3u), 1u);
+            ptx::fence_acq_rel_cluster();
+          } else {
+            *reinterpret_cast<volatile uint32_t*>(&ctl->redo_need[(nu - 1u) & 3u]) = 1u;
+          }
+        }
+      };
       // Columns c0 ... of the rows of O of this warp's 32 lanes, a row a lane, to `dst` (rows of `stride` elements of
       // 4 bytes, or of 2 and rounded); those from `rows` on do not exist.  Groups of lanes write a row's columns
       // together: with a row a lane every store of 16 bytes went to 32 lines, and the 2048 cycles that took held up
@@ -1279,11 +1312,12 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           if (c0 == 0) {
             // rows whose own keys lie 40 nats below a reference taken over other keys: their weights may
             // have lost their tail
+            if (!redo && half == 0) leave_ref(l);
             const bool low = kLazyRef && seen && l < kTileSafeLow;
             if ((kLazyRef || kSumCol) && !redo &&
                 __any_sync(0xffffffffu, low || (kSumCol && !(l <= kSplitSafeSum))) && lane == 0)
               hand_over();
-            // (against their maxima only rows that met a score that is not a number add up to that much)
+            // (run again only rows that met a score that is not a number add up to that much)
             if (redo && !(l <= kSplitSafeSum)) l = __int_as_float(0x7fc00000);
             inv = (l == 0.f) ? 0.f : 1.f / l;
             if (partial && half == 0 && T < p.nQt && LOSA_IN_RANGE(pslot, p.cap_part_rows)) p.part_ml[pslot] = make_float2(m_ref, l);
@@ -1329,10 +1363,12 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           for (int c = 0; c < kOC; ++c) r[c] = 0u;
         }
         if (kSumCol && !redo && __any_sync(0xffffffffu, !(l <= kSplitSafeSum)) && lane == 0) hand_over();
-        // (against their maxima only rows that met a score that is not a number add up to that much)
+        if (!redo && quarter == 0) leave_ref(l);
+        // (run again only rows that met a score that is not a number add up to that much)
         if (redo && !(l <= kSplitSafeSum)) l = __int_as_float(0x7fc00000);
         store_o(r, c0, (l == 0.f) ? 0.f : 1.f / l, std::integral_constant<int, kOC>());
       }
+      if (!kHasV && !redo && quarter == 0) leave_ref(l);
       if (kWantMass) {
         // ---- fused construction step: the block masses of this CTA's query tile (Eq. 1).  The
         // reference did not move during the item, so a row's weight is 1 / (its sum of unrounded

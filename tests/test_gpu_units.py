@@ -73,6 +73,40 @@ def test_short_items_cut_into_as_many_parts_as_there_can_be(D, R, C, tiles):
     check(1, 128 * tiles - 30, D, R, C, (0,), 1300 + tiles, again=1 if tiles == 9 else 0)
 
 
+@pytest.mark.parametrize("D,R,C", [(64, 64, 64), (64, 128, 32), (128, 128, 128), (128, 64, 64)])
+def test_units_run_again_with_and_without_their_maxima(D, R, C):
+    """Keys 60 nats above the first tile leave finite row sums, which the unit's rows are run again against; keys 150
+    nats above do not, and their maxima are taken first.  Both, and units that are not run again, in turn and several of
+    a kind behind one another, more than one to a work slot."""
+    losa = lib()
+    H, N = 2 * losa.losa_work_slots(losa.binding.LOSA_OP_ATTN, losa.make_problem(
+        torch.empty((1, 1, 256, D), dtype=torch.bfloat16, device="cuda"), R, C)) + 40, 250
+    g = torch.Generator("cpu").manual_seed(1600)
+    q = torch.randn(1, H, N, D, generator=g) * 0.3 + 1.0
+    k = torch.randn(1, H, N, D, generator=g) * 0.3
+    v = torch.randn(1, H, N, D, generator=g)
+    nats = torch.tensor([0.0, 60.0, 60.0, 150.0, 60.0, 150.0, 150.0])[torch.arange(H) * 5 // 3 % 7]
+    k[0, :, 140:] += (nats * D ** 0.5 / D)[:, None, None]
+    q, k, v = q.bfloat16(), k.bfloat16(), v.bfloat16()
+    qd, kd, vd = q.cuda(), k.cuda(), v.cuda()
+    qn, kn, vn = (util.to_np(x) for x in (q, k, v))
+    ref, ref_m = orc.dense_attn(qn, kn, vn), orc.block_mass(qn, kn, R, C)
+    off, idx = util.all_blocks_csr(H * -(-N // R), -(-N // C))
+    o = losa.losa_attn(qd, kd, vd, R, C, out_dtype=torch.float32)
+    o_s = losa.losa_sparse_attn(qd, kd, vd, torch.from_numpy(off).cuda(), torch.from_numpy(idx).cuda(), R, C,
+                                out_dtype=torch.float32)
+    mass, lse = losa.losa_block_mass(qd, kd, R, C, return_lse=True)
+    o_f, mass_f, lse_f = losa.losa_attn_mass(qd, kd, vd, R, C, return_lse=True, out_dtype=torch.float32)
+    assert losa.losa_async_status() == 0
+    for name, x in (("dense", o), ("sparse", o_s), ("fused", o_f)):
+        util.assert_output_close(x, ref, name)
+    for m in (mass, mass_f):
+        assert np.abs(m.cpu().numpy().reshape(ref_m.shape) - ref_m).max() <= util.MASS_TOL
+    want = torch.logsumexp(q[0].double() @ k[0].double().transpose(1, 2) / D ** 0.5, -1)
+    for x in (lse, lse_f):
+        assert (x[0].cpu().double() - want).abs().max() <= 1e-4  # 150 + 64 sums in fp32: 150 * 2^-23 each
+
+
 @pytest.mark.parametrize("H", [2, 80])
 @pytest.mark.parametrize("sparse", [False, True])
 def test_captured_behind_a_memset_and_behind_another_stream(H, sparse):
