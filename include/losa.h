@@ -239,9 +239,9 @@ size_t losa_workspace_bytes_batched(int op, const losa_problem_t* p, int32_t n_l
  * of kind `op` (a LOSA_OP_* attention call) occupies on the current device.  A call's work items -
  * pairs of 128-row query tiles per (batch, head) - are spread over these slots, and the items of
  * a last, partly filled wave are cut into parts and merged; callers that compare results bit for
- * bit across calls of different sizes need this number.  0 for an invalid problem or op.
- * (On a device that cannot hold a pair of CTAs the paired kernels fall back to single CTAs; the
- * number returned does not know that.) */
+ * bit across calls of different sizes need this number.  0 for an invalid problem or op,
+ * and on a device that cannot hold a pair of CTAs if the call needs pairs (head dimension 128): such calls return
+ * LOSA_ERR_UNSUPPORTED there. */
 int32_t losa_work_slots(int op, const losa_problem_t* p);
 
 /* Dense softmax attention o = softmax(q k^T * scale) v over the N valid keys: the paper's

@@ -230,11 +230,11 @@ __device__ __forceinline__ void transpose_chunks(uint32_t* r, int lane) {
 }
 
 template <int D, int R, int C_, int MODE, bool PAIR>
-__global__ void __launch_bounds__(Lay<true>::kThreads, 1)
+__global__ void __launch_bounds__(Lay::kThreads, 1)
 losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                  const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_kw,
                  const __grid_constant__ CUtensorMap map_vw, const Params p) {
-  using L = Lay<true>;
+  using L = Lay;
   static_assert(PAIR ? D == 128 : D == 64, "pairs at head dimension 128, one CTA at 64");
   constexpr int kQB = 128 / R;  // query blocks of the query tile
   constexpr int kC = C_, kG = 128 / C_, kW = 128;
@@ -268,9 +268,11 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   constexpr bool kWantMass = (MODE == kFused || MODE == kMass);  // the block masses (Eq. 1) are wanted
   // the mass pass alone has no V, no P and no O: its score buffers go back as soon as they are read
   constexpr bool kHasV = (MODE != kMass);
-  // When a unit's place is read from its header: at its end, but in some of the mass passes, whose registers hold it
-  // and which the compiler orders better around that (16384 tokens, 12 heads, us at the start / at the end: D = 64,
-  // C = 32 957 / 1014, C = 64 828 / 911, C = 128 885 / 870; D = 128, C = 32 2050 / 2070, C = 64 986 / 969, C = 128 998 / 1010).
+  // When a unit's place is read from its header: at its end, but in those mass passes that came out faster with it in
+  // registers from the unit's start.  That is the compiler's ordering of the exponentials, not the eight registers, so
+  // the line lies where it was measured, and has to be measured again when the loop changes (16384 tokens, 12 heads, us at
+  // the start / at the end: D = 64, C = 32 957 / 1004, C = 64 827 / 913, C = 128 879 / 830; D = 128, C = 32 1029 / 1034,
+  // C = 64 974 / 959, C = 128 985 / 999).
   constexpr bool kInfoEarly = MODE == kMass && (D == 64 ? C_ < 128 : C_ != 64);
   constexpr int kChunkTiles = (MODE == kSparse) ? 32 / kG : (1 << 28);  // K/V tiles per chunk of the list
   static_assert(offsetof(TileControl, tl) % 16 == 0, "the tile list is read with 16-byte loads");

@@ -498,10 +498,10 @@ def test_block_mass_with_one_key_far_above_the_reference(D, col):
 @pytest.mark.parametrize("D,BLK", [(128, 128), (64, 64)])
 def test_rows_that_outgrow_their_reference_in_whole_and_cut_work_units(D, BLK):
     """The forward keeps, per work unit, the reference of the unit's first tile; a unit whose scores
-    rise far above it is handed to a second launch that moves the reference.  More work items than
+    rise far above it is run again against a reference of its rows' own.  More work items than
     SMs, so that some units are whole items and the last ones are parts; half of the heads carry
     keys 60 nats above the rest from the third tile on, the other half do not (their units must
-    not be touched by the second launch: compared with the oracle all the same)."""
+    not be run again: compared with the oracle all the same)."""
     losa = lib()
     sms = torch.cuda.get_device_properties(0).multi_processor_count
     B, N = 1, 128 * 7 + 50
@@ -535,8 +535,8 @@ def test_rows_that_outgrow_their_reference_in_whole_and_cut_work_units(D, BLK):
 @pytest.mark.parametrize("D,R,C", [(128, 64, 64), (64, 64, 64), (64, 128, 32), (128, 128, 64)])
 def test_every_unit_outgrows_its_reference(D, R, C):
     """Units of two key tiles whose second lies 60 nats above the first, in every head: both query tiles
-    of every unit find it outgrown, several units apart from one another, and the list of the second
-    launch has to hold each unit once."""
+    of every unit find it outgrown, several units apart from one another, and each unit has to be
+    run again once."""
     losa = lib()
     sms = torch.cuda.get_device_properties(0).multi_processor_count
     B, H, N = 1, 2 * sms + 5, 256  # one pair of query tiles per head
@@ -563,8 +563,8 @@ def test_every_unit_outgrows_its_reference(D, R, C):
         else:
             mass = losa.losa_block_mass(qd, kd, R, C, ws=ws)
         assert np.abs(mass.cpu().numpy().reshape(ref_m.shape) - ref_m).max() <= util.MASS_TOL
-        # the head of the workspace: work items drawn, units listed
-        assert int(ws[:8].view(torch.int32)[1]) == B * H, "every unit is listed once"
+        # the head of the workspace: work items drawn, units run again
+        assert int(ws[:8].view(torch.int32)[1]) == B * H, "every unit is run again once"
     assert losa.losa_async_status() == 0
     util.assert_output_close(o, ref, "dense")
     util.assert_output_close(o_s, ref, "sparse")
@@ -633,7 +633,7 @@ def test_cut_items_of_which_some_parts_outgrow(D, R, C, heads):
     ws = torch.empty(losa.losa_workspace_bytes(losa.binding.LOSA_OP_ATTN, losa.make_problem(qd, R, C)),
                      dtype=torch.uint8, device="cuda")
     o = losa.losa_attn(qd, kd, vd, R, C, out_dtype=torch.float32, ws=ws)
-    assert int(ws[:8].view(torch.int32)[1]) >= len(heads)  # units were listed
+    assert int(ws[:8].view(torch.int32)[1]) >= len(heads)  # units were run again
     again = losa.losa_attn(qd, kd, vd, R, C, out_dtype=torch.float32, ws=ws)
     o_s = losa.losa_sparse_attn(qd, kd, vd, offd, idxd, R, C, out_dtype=torch.float32)
     again_s = losa.losa_sparse_attn(qd, kd, vd, offd, idxd, R, C, out_dtype=torch.float32)
