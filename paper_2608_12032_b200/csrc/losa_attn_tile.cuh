@@ -403,6 +403,7 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   // (its entries, of which there are few where a slot has 256 tokens or more, are read from shared memory the first
   // time; they lie behind what the first unit's end uses of that place)
   constexpr int kListAt = 512;
+  static_assert(2 * kQB * ((256 / C_ * (kMaxPersistentCtas / 2) + 31) / 32) <= kListAt, "room for the bitmaps");
   static_assert(sizeof(TileControl::xch) >= 4 * (kListAt + 256 / C_ * (kMaxPersistentCtas / 2) + 48), "room for a list");
   constexpr bool kOne = tile_lists_per_unit(D) == 2;
   constexpr int kListBlocks = (kOne ? 1 : 2) * kQB;  // query blocks of a list
@@ -805,7 +806,7 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         LOSA_WAIT_RELAXED(&ctl->hdr_next, (nu - 1u) & 1u);
       }
       if (!p.stall) TILE_HDR_PUT(kTlEnd, 0u, 0, 0, 0, 0, nullptr, 0);
-      if (p.one_wave && lane == 0)
+      if (p.one_wave && p.split_parts > 1 && lane == 0)
         p.redo_flag[PAIR ? blockIdx.x >> 1 : blockIdx.x] = *reinterpret_cast<volatile int*>(&ctl->redo_state[3]);
     }
   } else {
