@@ -103,7 +103,7 @@ size_t losa_workspace_bytes(int op, const losa_problem_t* p);
  * that each row of `mass` sums to 1 and Eq. 3's threshold theta*R becomes tau.
  * One pass over Q K^T: every row keeps a running sum of exponentials against a reference
  * score (the row's maximum over its first key tile; rows whose later scores outgrow the
- * fp32 range around it are recomputed against their maximum over all keys);
+ * fp32 range around it are recomputed against a reference from all their keys);
  * the per-key-block sums are taken in the same pass and normalised by the row's
  * final sum at the end.
  *   q, k    bf16 [B,H,N,D] (strides from p)
