@@ -104,6 +104,7 @@ struct Params {
   // Work units: items [0, split_first) whole, items [split_first, nWork) in split_parts parts of
   // their key-block lists each (the last, partly filled wave of the persistent grid is cut finer).
   int nUnits, split_first, split_parts;
+  Divisor by_parts, by_pairs, by_heads, by_problem;  // split_parts, nPairs, H, B * H
   // Sparse mode: the merged tile lists of all units, built by build_tile_lists_kernel before the
   // attention kernel: unit u owns tl_entries[u * tl_cap ...], tl_count[u] of them (padded to whole tiles).
   uint32_t* tl_entries;
@@ -168,6 +169,11 @@ struct Params {
     }                                                            \
   } while (0)
 
+// An item's place: the problem of a batched launch, the head (b * H + h) in it and the pair of query tiles.
+__device__ __forceinline__ void item_place(const Params& p, int w, int& problem, int& bh, int& pr) {
+  problem = p.by_problem.divmod(p.by_pairs.divmod(w, pr), bh);
+}
+
 // ---- merge of the partial units: for every row of the split items, combine the parts' unnormalised
 // O, reference maximum and row sum (the usual log-sum-exp merge) and write the attention output.
 // (slot0: of part 0; part s of the row lies 256 s slots further.  Lanes are the columns.)
@@ -183,10 +189,11 @@ __device__ __forceinline__ void load_part_row(const Params& p, int64_t slot, int
   }
 }
 template <int D>
-__device__ __forceinline__ void store_merged_row(const Params& p, int pbh, int grow, int lane, const float* acc, float inv) {
-  const int bh = pbh % (p.B * p.H);
-  void* const o_base = (p.problems != nullptr) ? p.problems[pbh / (p.B * p.H)].o : p.o;
-  const int64_t off = (int64_t)(bh / p.H) * p.sb + (int64_t)(bh % p.H) * p.sh + (int64_t)grow * p.sn + lane * (D / 32);
+__device__ __forceinline__ void store_merged_row(const Params& p, int problem, int bh, int grow, int lane, const float* acc, float inv) {
+  void* const o_base = (p.problems != nullptr) ? p.problems[problem].o : p.o;
+  int h;
+  const int b = p.by_heads.divmod(bh, h);
+  const int64_t off = (int64_t)b * p.sb + (int64_t)h * p.sh + (int64_t)grow * p.sn + lane * (D / 32);
   if (p.o_f32) {
     float* dst = static_cast<float*>(o_base) + off;
     if constexpr (D == 128)
@@ -217,8 +224,8 @@ __device__ __forceinline__ void merge_parts(const Params& p, int cta, int ctas) 
   const int rows = (p.nWork - p.split_first) * 256;
   for (int i = cta * warps + (threadIdx.x >> 5); i < rows; i += ctas * warps) {
     const int r = i >> 8, qt = (i >> 7) & 1, row = i & 127;
-    const int w = p.split_first + r;
-    const int pbh = w / p.nPairs, pr = w % p.nPairs;
+    int problem, bh, pr;
+    item_place(p, p.split_first + r, problem, bh, pr);
     const int T = 2 * pr + qt, grow = T * 128 + row;
     if (grow >= p.N) continue;
     const int64_t slot0 = ((int64_t)r * parts * 2 + qt) * 128 + row;
@@ -247,7 +254,7 @@ __device__ __forceinline__ void merge_parts(const Params& p, int cta, int ctas) 
         }
       }
     }
-    store_merged_row<D>(p, pbh, grow, lane, acc, (L != 0.f) ? 1.f / L : 0.f);
+    store_merged_row<D>(p, problem, bh, grow, lane, acc, (L != 0.f) ? 1.f / L : 0.f);
   }
 }
 
@@ -272,12 +279,11 @@ __device__ __forceinline__ void unit_item(const Params& p, int unit, int& w, int
   part = 0;
   parts = 1;
   if (unit >= p.split_first) {
-    const int r = unit - p.split_first;
     parts = p.split_parts;
-    part = r % parts;
-    w = p.split_first + r / parts;
+    w = p.split_first + p.by_parts.divmod(unit - p.split_first, part);
   }
 }
+
 
 // Bitmap of the n-th query block of a list (whole warp).
 template <int NB, bool ONE>
@@ -285,12 +291,12 @@ __device__ __forceinline__ void fill_tile_bitmap(const Params& p, int list, int 
   const int bit0 = ONE ? (list & 1) * NB : 0;  // membership bit of the first query block
   int w, part, parts;
   unit_item(p, ONE ? list >> 1 : list, w, part, parts);
-  const int pbh = w / p.nPairs, pr = w % p.nPairs;
-  const int bh = pbh % (p.B * p.H);
+  int problem, bh, pr;
+  item_place(p, w, problem, bh, pr);
   const int32_t* offsets = p.offsets;
   const int32_t* kv_idx = p.kv_idx;
   if (p.problems != nullptr) {
-    const ProblemEntry* pe = p.problems + pbh / (p.B * p.H);
+    const ProblemEntry* pe = p.problems + problem;
     offsets = pe->offsets;
     kv_idx = pe->kv_idx;
   }
@@ -311,8 +317,9 @@ __device__ __forceinline__ void fill_tile_bitmap(const Params& p, int list, int 
   for (int i = lane; i < W; i += 32) mine[i] = 0u;
   __syncwarp();
   {
-    const int b2 = b + (int)(((int64_t)(e - b) * part) / parts);
-    const int e2 = b + (int)(((int64_t)(e - b) * (part + 1)) / parts);
+    // (a list has fewer than 2^16 entries and is cut into kMaxParts parts at most)
+    const int b2 = (parts == 1) ? b : b + p.by_parts.div((e - b) * part);
+    const int e2 = (parts == 1) ? e : b + p.by_parts.div((e - b) * (part + 1));
 #pragma unroll 4
     for (int i = b2 + lane; i < e2; i += 32) {
       const int v = __ldg(kv_idx + i);
@@ -680,6 +687,10 @@ int launch_t(const Geometry& g, const void* q, const void* k, const void* v, Par
     }
   }
   prm.one_wave = (prm.nUnits <= slots) ? 1 : 0;
+  prm.by_parts = Divisor(prm.split_parts);
+  prm.by_pairs = Divisor(prm.nPairs);
+  prm.by_heads = Divisor(prm.H);
+  prm.by_problem = Divisor(prm.B * prm.H);
   // Every kernel is launched as a dependent of the one before.
   if (prm.one_wave) {
     rc = LOSA_OK;

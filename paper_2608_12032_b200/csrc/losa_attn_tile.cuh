@@ -99,10 +99,9 @@ struct TileControl {
 
 // Key blocks of a unit in the dense modes.
 __device__ __forceinline__ void tile_key_range(const Params& p, uint32_t ent, int& jlo, int& jhi) {
-  const int part = (ent & kTlPartial) ? (int)((ent >> 24) & 7u) : 0;
-  const int parts = (ent & kTlPartial) ? p.split_parts : 1;
-  jlo = (int)(((int64_t)p.nKb * part) / parts);
-  jhi = (int)(((int64_t)p.nKb * (part + 1)) / parts);
+  const int part = (int)((ent >> 24) & 7u);
+  jlo = (ent & kTlPartial) ? p.by_parts.div(p.nKb * part) : 0;
+  jhi = (ent & kTlPartial) ? p.by_parts.div(p.nKb * (part + 1)) : p.nKb;
 }
 
 // (a barrier whose data the other CTA of a pair may have written)
@@ -119,8 +118,10 @@ __device__ __forceinline__ void tile_key_range(const Params& p, uint32_t ent, in
 // What the roles are told.  Per work unit the scheduler of the first CTA publishes a header in both
 // CTAs: the item, and a word with the number of K/V tiles (kHdrTiles), which of the two query tiles
 // lists any (kHdrHas), and whether query tile 1 lists its first one in the unit's second tile instead
-// of its first (kHdrLate).  The dense modes need no more: a unit's tiles follow from its share of the
-// key range.  In the sparse mode the unit's tile list follows in chunks of 32 entries - GROUPS of
+// of its first (kHdrLate).  The dense modes need no more than the unit's share of the key range, which
+// is in the header as well (worked out by every warp with two 64-bit divisions, a unit of 4 K/V tiles
+// took 0.5 us longer: 37 heads of 512 tokens, D = 64, 10.1 -> 9.5 us; of 2048 55.2 -> 53.1, D = 128 83.4 -> 80.5).
+// In the sparse mode the unit's tile list follows in chunks of 32 entries - GROUPS of
 // kG = 128 / C, one per K/V tile, a unit beginning with a chunk of its own - which only the producers
 // and the softmax warps read, the latter only the tiles they work on.  (When every warp walked one
 // list of headers and tiles entry by entry, in the dense modes too, that took more instructions per
@@ -155,16 +156,16 @@ static_assert(2u * (kTlItemMask + 1u) - 1u <= kRedoList, "a tile list's number")
 // Scheduler of the first CTA: publish a header in both CTAs, a lane per word.  It says where the unit lies, so
 // that not every warp has to divide the item's number up again (five divisions, between two units).  A header
 // lies in one of four places in turn: it is there until its readers are done with the unit.
-#define TILE_HDR_PUT(ent, word, pr, bh, b, h, o, problem)                                  \
+#define TILE_HDR_PUT(ent, word, jlo, jhi, pr, bh, b, h, o, problem)                        \
   do {                                                                                     \
     const uint32_t s_ = nu & 1u;                                                           \
     LOSA_WAIT_RELAXED(&ctl->hdr_empty[s_], ((nu >> 1) & 1u) ^ 1u);                         \
     const uint64_t o_ = (uint64_t)reinterpret_cast<uintptr_t>(o);                          \
-    const uint32_t all_[9] = {(ent), (word), (uint32_t)(pr), (uint32_t)(bh), (uint32_t)(b), (uint32_t)(h), \
-                              (uint32_t)o_, (uint32_t)(o_ >> 32), (uint32_t)(problem)};    \
+    const uint32_t all_[11] = {(ent), (word), (uint32_t)(jlo), (uint32_t)(jhi), (uint32_t)(pr), (uint32_t)(bh), \
+                               (uint32_t)(b), (uint32_t)(h), (uint32_t)o_, (uint32_t)(o_ >> 32), (uint32_t)(problem)}; \
     uint32_t mine_ = 0u;                                                                   \
-    _Pragma("unroll") for (int i_ = 0; i_ < 9; ++i_) if (lane == i_) mine_ = all_[i_];     \
-    if (lane < 9) {                                                                        \
+    _Pragma("unroll") for (int i_ = 0; i_ < 11; ++i_) if (lane == i_) mine_ = all_[i_];    \
+    if (lane < 11) {                                                                        \
       ctl->hdr[nu & 3u][lane] = mine_;                                                     \
       if (PAIR) {                                                                          \
         ptx::st_cluster_u32(hdr1 + 48u * (nu & 3u) + 4u * lane, mine_);                    \
@@ -269,11 +270,11 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   // the mass pass alone has no V, no P and no O: its score buffers go back as soon as they are read
   constexpr bool kHasV = (MODE != kMass);
   // When a unit's place is read from its header: at its end, but in those mass passes that came out faster with it in
-  // registers from the unit's start.  That is the compiler's ordering of the exponentials, not the eight registers, so
+  // registers from the unit's start.  That is the compiler's ordering of the exponentials, not the seven registers, so
   // the line lies where it was measured, and has to be measured again when the loop changes (16384 tokens, 12 heads, us at
-  // the start / at the end: D = 64, C = 32 957 / 1004, C = 64 827 / 913, C = 128 879 / 830; D = 128, C = 32 1029 / 1034,
-  // C = 64 974 / 959, C = 128 985 / 999).
-  constexpr bool kInfoEarly = MODE == kMass && (D == 64 ? C_ < 128 : C_ != 64);
+  // the start / at the end: D = 64, C = 32 959 / 915, C = 64 823 / 855, C = 128 883 / 865; D = 128, C = 32 1006 / 977,
+  // C = 64 967 / 926, C = 128 968 / 1007).
+  constexpr bool kInfoEarly = MODE == kMass && C_ == (D == 64 ? 64 : 128);
   constexpr int kChunkTiles = (MODE == kSparse) ? 32 / kG : (1 << 28);  // K/V tiles per chunk of the list
   static_assert(offsetof(TileControl, tl) % 16 == 0, "the tile list is read with 16-byte loads");
   static_assert(offsetof(TileControl, redo_need) == offsetof(TileControl, redo_mark) + 16, "reached from the marks");
@@ -435,18 +436,18 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           continue;
         }
         if ((ent >> 28) != 1) break;
-        const int pr = (int)hdr[2], b = (int)hdr[4], h = (int)hdr[5];
+        const int pr = (int)hdr[4], b = (int)hdr[6], h = (int)hdr[7];
         // (map_kw: K in boxes of 64 keys, map_vw: V in boxes of 128 keys, for consecutive key blocks)
         const CUtensorMap *mq = &map_q, *mk = &map_k, *mv = &map_v, *mkw = &map_kw, *mvw = &map_vw;
         if (p.problems != nullptr) {
-          const ProblemEntry* pe = p.problems + hdr[8];
+          const ProblemEntry* pe = p.problems + hdr[10];
           mq = &pe->map_q;
           mk = PAIR ? &pe->map_kh : &pe->map_k;
           mv = &pe->map_v;
           mkw = PAIR ? &pe->map_k64 : &pe->map_k128;
           mvw = &pe->map_v128;
-          if (PAIR && (int)hdr[8] != problem) {
-            problem = (int)hdr[8];
+          if (PAIR && (int)hdr[10] != problem) {
+            problem = (int)hdr[10];
             acquire_tile_maps<D, C_, kHasV>(pe, lane);
             __syncwarp();
           }
@@ -463,8 +464,7 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         }
         ++nq;
         const int tiles = (int)(word & kHdrTiles);
-        int jlo, jhi;  // dense modes: the unit's key blocks
-        tile_key_range(p, ent, jlo, jhi);
+        const int jlo = (int)hdr[2], jhi = (int)hdr[3];  // dense modes: the unit's key blocks
         // the scheduler draws the next unit when this one is 16 tiles from its end
         const int call_at = max(0, tiles - 16);
         if (tiles == 0 && rank == 0 && leader) ptx::mbar_arrive(&ctl->hdr_next);
@@ -738,7 +738,7 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
             continue;
           }
           ++idle;
-          TILE_HDR_PUT(kTlSkip, 0u, 0, 0, 0, 0, nullptr, 0);
+          TILE_HDR_PUT(kTlSkip, 0u, 0, 0, 0, 0, 0, 0, nullptr, 0);
           LOSA_WAIT_RELAXED(&ctl->hdr_next, (nu - 1u) & 1u);
           continue;
         }
@@ -749,13 +749,13 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         if (again && !p.one_wave && lane == 0 && atomicExch(p.redo_flag + w, 1) == 0) atomicAdd(p.redo_count, 1);
         uint32_t flags = 0;
         if (w >= p.split_first) {
-          const int r = w - p.split_first;
-          flags = kTlPartial | ((uint32_t)(r % p.split_parts) << 24);
-          w = p.split_first + r / p.split_parts;
+          int part;
+          w = p.split_first + p.by_parts.divmod(w - p.split_first, part);
+          flags = kTlPartial | ((uint32_t)part << 24);
         }
-        const int pbh = w / p.nPairs, pr = w % p.nPairs;
-        const int problem = pbh / (p.B * p.H), bh = pbh % (p.B * p.H);
-        const int b = bh / p.H, h = bh % p.H;
+        int pr, problem, bh, h;
+        item_place(p, w, problem, bh, pr);
+        const int b = p.by_heads.divmod(bh, h);
         void* o = p.o;
         if (p.problems != nullptr) {
           o = p.problems[problem].o;
@@ -770,7 +770,7 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           const bool own = p.one_wave && mode == 0u;  // (made by this CTA)
           const uint32_t word = own ? own_word : LOSA_IN_RANGE(list, p.cap_units) ? (uint32_t)__ldcg(p.tl_count + list) : 0u;
           const int cnt = min((int)(word & kHdrTiles) * kG, p.tl_cap);
-          TILE_HDR_PUT(kTlItem | flags | (uint32_t)w, (word & ~kHdrTiles) | odd | (uint32_t)(cnt / kG), pr, bh, b, h, o, problem);
+          TILE_HDR_PUT(kTlItem | flags | (uint32_t)w, (word & ~kHdrTiles) | odd | (uint32_t)(cnt / kG), 0, 0, pr, bh, b, h, o, problem);
           const uint32_t* src = p.tl_entries + (int64_t)list * p.tl_cap;
           for (int base = 0; base < cnt; base += 32) {
             const uint32_t e = (base + lane >= cnt) ? 0u
@@ -796,16 +796,16 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           tile_key_range(p, ent, jlo, jhi);
           const bool two = 2 * pr + 1 < p.nQt;  // the pair's second query tile exists
           if (PAIR) {
-            TILE_HDR_PUT(ent, mode | (two ? 3u : 1u) * kHdrHas | (uint32_t)((jhi - jlo + kG - 1) / kG), pr, bh, b, h, o, problem);
+            TILE_HDR_PUT(ent, mode | (two ? 3u : 1u) * kHdrHas | (uint32_t)((jhi - jlo + kG - 1) / kG), jlo, jhi, pr, bh, b, h, o, problem);
           } else {
             // (a query tile that does not exist is a unit without tiles)
-            TILE_HDR_PUT(ent, odd | ((two || !(odd & kHdrOdd)) ? kHdrHas | (uint32_t)((jhi - jlo + kG - 1) / kG) : 0u), pr, bh, b, h, o,
-                         problem);
+            TILE_HDR_PUT(ent, odd | ((two || !(odd & kHdrOdd)) ? kHdrHas | (uint32_t)((jhi - jlo + kG - 1) / kG) : 0u), jlo, jhi, pr, bh, b, h,
+                         o, problem);
           }
         }
         LOSA_WAIT_RELAXED(&ctl->hdr_next, (nu - 1u) & 1u);
       }
-      if (!p.stall) TILE_HDR_PUT(kTlEnd, 0u, 0, 0, 0, 0, nullptr, 0);
+      if (!p.stall) TILE_HDR_PUT(kTlEnd, 0u, 0, 0, 0, 0, 0, 0, nullptr, 0);
       if (p.one_wave && p.split_parts > 1 && lane == 0)
         p.redo_flag[PAIR ? blockIdx.x >> 1 : blockIdx.x] = *reinterpret_cast<volatile int*>(&ctl->redo_state[3]);
     }
@@ -846,10 +846,11 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       const int tile = PAIR ? (int)rank : (int)((word & kHdrOdd) != 0u);  // of the item's two query tiles
       const int my_bit = tile * kQB + sub;
       // where the unit lies, and what else of its header only its end needs: read again then, not kept in registers
-      uint32_t info[8];
+      uint32_t info[7];
       auto read_info = [&]() {
-        ptx::ld_shared_volatile_vec<4>(&ctl->hdr[(nu - 1u) & 3u][0], info);
-        ptx::ld_shared_volatile_vec<4>(&ctl->hdr[(nu - 1u) & 3u][4], info + 4);
+        ptx::ld_shared_volatile_vec<4>(&ctl->hdr[(nu - 1u) & 3u][4], info);
+        ptx::ld_shared_volatile_vec<2>(&ctl->hdr[(nu - 1u) & 3u][8], info + 4);
+        if (kOneGroup) ptx::ld_shared_volatile_vec<1>(&ctl->hdr[(nu - 1u) & 3u][0], info + 6);
       };
       if (kInfoEarly) read_info();
       float m_ref = 0.f, l = 0.f, le = 0.f;  // le: row sum of the unrounded exponentials (masses, LSE)
@@ -859,8 +860,7 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       // does this query tile list any of the unit's tiles?
       const bool has = (word & (PAIR ? kHdrHas << tile : kHdrHas)) != 0;
       // dense modes: the unit's key blocks, the end of its keys
-      int jlo, jhi;
-      tile_key_range(p, ent, jlo, jhi);
+      const int jlo = (int)hdr[2], jhi = (int)hdr[3];
       const int kend = min(p.N, jhi * kC);
       // Score k of the launch (kq: of the unit's first tile) is worked on by group k % 2 and lies in
       // buffer k % 3, in that buffer's use k / 3.
@@ -1192,11 +1192,12 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
 #undef TILE_REF_GIVE
 #undef TILE_REF_TAKE
       if (!kInfoEarly) read_info();
-      const int w = (int)(info[0] & kTlItemMask);
-      const bool partial = (info[0] & kTlPartial) != 0;
-      const int part = (int)((info[0] >> 24) & 7u);
-      const int pr = (int)info[2], bh = (int)info[3], b = (int)info[4], h = (int)info[5];
-      void* const o_base = reinterpret_cast<void*>((uint64_t)info[6] | ((uint64_t)info[7] << 32));
+      const uint32_t item = kOneGroup ? info[6] : ent;
+      const int w = (int)(item & kTlItemMask);
+      const bool partial = (item & kTlPartial) != 0;
+      const int part = (int)((item >> 24) & 7u);
+      const int pr = (int)info[0], bh = (int)info[1], b = (int)info[2], h = (int)info[3];
+      void* const o_base = reinterpret_cast<void*>((uint64_t)info[4] | ((uint64_t)info[5] << 32));
       const int T = 2 * pr + tile;
       const int grow = T * 128 + row;
       auto hand_over = [&]() {

@@ -30,6 +30,25 @@ const DeviceState* device_state(int* rc);
 int check_device();
 const char* set_cuda_error(cudaError_t e, const char* what);
 
+// Division by a number that the host knows: the quotient of n < 2^31 is the high word of a product
+// (Granlund and Montgomery, "Division by invariant integers using multiplication": mul is 2^(31 + shift) / d rounded
+// up, d <= 2^shift < 2 d, so that n mul / 2^(31 + shift) exceeds n / d by less than 1 / d).  A work unit's place takes
+// five divisions, one behind the other, that every one of its warps waits for.
+struct Divisor {
+  uint32_t d, mul, shift;
+  Divisor() = default;
+  explicit Divisor(uint32_t by) : d(by), mul(0), shift(0) {
+    while ((1ull << shift) < d) ++shift;
+    mul = (uint32_t)(((1ull << (31 + shift)) + d - 1) / d);
+  }
+  __device__ __forceinline__ int div(int n) const { return (int)(__umulhi((uint32_t)n << 1, mul) >> shift); }
+  __device__ __forceinline__ int divmod(int n, int& rest) const {
+    const int q = div(n);
+    rest = n - q * (int)d;
+    return q;
+  }
+};
+
 __device__ __forceinline__ void report_error(int* status, int code) {
   atomicCAS_system(status, 0, code);
 }
