@@ -8,7 +8,8 @@
 // batched launch.  At head dimension 128 the key blocks the pair visits are the union of the index lists of its query
 // blocks (two lists, four when R = 64), so that a K/V tile needed by both tiles is loaded once; at head
 // dimension 64 each of the two tiles has a list of its own.  The items of the last, partly filled wave of the
-// persistent grid are cut into parts of their lists, merged behind (merge_parts_kernel).
+// persistent grid are cut into parts of their lists, merged behind (merge_parts_kernel) or, where all of a call is one
+// wave, by the clusters that they share (merge_in_cluster).
 //
 // Every wait is bounded; a wait that expires raises the CTA's abort flag, records
 // LOSA_ERR_TIMEOUT, and all roles leave through the common teardown that frees TMEM.
@@ -75,6 +76,7 @@ constexpr uint32_t kHdrTiles = 0x00ffffffu, kHdrMax = 1u << 26, kHdrRedo = 1u <<
 // one query tile at a time) one for each.
 __host__ __device__ constexpr int tile_lists_per_unit(int D) { return D == 64 ? 2 : 1; }
 constexpr int kMaxParts = 8;
+constexpr int kMaxClusterCtas = 2 * kMaxParts;
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLn2 = 0.6931471805599453f;
 // a tile's half-row sum (or, where it comes out of the product with V, a unit's row sum) beyond
@@ -131,6 +133,8 @@ struct Params {
   // nothing prepared for it (counters, flags, tile lists), which saves a launch: the CTAs make their unit's
   // tile list themselves, and each list's flag says whether its unit was run again (where parts are merged).
   int one_wave;
+  // ... and the parts of an item run in one cluster, whose CTAs merge them through each other's shared memory
+  int in_cluster;
   // extents of the buffers the kernels index into (elements), for the checked build
   long long cap_part_rows, cap_table_floats, cap_mass, cap_lse, cap_units;
   uint32_t wait_polls;  // bound of every device-side wait, in polls (ptx::kWaitPolls)
@@ -599,28 +603,30 @@ write_problems_kernel(const __grid_constant__ ProblemChunk chunk, ProblemEntry* 
 
 // Configures the tile kernel on the current device (once) and says how many clusters - pairs of CTAs, or (PAIR =
 // false) CTAs - a call may have at work there.
-template <int D, int R, int C_, int MODE, bool PAIR>
-int configure_tile(int sms, int* clusters, cudaLaunchConfig_t* cfg, cudaLaunchAttribute* attr) {
+// `ctas`: of a cluster.
+template <int D, int R, int C_, int MODE, bool PAIR, bool ONE>
+int configure_tile(int sms, int ctas, int* clusters, cudaLaunchConfig_t* cfg, cudaLaunchAttribute* attr) {
   using L = Lay;
   constexpr size_t smem = (size_t)tile_nq(D, MODE) * 256 * D + (size_t)(tile_nk(MODE) + tile_nv(MODE)) * kTileStage +
                           (D == 64 ? kTileOnes : 0) + sizeof(TileControl);
   static_assert(smem <= 227 * 1024, "shared memory of one CTA");
-  auto kern = losa_tile_kernel<D, R, C_, MODE, PAIR>;
-  static int max_on[kMaxDevices] = {};
+  auto kern = losa_tile_kernel<D, R, C_, MODE, PAIR, ONE>;
+  // how many clusters of so many CTAs the device holds at once
+  static std::atomic<int> max_on[kMaxDevices][kMaxClusterCtas + 1];
   int dev = 0;
   LOSA_CUDA_TRY(cudaGetDevice(&dev));
   *cfg = {};
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   attr[1].id = cudaLaunchAttributeClusterDimension;
-  attr[1].val.clusterDim.x = 2;
+  attr[1].val.clusterDim.x = ctas;
   attr[1].val.clusterDim.y = 1;
   attr[1].val.clusterDim.z = 1;
   cfg->blockDim = dim3(L::kThreads, 1, 1);
   cfg->dynamicSmemBytes = smem;
   cfg->attrs = attr;
-  cfg->numAttrs = PAIR ? 2 : 1;
-  if (max_on[dev] == 0) {
+  cfg->numAttrs = ctas > 1 ? 2 : 1;
+  if (max_on[dev][ctas].load(std::memory_order_acquire) == 0) {
     // the in-kernel register reallocation must fit the registers the CTA is launched with
     cudaFuncAttributes fa;
     LOSA_CUDA_TRY(cudaFuncGetAttributes(&fa, kern));
@@ -630,21 +636,21 @@ int configure_tile(int sms, int* clusters, cudaLaunchConfig_t* cfg, cudaLaunchAt
     }
     LOSA_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     int n = sms;
-    if (PAIR) {
+    if (ctas > 1) {
+      LOSA_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
       cudaLaunchConfig_t ask = *cfg;
-      ask.gridDim = dim3(2 * kMaxPersistentCtas, 1, 1);
+      ask.gridDim = dim3(ctas * kMaxPersistentCtas, 1, 1);
       ask.attrs = attr + 1;
       ask.numAttrs = 1;
       LOSA_CUDA_TRY(cudaOccupancyMaxActiveClusters(&n, kern, &ask));
     }
-    if (n < 1) {
-      set_cuda_error(cudaErrorLaunchOutOfResources, "no resident CTA pair of losa_tile_kernel");
-      return LOSA_ERR_UNSUPPORTED;
-    }
-    max_on[dev] = n;
+    max_on[dev][ctas].store(n < 1 ? -1 : n, std::memory_order_release);
   }
-  *clusters = PAIR ? min(min(sms / 2, max_on[dev]), kMaxPersistentCtas) : min(sms, kMaxPersistentCtas);
-  return LOSA_OK;
+  const int n = max_on[dev][ctas].load(std::memory_order_acquire);
+  *clusters = min(min(sms / ctas, n), kMaxPersistentCtas);
+  if (n >= 1) return LOSA_OK;
+  set_cuda_error(cudaErrorLaunchOutOfResources, "no resident cluster of losa_tile_kernel");
+  return LOSA_ERR_UNSUPPORTED;
 }
 
 // Work slots of a call: pairs of CTAs, one for the two query tiles of a work item together (head dimension 128, on a
@@ -655,7 +661,7 @@ int work_slots(int sms, int* slots) {
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute attr[2];
   int n = 0;
-  const int rc = configure_tile<D, R, C_, MODE, D == 128>(sms, &n, &cfg, attr);
+  const int rc = configure_tile<D, R, C_, MODE, D == 128, false>(sms, D == 128 ? 2 : 1, &n, &cfg, attr);
   *slots = (D == 128) ? n : max(1, n / 2);
   return rc;
 }
@@ -670,16 +676,38 @@ int launch_t(const Geometry& g, const void* q, const void* k, const void* v, Par
   if ((rc = work_slots<D, R, C_, MODE>(sms, &slots)) != LOSA_OK) return rc;
   // The items of the last, partly filled wave of the persistent grid (all items, if there are
   // fewer than slots) are cut into parts of the key range, so that the wave ends after 1/parts of
-  // an item; their partial results are merged by a launch behind.  Attention output
+  // an item; their partial results are merged by their clusters or by a launch behind.  Attention output
   // only: the mass epilogue needs a row's final statistics inside the kernel.
   prm.nUnits = prm.nWork;
   prm.split_first = prm.nWork;
   prm.split_parts = 1;
   constexpr bool kAttnOnly = (MODE == kDense || MODE == kSparse);
+  constexpr int kTileCtas = kPair ? 2 : 1;
+  int ctas = kTileCtas;  // of a cluster
+  cudaLaunchConfig_t cfg;
+  cudaLaunchAttribute attr[2];
+  prm.in_cluster = 0;
   if (kAttnOnly) {
     const int rest = (prm.nWork < slots) ? prm.nWork : prm.nWork % slots;
     int parts = rest > 0 ? slots / rest : 1;
     parts = min(min(parts, kMaxParts), prm.nKb);
+    if (parts >= 2 && rest == prm.nWork) {
+      // A single wave: as many parts of an item in one cluster as the device has room for (at head dimension 64 in one for
+      // each of its query tiles), if the units are not longer by more K/V tiles than a launch for the merge takes (4 us; a
+      // tile 0.65 us at head dimension 64, 0.8 at 128).
+      int n = 0, fit = parts;
+      for (; fit >= 2; --fit) {
+        if ((rc = configure_tile<D, R, C_, MODE, kPair, true>(sms, kTileCtas * fit, &n, &cfg, attr)) == LOSA_ERR_CUDA) return rc;
+        if (rc == LOSA_OK && n >= rest * (kPair ? 1 : 2)) break;
+      }
+      constexpr int kBlocks = 128 / C_, kMergeTiles = kPair ? 5 : 6;
+      const int tiles = (prm.nKb + kBlocks - 1) / kBlocks;
+      if (fit >= 2 && (tiles + fit - 1) / fit <= (tiles + parts - 1) / parts + kMergeTiles) {
+        prm.in_cluster = 1;
+        ctas = kTileCtas * fit;
+        parts = fit;
+      }
+    }
     if (parts >= 2) {
       prm.split_first = prm.nWork - rest;
       prm.split_parts = parts;
@@ -705,15 +733,19 @@ int launch_t(const Geometry& g, const void* q, const void* k, const void* v, Par
                 kInitThreads, 0, st, true, prm.work_counter, prm.redo_flag, prm.nUnits);
   }
   if (rc != LOSA_OK) return rc;
-  cudaLaunchConfig_t cfg;
-  cudaLaunchAttribute attr[2];
-  int n = 0;
-  if ((rc = configure_tile<D, R, C_, MODE, kPair>(sms, &n, &cfg, attr)) != LOSA_OK) return rc;
-  cfg.gridDim = dim3(2 * min(slots, prm.nUnits), 1, 1);
-  cfg.stream = st;
-  LOSA_CUDA_TRY(cudaLaunchKernelEx(&cfg, losa_tile_kernel<D, R, C_, MODE, kPair>, maps.map_q, kPair ? maps.map_kh : maps.map_k,
-                                   maps.map_v, kPair ? maps.map_k64 : maps.map_k128, maps.map_v128, prm));
-  if (prm.stall || prm.split_parts == 1) return LOSA_OK;
+  auto launch_tile = [&](auto one) -> int {
+    int n = 0;
+    const int rc = configure_tile<D, R, C_, MODE, kPair, decltype(one)::value>(sms, ctas, &n, &cfg, attr);
+    if (rc != LOSA_OK) return rc;
+    cfg.gridDim = dim3(2 * min(slots, prm.nUnits), 1, 1);
+    cfg.stream = st;
+    LOSA_CUDA_TRY(cudaLaunchKernelEx(&cfg, losa_tile_kernel<D, R, C_, MODE, kPair, decltype(one)::value>, maps.map_q,
+                                     kPair ? maps.map_kh : maps.map_k, maps.map_v, kPair ? maps.map_k64 : maps.map_k128,
+                                     maps.map_v128, prm));
+    return LOSA_OK;
+  };
+  if ((rc = prm.one_wave ? launch_tile(std::true_type()) : launch_tile(std::false_type())) != LOSA_OK) return rc;
+  if (prm.stall || prm.split_parts == 1 || prm.in_cluster) return LOSA_OK;
   constexpr int kRows = kMergeThreads / 32;  // a warp per row
   return launch(merge_parts_kernel<D>, dim3((prm.nWork - prm.split_first) * (256 / kRows)), kMergeThreads, 0, st, true, prm);
 }

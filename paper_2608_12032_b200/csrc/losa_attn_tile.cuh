@@ -84,6 +84,7 @@ struct TileControl {
   alignas(16) uint32_t tl[kTlChunks * 32];  // (read in groups of up to four entries with one vector load)
   uint32_t redo_mark[4];   // per unit (of four in turn): 1 + the tile list of one that outgrew its reference
   uint32_t redo_need[4];   // ... whether its rows' maxima have to be taken first (directly behind the marks)
+  uint32_t cluster_marked; // one_wave: a unit of this cluster has to be run again
   uint32_t redo_queue[4];  // the scheduler's: units to be run again (kRedoList ...), and (1 + the one whose maxima were
   alignas(16) uint32_t redo_state[4];  // taken last; head and tail of the queue; whether there ever was one)
   uint8_t seen[4][16];     // a warp met keys that its rows attend to
@@ -135,6 +136,7 @@ static_assert(2u * (kTlItemMask + 1u) - 1u <= kRedoList, "a tile list's number")
 // four words.
 #define TILE_HDR_NEXT(hdr_, N)                                                             \
   do {                                                                                     \
+    if (ONE && nu == 1u && unit_over()) goto teardown;                                     \
     const uint32_t s_ = nu & 1u;                                                           \
     TILE_WAIT(&ctl->hdr_full[s_], (nu >> 1) & 1u);                                         \
     _Pragma("unroll") for (int i_ = 0; i_ < (N); ++i_)                                     \
@@ -204,8 +206,8 @@ __device__ __forceinline__ void commit0(uint64_t* bar) {
   else ptx::mma_commit(bar);
 }
 template <bool PAIR>
-__device__ __forceinline__ void commit_all(uint64_t* bar) {
-  if (PAIR) ptx::mma2_commit_both(bar);
+__device__ __forceinline__ void commit_all(uint64_t* bar, uint32_t pair_ctas) {
+  if (PAIR) ptx::mma2_commit_both(bar, pair_ctas);
   else ptx::mma_commit(bar);
 }
 
@@ -230,7 +232,70 @@ __device__ __forceinline__ void transpose_chunks(uint32_t* r, int lane) {
   }
 }
 
-template <int D, int R, int C_, int MODE, bool PAIR>
+// The merge of an item's parts by the CTAs of their cluster, each of them its share of the query tile's rows: the
+// launch of its own that merges parts elsewhere cost a call 4 us, all of it latency (8 heads of 1024 tokens, D = 64, dense
+// 14.0 -> 10.3 us, D = 128 18.4 -> 13.6, with the headers written ahead and the shorter way out).  The same
+// arithmetic as merge_parts.  first, step: the ranks of the CTAs with parts 0, 1, ... of this query tile.
+template <int D>
+__device__ __forceinline__ void merge_in_cluster(const Params& p, int unit, int tile, uint32_t first, uint32_t step,
+                                                 uint32_t park_o, uint32_t park_ml, int warp, int lane) {
+  constexpr int kLanes = D / 4, kRows = 32 / kLanes;  // lanes of a row, rows of a warp
+  const int parts = p.split_parts;
+  int part, problem, bh, pr, h;
+  const int w = p.by_parts.divmod(unit, part);  // (all items are cut)
+  item_place(p, w, problem, bh, pr);
+  const int b = p.by_heads.divmod(bh, h);
+  const int T = 2 * pr + tile, sub = lane / kLanes, col = lane % kLanes;
+  if (T >= p.nQt) return;
+  const int row0 = p.by_parts.div(128 * part), row1 = p.by_parts.div(128 * (part + 1));
+  void* const o_base = (p.problems != nullptr) ? p.problems[problem].o : p.o;
+  const int64_t place = (int64_t)b * p.sb + (int64_t)h * p.sh + (int64_t)T * 128 * p.sn + 4 * col;
+  for (int r0 = row0 + warp * kRows; r0 < row1; r0 += 16 * kRows) {
+    const int row = r0 + sub;
+    const bool here = row < row1 && T * 128 + row < p.N;
+    const uint32_t at = (uint32_t)(row * kLanes + ((col & ~7) | ((col ^ row) & 7))) * 16u;
+    float2 ml = make_float2(0.f, 0.f);
+    if (here && col < parts) ml = ptx::ld_cluster_f32x2(ptx::mapa(park_ml + 8u * row, first + step * col));
+    // (a part without keys of the row has the sum 0; one that met NaN has the sum NaN, and so has the row)
+    float m = (ml.y != 0.f) ? ml.x : -INFINITY;
+#pragma unroll
+    for (int d = kMaxParts / 2; d > 0; d >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, d, kLanes));
+    const float mine = (ml.y != 0.f) ? ptx::ex2_approx(ml.x - m) : 0.f;
+    float L = 0.f;
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    // (two parts at a time: unrolled over all eight, the code that a short call runs once and cold took longer than its
+    // loads)
+#pragma unroll 1
+    for (int s0 = 0; s0 < parts; s0 += 2) {
+      float4 v[2];
+#pragma unroll
+      for (int j = 0; j < 2; ++j)
+        if (s0 + j < parts && here) v[j] = ptx::ld_cluster_f32x4(ptx::mapa(park_o + at, first + step * (s0 + j)));
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        if (s0 + j >= parts) break;
+        const float sc = __shfl_sync(0xffffffffu, mine, s0 + j, kLanes);
+        L += __shfl_sync(0xffffffffu, ml.y, s0 + j, kLanes) * sc;
+        if (sc != 0.f && here) {
+          acc.x += v[j].x * sc;
+          acc.y += v[j].y * sc;
+          acc.z += v[j].z * sc;
+          acc.w += v[j].w * sc;
+        }
+      }
+    }
+    if (!here) continue;
+    const float inv = (L != 0.f) ? 1.f / L : 0.f;
+    const int64_t off = place + (int64_t)row * p.sn;
+    if (p.o_f32)
+      *reinterpret_cast<float4*>(static_cast<float*>(o_base) + off) = make_float4(acc.x * inv, acc.y * inv, acc.z * inv, acc.w * inv);
+    else
+      *reinterpret_cast<uint2*>(static_cast<__nv_bfloat16*>(o_base) + off) =
+          make_uint2(ptx::pack_bf16x2(acc.x * inv, acc.y * inv), ptx::pack_bf16x2(acc.z * inv, acc.w * inv));
+  }
+}
+
+template <int D, int R, int C_, int MODE, bool PAIR, bool ONE>
 __global__ void __launch_bounds__(Lay::kThreads, 1)
 losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                  const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_kw,
@@ -285,17 +350,35 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   uint8_t* const sV = sK + kNK * kTileStage;
   uint8_t* const sOnes = sV + kNV * kTileStage;
   Ctl* const ctl = reinterpret_cast<Ctl*>(sOnes + (D == 64 ? kTileOnes : 0));
+  // what a part leaves for the others of its cluster, where its K tiles were: unnormalised O, 16 bytes at a time, and the
+  // rows' reference and sum
+  uint4* const park_o = reinterpret_cast<uint4*>(sK);
+  float2* const park_ml = reinterpret_cast<float2*>(&ctl->half_max[0][0][0]);
+  static_assert(!kOneGroup || kNK * kTileStage >= 128 * D * 4, "room for a part's O");
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint32_t rank = PAIR ? ptx::cluster_ctarank() : 0u;  // 0: the CTA that issues the MMAs; also the query tile
+  // The parts of an item that a single wave is cut into may share a cluster (p.in_cluster): pairs of CTAs, or CTAs, in
+  // the order of the parts.
+  const bool in_cluster = ONE && kOneGroup && p.in_cluster;
+  const uint32_t cta = PAIR ? ptx::cluster_ctarank() : 0u, cta0 = ONE ? cta & ~1u : 0u;
+  const uint32_t rank = cta - cta0;  // 0: the CTA that issues the MMAs; also the query tile
+  const uint32_t pair_ctas = 3u << cta0;
+  // the tile list, which says the unit, that the CTA works on first
+  auto first_list = [&]() {
+    if (PAIR || !in_cluster) return (int)(PAIR ? blockIdx.x >> 1 : blockIdx.x);
+    // (a cluster per query tile)
+    int part;
+    const int c = p.by_parts.divmod((int)blockIdx.x, part);
+    return 2 * ((c >> 1) * p.split_parts + part) + (c & 1);
+  };
   ptx::grid_launch_dependents();
   // (the swizzled tiles rely on the declared alignment of the dynamic shared memory)
   const bool misaligned = (ptx::smem_u32(smem_raw) & 1023u) != 0;
 
   // shared::cluster addresses of the first CTA's barriers that both CTAs arrive on, and of the
   // second CTA's copy of the tile list (used by the first CTA's scheduler)
-  auto at0 = [](const void* x) { return PAIR ? ptx::mapa(ptx::smem_u32(x), 0) : ptx::smem_u32(x); };
-  auto at1 = [](const void* x) { return PAIR ? ptx::mapa(ptx::smem_u32(x), 1) : 0u; };
+  auto at0 = [&](const void* x) { return PAIR ? ptx::mapa(ptx::smem_u32(x), cta0) : ptx::smem_u32(x); };
+  auto at1 = [&](const void* x) { return PAIR ? ptx::mapa(ptx::smem_u32(x), cta0 + 1u) : 0u; };
   const uint32_t q_full0 = at0(&ctl->q_full[0]);
   const uint32_t k_full0 = at0(&ctl->k_full[0]);
   const uint32_t v_full0 = at0(&ctl->v_full[0]);
@@ -308,7 +391,25 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   const uint32_t hdr_full1 = at1(&ctl->hdr_full[0]);
   const uint32_t hdr1 = at1(&ctl->hdr[0][0]);
   const uint32_t tl1 = at1(&ctl->tl[0]);
-  const uint32_t abort_peer = PAIR ? ptx::mapa(ptx::smem_u32(&ctl->abort_flag), rank ^ 1u) : 0u;
+  const uint32_t abort_peer = PAIR ? ptx::mapa(ptx::smem_u32(&ctl->abort_flag), cta ^ 1u) : 0u;
+
+  // One unit to a CTA, or pair of them (p.one_wave): where a warp is through with it, it meets the other warps of the
+  // cluster, and where no unit of the cluster has to be run again all may leave.  (Asking the scheduler for the next unit
+  // instead, and being told that there is none, took 1800 cycles of a 2048-token call's 26000.)
+  int over = -1;
+  auto unit_over = [&]() -> bool {
+    ptx::tc_fence_before_sync();
+    ptx::cluster_meet();
+    over = *reinterpret_cast<volatile uint32_t*>(&ctl->cluster_marked) == 0u ? 1 : 0;
+    return over != 0;
+  };
+  // (every CTA of the cluster is told)
+  auto mark_cluster = [&]() {
+    if (!ONE) return;
+    const uint32_t ctas = (PAIR ? 2u : 1u) * (in_cluster ? (uint32_t)p.split_parts : 1u);
+    for (uint32_t c = 0; c < ctas; ++c) ptx::st_cluster_u32(ptx::mapa(ptx::smem_u32(&ctl->cluster_marked), c), 1u);
+    ptx::fence_acq_rel_cluster();
+  };
 
   if (threadIdx.x == 0) {
     constexpr int kCtas = PAIR ? 2 : 1;
@@ -355,9 +456,37 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     ptx::mbar_init(&ctl->fold_bar, 16);
     ptx::mbar_init(&ctl->drain, 2);
     for (int i = 0; i < 4; ++i) ctl->redo_mark[i] = ctl->redo_need[i] = ctl->redo_state[i] = 0u;
+    ctl->cluster_marked = 0u;
     for (int i = 0; i < 16; ++i) ctl->max_uses[i] = 0;
     ctl->abort_flag = 0;
     ptx::fence_barrier_init();
+  }
+  // A call's first header says where the unit at this CTA's position lies, and is written ahead: in the dense modes it is
+  // all there is to say, and where the CTA makes its own list all but what that says.  (Where the list comes from the
+  // launch ahead, the header as well does: written here, that sparse kernel was up to 8 % slower in all of its units, the
+  // compiler's doing.)
+  const bool early = (ONE || MODE != kSparse) && p.problems == nullptr && !p.stall;
+  if (warp == kSchedulerWarp && early) {
+    int unit = first_list();
+    const uint32_t odd = (!PAIR && (unit & 1)) ? kHdrOdd : 0u;
+    if (!PAIR) unit >>= 1;
+    int w, part, parts, problem, bh, pr, h, jlo, jhi;
+    unit_item(p, unit, w, part, parts);
+    const uint32_t ent = kTlItem | (parts > 1 ? kTlPartial | ((uint32_t)part << 24) : 0u) | (uint32_t)w;
+    item_place(p, w, problem, bh, pr);
+    const int b = p.by_heads.divmod(bh, h);
+    tile_key_range(p, ent, jlo, jhi);
+    const bool two = 2 * pr + 1 < p.nQt;  // the pair's second query tile exists
+    const uint32_t tiles = (uint32_t)((jhi - jlo + kG - 1) / kG);
+    const uint32_t word = PAIR ? (two ? 3u : 1u) * kHdrHas | tiles : odd | ((two || odd == 0u) ? kHdrHas | tiles : 0u);
+    const uint64_t o = (uint64_t)reinterpret_cast<uintptr_t>(p.o);
+    const uint32_t all[11] = {ent, word, (uint32_t)jlo, (uint32_t)jhi, (uint32_t)pr, (uint32_t)bh, (uint32_t)b, (uint32_t)h,
+                              (uint32_t)o, (uint32_t)(o >> 32), 0u};
+    uint32_t mine = 0u;
+#pragma unroll
+    for (int i = 0; i < 11; ++i) if (lane == i) mine = all[i];
+    if (lane < 11) ctl->hdr[0][lane] = mine;
+    __syncwarp();
   }
   if (kSumCol && threadIdx.x < kTileOnes / 16) {
     reinterpret_cast<uint4*>(sOnes)[threadIdx.x] = make_uint4(0x3f803f80u, 0x3f803f80u, 0x3f803f80u, 0x3f803f80u);
@@ -384,13 +513,14 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   }
   ptx::tc_fence_before_sync();
   __syncthreads();
-  if (PAIR) ptx::cluster_sync();  // both CTAs' barriers are initialised before either signals the other
+  if (MODE != kSparse && early && warp == kSchedulerWarp && lane == 0) ptx::mbar_arrive(&ctl->hdr_full[0]);
+  if (PAIR || in_cluster) ptx::cluster_sync();  // both CTAs' barriers are initialised before either signals the other
   ptx::tc_fence_after_sync();
   const uint32_t tmem_base = ctl->tmem_base;
   {
     // the MMAs address both CTAs' tensor memory with one address
     const uint32_t other =
-        PAIR ? ptx::ld_cluster_u32(ptx::mapa(ptx::smem_u32(&ctl->tmem_base), rank ^ 1u)) : tmem_base;
+        PAIR ? ptx::ld_cluster_u32(ptx::mapa(ptx::smem_u32(&ctl->tmem_base), cta ^ 1u)) : tmem_base;
     if (misaligned || other != tmem_base) {
       if (threadIdx.x == 0) {
         ctl->abort_flag = 1;
@@ -408,11 +538,10 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   static_assert(sizeof(TileControl::xch) >= 4 * (kListAt + 256 / C_ * (kMaxPersistentCtas / 2) + 48), "room for a list");
   constexpr bool kOne = tile_lists_per_unit(D) == 2;
   constexpr int kListBlocks = (kOne ? 1 : 2) * kQB;  // query blocks of a list
-  if (MODE == kSparse && p.one_wave) {
+  if (MODE == kSparse && ONE) {
     // ... or the tile list of this CTA's unit from here: the bitmaps of its query blocks, in a place not in use yet
-    const int list = (int)(PAIR ? blockIdx.x >> 1 : blockIdx.x);
     if (rank == 0 && warp < kListBlocks)
-      fill_tile_bitmap<kListBlocks, kOne>(p, list, warp, lane, reinterpret_cast<uint32_t*>(&ctl->xch[0][0][0]));
+      fill_tile_bitmap<kListBlocks, kOne>(p, first_list(), warp, lane, reinterpret_cast<uint32_t*>(&ctl->xch[0][0][0]));
     __syncthreads();
   }
 
@@ -589,8 +718,8 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
               else
                 ptx::mma_ss_lo(tmem_base + bsel * 128, qd[kk] + q0, kd0 + (((kk & 3) * 32) >> 4), kDescHi, kIdescQK,
                                kk > 0 ? 1u : 0u);
-            commit_all<PAIR>(&ctl->s_full[bsel]);
-            commit_all<PAIR>(&ctl->k_empty[ks]);
+            commit_all<PAIR>(&ctl->s_full[bsel], pair_ctas);
+            commit_all<PAIR>(&ctl->k_empty[ks], pair_ctas);
           }
           ++nt;
         }
@@ -598,7 +727,7 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           // a unit without key tiles: the query tiles were loaded all the same
           LOSA_WAIT(&ctl->q_full[nq % kNQ], (nq / kNQ) & 1);
         }
-        if (leader) commit_all<PAIR>(&ctl->q_empty[nq % kNQ]);
+        if (leader) commit_all<PAIR>(&ctl->q_empty[nq % kNQ], pair_ctas);
         ++nq;
       }
     } else if (warp == kIssuerWarp + 1 && rank == 0) {
@@ -622,7 +751,7 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
             LOSA_WAIT(&ctl->p_ready[nt % 3u], (nt / 3u) & 1);
             if (leader) commit0<PAIR>(&ctl->pv_done[nt % 3u]);
           }
-          if (leader) commit_all<PAIR>(&ctl->o_done[od]);
+          if (leader) commit_all<PAIR>(&ctl->o_done[od], pair_ctas);
           continue;
         }
         uint32_t pv_item = 0;
@@ -647,13 +776,13 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
                                vd0 + kk * (kSumCol ? (2048u >> 4) - (2048u << 12) : 2048u >> 4), kDescHi, kIdescPV,
                                (kk > 0 || pv_item > 0) ? 1u : 0u);
             commit0<PAIR>(&ctl->pv_done[bsel]);
-            commit_all<PAIR>(&ctl->v_empty[vs]);
+            commit_all<PAIR>(&ctl->v_empty[vs], pair_ctas);
           }
           ++pv_item;
           ++nt;
           ++nv;
         }
-        if (leader) commit_all<PAIR>(&ctl->o_done[od]);  // every product of the item is done
+        if (leader) commit_all<PAIR>(&ctl->o_done[od], pair_ctas);  // every product of the item is done
         if (pv_item > 0) ++nof;
       }
     } else if (warp == kSchedulerWarp && rank == 0) {
@@ -667,13 +796,69 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       int acquired = -1;  // batched launch: whose tensor maps this warp has acquired
       bool first_item = true, drawn = false;
       uint32_t own_word = 0u;  // one_wave: what tl_count holds of the CTA's unit
-      if (MODE == kSparse && p.one_wave) {
+      // (how many units were run again is for tests to read: whoever adds to it has run two, ten microseconds later)
+      if (in_cluster && blockIdx.x == 0 && lane == 0) *p.redo_count = 0;
+      if (MODE == kSparse && ONE) {
         uint32_t* const bm = reinterpret_cast<uint32_t*>(&ctl->xch[0][0][0]);
-        own_word = emit_tile_list<kListBlocks, kG, kOne>(p, (int)(PAIR ? blockIdx.x >> 1 : blockIdx.x), lane, bm, bm + kListAt);
+        own_word = emit_tile_list<kListBlocks, kG, kOne>(p, first_list(), lane, bm, bm + kListAt);
         __syncwarp();
       }
+      // A unit's tile list, in chunks of 32 entries, to both CTAs; `own`: made by this CTA, in shared memory.  False: gave up.
+      auto publish_list = [&](int list, int cnt, bool own) -> bool {
+        const uint32_t* src = p.tl_entries + (int64_t)list * p.tl_cap;
+        for (int base = 0; base < cnt; base += 32) {
+          const uint32_t e = (base + lane >= cnt) ? 0u
+                             : own ? reinterpret_cast<const uint32_t*>(&ctl->xch[0][0][0])[kListAt + base + lane]
+                                   : __ldcg(src + base + lane);
+          const uint32_t c = nc & (kTlChunks - 1);
+          if (!ptx::mbar_wait_relaxed(&ctl->tl_empty[c], ((nc / kTlChunks) & 1u) ^ 1u, &ctl->abort_flag, p.wait_polls)) {
+            ctl->abort_flag = 1;
+            report_error(p.status, LOSA_ERR_TIMEOUT);
+            return false;
+          }
+          ctl->tl[c * 32 + lane] = e;
+          if (PAIR) {
+            ptx::st_cluster_u32(tl1 + 4u * (c * 32 + lane), e);
+            ptx::fence_acq_rel_cluster();
+          }
+          __syncwarp();
+          if (lane == 0) {
+            ptx::mbar_arrive(&ctl->tl_full[c]);
+            if (PAIR) ptx::mbar_arrive_cluster(tl_full1 + 8u * c);
+          }
+          ++nc;
+        }
+        return true;
+      };
       for (;;) {
         if (p.stall) break;  // diagnostic launch: nothing is published and every wait runs out
+        if (nu == 0u && early) {
+          // (the first unit's header is there: in the sparse mode without what its list says)
+          first_item = false;
+          if (MODE == kSparse) {
+            const int list = first_list();
+            const int cnt = min((int)(own_word & kHdrTiles) * kG, p.tl_cap);
+            if (lane == 0) {
+              const uint32_t word = (own_word & ~kHdrTiles) | ((!PAIR && (list & 1)) ? kHdrOdd : 0u) | (uint32_t)(cnt / kG);
+              *reinterpret_cast<volatile uint32_t*>(&ctl->hdr[0][1]) = word;
+              if (PAIR) {
+                ptx::st_cluster_u32(hdr1 + 4u, word);
+                ptx::fence_acq_rel_cluster();
+              }
+              ptx::mbar_arrive(&ctl->hdr_full[0]);
+              if (PAIR) ptx::mbar_arrive_cluster(hdr_full1);
+            }
+            __syncwarp();
+            if (!publish_list(list, cnt, true)) goto teardown;
+          }
+          ++nu;
+          LOSA_WAIT_RELAXED(&ctl->hdr_next, 0u);
+          continue;
+        }
+        if (ONE && nu == 1u && unit_over()) {
+          if (p.split_parts > 1 && !in_cluster && lane == 0) p.redo_flag[first_list()] = 0;
+          goto teardown;
+        }
         LOSA_WAIT_RELAXED(&ctl->hdr_empty[nu & 1u], ((nu >> 1) & 1u) ^ 1u);
         if (PAIR) ptx::fence_acq_rel_cluster();
         auto take_mark = [&](uint32_t unit_no) {
@@ -716,9 +901,9 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         } else if (!drawn) {
           // a first unit by position, then from the counter; without pairs of CTAs a unit's two query
           // tiles are drawn one by one
-          w = (int)(PAIR ? blockIdx.x >> 1 : blockIdx.x);
+          w = first_list();
           if (!first_item) {
-            if (p.one_wave) {
+            if (ONE) {
               w = INT_MAX;
             } else {
               if (lane == 0) w = (int)(PAIR ? gridDim.x >> 1 : gridDim.x) + atomicAdd(p.work_counter, 1);
@@ -746,7 +931,7 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         const int list = w;  // its tile list
         const uint32_t odd = ((!PAIR && (w & 1)) ? kHdrOdd : 0u) | mode;
         if (!PAIR) w >>= 1;
-        if (again && !p.one_wave && lane == 0 && atomicExch(p.redo_flag + w, 1) == 0) atomicAdd(p.redo_count, 1);
+        if (again && !ONE && lane == 0 && atomicExch(p.redo_flag + w, 1) == 0) atomicAdd(p.redo_count, 1);
         uint32_t flags = 0;
         if (w >= p.split_first) {
           int part;
@@ -767,29 +952,11 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           }
         }
         if (MODE == kSparse) {
-          const bool own = p.one_wave && mode == 0u;  // (made by this CTA)
+          const bool own = ONE && mode == 0u;  // (made by this CTA)
           const uint32_t word = own ? own_word : LOSA_IN_RANGE(list, p.cap_units) ? (uint32_t)__ldcg(p.tl_count + list) : 0u;
           const int cnt = min((int)(word & kHdrTiles) * kG, p.tl_cap);
           TILE_HDR_PUT(kTlItem | flags | (uint32_t)w, (word & ~kHdrTiles) | odd | (uint32_t)(cnt / kG), 0, 0, pr, bh, b, h, o, problem);
-          const uint32_t* src = p.tl_entries + (int64_t)list * p.tl_cap;
-          for (int base = 0; base < cnt; base += 32) {
-            const uint32_t e = (base + lane >= cnt) ? 0u
-                               : own ? reinterpret_cast<const uint32_t*>(&ctl->xch[0][0][0])[kListAt + base + lane]
-                                     : __ldcg(src + base + lane);
-            const uint32_t c = nc & (kTlChunks - 1);
-            LOSA_WAIT_RELAXED(&ctl->tl_empty[c], ((nc / kTlChunks) & 1u) ^ 1u);
-            ctl->tl[c * 32 + lane] = e;
-            if (PAIR) {
-              ptx::st_cluster_u32(tl1 + 4u * (c * 32 + lane), e);
-              ptx::fence_acq_rel_cluster();
-            }
-            __syncwarp();
-            if (lane == 0) {
-              ptx::mbar_arrive(&ctl->tl_full[c]);
-              if (PAIR) ptx::mbar_arrive_cluster(tl_full1 + 8u * c);
-            }
-            ++nc;
-          }
+          if (!publish_list(list, cnt, own)) goto teardown;
         } else {
           const uint32_t ent = kTlItem | flags | (uint32_t)w;
           int jlo, jhi;
@@ -806,8 +973,11 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         LOSA_WAIT_RELAXED(&ctl->hdr_next, (nu - 1u) & 1u);
       }
       if (!p.stall) TILE_HDR_PUT(kTlEnd, 0u, 0, 0, 0, 0, 0, 0, nullptr, 0);
-      if (p.one_wave && p.split_parts > 1 && lane == 0)
-        p.redo_flag[PAIR ? blockIdx.x >> 1 : blockIdx.x] = *reinterpret_cast<volatile int*>(&ctl->redo_state[3]);
+      if (ONE && p.split_parts > 1 && lane == 0) {
+        const int again = *reinterpret_cast<volatile int*>(&ctl->redo_state[3]);
+        if (!in_cluster) p.redo_flag[first_list()] = again;
+        else if (again != 0) atomicAdd(p.redo_count, 1);
+      }
     }
   } else {
     // ------------------------------------------------------------------ softmax warps (both CTAs)
@@ -1134,7 +1304,10 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           // (in the mass pass l is le once more; without it, and with a vote over the whole sums at the unit's end, the
           // compiler ordered the exponentials worse: 1024 key blocks 4090 us against 4300)
           if (!kSumCol) {
-            ovf = ovf || __any_sync(0xffffffffu, !(tsum <= kSplitSafeSum));
+            // (the same twice; which, is a matter of the order that the compiler finds: masses, 16384 tokens, 12 heads, D = 64
+            // with 128-key blocks 872 / 836 us, with 64 825 / 856; D = 128 969 - 1043 / 957 - 1010)
+            if (MODE == kMass && !(D == 64 && C_ == 64)) ovf = __any_sync(0xffffffffu, ovf || !(tsum <= kSplitSafeSum));
+            else ovf = ovf || __any_sync(0xffffffffu, !(tsum <= kSplitSafeSum));
             l += tsum;
           }
           if (kSumCol) ptx::tmem_st16(tS + 16, &sr[16]);
@@ -1201,6 +1374,7 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       const int T = 2 * pr + tile;
       const int grow = T * 128 + row;
       auto hand_over = [&]() {
+        mark_cluster();
         const int unit = partial ? p.split_first + (w - p.split_first) * p.split_parts + part : w;
         const uint32_t mark = 1u + (uint32_t)(PAIR ? unit : 2 * unit + tile);
         if (PAIR) {
@@ -1324,9 +1498,21 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
             // (run again only rows that met a score that is not a number add up to that much)
             if (redo && !(l <= kSplitSafeSum)) l = __int_as_float(0x7fc00000);
             inv = (l == 0.f) ? 0.f : 1.f / l;
-            if (partial && half == 0 && T < p.nQt && LOSA_IN_RANGE(pslot, p.cap_part_rows)) p.part_ml[pslot] = make_float2(m_ref, l);
+            if (in_cluster) {
+              if (half == 0) park_ml[row] = make_float2(m_ref, l);
+            } else if (partial && half == 0 && T < p.nQt && LOSA_IN_RANGE(pslot, p.cap_part_rows)) {
+              p.part_ml[pslot] = make_float2(m_ref, l);
+            }
           }
-          if (partial) {
+          if (in_cluster) {
+            // (16 bytes of a row lie where eight lanes' stores meet no bank twice)
+#pragma unroll
+            for (int c = 0; c < 32; c += 4)
+              park_o[row * (D / 4) + ((((half * kOC + c0 + c) >> 2) & ~7) | ((((half * kOC + c0 + c) >> 2) ^ row) & 7))] =
+                  make_uint4(r[c], r[c + 1], r[c + 2], r[c + 3]);
+            // (the copies of a unit that is run again come behind this)
+            if (c0 + 32 == kOC) ptx::fence_proxy_async();
+          } else if (partial) {
             const int64_t slot0 = pslot - lane;  // (of the warp's first row; 32 rows of it exist in any case)
             if (T < p.nQt)
               store_rows(r, p.part_o + (LOSA_IN_RANGE(pslot, p.cap_part_rows) ? slot0 : 0) * D + half * kOC + c0, D, 32,
@@ -1453,10 +1639,26 @@ teardown:
       for (uint32_t it = 0; it < (1u << 10); ++it) __nanosleep(1024);
     }
   }
-  ptx::tc_fence_before_sync();
-  __syncthreads();
   // neither CTA leaves, or frees its tensor memory, while the other may still signal into it
-  if (PAIR) ptx::cluster_sync();
+  if (ONE && over < 0) unit_over();
+  if (!ONE || over != 1) {
+    ptx::tc_fence_before_sync();
+    __syncthreads();
+    if (PAIR || in_cluster) ptx::cluster_sync();
+  }
+  if constexpr (ONE && kOneGroup) {
+    if (in_cluster) {
+      // (every part has left its rows; none leaves the cluster before they are read)
+      if (warp >= 4 && !ctl->abort_flag) {
+        const int list = first_list();
+        merge_in_cluster<D>(p, PAIR ? list : list >> 1, PAIR ? (int)rank : list & 1, PAIR ? rank : 0u, PAIR ? 2u : 1u,
+                            ptx::smem_u32(park_o), ptx::smem_u32(park_ml), warp - 4, lane);
+      }
+      __syncwarp();
+      ptx::cluster_arrive_relaxed();
+      ptx::cluster_wait();
+    }
+  }
   if (warp == kIssuerWarp) {
     ptx::tc_fence_after_sync();
     if (PAIR) ptx::tmem_dealloc2(tmem_base, kTmemCols);

@@ -329,6 +329,14 @@ __device__ __forceinline__ void cluster_sync() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
+// The same for warps at different places of the code; and in two halves, without ordering memory (a release at cluster
+// scope waits for the thread's stores to global memory, over a thousand cycles).
+__device__ __forceinline__ void cluster_meet() {
+  asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_arrive_relaxed() { asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait;" ::: "memory"); }
+
 __device__ __forceinline__ void fence_acq_rel_cluster() {
   asm volatile("fence.acq_rel.cluster;" ::: "memory");
 }
@@ -340,6 +348,18 @@ __device__ __forceinline__ void st_cluster_u32(uint32_t caddr, uint32_t v) {
 __device__ __forceinline__ uint32_t ld_cluster_u32(uint32_t caddr) {
   uint32_t v;
   asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(caddr) : "memory");
+  return v;
+}
+
+__device__ __forceinline__ float4 ld_cluster_f32x4(uint32_t caddr) {
+  float4 v;
+  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(caddr) : "memory");
+  return v;
+}
+
+__device__ __forceinline__ float2 ld_cluster_f32x2(uint32_t caddr) {
+  float2 v;
+  asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(caddr) : "memory");
   return v;
 }
 
@@ -461,19 +481,19 @@ __device__ __forceinline__ void mma2_ts_lo(uint32_t d_tmem, uint32_t a_tmem, uin
       : "memory");
 }
 
-// arrive on a barrier of the issuing CTA / on the same barrier in both CTAs of the pair, once every
-// MMA issued so far by this thread has completed
+// arrive on a barrier of the issuing CTA / on the same barrier in both CTAs of the pair (`ctas`: bits 2 i and 2 i + 1 for
+// pair i of the cluster), once every MMA issued so far by this thread has completed
 __device__ __forceinline__ void mma2_commit(uint64_t* bar) {
   asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
                    smem_u32(bar))
                : "memory");
 }
 
-__device__ __forceinline__ void mma2_commit_both(uint64_t* bar) {
+__device__ __forceinline__ void mma2_commit_both(uint64_t* bar, uint32_t ctas) {
   asm volatile(
       "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(
           smem_u32(bar)),
-      "h"((uint16_t)3)
+      "h"((uint16_t)ctas)
       : "memory");
 }
 

@@ -1,0 +1,41 @@
+"""Items that a single wave is cut into: their parts run in one cluster and are merged through its CTAs' shared memory,
+from two parts to as many as there can be, of an odd number of query tiles with a short last one; some parts outgrow their
+reference and are run again, the others of their cluster wait for them.  Against the fp64 oracle."""
+import pytest
+import torch
+
+from tests import util
+from tests.test_gpu_units import check, lib
+
+pytestmark = pytest.mark.gpu
+
+N = 1100  # 9 query tiles, of 5 items to a head; 9 K/V tiles
+
+
+@pytest.mark.parametrize("D,R,C", [(64, 64, 64), (64, 128, 32), (128, 128, 128), (128, 64, 64)])
+@pytest.mark.parametrize("H", [1, 2, 3, 4, 7])
+def test_parts_of_an_item_are_merged_in_their_cluster(D, R, C, H):
+    losa = lib()
+    prob = losa.make_problem(torch.empty((1, H, N, D), dtype=torch.bfloat16, device="cuda"), R, C)
+    assert 2 <= losa.losa_work_slots(losa.binding.LOSA_OP_ATTN, prob) // (5 * H)
+    check(H, N, D, R, C, (0, H - 1), 1700 + H)
+
+
+@pytest.mark.parametrize("D,R,C", [(64, 64, 64), (128, 128, 64)])
+def test_cut_items_of_a_batched_call_and_of_token_major_tensors(D, R, C):
+    """Two layers of two heads in one wave equal the single calls where both are cut alike; rows a head apart, a batch of
+    two, bf16 and fp32 output (the same, rounded once)."""
+    losa = lib()
+    nQb, nKb = -(-N // R), -(-N // C)
+    layers = []
+    for i in range(2):
+        q, k, v = (util.rand_bf16((2, N, 1, D), 1720 + 3 * i + j).cuda().transpose(1, 2) for j in range(3))
+        off, idx = util.random_csr(2 * nQb, nKb, 1730 + i, 0.6)
+        layers.append((q, k, v, torch.from_numpy(off).cuda(), torch.from_numpy(idx).cuda()))
+    outs = losa.losa_sparse_attn_batched(layers, R, C, out_dtype=torch.float32)
+    for (q, k, v, off, idx), o in zip(layers, outs):
+        single = losa.losa_sparse_attn(q, k, v, off, idx, R, C, out_dtype=torch.float32)
+        assert torch.equal(single.bfloat16(), losa.losa_sparse_attn(q, k, v, off, idx, R, C))
+        # 10 items in 7 parts, 20 in 3: P rounds against another reference, 2^-9 each at random
+        assert (o - single).norm() <= 4e-3 * single.norm()
+    assert losa.losa_async_status() == 0
