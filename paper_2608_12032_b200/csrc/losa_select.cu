@@ -7,9 +7,12 @@
 //                           over block indices plus its size.
 //   2. expand_rows_kernel   every CTA adds up the sizes of the rows before its own (offsets) and
 //                           turns its rows' bitmaps into ascending block indices.
+// Up to 256 rows of at most 1024 blocks take one launch of one cluster instead (select_small_kernel).
 // Each mass element is read once and each kept index written once; the bitmap adds 1/16
 // of the mass bytes.  The result is deterministic (no floating-point atomics).
 #include <limits.h>
+
+#include <atomic>
 
 #include "losa_common.cuh"
 #include "losa_ptx.cuh"
@@ -236,34 +239,23 @@ __device__ __forceinline__ void find_bin(RowShared* rs, unsigned long long targe
   row_sync<W>();
 }
 
-// W warps per row, K blocks per lane: warp w of the row owns blocks [w * 32 K, (w + 1) * 32 K), its
-// lane l the blocks l, l + 32, ... of those, so that a ballot is a bitmap word.  One row per CTA, or
-// four at W = 1.  COUNT: the fixed-ratio rule.
-template <int W, int K, bool COUNT>
-__global__ void __launch_bounds__(W == 1 ? 128 : 32 * W, W == 1 ? 7 : 28 / W)
-select_rows_kernel(const float* __restrict__ mass, int rows, int nKb, double tau, int fixed_count,
-                   int32_t* __restrict__ counts, uint32_t* __restrict__ bitmaps, int* status) {
-  constexpr int kRowsPerCta = (W == 1) ? 4 : 1;
+// What a row keeps.  W warps per row, K blocks per lane: warp w of the row owns blocks [w * 32 K, (w + 1) * 32 K), its
+// lane l the blocks l, l + 32, ... of those, so that a ballot is a bitmap word; lane k gets word k of its warp's K.
+// `src`: the lane's first block, `mine`: how many blocks of the warp exist (may be none).  COUNT: the fixed-ratio rule.
+template <int W, int K, bool COUNT, bool EARLY>
+__device__ __forceinline__ uint32_t kept_words(RowShared* rs, const float* src, int mine, int warp, int lane, int nKb,
+                                               double tau, int fixed_count, int* status) {
   constexpr int T = 32 * W;
   constexpr int kShift = COUNT ? kCountShift : kTauShift;
   constexpr int kBase = COUNT ? 0 : kTopBin - (kBins - 1);
   constexpr uint32_t kLowMask = (1u << kShift) - 1u;
-  __shared__ RowShared shared[kRowsPerCta];
-  const int lane = threadIdx.x & 31;
-  const int warp = (W == 1) ? 0 : threadIdx.x >> 5;     // of the row
   const int t = warp * 32 + lane;                       // thread of the row
-  RowShared* const rs = &shared[(W == 1) ? threadIdx.x >> 5 : 0];
-  const int64_t row = (int64_t)blockIdx.x * kRowsPerCta + ((W == 1) ? threadIdx.x >> 5 : 0);
-  ptx::grid_launch_dependents();
-  if (row >= rows) return;
-  const int words = (nKb + 31) >> 5;
-  const int mine = min(32 * K, nKb - warp * 32 * K);    // blocks of this warp (may be none)
-  const float* src = mass + row * nKb + warp * 32 * K + lane;
-
+  // EARLY: the kernel ahead may have written the masses while this one was starting, so that they are no read-only data.
+  auto load = [](const float* at) { return EARLY ? __ldca(at) : __ldg(at); };
   // (blocks past the row's end weigh nothing; they are told apart by their index where they could count)
   uint32_t bits[K];
 #pragma unroll
-  for (int k = 0; k < K; ++k) bits[k] = (k * 32 + lane < mine) ? __float_as_uint(__ldg(src + k * 32)) : 0u;
+  for (int k = 0; k < K; ++k) bits[k] = (k * 32 + lane < mine) ? __float_as_uint(load(src + k * 32)) : 0u;
   for (int i = t; i < kBins; i += T) {
     rs->cnt[i] = 0u;
     if (!COUNT) rs->low[i] = 0u;
@@ -411,7 +403,7 @@ select_rows_kernel(const float* __restrict__ mass, int rows, int nKb, double tau
         while (in != 0u) {
           const int k = __ffs(in) - 1;
           in &= in - 1u;
-          uint32_t x = __float_as_uint(__ldg(src + k * 32));
+          uint32_t x = __float_as_uint(load(src + k * 32));
           if (x > kMaxMassBits) x = 0u;
           rs->list[atomicAdd(&rs->list_len, 1)] = x & ((1u << rest) - 1u);
         }
@@ -439,7 +431,7 @@ select_rows_kernel(const float* __restrict__ mass, int rows, int nKb, double tau
         unsigned long long a = 0ull;
 #pragma unroll 1
         for (int k = 0; k * 32 + lane < mine; ++k) {
-          uint32_t x = __float_as_uint(__ldg(src + k * 32));
+          uint32_t x = __float_as_uint(load(src + k * 32));
           if (x > kMaxMassBits) x = 0u;
           if (x >= from) a += fixed_weight(x, scale, cap);
         }
@@ -502,6 +494,27 @@ select_rows_kernel(const float* __restrict__ mass, int rows, int nKb, double tau
   const int valid = mine - lane * 32;
   if (lane >= K || valid <= 0) out = 0u;
   else if (valid < 32) out &= (1u << valid) - 1u;
+  return out;
+}
+
+// One row per CTA, or four at W = 1.
+template <int W, int K, bool COUNT>
+__global__ void __launch_bounds__(W == 1 ? 128 : 32 * W, W == 1 ? 7 : 28 / W)
+select_rows_kernel(const float* __restrict__ mass, int rows, int nKb, double tau, int fixed_count,
+                   int32_t* __restrict__ counts, uint32_t* __restrict__ bitmaps, int* status) {
+  constexpr int kRowsPerCta = (W == 1) ? 4 : 1;
+  __shared__ RowShared shared[kRowsPerCta];
+  const int lane = threadIdx.x & 31;
+  const int warp = (W == 1) ? 0 : threadIdx.x >> 5;     // of the row
+  RowShared* const rs = &shared[(W == 1) ? threadIdx.x >> 5 : 0];
+  const int64_t row = (int64_t)blockIdx.x * kRowsPerCta + ((W == 1) ? threadIdx.x >> 5 : 0);
+  ptx::grid_launch_dependents();
+  ptx::grid_dependency_wait();
+  if (row >= rows) return;
+  const int words = (nKb + 31) >> 5;
+  const int mine = min(32 * K, nKb - warp * 32 * K);
+  const float* src = mass + row * nKb + warp * 32 * K + lane;
+  const uint32_t out = kept_words<W, K, COUNT, !COUNT>(rs, src, mine, warp, lane, nKb, tau, fixed_count, status);
   if (lane < K && warp * K + lane < words) bitmaps[row * words + warp * K + lane] = out;
   int kept = __reduce_add_sync(0xffffffffu, __popc(out));
   if (W > 1) {
@@ -511,7 +524,68 @@ select_rows_kernel(const float* __restrict__ mass, int rows, int nKb, double tau
 #pragma unroll
     for (int w = 0; w < W; ++w) kept += rs->part[w];
   }
-  if (t == 0) counts[row] = kept;
+  if (warp * 32 + lane == 0) counts[row] = kept;
+}
+
+// Few rows: one launch, of one cluster.  A warp per row, two rows at most; the sizes of all rows meet in every CTA's
+// shared memory, and each warp writes the indices of its own rows.  The two launches of the general way are all latency
+// there (masses, selection and attention of 256 tokens, 27.8 -> 24.5 us; 4 x 32 rows of 32 blocks,
+// calls in a row, 9.1 -> 6.1).
+constexpr int kSmallWarps = 16, kSmallCtas = 8, kSmallRows = 2 * kSmallWarps * kSmallCtas;
+struct SmallShared {
+  RowShared rows[kSmallWarps];
+  int counts[kSmallRows];
+};
+template <int K, bool COUNT>
+__global__ void __launch_bounds__(32 * kSmallWarps)
+select_small_kernel(const float* __restrict__ mass, int rows, int nKb, double tau, int fixed_count,
+                    int32_t* __restrict__ offsets, int32_t* __restrict__ kv_idx, int64_t kv_capacity, int* status) {
+  extern __shared__ __align__(16) unsigned char small_raw[];
+  SmallShared* const sh = reinterpret_cast<SmallShared*>(small_raw);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, ctas = gridDim.x;
+  ptx::grid_launch_dependents();
+  ptx::cluster_sync();  // (the other CTAs' shared memory is there)
+  ptx::grid_dependency_wait();
+  uint32_t word[2] = {0u, 0u};
+  int kept[2] = {0, 0};
+#pragma unroll 1
+  for (int i = 0; i < 2; ++i) {
+    const int row = (i * ctas + (int)blockIdx.x) * kSmallWarps + warp;
+    if (row >= rows) break;
+    const uint32_t out = kept_words<1, K, COUNT, true>(&sh->rows[warp], mass + (int64_t)row * nKb + lane, nKb, 0, lane, nKb, tau,
+                                                 fixed_count, status);
+    const int n = __reduce_add_sync(0xffffffffu, __popc(out));
+    if (lane < ctas) ptx::st_cluster_u32(ptx::mapa(ptx::smem_u32(&sh->counts[row]), lane), (uint32_t)n);
+    if (i == 0) word[0] = out, kept[0] = n;
+    else word[1] = out, kept[1] = n;
+    __syncwarp();
+  }
+  ptx::cluster_sync();
+  const uint32_t bit = 1u << lane, below = bit - 1u;
+  const int words = (nKb + 31) >> 5;
+#pragma unroll 1
+  for (int i = 0; i < 2; ++i) {
+    const int row = (i * ctas + (int)blockIdx.x) * kSmallWarps + warp;
+    if (row >= rows) break;
+    int at = 0;
+    for (int r = lane; r < row; r += 32) at += sh->counts[r];
+    at = __reduce_add_sync(0xffffffffu, at);
+    const uint32_t mine = (i == 0) ? word[0] : word[1];
+    const int n = (i == 0) ? kept[0] : kept[1];
+    if (lane == 0) {
+      offsets[row] = at;
+      if (row == rows - 1) {
+        offsets[rows] = at + n;
+        if ((int64_t)at + n > kv_capacity) report_error(status, LOSA_ERR_CAPACITY);
+      }
+    }
+    for (int w = 0; w < words; ++w) {
+      const uint32_t x = __shfl_sync(0xffffffffu, mine, w);
+      const int to = at + __popc(x & below);
+      if ((x & bit) && to < kv_capacity) kv_idx[to] = w * 32 + lane;
+      at += __popc(x);
+    }
+  }
 }
 
 // Bitmaps -> ascending indices, `per_cta` consecutive rows per CTA.  The CTA first adds up the sizes
@@ -651,21 +725,61 @@ size_t select_workspace_bytes(int64_t rows, int nKb) {
   return align_up((size_t)rows * sizeof(int32_t), 256) + (size_t)rows * words * sizeof(uint32_t);
 }
 
+template <int K, bool COUNT>
+static int launch_small(int ctas, const float* mass, int rows, int nKb, double tau, int fixed_count, int32_t* offsets,
+                        int32_t* kv_idx, int64_t kv_capacity, int* status, cudaStream_t st) {
+  auto kern = select_small_kernel<K, COUNT>;
+  static std::atomic<int> ready[kMaxDevices];
+  int dev = 0;
+  LOSA_CUDA_TRY(cudaGetDevice(&dev));
+  if (!ready[dev].load(std::memory_order_acquire)) {
+    LOSA_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SmallShared)));
+    ready[dev].store(1, std::memory_order_release);
+  }
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = ctas;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
+  cfg.gridDim = dim3(ctas, 1, 1);
+  cfg.blockDim = dim3(32 * kSmallWarps, 1, 1);
+  cfg.dynamicSmemBytes = sizeof(SmallShared);
+  cfg.stream = st;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  LOSA_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, mass, rows, nKb, tau, fixed_count, offsets, kv_idx, kv_capacity, status));
+  return LOSA_OK;
+}
+
 int launch_select(int rows, int nKb, const float* mass, double tau, int fixed_count,
                   int32_t* offsets, int32_t* kv_idx, int64_t kv_capacity, void* ws, int* status,
                   cudaStream_t st) {
   int32_t* counts = static_cast<int32_t*>(ws);
   uint32_t* bitmaps = reinterpret_cast<uint32_t*>(static_cast<char*>(ws) +
                                                   align_up((size_t)rows * sizeof(int32_t), 256));
-  // (registers hold 32 blocks per lane at most: longer rows take more warps)
+  if (rows <= kSmallRows && nKb <= 1024) {
+    const int ctas = min(kSmallCtas, (rows + kSmallWarps - 1) / kSmallWarps);
+#define LOSA_SELECT_SMALL(k)                                                                                  \
+  (fixed_count > 0 ? launch_small<k, true>(ctas, mass, rows, nKb, tau, fixed_count, offsets, kv_idx, kv_capacity, status, st) \
+                   : launch_small<k, false>(ctas, mass, rows, nKb, tau, 0, offsets, kv_idx, kv_capacity, status, st))
+    return nKb <= 256 ? LOSA_SELECT_SMALL(8) : nKb <= 512 ? LOSA_SELECT_SMALL(16) : LOSA_SELECT_SMALL(32);
+#undef LOSA_SELECT_SMALL
+  }
+  // (registers hold 32 blocks per lane at most: longer rows take more warps.  Under the retained-mass rule the launch is a
+  // dependent: 1024 key blocks of 1536 rows 14.3 -> 11.6 us, 928 of 3716 22.4 -> 19.8.  Under the fixed-ratio rule its
+  // kernel is 13 - 17 % slower with loads that are not read-only ones, and waits for the kernel ahead.)
 #define LOSA_SELECT_ROWS(w, k)                                                                                 \
   do {                                                                                                         \
     const int ctas = (w) == 1 ? (rows + 3) / 4 : rows, threads = (w) == 1 ? 128 : 32 * (w);                    \
-    if (fixed_count > 0)                                                                                       \
-      select_rows_kernel<w, k, true><<<ctas, threads, 0, st>>>(mass, rows, nKb, tau, fixed_count, counts, bitmaps, status); \
-    else                                                                                                       \
-      select_rows_kernel<w, k, false><<<ctas, threads, 0, st>>>(mass, rows, nKb, tau, 0, counts, bitmaps, status); \
+    rc = fixed_count > 0 ? launch(select_rows_kernel<w, k, true>, dim3(ctas), threads, 0, st, false, mass, rows, nKb, tau,  \
+                                  fixed_count, counts, bitmaps, status)                                        \
+                         : launch(select_rows_kernel<w, k, false>, dim3(ctas), threads, 0, st, true, mass, rows, nKb, tau, \
+                                  0, counts, bitmaps, status);                                                 \
   } while (0)
+  int rc;
   if (nKb <= 256) LOSA_SELECT_ROWS(1, 8);
   else if (nKb <= 512) LOSA_SELECT_ROWS(1, 16);
   else if (nKb <= 1024) LOSA_SELECT_ROWS(1, 32);
@@ -676,7 +790,7 @@ int launch_select(int rows, int nKb, const float* mass, double tau, int fixed_co
   // four CTAs per SM at most (but no fewer rows than warps): adding up the sizes of the rows before
   // costs every CTA the same, so more of them only read more
   const int per_cta = max(kExpandThreads / 32, (rows + 591) / 592);
-  LOSA_CUDA_TRY(cudaGetLastError());
+  if (rc != LOSA_OK) return rc;
   return launch(expand_rows_kernel, dim3((rows + per_cta - 1) / per_cta), kExpandThreads, 0, st, true, counts, bitmaps, rows,
                 nKb, per_cta, offsets, kv_idx, kv_capacity, status);
 }
