@@ -367,12 +367,9 @@ __device__ __forceinline__ uint32_t emit_tile_list(const Params& p, int list, in
     na += __popc(ta & ~tb);
     nbb += __popc(tb & ~ta);
   }
-#pragma unroll
-  for (int d = 16; d > 0; d >>= 1) {
-    nb += __shfl_xor_sync(0xffffffffu, nb, d);
-    na += __shfl_xor_sync(0xffffffffu, na, d);
-    nbb += __shfl_xor_sync(0xffffffffu, nbb, d);
-  }
+  nb = __reduce_add_sync(0xffffffffu, nb);
+  na = ONE ? 0 : __reduce_add_sync(0xffffffffu, na);  // (a query tile's own list has one class)
+  nbb = ONE ? 0 : __reduce_add_sync(0xffffffffu, nbb);
   const int s1 = (nb + G - 1) / G * G;                       // entries of the first section
   const int tA = (na + G - 1) / G, tB = (nbb + G - 1) / G;   // K/V tiles of the single-tile classes
   const int tmin = min(tA, tB);

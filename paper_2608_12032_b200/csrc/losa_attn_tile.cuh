@@ -254,8 +254,15 @@ __device__ __forceinline__ void merge_in_cluster(const Params& p, int unit, int 
     const int row = r0 + sub;
     const bool here = row < row1 && T * 128 + row < p.N;
     const uint32_t at = (uint32_t)(row * kLanes + ((col & ~7) | ((col ^ row) & 7))) * 16u;
+    float4 v[2];
+    auto fetch = [&](int s0) {
+#pragma unroll
+      for (int j = 0; j < 2; ++j)
+        if (s0 + j < parts && here) v[j] = ptx::ld_cluster_f32x4(ptx::mapa(park_o + at, first + step * (s0 + j)));
+    };
     float2 ml = make_float2(0.f, 0.f);
     if (here && col < parts) ml = ptx::ld_cluster_f32x2(ptx::mapa(park_ml + 8u * row, first + step * col));
+    fetch(0);
     // (a part without keys of the row has the sum 0; one that met NaN has the sum NaN, and so has the row)
     float m = (ml.y != 0.f) ? ml.x : -INFINITY;
 #pragma unroll
@@ -263,14 +270,10 @@ __device__ __forceinline__ void merge_in_cluster(const Params& p, int unit, int 
     const float mine = (ml.y != 0.f) ? ptx::ex2_approx(ml.x - m) : 0.f;
     float L = 0.f;
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-    // (two parts at a time: unrolled over all eight, the code that a short call runs once and cold took longer than its
-    // loads)
+    // (two parts at a time, the first two ahead: unrolled over all eight, the code that a short call runs once and cold took
+    // longer than its loads)
 #pragma unroll 1
     for (int s0 = 0; s0 < parts; s0 += 2) {
-      float4 v[2];
-#pragma unroll
-      for (int j = 0; j < 2; ++j)
-        if (s0 + j < parts && here) v[j] = ptx::ld_cluster_f32x4(ptx::mapa(park_o + at, first + step * (s0 + j)));
 #pragma unroll
       for (int j = 0; j < 2; ++j) {
         if (s0 + j >= parts) break;
@@ -283,6 +286,7 @@ __device__ __forceinline__ void merge_in_cluster(const Params& p, int unit, int 
           acc.w += v[j].w * sc;
         }
       }
+      fetch(s0 + 2);
     }
     if (!here) continue;
     const float inv = (L != 0.f) ? 1.f / L : 0.f;
@@ -399,7 +403,15 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   int over = -1;
   auto unit_over = [&]() -> bool {
     ptx::tc_fence_before_sync();
-    ptx::cluster_meet();
+    // What was stored into another CTA's shared memory - arrivals on a pair's barriers, the abort flag - has to be there
+    // before that CTA may leave, and what is left for the other parts before they read it.  (Elsewhere a release would only
+    // wait for O's way to memory.)
+    if (PAIR || (in_cluster && warp >= 4)) {
+      ptx::cluster_meet();
+    } else {
+      ptx::cluster_arrive_relaxed();
+      ptx::cluster_wait();
+    }
     over = *reinterpret_cast<volatile uint32_t*>(&ctl->cluster_marked) == 0u ? 1 : 0;
     return over != 0;
   };
