@@ -255,7 +255,9 @@ __device__ __forceinline__ uint32_t kept_words(RowShared* rs, const float* src, 
   // (blocks past the row's end weigh nothing; they are told apart by their index where they could count)
   uint32_t bits[K];
 #pragma unroll
-  for (int k = 0; k < K; ++k) bits[k] = (k * 32 + lane < mine) ? __float_as_uint(load(src + k * 32)) : 0u;
+  for (int k = 0; k < K; ++k) bits[k] = 0u;
+#pragma unroll
+  for (int k = 0; k < K; ++k) if (k * 32 + lane < mine) bits[k] = __float_as_uint(load(src + k * 32));
   for (int i = t; i < kBins; i += T) {
     rs->cnt[i] = 0u;
     if (!COUNT) rs->low[i] = 0u;
@@ -265,14 +267,24 @@ __device__ __forceinline__ uint32_t kept_words(RowShared* rs, const float* src, 
     rs->bin = -1;
   }
   row_sync<W>();
+  // (what is no mass is looked for one by one only where there is any: 22296 rows of 3713, fixed ratio 258 -> 245 us, 3716 of
+  // 929 18.4 -> 16.9; retained mass 211.3 -> 210.4, 2200 of 275 30.5 -> 29.9)
   bool bad = false;
   float sum = 0.0f;
+  uint32_t top = 0u;
+#pragma unroll
+  for (int k = 0; k < K; ++k) top = max(top, bits[k]);
+  if (__any_sync(0xffffffffu, top > kMaxMassBits)) {
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+      if (bits[k] > kMaxMassBits) {  // negative, NaN, or far beyond any mass; -0 becomes +0
+        bad |= bits[k] != 0x80000000u;
+        bits[k] = 0u;
+      }
+    }
+  }
 #pragma unroll
   for (int k = 0; k < K; ++k) {
-    if (bits[k] > kMaxMassBits) {  // negative, NaN, or far beyond any mass; -0 becomes +0
-      bad |= bits[k] != 0x80000000u;
-      bits[k] = 0u;
-    }
     sum += __uint_as_float(bits[k]);
     // (a mass of zero changes no sum: only the fixed-ratio rule counts it)
     if (COUNT ? k * 32 + lane < mine : bits[k] != 0u) {
