@@ -339,11 +339,13 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   // the mass pass alone has no V, no P and no O: its score buffers go back as soon as they are read
   constexpr bool kHasV = (MODE != kMass);
   // When a unit's place is read from its header: at its end, but in those mass passes that came out faster with it in
-  // registers from the unit's start.  That is the compiler's ordering of the exponentials, not the seven registers, so
-  // the line lies where it was measured, and has to be measured again when the loop changes (16384 tokens, 12 heads, us at
-  // the start / at the end: D = 64, C = 32 959 / 915, C = 64 823 / 855, C = 128 883 / 865; D = 128, C = 32 1006 / 977,
-  // C = 64 967 / 926, C = 128 968 / 1007).
-  constexpr bool kInfoEarly = MODE == kMass && C_ == (D == 64 ? 64 : 128);
+  // registers from the unit's start; and which four of 16 scores the mass pass takes from the polynomial.  That is the
+  // compiler's ordering of the exponentials, so the lines lie where they were measured, and have to be measured again when
+  // the loop changes (masses, 16384 tokens, 12 heads, us: at the start / at the end, and with the second four instead of the
+  // first: D = 64, C = 32 908 / 917, 920 / 929, C = 64 826 / 854, 886 / 826, C = 128 851 / 843, 818 / 843; D = 128, C = 32
+  // 1059 / 992, 1023 / 1054, C = 64 963 / 948, 965 / 945, C = 128 946 / 961, 918 / 956).
+  constexpr bool kInfoEarly = MODE == kMass && (C_ == 128 || (D == 64 && C_ == 64));
+  constexpr int kPolyAt = (MODE == kMass && C_ == 128) ? 1 : 0;
   constexpr int kChunkTiles = (MODE == kSparse) ? 32 / kG : (1 << 28);  // K/V tiles per chunk of the list
   static_assert(offsetof(TileControl, tl) % 16 == 0, "the tile list is read with 16-byte loads");
   static_assert(offsetof(TileControl, redo_need) == offsetof(TileControl, redo_mark) + 16, "reached from the marks");
@@ -1288,7 +1290,7 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
             float2 x1 = ptx::fma2(make_float2(__uint_as_float(sr[c + 2]), __uint_as_float(sr[c + 3])), sc2,
                                   nm2[c / kBW]);
             // (at head dimension 128 a share of these on the FMA pipe measured -1 % at 12.5 % and +5 % at 25 %)
-            if (kPolyOf > 0 && (c >> 2) % (kPolyOf > 0 ? kPolyOf : 1) == 0) {
+            if (kPolyOf > 0 && (c >> 2) % (kPolyOf > 0 ? kPolyOf : 1) == kPolyAt) {
               x0 = ptx::ex2_poly2(x0);
               x1 = ptx::ex2_poly2(x1);
             } else {
