@@ -21,7 +21,7 @@ def masses(rows, nKb, seed):
 
 
 @pytest.mark.parametrize("rows", [1, 15, 16, 17, 128, 129, 255, 256, 257])
-@pytest.mark.parametrize("nKb", [1, 33, 256, 257, 1024])
+@pytest.mark.parametrize("nKb", [1, 4, 32, 33, 256, 257, 1024])
 def test_row_counts_around_the_cluster(rows, nKb):
     losa = lib()
     m = masses(rows, nKb, rows + nKb)
@@ -53,3 +53,22 @@ def test_a_capacity_that_is_too_small_and_masses_that_are_none():
     a, b = offsets.tolist(), offsets2.tolist()
     for r in set(range(40)) - {3, 39}:  # the other rows are untouched
         assert torch.equal(idx[a[r]:a[r + 1]], idx2[b[r]:b[r + 1]])
+
+
+@pytest.mark.parametrize("nKb", [2, 8, 31, 32, 33])
+@pytest.mark.parametrize("tau", [1e-7, 0.25, 0.5, 0.515625, 1.0])
+def test_ties_zeros_and_sums_that_just_reach_tau(nKb, tau):
+    """Masses in units of 2^-6, many of them equal or zero, some rows adding up to less than tau: whole in every arithmetic."""
+    losa = lib()
+    rng = np.random.default_rng(nKb)
+    m = rng.integers(0, 4, (20, nKb)).astype(np.float64)
+    m[0], m[1], m[2] = 0.0, 1.0, 0.0
+    m[2, nKb // 2] = 64.0
+    for r in range(3, 20):
+        m[r, rng.integers(nKb)] += max(0.0, 64.0 - m[r].sum()) if r < 17 else 0.0
+    m /= 64.0
+    offsets, idx = losa.losa_select(torch.from_numpy(m).float().reshape(1, 1, 20, nKb).cuda(), tau)
+    ref = orc.select(m, tau)
+    assert np.array_equal(offsets.cpu().numpy(), ref.offsets)
+    assert np.array_equal(idx.cpu().numpy()[:ref.offsets[-1]], ref.kv_idx)
+    assert losa.losa_async_status() == 0
