@@ -51,21 +51,22 @@ FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustain
 
 
 def launches_per_call(wl, slots: int, attention_only: bool) -> int:
-    """Kernels launched by one attention-shaped call: its kernel; before it the work units' tile lists (sparse)
-    or the launch's counters, if there are more units than work slots; behind it the merge of the last wave's
-    units, if they are cut into parts."""
+    """Kernels launched by one attention-shaped call: its kernel; and if there are more units than work slots, before it
+    the work units' tile lists (sparse) or the launch's counters, behind it the merge of the last wave's units, where they
+    are cut into parts.  (In a single wave the clusters merge them.)"""
     items = wl.B * wl.H * ((-(-wl.N // 128) + 1) // 2)
     rest = items if items < slots else items % slots
     parts = min(slots // rest if rest else 1, 8, wl.nKb)
     cut = attention_only and parts >= 2
     units = items + rest * (parts - 1) if cut else items
-    return 1 + (units > slots) + cut
+    return 1 + (units > slots) * (1 + cut)
 
 
 def launches_per_step(wl, slots: int, draws: int) -> int:
-    """Kernels of the library launched by one step: mass pass, selection (two), the sparse draws, the dense and
-    the fused call."""
-    return (launches_per_call(wl, slots, False) + 2 + (draws + 1) * launches_per_call(wl, slots, True)
+    """Kernels of the library launched by one step: mass pass, selection (two, or one for a few rows), the sparse draws,
+    the dense and the fused call."""
+    select = 1 if wl.rows <= 256 and wl.nKb <= 1024 else 2
+    return (launches_per_call(wl, slots, False) + select + (draws + 1) * launches_per_call(wl, slots, True)
             + launches_per_call(wl, slots, False))
 
 
