@@ -689,20 +689,15 @@ int launch_t(const Geometry& g, const void* q, const void* k, const void* v, Par
     int parts = rest > 0 ? slots / rest : 1;
     parts = min(min(parts, kMaxParts), prm.nKb);
     if (parts >= 2 && rest == prm.nWork) {
-      // A single wave: as many parts of an item in one cluster as the device has room for (at head dimension 64 in one for
-      // each of its query tiles), if the units are not longer by more K/V tiles than a launch for the merge takes (4 us; a
-      // tile 0.65 us at head dimension 64, 0.8 at 128).
-      int n = 0, fit = parts;
-      for (; fit >= 2; --fit) {
-        if ((rc = configure_tile<D, R, C_, MODE, kPair, true>(sms, kTileCtas * fit, &n, &cfg, attr)) == LOSA_ERR_CUDA) return rc;
-        if (rc == LOSA_OK && n >= rest * (kPair ? 1 : 2)) break;
-      }
-      constexpr int kBlocks = 128 / C_, kMergeTiles = kPair ? 5 : 6;
-      const int tiles = (prm.nKb + kBlocks - 1) / kBlocks;
-      if (fit >= 2 && (tiles + fit - 1) / fit <= (tiles + parts - 1) / parts + kMergeTiles) {
+      // A single wave: the parts of an item in one cluster (at head dimension 64 of each of its query tiles), where the
+      // device holds all of them at once - of 16 CTAs 7, of 8 15, of 6 22, of 4 33, of 3 45.  Elsewhere a launch behind
+      // merges them: with fewer parts, which would fit, calls were up to 30 % faster, but a part's largest weights round to
+      // themselves, and the error against 64 bits grew (264 tokens, 4 heads, D = 64, 8 parts / 7: 1.7e-3 / 1.8e-3).
+      int n = 0;
+      if ((rc = configure_tile<D, R, C_, MODE, kPair, true>(sms, kTileCtas * parts, &n, &cfg, attr)) == LOSA_ERR_CUDA) return rc;
+      if (rc == LOSA_OK && n >= rest * (kPair ? 1 : 2)) {
         prm.in_cluster = 1;
-        ctas = kTileCtas * fit;
-        parts = fit;
+        ctas = kTileCtas * parts;
       }
     }
     if (parts >= 2) {
