@@ -191,7 +191,8 @@ int losa_select_noalloc(int32_t B, int32_t H, int32_t nQb, int32_t nKb, const fl
  *            plus the work units' tile lists: the counter the persistent CTAs draw work
  *            items from, the partial results of the last work items, which are processed in
  *            parts and merged by a second launch on the same stream (by the same launch, where
- *            the call has no more work units than slots), and a word per work
+ *            the call has no more work units than slots and the device holds the clusters that
+ *            the parts of an item then share), and a word per work
  *            unit for those that are recomputed because their scores outgrew the reference
  *            of their first tile); not shared between calls that may run
  *            concurrently; contents undefined afterwards.  The result does not depend on

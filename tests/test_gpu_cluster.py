@@ -1,6 +1,7 @@
-"""Items that a single wave is cut into: their parts run in one cluster and are merged through its CTAs' shared memory,
-from two parts to as many as there can be, of an odd number of query tiles with a short last one; some parts outgrow their
-reference and are run again, the others of their cluster wait for them.  Against the fp64 oracle."""
+"""Items that a single wave is cut into: their parts run in one cluster and are merged through its CTAs' shared memory
+(or, where the device does not hold all these clusters at once, by a launch behind: 10 items), from two parts to as many as
+there can be, of an odd number of query tiles with a short last one; some parts outgrow their reference and are run again,
+the others of their cluster wait for them.  Against the fp64 oracle."""
 import pytest
 import torch
 
