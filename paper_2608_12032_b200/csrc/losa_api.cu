@@ -23,9 +23,7 @@ const char* set_cuda_error(cudaError_t e, const char* what) {
   return g_cuda_error;
 }
 
-int check_device() {
-  int dev = 0;
-  LOSA_CUDA_TRY(cudaGetDevice(&dev));
+static int check_device(int dev) {
   if (dev < 0 || dev >= kMaxDevices) return LOSA_ERR_UNSUPPORTED;
   int ok = g_device_ok[dev].load(std::memory_order_acquire);
   if (ok == 0) {
@@ -42,18 +40,27 @@ int check_device() {
   return LOSA_OK;
 }
 
+int check_device() {
+  int dev = 0;
+  LOSA_CUDA_TRY(cudaGetDevice(&dev));
+  return check_device(dev);
+}
+
 const DeviceState* device_state(int* rc) {
   int dev = 0;
-  *rc = check_device();
-  if (*rc != LOSA_OK) return nullptr;
-  if (cudaGetDevice(&dev) != cudaSuccess) {
+  const cudaError_t got = cudaGetDevice(&dev);
+  if (got != cudaSuccess) {
+    set_cuda_error(got, "cudaGetDevice");
     *rc = LOSA_ERR_CUDA;
     return nullptr;
   }
+  *rc = check_device(dev);
+  if (*rc != LOSA_OK) return nullptr;
   if (g_state_ready[dev].load(std::memory_order_acquire)) return &g_state[dev];
   std::lock_guard<std::mutex> lock(g_state_mutex);
   if (g_state_ready[dev].load(std::memory_order_acquire)) return &g_state[dev];
   DeviceState st{};
+  st.ordinal = dev;
   cudaError_t e = cudaDeviceGetAttribute(&st.sm_count, cudaDevAttrMultiProcessorCount, dev);
   if (e == cudaSuccess) {
     int* h = nullptr;
@@ -137,10 +144,10 @@ int32_t losa_work_slots(int op, const losa_problem_t* p) {
   const DeviceState* dev = device_state(&rc);
   if (!dev) return 0;
   switch (op) {
-    case LOSA_OP_BLOCK_MASS: return attn_work_slots(kMass, g, dev->sm_count);
-    case LOSA_OP_SPARSE_ATTN: return attn_work_slots(kSparse, g, dev->sm_count);
-    case LOSA_OP_ATTN: return attn_work_slots(kDense, g, dev->sm_count);
-    case LOSA_OP_ATTN_MASS: return attn_work_slots(kFused, g, dev->sm_count);
+    case LOSA_OP_BLOCK_MASS: return attn_work_slots(kMass, g, *dev);
+    case LOSA_OP_SPARSE_ATTN: return attn_work_slots(kSparse, g, *dev);
+    case LOSA_OP_ATTN: return attn_work_slots(kDense, g, *dev);
+    case LOSA_OP_ATTN_MASS: return attn_work_slots(kFused, g, *dev);
   }
   return 0;
 }

@@ -602,7 +602,7 @@ write_problems_kernel(const __grid_constant__ ProblemChunk chunk, ProblemEntry* 
 // false) CTAs - a call may have at work there.
 // `ctas`: of a cluster.
 template <int D, int R, int C_, int MODE, bool PAIR, bool ONE>
-int configure_tile(int sms, int ctas, int* clusters, cudaLaunchConfig_t* cfg, cudaLaunchAttribute* attr) {
+int configure_tile(const DeviceState& on, int ctas, int* clusters, cudaLaunchConfig_t* cfg, cudaLaunchAttribute* attr) {
   using L = Lay;
   constexpr size_t smem = (size_t)tile_nq(D, MODE) * 256 * D + (size_t)(tile_nk(MODE) + tile_nv(MODE)) * kTileStage +
                           (D == 64 ? kTileOnes : 0) + sizeof(TileControl);
@@ -610,8 +610,7 @@ int configure_tile(int sms, int ctas, int* clusters, cudaLaunchConfig_t* cfg, cu
   auto kern = losa_tile_kernel<D, R, C_, MODE, PAIR, ONE>;
   // how many clusters of so many CTAs the device holds at once
   static std::atomic<int> max_on[kMaxDevices][kMaxClusterCtas + 1];
-  int dev = 0;
-  LOSA_CUDA_TRY(cudaGetDevice(&dev));
+  const int dev = on.ordinal, sms = on.sm_count;
   *cfg = {};
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
@@ -654,23 +653,23 @@ int configure_tile(int sms, int ctas, int* clusters, cudaLaunchConfig_t* cfg, cu
 // cluster) or one CTA for each (head dimension 64).  Head dimension 128 with 64-row query blocks, 9600 tokens, 12 heads,
 // against two query tiles on one CTA: dense 557 -> 487 us, sparse 457 -> 419, masses 474 -> 359, construction step 703 -> 538.
 template <int D, int R, int C_, int MODE>
-int work_slots(int sms, int* slots) {
+int work_slots(const DeviceState& dev, int* slots) {
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute attr[2];
   int n = 0;
-  const int rc = configure_tile<D, R, C_, MODE, D == 128, false>(sms, D == 128 ? 2 : 1, &n, &cfg, attr);
+  const int rc = configure_tile<D, R, C_, MODE, D == 128, false>(dev, D == 128 ? 2 : 1, &n, &cfg, attr);
   *slots = (D == 128) ? n : max(1, n / 2);
   return rc;
 }
 
 template <int D, int R, int C_, int MODE>
-int launch_t(const Geometry& g, const void* q, const void* k, const void* v, Params prm, int sms,
-             cudaStream_t st) {
+int launch_t(const Geometry& g, const void* q, const void* k, const void* v, Params prm,
+             const DeviceState& dev, cudaStream_t st) {
   constexpr bool kPair = D == 128;
   ProblemEntry maps;
   int rc, slots;
   if ((rc = make_maps(&maps, g, q, k, MODE != kMass ? v : nullptr)) != LOSA_OK) return rc;
-  if ((rc = work_slots<D, R, C_, MODE>(sms, &slots)) != LOSA_OK) return rc;
+  if ((rc = work_slots<D, R, C_, MODE>(dev, &slots)) != LOSA_OK) return rc;
   // The items of the last, partly filled wave of the persistent grid (all items, if there are
   // fewer than slots) are cut into parts of the key range, so that the wave ends after 1/parts of
   // an item; their partial results are merged by their clusters or by a launch behind.  Attention output
@@ -694,7 +693,7 @@ int launch_t(const Geometry& g, const void* q, const void* k, const void* v, Par
       // merges them: with fewer parts, which would fit, calls were up to 30 % faster, but a part's largest weights round to
       // themselves, and the error against 64 bits grew (264 tokens, 4 heads, D = 64, 8 parts / 7: 1.7e-3 / 1.8e-3).
       int n = 0;
-      if ((rc = configure_tile<D, R, C_, MODE, kPair, true>(sms, kTileCtas * parts, &n, &cfg, attr)) == LOSA_ERR_CUDA) return rc;
+      if ((rc = configure_tile<D, R, C_, MODE, kPair, true>(dev, kTileCtas * parts, &n, &cfg, attr)) == LOSA_ERR_CUDA) return rc;
       if (rc == LOSA_OK && n >= rest * (kPair ? 1 : 2)) {
         prm.in_cluster = 1;
         ctas = kTileCtas * parts;
@@ -727,7 +726,7 @@ int launch_t(const Geometry& g, const void* q, const void* k, const void* v, Par
   if (rc != LOSA_OK) return rc;
   auto launch_tile = [&](auto one) -> int {
     int n = 0;
-    const int rc = configure_tile<D, R, C_, MODE, kPair, decltype(one)::value>(sms, ctas, &n, &cfg, attr);
+    const int rc = configure_tile<D, R, C_, MODE, kPair, decltype(one)::value>(dev, ctas, &n, &cfg, attr);
     if (rc != LOSA_OK) return rc;
     cfg.gridDim = dim3(2 * min(slots, prm.nUnits), 1, 1);
     cfg.stream = st;
@@ -748,19 +747,19 @@ int launch_t(const Geometry& g, const void* q, const void* k, const void* v, Par
 
 template <int MODE>
 int dispatch(const Geometry& g, const void* q, const void* k, const void* v, const Params& prm,
-             int sms, cudaStream_t st) {
+             const DeviceState& dev, cudaStream_t st) {
 #define LOSA_CASE(d, r, c) \
-  if (g.D == d && g.R == r && g.C == c) return launch_t<d, r, c, MODE>(g, q, k, v, prm, sms, st);
+  if (g.D == d && g.R == r && g.C == c) return launch_t<d, r, c, MODE>(g, q, k, v, prm, dev, st);
   LOSA_GEOMETRIES(LOSA_CASE)
 #undef LOSA_CASE
   return LOSA_ERR_UNSUPPORTED;
 }
 
 template <int MODE>
-int slots_of(const Geometry& g, int sms) {
+int slots_of(const Geometry& g, const DeviceState& dev) {
   int slots = 0;
 #define LOSA_CASE(d, r, c) \
-  if (g.D == d && g.R == r && g.C == c) return work_slots<d, r, c, MODE>(sms, &slots) == LOSA_OK ? slots : 0;
+  if (g.D == d && g.R == r && g.C == c) return work_slots<d, r, c, MODE>(dev, &slots) == LOSA_OK ? slots : 0;
   LOSA_GEOMETRIES(LOSA_CASE)
 #undef LOSA_CASE
   return 0;
@@ -792,14 +791,14 @@ size_t tl_entries_bytes(const Geometry& g, int n_prob) {
 
 void arm_stalled_launch(uint32_t polls) { g_stall_polls.store(polls); }
 
-// Work slots that a call of this kind occupies on the current device, which has `sms` multiprocessors, for callers that
+// Work slots that a call of this kind occupies on the current device, for callers that
 // want to know how the work items are spread (which of them the last wave cuts into parts); 0 where it cannot run.
-int attn_work_slots(AttnMode mode, const Geometry& g, int sms) {
+int attn_work_slots(AttnMode mode, const Geometry& g, const DeviceState& dev) {
   switch (mode) {
-    case kDense: return slots_of<kDense>(g, sms);
-    case kSparse: return slots_of<kSparse>(g, sms);
-    case kMass: return slots_of<kMass>(g, sms);
-    case kFused: return slots_of<kFused>(g, sms);
+    case kDense: return slots_of<kDense>(g, dev);
+    case kSparse: return slots_of<kSparse>(g, dev);
+    case kMass: return slots_of<kMass>(g, dev);
+    case kFused: return slots_of<kFused>(g, dev);
   }
   return 0;
 }
@@ -900,16 +899,15 @@ int launch_attn(AttnMode mode, const Geometry& g, const void* q, const void* k, 
   const DeviceState* dev = device_state(&rc);
   if (!dev) return rc;
   prm.status = dev->status_dev;
-  const int sms = dev->sm_count;
   // one-shot diagnostic armed by losa_debug_stall_next_launch()
   const uint32_t stall_polls = g_stall_polls.exchange(0u);
   prm.stall = stall_polls > 0u ? 1 : 0;
   prm.wait_polls = stall_polls > 0u ? stall_polls : ptx::kWaitPolls;
   switch (mode) {
-    case kDense: return dispatch<kDense>(g, q, k, v, prm, sms, st);
-    case kSparse: return dispatch<kSparse>(g, q, k, v, prm, sms, st);
-    case kMass: return dispatch<kMass>(g, q, k, v, prm, sms, st);
-    case kFused: return dispatch<kFused>(g, q, k, v, prm, sms, st);
+    case kDense: return dispatch<kDense>(g, q, k, v, prm, *dev, st);
+    case kSparse: return dispatch<kSparse>(g, q, k, v, prm, *dev, st);
+    case kMass: return dispatch<kMass>(g, q, k, v, prm, *dev, st);
+    case kFused: return dispatch<kFused>(g, q, k, v, prm, *dev, st);
   }
   return LOSA_ERR_INVALID_ARG;
 }
