@@ -571,7 +571,40 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       const uint32_t tl_a = ptx::smem_u32(&ctl->tl[0]);
       uint32_t nq = 0, nk = 0, vs = 0, v_par = 1u, nu = 0, nc = 0, hdr[12];
       int problem = -1;  // batched launch: whose tensor maps this warp has acquired
+      // One wave: every stage and score buffer is free again.  The tensor cores say so, in both CTAs of a pair, some time
+      // after the MMAs were issued, and nobody else waits for the last of it: a CTA must not leave before.  A lane for each;
+      // false: gave up.  (In the other kernels two headers lie between the last of it and the end.)
+      auto all_returned = [&]() -> bool {
+        const int who = __ffs(__ballot_sync(0xffffffffu, leader)) - 1;  // (it alone has counted)
+        const uint32_t k0 = __shfl_sync(0xffffffffu, nk, who), v0 = __shfl_sync(0xffffffffu, vs, who);
+        const uint32_t v0_par = __shfl_sync(0xffffffffu, v_par, who);
+        uint32_t bar = 0u, par = 0u;
+        if (lane < kNQ) {
+          const uint32_t i = nq + lane;
+          bar = ptx::smem_u32(&ctl->q_empty[i % kNQ]);
+          par = ((i / kNQ) & 1u) ^ 1u;
+        } else if (lane < kNQ + kNK) {
+          const uint32_t i = k0 + lane - kNQ;
+          bar = k_empty_a + 8u * (i % kNK);
+          par = ((i / kNK) & 1u) ^ 1u;
+        } else if (lane < kNQ + kNK + kNV) {
+          const uint32_t i = lane - kNQ - kNK;
+          bar = v_empty_a + 8u * i;
+          par = i >= v0 ? v0_par : v0_par ^ 1u;
+        } else if (kHasV && rank == 0 && lane < kNQ + kNK + kNV + 3) {
+          const uint32_t i = k0 + lane - kNQ - kNK - kNV;  // (a product for each K tile)
+          bar = ptx::smem_u32(&ctl->pv_done[i % 3u]);
+          par = ((i / 3u) & 1u) ^ 1u;
+        }
+        if (bar != 0u && !ptx::mbar_wait_relaxed_u32(bar, par, &ctl->abort_flag, p.wait_polls)) {
+          ctl->abort_flag = 1;
+          report_error(p.status, LOSA_ERR_TIMEOUT);
+        }
+        __syncwarp();
+        return *reinterpret_cast<volatile int*>(&ctl->abort_flag) == 0;
+      };
       for (;;) {
+        if (ONE && nu == 1u && !all_returned()) goto teardown;
         TILE_HDR_NEXT(hdr, 3);
         const uint32_t ent = hdr[0], word = hdr[1];
         if (ent == kTlSkip) {
@@ -690,6 +723,7 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           if (MODE == kSparse) TILE_CHUNK_DONE();
         }
       }
+      if (ONE) all_returned();
     } else if (warp == kIssuerWarp && rank == 0) {
       // ------------------------------------------------------------------ S = Q K^T of the pair
       // Score k of the launch goes into buffer k % 3, which holds the P of score k - 3 until the
@@ -754,6 +788,13 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       auto v_desc = [&](uint32_t bytes) { return v_lo + (bytes >> 4) - (kSumCol ? (bytes >> 4) << 16 : 0u); };
       const uint32_t tO = tmem_base + 384;
       uint32_t nof = 0, nt = 0, nv = 0, nu = 0, hdr[4];
+      // one wave, no products to wait for: this thread's own arrivals, which are there before it meets the other warps, not
+      // the tensor cores', which nobody waits for
+      const uint32_t o_done1 = at1(&ctl->o_done[0]);
+      auto no_products = [&](uint32_t od) {
+        ptx::mbar_arrive(&ctl->o_done[od]);
+        if (PAIR) ptx::mbar_arrive_cluster(o_done1 + 8u * od);
+      };
       for (;;) {
         TILE_HDR_NEXT(hdr, 1);
         const uint32_t ent = hdr[0], word = hdr[1];
@@ -765,7 +806,10 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
             LOSA_WAIT(&ctl->p_ready[nt % 3u], (nt / 3u) & 1);
             if (leader) commit0<PAIR>(&ctl->pv_done[nt % 3u]);
           }
-          if (leader) commit_all<PAIR>(&ctl->o_done[od], pair_ctas);
+          if (leader) {
+            if (ONE) no_products(od);
+            else commit_all<PAIR>(&ctl->o_done[od], pair_ctas);
+          }
           continue;
         }
         uint32_t pv_item = 0;
@@ -796,7 +840,10 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           ++nt;
           ++nv;
         }
-        if (leader) commit_all<PAIR>(&ctl->o_done[od], pair_ctas);  // every product of the item is done
+        if (leader) {
+          if (ONE && pv_item == 0) no_products(od);
+          else commit_all<PAIR>(&ctl->o_done[od], pair_ctas);  // every product of the item is done
+        }
         if (pv_item > 0) ++nof;
       }
     } else if (warp == kSchedulerWarp && rank == 0) {

@@ -2,9 +2,11 @@
 (or, where the device does not hold all these clusters at once, by a launch behind: 10 items), from two parts to as many as
 there can be, of an odd number of query tiles with a short last one; some parts outgrow their reference and are run again,
 the others of their cluster wait for them.  Against the fp64 oracle."""
+import numpy as np
 import pytest
 import torch
 
+from oracle import losa_oracle as orc
 from tests import util
 from tests.test_gpu_units import check, lib
 
@@ -40,3 +42,23 @@ def test_cut_items_of_a_batched_call_and_of_token_major_tensors(D, R, C):
         # 10 items in 7 parts, 20 in 3: P rounds against another reference, 2^-9 each at random
         assert (o - single).norm() <= 4e-3 * single.norm()
     assert losa.losa_async_status() == 0
+
+
+@pytest.mark.parametrize("D,R,C", [(64, 64, 64), (64, 128, 32), (128, 128, 128), (128, 64, 64)])
+@pytest.mark.parametrize("H", [2])
+def test_parts_that_list_nothing(D, R, C, H):
+    """Lists of one to three key blocks cut into seven parts (10 items, merged by a launch behind): most units have no K/V
+    tile and end as soon as their query tile is there."""
+    losa = lib()
+    nQb, nKb = -(-N // R), -(-N // C)
+    q, k, v = (util.rand_bf16((1, H, N, D), 1740 + i) for i in range(3))
+    rng = np.random.default_rng(1750 + H)
+    rows = [np.sort(rng.choice(nKb, rng.integers(1, 4), replace=False)) for _ in range(H * nQb)]
+    off = np.concatenate([[0], np.cumsum([len(r) for r in rows])]).astype(np.int32)
+    idx = np.concatenate(rows).astype(np.int32)
+    args = [x.cuda() for x in (q, k, v, torch.from_numpy(off), torch.from_numpy(idx))]
+    outs = [losa.losa_sparse_attn(*args, R, C, out_dtype=torch.float32) for _ in range(20)]
+    assert losa.losa_async_status() == 0
+    want = orc.blocks_to_tokens(orc.sparse_attn(*(util.to_np(x) for x in (q, k, v)), R, C, off, idx), 1, H, N)
+    util.assert_output_close(outs[0], want, "short lists")
+    assert all(torch.equal(outs[0], o) for o in outs[1:])
