@@ -254,7 +254,7 @@ __device__ __forceinline__ void merge_in_cluster(const Params& p, int unit, int 
     const int row = r0 + sub;
     const bool here = row < row1 && T * 128 + row < p.N;
     const uint32_t at = (uint32_t)(row * kLanes + ((col & ~7) | ((col ^ row) & 7))) * 16u;
-    float4 v[2];
+    float4 v[2] = {make_float4(0.f, 0.f, 0.f, 0.f), make_float4(0.f, 0.f, 0.f, 0.f)};
     auto fetch = [&](int s0) {
 #pragma unroll
       for (int j = 0; j < 2; ++j)
@@ -279,12 +279,13 @@ __device__ __forceinline__ void merge_in_cluster(const Params& p, int unit, int 
         if (s0 + j >= parts) break;
         const float sc = __shfl_sync(0xffffffffu, mine, s0 + j, kLanes);
         L += __shfl_sync(0xffffffffu, ml.y, s0 + j, kLanes) * sc;
-        if (sc != 0.f && here) {
-          acc.x += v[j].x * sc;
-          acc.y += v[j].y * sc;
-          acc.z += v[j].z * sc;
-          acc.w += v[j].w * sc;
-        }
+        // (What was fetched is used, also where it weighs nothing: the last meeting waits for no reads, and the CTA that is
+        // read from must not leave before they have come.  A zero adds nothing to a sum that is never -0.)
+        const bool none = sc == 0.f;
+        acc.x += (none ? 0.f : v[j].x) * sc;
+        acc.y += (none ? 0.f : v[j].y) * sc;
+        acc.z += (none ? 0.f : v[j].z) * sc;
+        acc.w += (none ? 0.f : v[j].w) * sc;
       }
       fetch(s0 + 2);
     }

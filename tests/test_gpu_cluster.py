@@ -45,10 +45,11 @@ def test_cut_items_of_a_batched_call_and_of_token_major_tensors(D, R, C):
 
 
 @pytest.mark.parametrize("D,R,C", [(64, 64, 64), (64, 128, 32), (128, 128, 128), (128, 64, 64)])
-@pytest.mark.parametrize("H", [2])
+@pytest.mark.parametrize("H", [1, 2])
 def test_parts_that_list_nothing(D, R, C, H):
-    """Lists of one to three key blocks cut into seven parts (10 items, merged by a launch behind): most units have no K/V
-    tile and end as soon as their query tile is there."""
+    """Lists of one to three key blocks cut into eight parts (5 items, in clusters) or seven (10 items at D = 128 and 64,
+    merged by a launch behind): most units have no K/V tile and end as soon as their query tile is there, and others
+    list blocks of one of their query blocks only, so that the other's rows have no weight in that part."""
     losa = lib()
     nQb, nKb = -(-N // R), -(-N // C)
     q, k, v = (util.rand_bf16((1, H, N, D), 1740 + i) for i in range(3))
