@@ -1686,8 +1686,9 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
 
 teardown:
   if (ctl->abort_flag) {
-    // the other CTA's waits give up at their next look at the flag
-    if (PAIR && lane == 0) ptx::st_cluster_u32(abort_peer, 1u);
+    // the other CTA's waits give up at their next look at the flag (where all have met already, none is left to be told,
+    // and that CTA may be gone)
+    if (PAIR && lane == 0 && !(ONE && over == 1)) ptx::st_cluster_u32(abort_peer, 1u);
     // give MMAs and bulk copies still in flight a bounded time to land before shared memory and
     // tensor memory are released
     if (rank == 0 && (warp == kIssuerWarp || warp == kIssuerWarp + 1) && ptx::elect_one()) {
