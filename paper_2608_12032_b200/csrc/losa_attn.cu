@@ -128,7 +128,7 @@ struct Params {
   // How many work units were run again because their scores outgrew the reference, and a flag for each, so that one
   // is counted once.  Where units are neither drawn nor merged nobody counts them.
   int* redo_count;
-  int* redo_flag;  // [nUnits], or a word per tile list (one_wave)
+  int* redo_flag;  // [nUnits], or a word per tile list (one_wave, where items are cut)
   // No more work units than work slots: each slot takes the one at its position, and needs
   // nothing prepared for it (counters, flags, tile lists), which saves a launch: the CTAs make their unit's
   // tile list themselves, and each list's flag says whether its unit was run again (where parts are merged).

@@ -858,8 +858,8 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       int acquired = -1;  // batched launch: whose tensor maps this warp has acquired
       bool first_item = true, drawn = false;
       uint32_t own_word = 0u;  // one_wave: what tl_count holds of the CTA's unit
-      // (how many units were run again is for tests to read: whoever adds to it has run two, ten microseconds later)
-      if (in_cluster && blockIdx.x == 0 && lane == 0) *p.redo_count = 0;
+      // (how many units were run again is for tests to read: where no launch behind adds their flags up, the flags say it)
+      if (in_cluster && blockIdx.x == 0 && lane == 0) *p.redo_count = -1;
       if (MODE == kSparse && ONE) {
         uint32_t* const bm = reinterpret_cast<uint32_t*>(&ctl->xch[0][0][0]);
         own_word = emit_tile_list<kListBlocks, kG, kOne>(p, first_list(), lane, bm, bm + kListAt);
@@ -918,7 +918,7 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           continue;
         }
         if (ONE && nu == 1u && unit_over()) {
-          if (p.split_parts > 1 && !in_cluster && lane == 0) p.redo_flag[first_list()] = 0;
+          if (p.split_parts > 1 && lane == 0) p.redo_flag[first_list()] = 0;
           goto teardown;
         }
         LOSA_WAIT_RELAXED(&ctl->hdr_empty[nu & 1u], ((nu >> 1) & 1u) ^ 1u);
@@ -1035,11 +1035,8 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         LOSA_WAIT_RELAXED(&ctl->hdr_next, (nu - 1u) & 1u);
       }
       if (!p.stall) TILE_HDR_PUT(kTlEnd, 0u, 0, 0, 0, 0, 0, 0, nullptr, 0);
-      if (ONE && p.split_parts > 1 && lane == 0) {
-        const int again = *reinterpret_cast<volatile int*>(&ctl->redo_state[3]);
-        if (!in_cluster) p.redo_flag[first_list()] = again;
-        else if (again != 0) atomicAdd(p.redo_count, 1);
-      }
+      if (ONE && p.split_parts > 1 && lane == 0)
+        p.redo_flag[first_list()] = *reinterpret_cast<volatile int*>(&ctl->redo_state[3]);
     }
   } else {
     // ------------------------------------------------------------------ softmax warps (both CTAs)

@@ -8,7 +8,7 @@ import torch
 
 from oracle import losa_oracle as orc
 from tests import util
-from tests.test_gpu_units import check, lib
+from tests.test_gpu_units import check, lib, problem
 
 pytestmark = pytest.mark.gpu
 
@@ -63,3 +63,20 @@ def test_parts_that_list_nothing(D, R, C, H):
     want = orc.blocks_to_tokens(orc.sparse_attn(*(util.to_np(x) for x in (q, k, v)), R, C, off, idx), 1, H, N)
     util.assert_output_close(outs[0], want, "short lists")
     assert all(torch.equal(outs[0], o) for o in outs[1:])
+
+
+@pytest.mark.parametrize("D,R,C", [(64, 64, 64), (64, 128, 32), (128, 128, 128), (128, 64, 64)])
+@pytest.mark.parametrize("H", [1, 2])
+def test_a_unit_whose_two_query_tiles_are_run_again_counts_once(D, R, C, H):
+    """One row of each query tile of an item meets its far key in the second K/V tile of the item's last part, in every head;
+    merged in clusters (5 items) and by a launch behind (10)."""
+    losa = lib()
+    q, k, v = problem(H, N, D, 1760, range(H))
+    q[0, :, 128 + 7] = q[0, :, 7]
+    prob = losa.make_problem(q.cuda(), R, C)
+    for fill in (0, 255):  # whatever the workspace held before
+        ws = torch.full((losa.losa_workspace_bytes(losa.binding.LOSA_OP_ATTN, prob),), fill, dtype=torch.uint8, device="cuda")
+        o = losa.losa_attn(q.cuda(), k.cuda(), v.cuda(), R, C, out_dtype=torch.float32, ws=ws)
+        assert losa.losa_async_status() == 0
+        assert util.units_run_again(losa, ws, prob) == H
+        util.assert_output_close(o, orc.dense_attn(*(util.to_np(x) for x in (q, k, v))), "two tiles again")

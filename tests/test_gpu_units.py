@@ -36,11 +36,11 @@ def check(H, N, D, R, C, heads, seed, again=None):
     qn, kn, vn = (util.to_np(x) for x in (q, k, v))
     nQb, nKb = -(-N // R), -(-N // C)
     off, idx = util.random_csr(H * nQb, nKb, seed, 0.6)
-    ws = torch.empty(losa.losa_workspace_bytes(losa.binding.LOSA_OP_ATTN, losa.make_problem(qd, R, C)), dtype=torch.uint8,
-                     device="cuda")
+    prob = losa.make_problem(qd, R, C)
+    ws = torch.empty(losa.losa_workspace_bytes(losa.binding.LOSA_OP_ATTN, prob), dtype=torch.uint8, device="cuda")
     o = losa.losa_attn(qd, kd, vd, R, C, out_dtype=torch.float32, ws=ws)
     if again is not None:
-        assert int(ws[:8].view(torch.int32)[1]) == again
+        assert util.units_run_again(losa, ws, prob) == again
     o_s = losa.losa_sparse_attn(qd, kd, vd, torch.from_numpy(off).cuda(), torch.from_numpy(idx).cuda(), R, C,
                                 out_dtype=torch.float32)
     mass = losa.losa_block_mass(qd, kd, R, C)

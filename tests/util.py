@@ -66,3 +66,17 @@ def assert_output_close(o_gpu: torch.Tensor, o_ref: np.ndarray, what=""):
     assert diff.max() <= MAX_ABS_TOL, f"{what}: max-abs {diff.max():.3e}"
     assert diff.mean() <= MEAN_ABS_TOL, f"{what}: mean-abs {diff.mean():.3e}"
     return diff.max(), diff.mean()
+
+
+def units_run_again(losa, ws, problem):
+    """How many work units a dense call has run again, from its workspace of exactly the size that was asked for: word 1, or
+    where that is -1 (the parts of an item were merged in their cluster) the flags of the tile lists, which are its last part."""
+    n = int(ws[:8].view(torch.int32)[1])
+    if n >= 0:
+        return n
+    items = problem.B * problem.H * ((-(-problem.N // 128) + 1) // 2)
+    slots, lists = losa.losa_work_slots(losa.binding.LOSA_OP_ATTN, problem), 2 if problem.D == 64 else 1
+    parts = min(slots // items, 8, -(-problem.N // problem.C))
+    room = -(-4 * (items + 160) // 256) * 256
+    flags = ws[ws.numel() - room:].view(torch.int32)[:items * parts * lists].view(-1, lists)
+    return int(flags.any(1).sum())
