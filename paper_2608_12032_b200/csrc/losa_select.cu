@@ -7,7 +7,7 @@
 //                           over block indices plus its size.
 //   2. expand_rows_kernel   every CTA adds up the sizes of the rows before its own (offsets) and
 //                           turns its rows' bitmaps into ascending block indices.
-// Up to 256 rows of at most 1024 blocks take one launch of one cluster instead (select_small_kernel).
+// Few rows take one launch of one cluster instead (select_small_kernel).
 // Each mass element is read once and each kept index written once; the bitmap adds 1/16
 // of the mass bytes.  The result is deterministic (no floating-point atomics).
 #include <limits.h>
@@ -274,7 +274,8 @@ __device__ __forceinline__ uint32_t kept_word(const float* src, int nKb, int lan
 // What a row keeps.  W warps per row, K blocks per lane: warp w of the row owns blocks [w * 32 K, (w + 1) * 32 K), its
 // lane l the blocks l, l + 32, ... of those, so that a ballot is a bitmap word; lane k gets word k of its warp's K.
 // `src`: the lane's first block, `mine`: how many blocks of the warp exist (may be none).  COUNT: the fixed-ratio rule.
-template <int W, int K, bool COUNT, bool EARLY>
+// PICK: see below.
+template <int W, int K, bool COUNT, bool EARLY, bool PICK>
 __device__ __forceinline__ uint32_t kept_words(RowShared* rs, const float* src, int mine, int warp, int lane, int nKb,
                                                double tau, int fixed_count, int* status) {
   constexpr int T = 32 * W;
@@ -443,7 +444,15 @@ __device__ __forceinline__ uint32_t kept_words(RowShared* rs, const float* src, 
 #pragma unroll
         for (int k = 0; k < K; ++k) in |= ((bits[k] >> rest) == lead) ? 1u << k : 0u;
         if (COUNT) in &= (mine_k >= 32) ? 0xffffffffu : (1u << max(mine_k, 0)) - 1u;
-        // (a lane has one or two of them: their values are read again instead of picked out of registers)
+        // (A lane has one or two of them: their values are read again instead of picked out of registers.  Where few warps
+        // share an SM and the loads are not read-only ones, nothing hides these reads - 64 rows of 256 blocks, a third of
+        // them, 7.6 us a call instead of 4.3 - and they are picked; of long rows among many that costs 10 - 14 %.)
+        if (PICK) {
+#pragma unroll
+          for (int k = 0; k < K; ++k)
+            if ((in >> k) & 1u) rs->list[atomicAdd(&rs->list_len, 1)] = bits[k] & ((1u << rest) - 1u);
+          in = 0u;
+        }
         while (in != 0u) {
           const int k = __ffs(in) - 1;
           in &= in - 1u;
@@ -558,7 +567,7 @@ select_rows_kernel(const float* __restrict__ mass, int rows, int nKb, double tau
   const int words = (nKb + 31) >> 5;
   const int mine = min(32 * K, nKb - warp * 32 * K);
   const float* src = mass + row * nKb + warp * 32 * K + lane;
-  const uint32_t out = kept_words<W, K, COUNT, !COUNT>(rs, src, mine, warp, lane, nKb, tau, fixed_count, status);
+  const uint32_t out = kept_words<W, K, COUNT, !COUNT, false>(rs, src, mine, warp, lane, nKb, tau, fixed_count, status);
   if (lane < K && warp * K + lane < words) bitmaps[row * words + warp * K + lane] = out;
   int kept = __reduce_add_sync(0xffffffffu, __popc(out));
   if (W > 1) {
@@ -571,11 +580,24 @@ select_rows_kernel(const float* __restrict__ mass, int rows, int nKb, double tau
   if (warp * 32 + lane == 0) counts[row] = kept;
 }
 
-// Few rows: one launch, of one cluster.  A warp per row, two rows at most; the sizes of all rows meet in every CTA's
-// shared memory, and each warp writes the indices of its own rows.  The two launches of the general way are all latency
-// there (masses, selection and attention of 256 tokens, 27.8 -> 24.5 us; 4 x 32 rows of 32 blocks,
+// Few rows: one launch, of one cluster.  A warp per row, two rows at most, spread over the cluster's CTAs; the sizes of all
+// rows meet in every CTA's shared memory, and each warp writes the indices of its own rows.  The two launches of the general
+// way are all latency there (masses, selection and attention of 256 tokens, 27.8 -> 24.5 us; 4 x 32 rows of 32 blocks,
 // calls in a row, 9.1 -> 6.1).
 constexpr int kSmallWarps = 16, kSmallCtas = 8, kSmallRows = 2 * kSmallWarps * kSmallCtas;
+// Which calls: those that the eight SMs get through about as fast as the general way gets through its two launches; us a
+// call in a captured graph, that way / this one (from the host a call of either rule is 2 - 2.6 us shorter this way).
+//   256 rows of 32 blocks, all compared with all   5.6 / 5.6 (retained mass), 5.4 / 4.9 (fixed ratio)
+//   128 rows of 256 blocks, a row a warp           6.1 / 6.2, 6.4 / 5.0;  64 of 128 5.8 / 4.4, 5.9 / 3.9
+//   128 of 512                                     6.6 - 10.5 / 7.4 - 8.2 by the masses (on average 8.4 / 7.7), 7.4 / 6.5
+//   64 of 1024, half as many warps to an SM        8.0 - 11.7 / 7.0 - 8.0, 10.0 / 8.0;  128 7.8 - 12.5 / 9.8 - 10.9
+//   256 of 64, two rows a warp                     5.8 / 9.5, 5.8 / 6.8;  of 128 5.8 / 9.7, 6.0 / 7.5;  of 256 6.1 / 10.5, 6.4 / 8.5
+// Under the fixed-ratio rule two rows a warp are taken up to 128 blocks all the same: what they lose on the device is less
+// than what they save on the host.
+static bool small_selection(int rows, int nKb, bool fixed) {
+  if (nKb <= (fixed ? 128 : 32)) return rows <= kSmallRows;
+  return nKb <= 512 ? rows <= kSmallRows / 2 : nKb <= 1024 && rows <= kSmallRows / 4;
+}
 struct SmallShared {
   RowShared rows[kSmallWarps];
   int counts[kSmallRows];
@@ -586,7 +608,7 @@ select_small_kernel(const float* __restrict__ mass, int rows, int nKb, double ta
                     int32_t* __restrict__ offsets, int32_t* __restrict__ kv_idx, int64_t kv_capacity, int* status) {
   extern __shared__ __align__(16) unsigned char small_raw[];
   SmallShared* const sh = reinterpret_cast<SmallShared*>(small_raw);
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, ctas = gridDim.x;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, ctas = gridDim.x, warps = blockDim.x >> 5;
   ptx::grid_launch_dependents();
   ptx::cluster_sync();  // (the other CTAs' shared memory is there)
   ptx::grid_dependency_wait();
@@ -594,7 +616,7 @@ select_small_kernel(const float* __restrict__ mass, int rows, int nKb, double ta
   int kept[2] = {0, 0};
 #pragma unroll 1
   for (int i = 0; i < 2; ++i) {
-    const int row = (i * ctas + (int)blockIdx.x) * kSmallWarps + warp;
+    const int row = (i * ctas + (int)blockIdx.x) * warps + warp;
     if (row >= rows) break;
     const float* const src = mass + (int64_t)row * nKb + lane;
     uint32_t out;  // (lane k: word k)
@@ -602,7 +624,7 @@ select_small_kernel(const float* __restrict__ mass, int rows, int nKb, double ta
       out = kept_word<COUNT, true>(src, nKb, lane, tau, fixed_count, status);
       if (lane > 0) out = 0u;
     } else {
-      out = kept_words<1, K, COUNT, true>(&sh->rows[warp], src, nKb, 0, lane, nKb, tau, fixed_count, status);
+      out = kept_words<1, K, COUNT, true, true>(&sh->rows[warp], src, nKb, 0, lane, nKb, tau, fixed_count, status);
     }
     const int n = __reduce_add_sync(0xffffffffu, __popc(out));
     if (lane < ctas) ptx::st_cluster_u32(ptx::mapa(ptx::smem_u32(&sh->counts[row]), lane), (uint32_t)n);
@@ -615,7 +637,7 @@ select_small_kernel(const float* __restrict__ mass, int rows, int nKb, double ta
   const int words = (nKb + 31) >> 5;
 #pragma unroll 1
   for (int i = 0; i < 2; ++i) {
-    const int row = (i * ctas + (int)blockIdx.x) * kSmallWarps + warp;
+    const int row = (i * ctas + (int)blockIdx.x) * warps + warp;
     if (row >= rows) break;
     int at = 0;
     for (int r = lane; r < row; r += 32) at += sh->counts[r];
@@ -795,7 +817,7 @@ static int launch_small(int ctas, const float* mass, int rows, int nKb, double t
   attr[1].val.clusterDim.y = 1;
   attr[1].val.clusterDim.z = 1;
   cfg.gridDim = dim3(ctas, 1, 1);
-  cfg.blockDim = dim3(32 * kSmallWarps, 1, 1);
+  cfg.blockDim = dim3(32 * min(kSmallWarps, (rows + ctas - 1) / ctas), 1, 1);
   cfg.dynamicSmemBytes = sizeof(SmallShared);
   cfg.stream = st;
   cfg.attrs = attr;
@@ -810,8 +832,8 @@ int launch_select(int rows, int nKb, const float* mass, double tau, int fixed_co
   int32_t* counts = static_cast<int32_t*>(ws);
   uint32_t* bitmaps = reinterpret_cast<uint32_t*>(static_cast<char*>(ws) +
                                                   align_up((size_t)rows * sizeof(int32_t), 256));
-  if (rows <= kSmallRows && nKb <= 1024) {
-    const int ctas = min(kSmallCtas, (rows + kSmallWarps - 1) / kSmallWarps);
+  if (small_selection(rows, nKb, fixed_count > 0)) {
+    const int ctas = min(kSmallCtas, rows);
 #define LOSA_SELECT_SMALL(k)                                                                                  \
   (fixed_count > 0 ? launch_small<k, true>(ctas, mass, rows, nKb, tau, fixed_count, offsets, kv_idx, kv_capacity, status, st) \
                    : launch_small<k, false>(ctas, mass, rows, nKb, tau, 0, offsets, kv_idx, kv_capacity, status, st))

@@ -1,5 +1,5 @@
-"""Selection of few rows by one cluster, and of one row more by the general way: both against the oracle's rule, over row
-counts around a warp's, a CTA's and the cluster's, with a capacity that is too small and with masses that are none."""
+"""Selection of few rows by one cluster, and of more or longer ones by the general way: both against the oracle's rule, over
+row counts and lengths on both sides of the lines between them, with a capacity that is too small and with masses that are none."""
 import numpy as np
 import pytest
 import torch
@@ -20,8 +20,8 @@ def masses(rows, nKb, seed):
     return (m / m.sum(1, keepdim=True)).reshape(1, 1, rows, nKb)
 
 
-@pytest.mark.parametrize("rows", [1, 15, 16, 17, 128, 129, 255, 256, 257])
-@pytest.mark.parametrize("nKb", [1, 4, 32, 33, 256, 257, 1024])
+@pytest.mark.parametrize("rows", [1, 7, 8, 9, 15, 16, 17, 64, 65, 128, 129, 255, 256, 257])
+@pytest.mark.parametrize("nKb", [1, 4, 32, 33, 128, 129, 256, 257, 512, 513, 1024, 1025])
 def test_row_counts_around_the_cluster(rows, nKb):
     losa = lib()
     m = masses(rows, nKb, rows + nKb)
@@ -53,6 +53,25 @@ def test_a_capacity_that_is_too_small_and_masses_that_are_none():
     a, b = offsets.tolist(), offsets2.tolist()
     for r in set(range(40)) - {3, 39}:  # the other rows are untouched
         assert torch.equal(idx[a[r]:a[r + 1]], idx2[b[r]:b[r + 1]])
+
+
+@pytest.mark.parametrize("rows,nKb", [(8, 256), (64, 1024), (128, 512), (256, 128), (65, 1024), (129, 130)])
+def test_thresholds_among_many_close_masses(rows, nKb):
+    """Masses within a few per cent of each other, of which half are kept: the threshold's bin holds most of the row, so
+    that its list is long and split again.  The last two by the general way."""
+    losa = lib()
+    g = torch.Generator("cpu").manual_seed(rows + nKb)
+    m = torch.exp(0.01 * torch.randn(rows, nKb, generator=g))
+    m = (m / m.sum(1, keepdim=True)).reshape(1, 1, rows, nKb)
+    offsets, idx = losa.losa_select(m.cuda(), 0.5)
+    ref = orc.select(m.reshape(rows, nKb).numpy().astype(np.float64), 0.5)
+    assert np.array_equal(offsets.cpu().numpy(), ref.offsets)
+    assert np.array_equal(idx.cpu().numpy()[:ref.offsets[-1]], ref.kv_idx)
+    k = nKb // 2
+    offsets, idx = losa.losa_select_topk(m.cuda(), k)
+    order = torch.sort(m.reshape(rows, nKb), dim=1, descending=True, stable=True)[1][:, :k]
+    assert torch.equal(idx.cpu().reshape(rows, k).long(), order.sort(1)[0])
+    assert losa.losa_async_status() == 0
 
 
 @pytest.mark.parametrize("nKb", [2, 8, 31, 32, 33])
