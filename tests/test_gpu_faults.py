@@ -22,9 +22,15 @@ def lib():
 
 
 @pytest.mark.parametrize("mode", ["dense", "sparse", "mass", "fused"])
-def test_a_wait_that_runs_out_is_reported_and_the_next_call_is_fine(mode):
+@pytest.mark.parametrize("D,BLK,H,N", [
+    (128, 128, 2, 700),   # one wave, its 6 items in 8 parts that share clusters
+    (128, 128, 2, 1100),  # 10 items in 7 parts, merged by a launch behind
+    (64, 64, 2, 700), (64, 64, 2, 1100),  # the same without pairs of CTAs
+    (64, 64, 80, 200), (128, 128, 80, 200),  # more work units than slots
+])
+def test_a_wait_that_runs_out_is_reported_and_the_next_call_is_fine(mode, D, BLK, H, N):
     losa = lib()
-    B, H, N, D, BLK = 1, 2, 700, 128, 128
+    B = 1
     q = util.rand_bf16((B, H, N, D), 1, 1.5)
     k = util.rand_bf16((B, H, N, D), 2, 1.5)
     v = util.rand_bf16((B, H, N, D), 3)
