@@ -50,24 +50,12 @@ NCU_TRAFFIC_SOURCE = "ncu capture of the sparse forward at the Wan2.1 shape (dra
 FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustained": 1400.0}
 
 
-def launches_per_call(wl, slots: int, attention_only: bool) -> int:
-    """Kernels launched by one attention-shaped call: its kernel; and if there are more units than work slots, before it
-    the work units' tile lists (sparse) or the launch's counters, behind it the merge of the last wave's units, where they
-    are cut into parts.  (In a single wave the clusters merge them.)"""
-    items = wl.B * wl.H * ((-(-wl.N // 128) + 1) // 2)
-    rest = items if items < slots else items % slots
-    parts = min(slots // rest if rest else 1, 8, wl.nKb)
-    cut = attention_only and parts >= 2
-    units = items + rest * (parts - 1) if cut else items
-    return 1 + (units > slots) * (1 + cut)
-
-
-def launches_per_step(wl, slots: int, draws: int) -> int:
-    """Kernels of the library launched by one step: mass pass, selection (two, or one for a few rows), the sparse draws,
-    the dense and the fused call."""
-    select = 1 if wl.rows <= 256 and wl.nKb <= 1024 else 2
-    return (launches_per_call(wl, slots, False) + select + (draws + 1) * launches_per_call(wl, slots, True)
-            + launches_per_call(wl, slots, False))
+def launches_per_step(losa, prob, draws: int) -> int:
+    """Kernels of the library launched by one step: mass pass, selection, the sparse draws, the dense and the fused call."""
+    b = losa.binding
+    return (losa.losa_kernel_launches(b.LOSA_OP_BLOCK_MASS, prob) + losa.losa_kernel_launches(b.LOSA_OP_SELECT, prob)
+            + draws * losa.losa_kernel_launches(b.LOSA_OP_SPARSE_ATTN, prob)
+            + losa.losa_kernel_launches(b.LOSA_OP_ATTN, prob) + losa.losa_kernel_launches(b.LOSA_OP_ATTN_MASS, prob))
 
 
 def cpu_model() -> str:
@@ -646,8 +634,7 @@ def main():
             "algorithmic_bytes_per_launch": 4 * q0.numel() * 2,
         },
         "clocks": clocks.summary(),
-        "gpu_launches": args.steps * launches_per_step(
-            wl, losa.losa_work_slots(losa.binding.LOSA_OP_SPARSE_ATTN, prob), args.draws),
+        "gpu_launches": args.steps * launches_per_step(losa, prob, args.draws),
     }
     if batched is not None:
         line["batched"] = batched

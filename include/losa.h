@@ -246,6 +246,13 @@ size_t losa_workspace_bytes_batched(int op, const losa_problem_t* p, int32_t n_l
  * LOSA_ERR_UNSUPPORTED there. */
 int32_t losa_work_slots(int op, const losa_problem_t* p);
 
+/* How many kernels a call of kind `op` (a LOSA_OP_* constant; LOSA_OP_SELECT: under the retained-mass rule)
+ * launches on the current device: for callers that account for launches.  An attention call takes one
+ * kernel, one ahead of it if it has more work units than slots, and one behind it that merges the parts of
+ * the last wave's items - unless all of the call is one wave and the device holds the clusters in which
+ * these parts merge themselves.  0 where losa_work_slots is 0. */
+int32_t losa_kernel_launches(int op, const losa_problem_t* p);
+
 /* Dense softmax attention o = softmax(q k^T * scale) v over the N valid keys: the paper's
  * dense steps up to the construction step, and this library's own dense baseline.
  * Same tensors and workspace rule as losa_sparse_attn, without the CSR. */

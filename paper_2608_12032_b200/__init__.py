@@ -10,6 +10,7 @@ from .binding import (  # noqa: F401
     losa_attn,
     losa_attn_mass,
     losa_block_mass,
+    losa_kernel_launches,
     losa_debug_stall_next_launch,
     losa_select,
     losa_select_noalloc,

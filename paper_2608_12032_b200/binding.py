@@ -27,6 +27,7 @@ EXPORTS = (
     "losa_select_noalloc", "losa_validate_csr", "losa_async_status", "losa_status_string", "losa_last_cuda_error",
     "losa_debug_stall_next_launch", "losa_sparse_attn_batched", "losa_workspace_bytes_batched",
     "losa_work_slots",
+    "losa_kernel_launches",
 )
 
 
@@ -89,6 +90,8 @@ def _lib():
         lib.losa_workspace_bytes_batched.argtypes = [ctypes.c_int, pp, i32]
         lib.losa_work_slots.restype = i32
         lib.losa_work_slots.argtypes = [ctypes.c_int, pp]
+        lib.losa_kernel_launches.restype = i32
+        lib.losa_kernel_launches.argtypes = [ctypes.c_int, pp]
         lib.losa_attn.restype = ctypes.c_int
         lib.losa_attn.argtypes = [pp, vp, vp, vp, vp, ctypes.c_int, vp, sz, vp]
         lib.losa_attn_mass.restype = ctypes.c_int
@@ -161,6 +164,11 @@ def losa_workspace_bytes(op: int, problem: Problem) -> int:
 def losa_work_slots(op: int, problem: Problem) -> int:
     """Work slots (persistent CTAs, or pairs of them) an attention call of this kind occupies."""
     return int(_lib().losa_work_slots(op, ctypes.byref(problem)))
+
+
+def losa_kernel_launches(op: int, problem: Problem) -> int:
+    """Kernels that a call of this kind launches (LOSA_OP_SELECT: under the retained-mass rule)."""
+    return int(_lib().losa_kernel_launches(op, ctypes.byref(problem)))
 
 
 def _workspace(need: int, device, ws: Optional[torch.Tensor]) -> Tuple[Optional[torch.Tensor], int]:

@@ -152,6 +152,27 @@ int32_t losa_work_slots(int op, const losa_problem_t* p) {
   return 0;
 }
 
+int32_t losa_kernel_launches(int op, const losa_problem_t* p) {
+  if (!p) return 0;
+  if (op == LOSA_OP_SELECT) {
+    if (losa_workspace_bytes(op, p) == 0) return 0;
+    const int64_t nQb = (p->N + p->R - 1) / p->R, nKb = (p->N + p->C - 1) / p->C;
+    return select_launches((int64_t)p->B * p->H * nQb, (int)nKb, false);
+  }
+  Geometry g;
+  if (make_geometry(p, &g) != LOSA_OK) return 0;
+  int rc = LOSA_OK;
+  const DeviceState* dev = device_state(&rc);
+  if (!dev) return 0;
+  switch (op) {
+    case LOSA_OP_BLOCK_MASS: return attn_launches(kMass, g, *dev);
+    case LOSA_OP_SPARSE_ATTN: return attn_launches(kSparse, g, *dev);
+    case LOSA_OP_ATTN: return attn_launches(kDense, g, *dev);
+    case LOSA_OP_ATTN_MASS: return attn_launches(kFused, g, *dev);
+  }
+  return 0;
+}
+
 int losa_block_mass(const losa_problem_t* p, const void* q, const void* k, float* mass, float* lse,
                     void* ws, size_t ws_bytes, void* cuda_stream) {
   Geometry g;

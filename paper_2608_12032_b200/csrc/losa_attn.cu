@@ -18,6 +18,7 @@
 #include <limits.h>
 #include <math.h>
 
+#include <algorithm>
 #include <atomic>
 #include <cstddef>
 #include <type_traits>
@@ -662,50 +663,71 @@ int work_slots(const DeviceState& dev, int* slots) {
   return rc;
 }
 
+// How a call's work items are spread over the slots.
+struct Waves {
+  int slots, units, split_first, parts;
+  int ctas;  // of a cluster
+  bool one_wave, in_cluster;
+  // kernels: the tile kernel, ahead of it what prepares several waves, behind it the merge of parts that share no cluster
+  int launches() const { return 1 + (one_wave ? 0 : 1) + (parts > 1 && !in_cluster ? 1 : 0); }
+};
+
 template <int D, int R, int C_, int MODE>
-int launch_t(const Geometry& g, const void* q, const void* k, const void* v, Params prm,
-             const DeviceState& dev, cudaStream_t st) {
+int plan_waves(int items, int nKb, const DeviceState& dev, Waves* waves) {
   constexpr bool kPair = D == 128;
-  ProblemEntry maps;
+  constexpr int kTileCtas = kPair ? 2 : 1;
   int rc, slots;
-  if ((rc = make_maps(&maps, g, q, k, MODE != kMass ? v : nullptr)) != LOSA_OK) return rc;
   if ((rc = work_slots<D, R, C_, MODE>(dev, &slots)) != LOSA_OK) return rc;
+  Waves w = {slots, items, items, 1, kTileCtas, false, false};
   // The items of the last, partly filled wave of the persistent grid (all items, if there are
   // fewer than slots) are cut into parts of the key range, so that the wave ends after 1/parts of
   // an item; their partial results are merged by their clusters or by a launch behind.  Attention output
   // only: the mass epilogue needs a row's final statistics inside the kernel.
-  prm.nUnits = prm.nWork;
-  prm.split_first = prm.nWork;
-  prm.split_parts = 1;
   constexpr bool kAttnOnly = (MODE == kDense || MODE == kSparse);
-  constexpr int kTileCtas = kPair ? 2 : 1;
-  int ctas = kTileCtas;  // of a cluster
-  cudaLaunchConfig_t cfg;
-  cudaLaunchAttribute attr[2];
-  prm.in_cluster = 0;
   if (kAttnOnly) {
-    const int rest = (prm.nWork < slots) ? prm.nWork : prm.nWork % slots;
+    const int rest = (items < slots) ? items : items % slots;
     int parts = rest > 0 ? slots / rest : 1;
-    parts = min(min(parts, kMaxParts), prm.nKb);
-    if (parts >= 2 && rest == prm.nWork) {
+    parts = min(min(parts, kMaxParts), nKb);
+    if (parts >= 2 && rest == items) {
       // A single wave: the parts of an item in one cluster (at head dimension 64 of each of its query tiles), where the
       // device holds all of them at once - of 16 CTAs 7, of 8 15, of 6 22, of 4 33, of 3 45.  Elsewhere a launch behind
       // merges them: with fewer parts, which would fit, calls were up to 30 % faster, but a part's largest weights round to
       // themselves, and the error against 64 bits grew (264 tokens, 4 heads, D = 64, 8 parts / 7: 1.7e-3 / 1.8e-3).
       int n = 0;
+      cudaLaunchConfig_t cfg;
+      cudaLaunchAttribute attr[2];
       if ((rc = configure_tile<D, R, C_, MODE, kPair, true>(dev, kTileCtas * parts, &n, &cfg, attr)) == LOSA_ERR_CUDA) return rc;
       if (rc == LOSA_OK && n >= rest * (kPair ? 1 : 2)) {
-        prm.in_cluster = 1;
-        ctas = kTileCtas * parts;
+        w.in_cluster = true;
+        w.ctas = kTileCtas * parts;
       }
     }
     if (parts >= 2) {
-      prm.split_first = prm.nWork - rest;
-      prm.split_parts = parts;
-      prm.nUnits = prm.split_first + rest * parts;
+      w.split_first = items - rest;
+      w.parts = parts;
+      w.units = w.split_first + rest * parts;
     }
   }
-  prm.one_wave = (prm.nUnits <= slots) ? 1 : 0;
+  w.one_wave = w.units <= slots;
+  *waves = w;
+  return LOSA_OK;
+}
+
+template <int D, int R, int C_, int MODE>
+int launch_t(const Geometry& g, const void* q, const void* k, const void* v, Params prm,
+             const DeviceState& dev, cudaStream_t st) {
+  constexpr bool kPair = D == 128;
+  ProblemEntry maps;
+  Waves w;
+  int rc;
+  if ((rc = make_maps(&maps, g, q, k, MODE != kMass ? v : nullptr)) != LOSA_OK) return rc;
+  if ((rc = plan_waves<D, R, C_, MODE>(prm.nWork, prm.nKb, dev, &w)) != LOSA_OK) return rc;
+  const int slots = w.slots;
+  prm.nUnits = w.units;
+  prm.split_first = w.split_first;
+  prm.split_parts = w.parts;
+  prm.in_cluster = w.in_cluster ? 1 : 0;
+  prm.one_wave = w.one_wave ? 1 : 0;
   prm.by_parts = Divisor(prm.split_parts);
   prm.by_pairs = Divisor(prm.nPairs);
   prm.by_heads = Divisor(prm.H);
@@ -726,7 +748,9 @@ int launch_t(const Geometry& g, const void* q, const void* k, const void* v, Par
   if (rc != LOSA_OK) return rc;
   auto launch_tile = [&](auto one) -> int {
     int n = 0;
-    const int rc = configure_tile<D, R, C_, MODE, kPair, decltype(one)::value>(dev, ctas, &n, &cfg, attr);
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr[2];
+    const int rc = configure_tile<D, R, C_, MODE, kPair, decltype(one)::value>(dev, w.ctas, &n, &cfg, attr);
     if (rc != LOSA_OK) return rc;
     cfg.gridDim = dim3(2 * min(slots, prm.nUnits), 1, 1);
     cfg.stream = st;
@@ -756,13 +780,24 @@ int dispatch(const Geometry& g, const void* q, const void* k, const void* v, con
 }
 
 template <int MODE>
-int slots_of(const Geometry& g, const DeviceState& dev) {
-  int slots = 0;
+int plan_of(const Geometry& g, int items, const DeviceState& dev, Waves* w) {
 #define LOSA_CASE(d, r, c) \
-  if (g.D == d && g.R == r && g.C == c) return work_slots<d, r, c, MODE>(dev, &slots) == LOSA_OK ? slots : 0;
+  if (g.D == d && g.R == r && g.C == c) return plan_waves<d, r, c, MODE>(items, g.nKb, dev, w);
   LOSA_GEOMETRIES(LOSA_CASE)
 #undef LOSA_CASE
-  return 0;
+  return LOSA_ERR_UNSUPPORTED;
+}
+
+int plan_of(AttnMode mode, const Geometry& g, const DeviceState& dev, Waves* w) {
+  // (calls of more items than the mask holds are refused)
+  const int items = (int)std::min<int64_t>((int64_t)g.B * g.H * g.nPairs, kTlItemMask);
+  switch (mode) {
+    case kDense: return plan_of<kDense>(g, items, dev, w);
+    case kSparse: return plan_of<kSparse>(g, items, dev, w);
+    case kMass: return plan_of<kMass>(g, items, dev, w);
+    case kFused: return plan_of<kFused>(g, items, dev, w);
+  }
+  return LOSA_ERR_UNSUPPORTED;
 }
 
 }  // namespace
@@ -794,13 +829,15 @@ void arm_stalled_launch(uint32_t polls) { g_stall_polls.store(polls); }
 // Work slots that a call of this kind occupies on the current device, for callers that
 // want to know how the work items are spread (which of them the last wave cuts into parts); 0 where it cannot run.
 int attn_work_slots(AttnMode mode, const Geometry& g, const DeviceState& dev) {
-  switch (mode) {
-    case kDense: return slots_of<kDense>(g, dev);
-    case kSparse: return slots_of<kSparse>(g, dev);
-    case kMass: return slots_of<kMass>(g, dev);
-    case kFused: return slots_of<kFused>(g, dev);
-  }
-  return 0;
+  Waves w;
+  return plan_of(mode, g, dev, &w) == LOSA_OK ? w.slots : 0;
+}
+
+// Kernels that such a call launches; 0 where it cannot run.
+int attn_launches(AttnMode mode, const Geometry& g, const DeviceState& dev) {
+  Waves w;
+  if ((int64_t)g.B * g.H * g.nPairs > (int64_t)kTlItemMask) return 0;
+  return plan_of(mode, g, dev, &w) == LOSA_OK ? w.launches() : 0;
 }
 
 size_t attn_workspace_bytes(AttnMode mode, const Geometry& g, int n_prob) {

@@ -97,6 +97,7 @@ inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 
 // ---- entry points of the kernel translation units (host launchers) -------------------
 
 size_t select_workspace_bytes(int64_t rows, int nKb);
+int select_launches(int64_t rows, int nKb, bool fixed);  // kernels that such a call launches
 int launch_select(int rows, int nKb, const float* mass, double tau, int fixed_count,
                   int32_t* offsets, int32_t* kv_idx, int64_t kv_capacity, void* ws, int* status,
                   cudaStream_t st);  // fixed_count > 0: keep that many blocks per row instead;
@@ -115,6 +116,7 @@ enum AttnMode { kDense = 0, kSparse = 1, kMass = 2, kFused = 3 };  // kFused: de
 size_t attn_workspace_bytes(AttnMode mode, const Geometry& g, int n_prob = 1);
 void arm_stalled_launch(uint32_t polls);  // the next attention launch publishes no work (diagnostic)
 int attn_work_slots(AttnMode mode, const Geometry& g, const DeviceState& dev);
+int attn_launches(AttnMode mode, const Geometry& g, const DeviceState& dev);
 int launch_attn(AttnMode mode, const Geometry& g, const void* q, const void* k, const void* v,
                 const int32_t* offsets, const int32_t* kv_idx, void* o, int o_dtype, float* mass,
                 float* lse, void* ws, cudaStream_t st, int n_prob = 1,

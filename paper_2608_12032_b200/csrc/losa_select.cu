@@ -594,7 +594,7 @@ constexpr int kSmallWarps = 16, kSmallCtas = 8, kSmallRows = 2 * kSmallWarps * k
 //   256 of 64, two rows a warp                     5.8 / 9.5, 5.8 / 6.8;  of 128 5.8 / 9.7, 6.0 / 7.5;  of 256 6.1 / 10.5, 6.4 / 8.5
 // Under the fixed-ratio rule two rows a warp are taken up to 128 blocks all the same: what they lose on the device is less
 // than what they save on the host.
-static bool small_selection(int rows, int nKb, bool fixed) {
+bool small_selection(int64_t rows, int nKb, bool fixed) {
   if (nKb <= (fixed ? 128 : 32)) return rows <= kSmallRows;
   return nKb <= 512 ? rows <= kSmallRows / 2 : nKb <= 1024 && rows <= kSmallRows / 4;
 }
@@ -796,6 +796,8 @@ size_t select_workspace_bytes(int64_t rows, int nKb) {
   const size_t words = (size_t)(nKb + 31) / 32;
   return align_up((size_t)rows * sizeof(int32_t), 256) + (size_t)rows * words * sizeof(uint32_t);
 }
+
+int select_launches(int64_t rows, int nKb, bool fixed) { return small_selection(rows, nKb, fixed) ? 1 : 2; }
 
 template <int K, bool COUNT>
 static int launch_small(int ctas, const float* mass, int rows, int nKb, double tau, int fixed_count, int32_t* offsets,

@@ -1,7 +1,7 @@
-"""Items that a single wave is cut into: their parts run in one cluster and are merged through its CTAs' shared memory
-(or, where the device does not hold all these clusters at once, by a launch behind: 10 items), from two parts to as many as
-there can be, of an odd number of query tiles with a short last one; some parts outgrow their reference and are run again,
-the others of their cluster wait for them.  Against the fp64 oracle."""
+"""Items that a single wave is cut into: their parts run in one cluster and are merged through its CTAs' shared memory, or,
+where the device does not hold all these clusters at once, by a launch behind (the library says how many kernels a call
+takes): from two parts to as many as there can be, of an odd number of query tiles with a short last one, and parts that
+outgrow their reference and are run again while the others of their cluster wait for them.  Against the fp64 oracle."""
 import numpy as np
 import pytest
 import torch
@@ -15,33 +15,50 @@ pytestmark = pytest.mark.gpu
 N = 1100  # 9 query tiles, of 5 items to a head; 9 K/V tiles
 
 
+def merged_in_cluster(losa, prob, op):
+    """Of a call that is one wave and cut: whether it takes one kernel or a second one that merges."""
+    launches = losa.losa_kernel_launches(op, prob)
+    assert launches in (1, 2)
+    return launches == 1
+
+
+# 5, 10, 15, 20 and 35 items in 8, 7, 4, 3 and 2 parts.  Of the first a B200 holds more clusters than there are, of the second
+# (14 CTAs, or 7) fewer whichever of its SMs are there; the others fit on some.
 @pytest.mark.parametrize("D,R,C", [(64, 64, 64), (64, 128, 32), (128, 128, 128), (128, 64, 64)])
-@pytest.mark.parametrize("H", [1, 2, 3, 4, 7])
-def test_parts_of_an_item_are_merged_in_their_cluster(D, R, C, H):
+@pytest.mark.parametrize("H,clusters", [(1, True), (2, False), (3, None), (4, None), (7, None)])
+def test_parts_of_an_item_are_merged_in_their_cluster(D, R, C, H, clusters):
+    """Heads whose first query block has a row that meets a far key in the last part only, which is run again."""
     losa = lib()
     prob = losa.make_problem(torch.empty((1, H, N, D), dtype=torch.bfloat16, device="cuda"), R, C)
     assert 2 <= losa.losa_work_slots(losa.binding.LOSA_OP_ATTN, prob) // (5 * H)
-    check(H, N, D, R, C, (0, H - 1), 1700 + H)
+    for op in (losa.binding.LOSA_OP_ATTN, losa.binding.LOSA_OP_SPARSE_ATTN):
+        assert clusters is None or merged_in_cluster(losa, prob, op) == clusters
+    check(H, N, D, R, C, (0, H - 1), 1700 + H, again=len({0, H - 1}))
 
 
 @pytest.mark.parametrize("D,R,C", [(64, 64, 64), (128, 128, 64)])
-def test_cut_items_of_a_batched_call_and_of_token_major_tensors(D, R, C):
-    """Two layers of two heads in one wave equal the single calls where both are cut alike; rows a head apart, a batch of
-    two, bf16 and fp32 output (the same, rounded once)."""
+@pytest.mark.parametrize("layers,B,H", [(2, 2, 1), (2, 1, 2), (3, 1, 1)])
+def test_cut_items_of_a_batched_call_and_of_token_major_tensors(D, R, C, layers, B, H):
+    """20 or 15 items of all the layers together in one wave, rows a head apart: against the oracle, in bf16 the fp32 output
+    rounded once, and bit for bit what one call on all the layers as one batch gives, which is cut alike."""
     losa = lib()
     nQb, nKb = -(-N // R), -(-N // C)
-    layers = []
-    for i in range(2):
-        q, k, v = (util.rand_bf16((2, N, 1, D), 1720 + 3 * i + j).cuda().transpose(1, 2) for j in range(3))
-        off, idx = util.random_csr(2 * nQb, nKb, 1730 + i, 0.6)
-        layers.append((q, k, v, torch.from_numpy(off).cuda(), torch.from_numpy(idx).cuda()))
-    outs = losa.losa_sparse_attn_batched(layers, R, C, out_dtype=torch.float32)
-    for (q, k, v, off, idx), o in zip(layers, outs):
-        single = losa.losa_sparse_attn(q, k, v, off, idx, R, C, out_dtype=torch.float32)
-        assert torch.equal(single.bfloat16(), losa.losa_sparse_attn(q, k, v, off, idx, R, C))
-        # 10 items in 7 parts, 20 in 3: P rounds against another reference, 2^-9 each at random
-        assert (o - single).norm() <= 4e-3 * single.norm()
+    args, want = [], []
+    for i in range(layers):
+        q, k, v = (util.rand_bf16((B, N, H, D), 1720 + 3 * i + j).transpose(1, 2) for j in range(3))
+        off, idx = util.random_csr(B * H * nQb, nKb, 1730 + i, 0.6)
+        want.append(orc.blocks_to_tokens(orc.sparse_attn(*(util.to_np(x) for x in (q, k, v)), R, C, off, idx), B, H, N))
+        args.append((*(x.cuda() for x in (q, k, v)), torch.from_numpy(off).cuda(), torch.from_numpy(idx).cuda()))
+    outs = losa.losa_sparse_attn_batched(args, R, C, out_dtype=torch.float32)
+    low = losa.losa_sparse_attn_batched(args, R, C)
     assert losa.losa_async_status() == 0
+    for o, ref in zip(outs, want):
+        util.assert_output_close(o, ref, "batched")
+    assert all(torch.equal(o.bfloat16(), x) for o, x in zip(outs, low))
+    q, k, v = (torch.cat([a[j] for a in args]) for j in range(3))
+    off = torch.cat([torch.zeros(1, dtype=torch.int32, device="cuda")] + [a[3].diff() for a in args]).cumsum(0).int()
+    one = losa.losa_sparse_attn(q, k, v, off, torch.cat([a[4] for a in args]), R, C, out_dtype=torch.float32)
+    assert torch.equal(torch.cat(outs), one)
 
 
 @pytest.mark.parametrize("D,R,C", [(64, 64, 64), (64, 128, 32), (128, 128, 128), (128, 64, 64)])
@@ -53,6 +70,7 @@ def test_parts_that_list_nothing(D, R, C, H):
     losa = lib()
     nQb, nKb = -(-N // R), -(-N // C)
     q, k, v = (util.rand_bf16((1, H, N, D), 1740 + i) for i in range(3))
+    assert merged_in_cluster(losa, losa.make_problem(q.cuda(), R, C), losa.binding.LOSA_OP_SPARSE_ATTN) == (H == 1)
     rng = np.random.default_rng(1750 + H)
     rows = [np.sort(rng.choice(nKb, rng.integers(1, 4), replace=False)) for _ in range(H * nQb)]
     off = np.concatenate([[0], np.cumsum([len(r) for r in rows])]).astype(np.int32)
@@ -74,6 +92,7 @@ def test_a_unit_whose_two_query_tiles_are_run_again_counts_once(D, R, C, H):
     q, k, v = problem(H, N, D, 1760, range(H))
     q[0, :, 128 + 7] = q[0, :, 7]
     prob = losa.make_problem(q.cuda(), R, C)
+    assert merged_in_cluster(losa, prob, losa.binding.LOSA_OP_ATTN) == (H == 1)
     for fill in (0, 255):  # whatever the workspace held before
         ws = torch.full((losa.losa_workspace_bytes(losa.binding.LOSA_OP_ATTN, prob),), fill, dtype=torch.uint8, device="cuda")
         o = losa.losa_attn(q.cuda(), k.cuda(), v.cuda(), R, C, out_dtype=torch.float32, ws=ws)
