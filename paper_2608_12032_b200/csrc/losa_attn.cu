@@ -276,7 +276,7 @@ __device__ __forceinline__ void merge_parts(const Params& p, int cta, int ctas) 
 // One warp per list fills its bitmap (a list of a small layer is nothing but the latency of its two
 // dependent loads), then the first warp writes the tile list.  The first CTA also zeroes the
 // launch's counters, and every CTA its unit's flag.
-// ONE: a list is that of one query tile of the unit (its NB query blocks), in ascending order.
+// PER_TILE: a list is that of one query tile of the unit (its NB query blocks), in ascending order.
 
 // A list's unit as (item, part of it).
 __device__ __forceinline__ void unit_item(const Params& p, int unit, int& w, int& part, int& parts) {
@@ -289,13 +289,12 @@ __device__ __forceinline__ void unit_item(const Params& p, int unit, int& w, int
   }
 }
 
-
 // Bitmap of the n-th query block of a list (whole warp).
-template <int NB, bool ONE>
+template <int NB, bool PER_TILE>
 __device__ __forceinline__ void fill_tile_bitmap(const Params& p, int list, int n, int lane, uint32_t* bm) {
-  const int bit0 = ONE ? (list & 1) * NB : 0;  // membership bit of the first query block
+  const int bit0 = PER_TILE ? (list & 1) * NB : 0;  // membership bit of the first query block
   int w, part, parts;
-  unit_item(p, ONE ? list >> 1 : list, w, part, parts);
+  unit_item(p, PER_TILE ? list >> 1 : list, w, part, parts);
   int problem, bh, pr;
   item_place(p, w, problem, bh, pr);
   const int32_t* offsets = p.offsets;
@@ -307,7 +306,7 @@ __device__ __forceinline__ void fill_tile_bitmap(const Params& p, int list, int 
   }
   const int W = (p.nKb + 31) >> 5;
   uint32_t* const mine = bm + n * W;
-  const int g = pr * (ONE ? 2 * NB : NB) + bit0 + n;
+  const int g = pr * (PER_TILE ? 2 * NB : NB) + bit0 + n;
   int b = 0, e = 0;
   if (g < p.nQb) {
     const int64_t row = (int64_t)bh * p.nQb + g;
@@ -336,11 +335,11 @@ __device__ __forceinline__ void fill_tile_bitmap(const Params& p, int list, int 
 
 // The tile list from its query blocks' bitmaps (whole warp).
 // Returns what goes into tl_count; `copy`, if not null, receives the entries as well.
-template <int NB, int G, bool ONE>
+template <int NB, int G, bool PER_TILE>
 __device__ __forceinline__ uint32_t emit_tile_list(const Params& p, int list, int lane, const uint32_t* bm,
                                                    uint32_t* copy) {
   const int W = (p.nKb + 31) >> 5;
-  const int bit0 = ONE ? (list & 1) * NB : 0;
+  const int bit0 = PER_TILE ? (list & 1) * NB : 0;
   // Order of the entries.  A key block that only ONE of the unit's two query tiles lists is
   // processed by that tile alone, at half the CTA's rate; two such blocks, one of each tile, can
   // be in flight at the same time (the tiles' chains are independent).  So the list holds first
@@ -360,7 +359,7 @@ __device__ __forceinline__ uint32_t emit_tile_list(const Params& p, int list, in
 #pragma unroll
     for (int n = 0; n < NB; ++n) {
       const uint32_t m = (wi < W) ? bm[n * W + wi] : 0u;
-      if (ONE) ta |= m, tb |= m;
+      if (PER_TILE) ta |= m, tb |= m;
       else if (n < NB / 2) ta |= m;
       else tb |= m;
     }
@@ -369,8 +368,8 @@ __device__ __forceinline__ uint32_t emit_tile_list(const Params& p, int list, in
     nbb += __popc(tb & ~ta);
   }
   nb = __reduce_add_sync(0xffffffffu, nb);
-  na = ONE ? 0 : __reduce_add_sync(0xffffffffu, na);  // (a query tile's own list has one class)
-  nbb = ONE ? 0 : __reduce_add_sync(0xffffffffu, nbb);
+  na = PER_TILE ? 0 : __reduce_add_sync(0xffffffffu, na);  // (a query tile's own list has one class)
+  nbb = PER_TILE ? 0 : __reduce_add_sync(0xffffffffu, nbb);
   const int s1 = (nb + G - 1) / G * G;                       // entries of the first section
   const int tA = (na + G - 1) / G, tB = (nbb + G - 1) / G;   // K/V tiles of the single-tile classes
   const int tmin = min(tA, tB);
@@ -396,7 +395,7 @@ __device__ __forceinline__ uint32_t emit_tile_list(const Params& p, int list, in
 #pragma unroll
       for (int n = 0; n < NB; ++n) {
         const uint32_t m = bm[n * W + wi];
-        if (ONE) ta |= m, tb |= m;
+        if (PER_TILE) ta |= m, tb |= m;
         else if (n < NB / 2) ta |= m;
         else tb |= m;
         memb |= ((m >> lane) & 1u) << (bit0 + n);
@@ -420,7 +419,7 @@ __device__ __forceinline__ uint32_t emit_tile_list(const Params& p, int list, in
 #pragma unroll
     for (int n = 0; n < NB; ++n) {
       m[n] = (wi < W) ? bm[n * W + wi] : 0u;
-      if (ONE) ta |= m[n], tb |= m[n];
+      if (PER_TILE) ta |= m[n], tb |= m[n];
       else if (n < NB / 2) ta |= m[n];
       else tb |= m[n];
     }
@@ -463,18 +462,18 @@ __device__ __forceinline__ uint32_t emit_tile_list(const Params& p, int list, in
   return word;
 }
 
-template <int NB, int G, bool ONE>
+template <int NB, int G, bool PER_TILE>
 __global__ void __launch_bounds__(32 * NB) build_tile_lists_kernel(const Params p) {
   extern __shared__ uint32_t bm[];  // [NB][W] bitmaps
   ptx::grid_launch_dependents();
   ptx::grid_dependency_wait();
   const int lane = threadIdx.x & 31, n = threadIdx.x >> 5;
-  const int list = blockIdx.x, unit = ONE ? list >> 1 : list;
+  const int list = blockIdx.x, unit = PER_TILE ? list >> 1 : list;
   if (list == 0 && threadIdx.x < kCounters) p.work_counter[threadIdx.x] = 0;
-  fill_tile_bitmap<NB, ONE>(p, list, n, lane, bm);
+  fill_tile_bitmap<NB, PER_TILE>(p, list, n, lane, bm);
   __syncthreads();
   if (n != 0) return;
-  emit_tile_list<NB, G, ONE>(p, list, lane, bm, nullptr);
+  emit_tile_list<NB, G, PER_TILE>(p, list, lane, bm, nullptr);
   if (lane == 0) p.redo_flag[unit] = 0;
 }
 

@@ -551,12 +551,12 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   constexpr int kListAt = 512;
   static_assert(2 * kQB * ((256 / C_ * (kMaxPersistentCtas / 2) + 31) / 32) <= kListAt, "room for the bitmaps");
   static_assert(sizeof(TileControl::xch) >= 4 * (kListAt + 256 / C_ * (kMaxPersistentCtas / 2) + 48), "room for a list");
-  constexpr bool kOne = tile_lists_per_unit(D) == 2;
-  constexpr int kListBlocks = (kOne ? 1 : 2) * kQB;  // query blocks of a list
+  constexpr bool kPerTile = tile_lists_per_unit(D) == 2;
+  constexpr int kListBlocks = (kPerTile ? 1 : 2) * kQB;  // query blocks of a list
   if (MODE == kSparse && ONE) {
     // ... or the tile list of this CTA's unit from here: the bitmaps of its query blocks, in a place not in use yet
     if (rank == 0 && warp < kListBlocks)
-      fill_tile_bitmap<kListBlocks, kOne>(p, first_list(), warp, lane, reinterpret_cast<uint32_t*>(&ctl->xch[0][0][0]));
+      fill_tile_bitmap<kListBlocks, kPerTile>(p, first_list(), warp, lane, reinterpret_cast<uint32_t*>(&ctl->xch[0][0][0]));
     __syncthreads();
   }
 
@@ -862,7 +862,7 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       if (in_cluster && blockIdx.x == 0 && lane == 0) *p.redo_count = -1;
       if (MODE == kSparse && ONE) {
         uint32_t* const bm = reinterpret_cast<uint32_t*>(&ctl->xch[0][0][0]);
-        own_word = emit_tile_list<kListBlocks, kG, kOne>(p, first_list(), lane, bm, bm + kListAt);
+        own_word = emit_tile_list<kListBlocks, kG, kPerTile>(p, first_list(), lane, bm, bm + kListAt);
         __syncwarp();
       }
       // A unit's tile list, in chunks of 32 entries, to both CTAs; `own`: made by this CTA, in shared memory.  False: gave up.
