@@ -203,7 +203,7 @@ int losa_select(int32_t B, int32_t H, int32_t nQb, int32_t nKb, const float* mas
   const DeviceState* dev = device_state(&rc);
   if (!dev) return rc;
   return launch_select((int)rows, nKb, mass, tau, 0, offsets, kv_idx, kv_capacity, ws,
-                       dev->status_dev, static_cast<cudaStream_t>(cuda_stream));
+                       dev->status_dev, dev->ordinal, static_cast<cudaStream_t>(cuda_stream));
 }
 
 int losa_select_topk(int32_t B, int32_t H, int32_t nQb, int32_t nKb, const float* mass, int32_t k,
@@ -221,7 +221,7 @@ int losa_select_topk(int32_t B, int32_t H, int32_t nQb, int32_t nKb, const float
   const DeviceState* dev = device_state(&rc);
   if (!dev) return rc;
   return launch_select((int)rows, nKb, mass, 0.5, k, offsets, kv_idx, kv_capacity, ws,
-                       dev->status_dev, static_cast<cudaStream_t>(cuda_stream));
+                       dev->status_dev, dev->ordinal, static_cast<cudaStream_t>(cuda_stream));
 }
 
 int losa_row_recall(int32_t rows, int32_t nKb, const float* mass, const int32_t* offsets,

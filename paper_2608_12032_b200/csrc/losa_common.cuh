@@ -100,8 +100,8 @@ size_t select_workspace_bytes(int64_t rows, int nKb);
 int select_launches(int64_t rows, int nKb, bool fixed);  // kernels that such a call launches
 int launch_select(int rows, int nKb, const float* mass, double tau, int fixed_count,
                   int32_t* offsets, int32_t* kv_idx, int64_t kv_capacity, void* ws, int* status,
-                  cudaStream_t st);  // fixed_count > 0: keep that many blocks per row instead;
-                                     // status: device-visible word that receives device-side errors
+                  int dev, cudaStream_t st);  // fixed_count > 0: keep that many blocks per row instead;
+                                              // status: device-visible word that receives device-side errors
 int launch_row_recall(int rows, int nKb, const float* mass, const int32_t* offsets,
                       const int32_t* kv_idx, double* retained, double* total, cudaStream_t st);
 size_t select_noalloc_workspace_limit();

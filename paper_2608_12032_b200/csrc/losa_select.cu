@@ -801,11 +801,9 @@ int select_launches(int64_t rows, int nKb, bool fixed) { return small_selection(
 
 template <int K, bool COUNT>
 static int launch_small(int ctas, const float* mass, int rows, int nKb, double tau, int fixed_count, int32_t* offsets,
-                        int32_t* kv_idx, int64_t kv_capacity, int* status, cudaStream_t st) {
+                        int32_t* kv_idx, int64_t kv_capacity, int* status, int dev, cudaStream_t st) {
   auto kern = select_small_kernel<K, COUNT>;
   static std::atomic<int> ready[kMaxDevices];
-  int dev = 0;
-  LOSA_CUDA_TRY(cudaGetDevice(&dev));
   if (!ready[dev].load(std::memory_order_acquire)) {
     LOSA_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SmallShared)));
     ready[dev].store(1, std::memory_order_release);
@@ -829,7 +827,7 @@ static int launch_small(int ctas, const float* mass, int rows, int nKb, double t
 }
 
 int launch_select(int rows, int nKb, const float* mass, double tau, int fixed_count,
-                  int32_t* offsets, int32_t* kv_idx, int64_t kv_capacity, void* ws, int* status,
+                  int32_t* offsets, int32_t* kv_idx, int64_t kv_capacity, void* ws, int* status, int dev,
                   cudaStream_t st) {
   int32_t* counts = static_cast<int32_t*>(ws);
   uint32_t* bitmaps = reinterpret_cast<uint32_t*>(static_cast<char*>(ws) +
@@ -837,8 +835,8 @@ int launch_select(int rows, int nKb, const float* mass, double tau, int fixed_co
   if (small_selection(rows, nKb, fixed_count > 0)) {
     const int ctas = min(kSmallCtas, rows);
 #define LOSA_SELECT_SMALL(k)                                                                                  \
-  (fixed_count > 0 ? launch_small<k, true>(ctas, mass, rows, nKb, tau, fixed_count, offsets, kv_idx, kv_capacity, status, st) \
-                   : launch_small<k, false>(ctas, mass, rows, nKb, tau, 0, offsets, kv_idx, kv_capacity, status, st))
+  (fixed_count > 0 ? launch_small<k, true>(ctas, mass, rows, nKb, tau, fixed_count, offsets, kv_idx, kv_capacity, status, dev, st) \
+                   : launch_small<k, false>(ctas, mass, rows, nKb, tau, 0, offsets, kv_idx, kv_capacity, status, dev, st))
     return nKb <= 256 ? LOSA_SELECT_SMALL(8) : nKb <= 512 ? LOSA_SELECT_SMALL(16) : LOSA_SELECT_SMALL(32);
 #undef LOSA_SELECT_SMALL
   }
@@ -904,7 +902,7 @@ int launch_select_noalloc(int rows, int nKb, const float* mass, double tau, int3
   // and bitmaps are fully rewritten by the first kernel before anything reads them
   LOSA_CUDA_TRY(cudaMemsetAsync(status, 0, sizeof(int), st));
   // the same kernels, dispatch and workspace layout as losa_select
-  const int rc = launch_select(rows, nKb, mass, tau, 0, offsets, kv_idx, kv_capacity, ws, status, st);
+  const int rc = launch_select(rows, nKb, mass, tau, 0, offsets, kv_idx, kv_capacity, ws, status, dev, st);
   if (rc != LOSA_OK) return rc;
   if (device_status)
     LOSA_CUDA_TRY(cudaMemcpyAsync(device_status, status, sizeof(int), cudaMemcpyDeviceToDevice, st));
