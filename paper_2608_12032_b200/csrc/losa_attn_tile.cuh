@@ -345,7 +345,7 @@ losa_tile_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   // the loop changes (masses, 16384 tokens, 12 heads, us: at the start / at the end, and with the second four instead of the
   // first: D = 64, C = 32 908 / 917, 920 / 929, C = 64 826 / 854, 886 / 826, C = 128 851 / 843, 818 / 843; D = 128, C = 32
   // 1059 / 992, 1023 / 1054, C = 64 963 / 948, 965 / 945, C = 128 946 / 961, 918 / 956).
-  constexpr bool kInfoEarly = MODE == kMass && (C_ == 128 || (D == 64 && C_ == 64));
+  constexpr bool kInfoEarly = MODE == kMass && (D == 64 || C_ == 128);
   constexpr int kPolyAt = (MODE == kMass && C_ == 128) ? 1 : 0;
   constexpr int kChunkTiles = (MODE == kSparse) ? 32 / kG : (1 << 28);  // K/V tiles per chunk of the list
   static_assert(offsetof(TileControl, tl) % 16 == 0, "the tile list is read with 16-byte loads");
