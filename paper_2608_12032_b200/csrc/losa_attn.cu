@@ -695,7 +695,8 @@ int plan_waves(int items, int nKb, const DeviceState& dev, Waves* waves) {
       int n = 0;
       cudaLaunchConfig_t cfg;
       cudaLaunchAttribute attr[2];
-      if ((rc = configure_tile<D, R, C_, MODE, kPair, true>(dev, kTileCtas * parts, &n, &cfg, attr)) == LOSA_ERR_CUDA) return rc;
+      rc = configure_tile<D, R, C_, MODE, kPair, true>(dev, kTileCtas * parts, &n, &cfg, attr);
+      if (rc == LOSA_ERR_CUDA) (void)cudaGetLastError();  // (a device that cannot say how many it holds: none)
       if (rc == LOSA_OK && n >= rest * (kPair ? 1 : 2)) {
         w.in_cluster = true;
         w.ctas = kTileCtas * parts;
